@@ -86,19 +86,28 @@ typedef struct {
 /* ---- Operators ---------------------------------------------------------- */
 
 /* Forward operator A (Eq. core:formula):  s[k][t] = sum_ij c[j][i] p_k^T
- * beta K(beta G(x_ij - r_t)) G v_t.  c is [ny][nx], s is [n_ch][T].  The sum
- * over voxels is a direct (exact, untruncated) sum, reduced deterministically:
- * the same inputs give bit-identical outputs.  T == 0 is a no-op. */
+ * beta K(beta G(x_ij - r_t)) G v_t.  c is [ny][nx], s is [n_ch][T].  FP64 and
+ * small FP32 problems are summed pair by pair; large FP32 problems are
+ * evaluated as convolutions on a grid with interpolation at the samples, to
+ * the same accuracy (nothing is truncated: errors are FP32 rounding, about
+ * 5e-8 in relative L2).  The route depends on sizes, model and alignment (r
+ * and v on 8 bytes) only.  Deterministic: the same inputs give bit-identical
+ * outputs.  T == 0 is a no-op. */
 int mpi_forward(const mpi_model *model, const mpi_grid_desc *grid,
                 const mpi_traj *traj, mpi_dtype dtype, const void *c, void *s,
                 void *stream);
 
-/* mpi_forward without any device allocation.  The paper has no counterpart:
+/* mpi_forward by the pair-by-pair sums at every size. */
+int mpi_forward_sums(const mpi_model *model, const mpi_grid_desc *grid,
+                     const mpi_traj *traj, mpi_dtype dtype, const void *c, void *s,
+                     void *stream);
+
+/* mpi_forward_sums without any device allocation.  The paper has no counterpart:
  * this entry point exists for callers that cannot let a library allocate
  * device memory while they run (a scan loop with a memory budget fixed at
  * start-up, a framework that owns all device memory through its own pool, code
  * that must avoid the implicit synchronisation of cudaFree).  Same inputs,
- * outputs and results as mpi_forward; its scratch is a fixed 32 MiB array in
+ * outputs and results as mpi_forward_sums; its scratch is a fixed 32 MiB array in
  * device global memory that every GPU loading the library keeps until the
  * process exits.  Problems whose scratch does not fit are rejected with
  * MPI_ERR_UNSUPPORTED before anything is enqueued: the limit is about

@@ -117,6 +117,7 @@ _lock = threading.Lock()
 
 _SIGS = {
     "mpi_forward": [ctypes.c_void_p] * 3 + [ctypes.c_int] + [ctypes.c_void_p] * 3,
+    "mpi_forward_sums": [ctypes.c_void_p] * 3 + [ctypes.c_int] + [ctypes.c_void_p] * 3,
     "mpi_forward_noalloc": [ctypes.c_void_p] * 3 + [ctypes.c_int] + [ctypes.c_void_p] * 3,
     "mpi_adjoint": [ctypes.c_void_p] * 3 + [ctypes.c_int] + [ctypes.c_void_p] * 3,
     "mpi_dbeta": [ctypes.c_void_p] * 3 + [ctypes.c_int] + [ctypes.c_void_p] * 4,
@@ -312,8 +313,22 @@ def mpi_forward(model, grid, r, v, c, s=None, stream=None):
     return s
 
 
+def mpi_forward_sums(model, grid, r, v, c, s=None, stream=None):
+    """mpi_forward by the pair-by-pair sums at every size."""
+    dt = c.dtype
+    n_ch = len(_get(model, "p"))
+    if s is None:
+        s = torch.empty((n_ch, r.shape[0]), dtype=dt, device=c.device)
+    tr = _traj(r, v, dt)
+    m, g = make_model(model), make_grid(grid)
+    _check(load().mpi_forward_sums(ctypes.byref(m), ctypes.byref(g), ctypes.byref(tr), _dtype(c),
+                                   _dev(c, dt, "c"), _dev(s, dt, "s") if s.numel() else None,
+                                   _stream(stream)))
+    return s
+
+
 def mpi_forward_noalloc(model, grid, r, v, c, s=None, stream=None):
-    """Like mpi_forward, for callers that cannot let the library allocate
+    """Like mpi_forward_sums, for callers that cannot let the library allocate
     device memory while they run: the library's scratch is a fixed 32 MiB
     device array (see include/mpi_recon.h for the size limit and the rule
     that overlapping calls race).  ``s`` should be preallocated by such a

@@ -29,7 +29,9 @@ class MPIForward(torch.autograd.Function):
     def forward(ctx, c, beta, model, grid, r, v):
         m = _model_with_beta(model, beta.item() if isinstance(beta, torch.Tensor) else beta)
         c_ = c.detach().contiguous()
-        s = api.mpi_forward(m, grid, r, v, c_)
+        # the same pair sums that mpi_dbeta differentiates: dL/dbeta is an FP64
+        # value of small residuals s - data, and follows every rounding of s
+        s = api.mpi_forward_sums(m, grid, r, v, c_)
         ctx.save_for_backward(c_)
         ctx.m, ctx.grid, ctx.r, ctx.v = m, grid, r, v
         ctx.beta_is_tensor = isinstance(beta, torch.Tensor)

@@ -7,6 +7,7 @@
 #include <mutex>
 #include <vector>
 
+#include "field_ops.cuh"
 #include "graph.cuh"
 #include "pair_ops.cuh"
 
@@ -227,12 +228,39 @@ GridH to_host(const mpi_grid_desc *g) { return GridH{g->nx, g->ny, g->x0, g->y0,
 
 // ---------------------------------------------------------------------------
 
+// Scratch of a gridded operator call: true once the plan's buffers point into
+// `scr`.  False (the direct sums then run) when the problem is not one for
+// that route, the trajectory is not 8-byte aligned or the scratch is not to
+// be had.
+static bool take_field(const ModelH &m, const GridH &g, const mpi_traj *tr, bool forward, bool adjoint, FieldPlan &plan,
+                       Scratch &scr)
+{
+    if (((uintptr_t)tr->r | (uintptr_t)tr->v) & 7) return false;
+    if (!field_worth(g, tr->T) || field_plan(m, g, tr->T, forward, adjoint, plan) != MPI_OK) return false;
+    if (!field_route(plan, adjoint)) return false;
+    const size_t o = scr.reserve(plan.bytes);
+    if (scr.allocate() != MPI_OK) {
+        (void)cudaGetLastError();
+        return false;
+    }
+    field_carve(plan, scr.at<char>(o));
+    return true;
+}
+
 template <typename R>
 static int forward_impl(const ModelH &m, const GridH &g, const mpi_traj *tr, const void *c, void *s,
-                        cudaStream_t st)
+                        bool sums, cudaStream_t st)
 {
     const int64_t T = tr->T;
     if (T == 0) return MPI_OK;
+    if constexpr (sizeof(R) == 4) {
+        FieldPlan plan;
+        Scratch fscr(st);
+        if (!sums && take_field(m, g, tr, true, false, plan, fscr)) {
+            return field_forward(plan, static_cast<const float *>(c), static_cast<const float *>(tr->r),
+                                 static_cast<const float *>(tr->v), static_cast<float *>(s), st);
+        }
+    }
     FwdSplit sp = forward_split(T, g.nx, g.ny, sizeof(R), forward_target_items());
     Scratch scr(st);
     const size_t o_geo = scr.reserve(geometry_bytes<R>(T, g.nx, g.ny));
@@ -251,6 +279,16 @@ static int adjoint_impl(const ModelH &m, const GridH &g, const mpi_traj *tr, con
                         cudaStream_t st)
 {
     const int64_t T = tr->T;
+    if constexpr (sizeof(R) == 4) {
+        FieldPlan plan;
+        Scratch fscr(st);
+        if (T > 0 && take_field(m, g, tr, false, true, plan, fscr)) {
+            const float *r = static_cast<const float *>(tr->r), *v = static_cast<const float *>(tr->v);
+            MPI_TRY(field_prepare(plan, nullptr, r, v, st));
+            MPI_TRY(field_order(plan, r, v, static_cast<const float *>(s), st));
+            return field_adjoint<float>(plan, static_cast<float *>(c), nullptr, nullptr, nullptr, st);
+        }
+    }
     AdjSplit sp = adjoint_split(T, g.nx, g.ny, default_target_items(), sizeof(R));
     Scratch scr(st);
     const size_t o_geo = scr.reserve(geometry_bytes<R>(T, g.nx, g.ny));
@@ -288,8 +326,8 @@ using namespace mpi;
 
 extern "C" {
 
-int mpi_forward(const mpi_model *model, const mpi_grid_desc *grid, const mpi_traj *traj,
-                mpi_dtype dtype, const void *c, void *s, void *stream)
+static int forward_call(const mpi_model *model, const mpi_grid_desc *grid, const mpi_traj *traj,
+                        mpi_dtype dtype, const void *c, void *s, bool sums, void *stream)
 {
     MPI_TRY(check_model(model));
     MPI_TRY(check_grid(grid));
@@ -298,8 +336,20 @@ int mpi_forward(const mpi_model *model, const mpi_grid_desc *grid, const mpi_tra
     if (traj->T > 0 && (!c || !s)) { set_error("c or s is NULL"); return MPI_ERR_INVALID; }
     const ModelH m = to_host(model);
     const GridH g = to_host(grid);
-    return dtype == MPI_F32 ? forward_impl<float>(m, g, traj, c, s, as_stream(stream))
-                            : forward_impl<double>(m, g, traj, c, s, as_stream(stream));
+    return dtype == MPI_F32 ? forward_impl<float>(m, g, traj, c, s, sums, as_stream(stream))
+                            : forward_impl<double>(m, g, traj, c, s, sums, as_stream(stream));
+}
+
+int mpi_forward(const mpi_model *model, const mpi_grid_desc *grid, const mpi_traj *traj,
+                mpi_dtype dtype, const void *c, void *s, void *stream)
+{
+    return forward_call(model, grid, traj, dtype, c, s, false, stream);
+}
+
+int mpi_forward_sums(const mpi_model *model, const mpi_grid_desc *grid, const mpi_traj *traj,
+                     mpi_dtype dtype, const void *c, void *s, void *stream)
+{
+    return forward_call(model, grid, traj, dtype, c, s, true, stream);
 }
 
 int mpi_adjoint(const mpi_model *model, const mpi_grid_desc *grid, const mpi_traj *traj,
