@@ -90,9 +90,9 @@ typedef struct {
  * small FP32 problems are summed pair by pair; large FP32 problems are
  * evaluated as convolutions on a grid with interpolation at the samples, to
  * the same accuracy (nothing is truncated: errors are FP32 rounding, about
- * 5e-8 in relative L2).  The route depends on sizes, model and alignment (r
- * and v on 8 bytes) only.  Deterministic: the same inputs give bit-identical
- * outputs.  T == 0 is a no-op. */
+ * 5e-8 in relative L2).  The route depends on sizes and model only.
+ * Deterministic: the same inputs give bit-identical outputs.  T == 0 is a
+ * no-op. */
 int mpi_forward(const mpi_model *model, const mpi_grid_desc *grid,
                 const mpi_traj *traj, mpi_dtype dtype, const void *c, void *s,
                 void *stream);
@@ -430,8 +430,9 @@ int mpi_grid3(const mpi_grid3_desc *grid, const mpi_traj *traj, mpi_dtype dtype,
 /* A plan runs Algorithm 1 with the forward operator (FP32 operator, FP64 CG
  * vectors, inner products and PnP scalars, built-in Gaussian denoiser) for up
  * to MPI_BATCH_MAX_FRAMES independent frames of different grid sizes and
- * trajectory lengths at once: every operator application over all frames is
- * one launch of the pair kernel over a frame table, the CG, percentile and
+ * trajectory lengths at once: large frames apply the gridded operators one by
+ * one, over all others every operator application is one launch of the pair
+ * kernel over a frame table, the CG, percentile and
  * denoiser steps are batched the same way, and one PnP iteration of all frames
  * is captured once as a CUDA graph and replayed n_iter times.  Each frame
  * has its own model, grid, T and nu0 (host arrays of n_frames entries); opts
@@ -441,7 +442,7 @@ int mpi_grid3(const mpi_grid3_desc *grid, const mpi_traj *traj, mpi_dtype dtype,
  * launch forms (one block per item, or a persistent grid pulling items from a
  * device counter) on the first run, which then synchronises the stream once;
  * the choice is cached in the file named by $MPI_AUTOTUNE_CACHE when set.
- * MPI_BATCH_MATCH_SINGLE splits every frame exactly as mpi_pnp_solve does,
+ * MPI_BATCH_MATCH_SINGLE routes and splits every frame exactly as mpi_pnp_solve does,
  * so each frame's result is bit-identical to its single-frame solve. */
 #define MPI_BATCH_MAX_FRAMES 64
 #define MPI_BATCH_AUTOTUNE 1

@@ -230,20 +230,18 @@ GridH to_host(const mpi_grid_desc *g) { return GridH{g->nx, g->ny, g->x0, g->y0,
 
 // Scratch of a gridded operator call: true once the plan's buffers point into
 // `scr`.  False (the direct sums then run) when the problem is not one for
-// that route, the trajectory is not 8-byte aligned or the scratch is not to
-// be had.
+// that route or the scratch is not to be had.
 static bool take_field(const ModelH &m, const GridH &g, const mpi_traj *tr, bool forward, bool adjoint, FieldPlan &plan,
                        Scratch &scr)
 {
-    if (((uintptr_t)tr->r | (uintptr_t)tr->v) & 7) return false;
     if (!field_worth(g, tr->T) || field_plan(m, g, tr->T, forward, adjoint, plan) != MPI_OK) return false;
-    if (!field_route(plan, adjoint)) return false;
-    const size_t o = scr.reserve(plan.bytes);
+    if (!field_route(plan)) return false;
+    const size_t o_keep = scr.reserve(plan.keep_bytes), o_work = scr.reserve(plan.work_bytes);
     if (scr.allocate() != MPI_OK) {
         (void)cudaGetLastError();
         return false;
     }
-    field_carve(plan, scr.at<char>(o));
+    field_carve(plan, scr.at<char>(o_keep), scr.at<char>(o_work));
     return true;
 }
 

@@ -2,8 +2,9 @@
 // independent frames of uneven grid size and trajectory length, FP32
 // operator with FP64 CG vectors and inner products.
 //
-// Every operator application over all frames is ONE launch of the pair
-// kernel over a frame table (the work items of all frames in one grid, or one
+// Frames whose gridded operators (field_ops.cu) cost less than their share of
+// the pair sums run those, frame by frame; over all other frames every
+// operator application is ONE launch of the pair kernel over a frame table (the work items of all frames in one grid, or one
 // persistent grid pulling items from a device counter), followed by one
 // batched chunk reduction.  The CG vector kernels, the percentile/variance
 // step and the Gaussian denoiser are batched the same way (a block belongs to
@@ -22,6 +23,7 @@
 #include <string>
 #include <vector>
 
+#include "field_ops.cuh"
 #include "pair_kernels.cuh"
 #include "pnp_device.cuh"
 
@@ -299,6 +301,10 @@ struct mpi_batch_plan {
     float *rho1 = nullptr, *rho2 = nullptr;
     unsigned long long *queues = nullptr;  // [forward 2][adjoint 2]
     std::vector<int> nvblk, npq;
+    // Frames on the gridded operators: launched frame by frame, so they share
+    // one work area; no pair items.
+    std::vector<char> gridded;
+    std::vector<FieldPlan> fld;
     // chosen configuration
     bool tuned = false;
     int64_t fwd_budget = kDefaultBudget, adj_budget = kDefaultBudget;
@@ -341,6 +347,9 @@ static void configure(mpi_batch_plan &P, int64_t fb, int64_t ab, bool fpers, boo
     P.as.resize(P.n);
     const bool single = (P.flags & MPI_BATCH_MATCH_SINGLE) != 0;
     for (int f = 0; f < P.n; ++f) {
+        P.fs[f] = FwdSplit{0, 0, 0, 1};
+        P.as[f] = AdjSplit{0, 0, 0, kAdjBlock};
+        if (P.gridded[f]) continue;
         P.fs[f] = single ? forward_split(P.T[f], P.g[f].nx, P.g[f].ny, 4, forward_target_items())
                          : fwd_split_budget(P.T[f], P.g[f].nx, P.g[f].ny, fb);
         P.as[f] = single ? adjoint_split(P.T[f], P.g[f].nx, P.g[f].ny, default_target_items(), 4)
@@ -373,7 +382,7 @@ static void configure(mpi_batch_plan &P, int64_t fb, int64_t ab, bool fpers, boo
         P.fwd_tab[1].f[f] = fw;
         P.fwd_tab[1].f[f].in = P.p + P.voff[f];
         fi += frame_items_fwd(P.fs[f]);
-        smem = std::max(smem, fwd_smem_bytes(P.g[f].nx, P.fs[f].rows_staged, sizeof(float)));
+        if (!P.gridded[f]) smem = std::max(smem, fwd_smem_bytes(P.g[f].nx, P.fs[f].rows_staged, sizeof(float)));
         PairFrame<float> ad = base;
         ad.item0 = ai;
         ad.in = P.sA[f];
@@ -395,7 +404,7 @@ static void configure(mpi_batch_plan &P, int64_t fb, int64_t ab, bool fpers, boo
         R = RedFrame{};
         R.part = P.fwd_part[f];
         R.out = P.sA[f];
-        R.len = (int64_t)P.m[f].n_ch * P.T[f];
+        R.len = P.gridded[f] ? 0 : (int64_t)P.m[f].n_ch * P.T[f];
         R.n_chunks = P.fs[f].n_chunks;
         R.blk0 = b;
         b += (R.len + 31) / 32;
@@ -411,7 +420,7 @@ static void configure(mpi_batch_plan &P, int64_t fb, int64_t ab, bool fpers, boo
             R.p = (t == 0 ? P.x : P.p) + P.voff[f];
             R.nu = P.scal[f] + kScalNu;
             R.dot = P.pq[f];
-            R.len = P.N[f];
+            R.len = P.gridded[f] ? 0 : P.N[f];
             R.n_chunks = P.as[f].n_chunks;
             R.blk0 = bb;
             bb += (R.len + 31) / 32;
@@ -476,6 +485,7 @@ static int prepare_launch(mpi_batch_plan &P)
 
 static int launch_fwd(mpi_batch_plan &P, int which, cudaStream_t st)
 {
+    if (P.fwd_items == 0) return MPI_OK;
     const PairTab &B = P.fwd_tab[which];
     {
         ProfScope prof(kProfForward, st);
@@ -495,6 +505,7 @@ static int launch_fwd(mpi_batch_plan &P, int which, cudaStream_t st)
 
 static int launch_adj_kernel(mpi_batch_plan &P, const PairTab &B, cudaStream_t st)
 {
+    if (P.adj_items == 0) return MPI_OK;
     ProfScope prof(kProfAdjoint, st);
     if (P.adj_persist) {
         auto k = adj_kernel_persistent(P);
@@ -512,8 +523,16 @@ static int apply_normal_b(mpi_batch_plan &P, int which, cudaStream_t st)
 {
     MPI_TRY(launch_fwd(P, which, st));
     MPI_TRY(launch_adj_kernel(P, P.adj_tab, st));
-    k_reduce_batch<double, true><<<(unsigned)red_blocks(P.red_adj[which]), 256, 0, st>>>(P.red_adj[which]);
-    MPI_CHECK_LAUNCH();
+    if (P.adj_items > 0) {
+        k_reduce_batch<double, true><<<(unsigned)red_blocks(P.red_adj[which]), 256, 0, st>>>(P.red_adj[which]);
+        MPI_CHECK_LAUNCH();
+    }
+    for (int f = 0; f < P.n; ++f) {
+        if (!P.gridded[f]) continue;
+        const double *v = (which == 0 ? P.x : P.p) + P.voff[f];
+        MPI_TRY(field_forward_ordered<double>(P.fld[f], v, st));
+        MPI_TRY(field_adjoint<double>(P.fld[f], P.q + P.voff[f], v, P.scal[f] + kScalNu, P.pq[f], st));
+    }
     return MPI_OK;
 }
 
@@ -552,7 +571,8 @@ static std::string tune_key(const mpi_batch_plan &P)
     cudaGetDeviceProperties(&prop, dev);
     std::ostringstream os;
     os << prop.name << "|sm" << prop.multiProcessorCount << "|f32|" << (P.mixed ? "m" : P.diag ? "d" : "g");
-    for (int f = 0; f < P.n; ++f) os << "|" << P.g[f].nx << "x" << P.g[f].ny << "x" << P.T[f] << "c" << P.m[f].n_ch;
+    for (int f = 0; f < P.n; ++f)
+        if (!P.gridded[f]) os << "|" << P.g[f].nx << "x" << P.g[f].ny << "x" << P.T[f] << "c" << P.m[f].n_ch;
     const size_t h = std::hash<std::string>{}(os.str());
     char buf[32];
     snprintf(buf, sizeof(buf), "%016zx", h);
@@ -590,6 +610,10 @@ static void cache_store(const std::string &key, int64_t fb, int fp, int64_t ab, 
 // work items, not what is summed.
 static int autotune(mpi_batch_plan &P, cudaStream_t st)
 {
+    if (P.fwd_items == 0) {  // every frame gridded: nothing to choose
+        P.tuned = true;
+        return MPI_OK;
+    }
     const std::string key = tune_key(P);
     int64_t fb, ab;
     int fp, ap;
@@ -734,21 +758,28 @@ int mpi_batch_plan_create(int n_frames, const mpi_model *models, const mpi_grid_
     }
     // Device memory: sized for the smallest work-item budget (most chunks).
     const int64_t bmin = kBudgets[0];
-    std::vector<size_t> o_geo, o_fp, o_ap, o_sA, o_pq, o_rr0, o_rr1, o_sc;
-    size_t tot = 0;
+    std::vector<size_t> o_geo, o_fp, o_ap, o_sA, o_pq, o_rr0, o_rr1, o_sc, o_keep;
+    size_t tot = 0, field_work = 0;
     auto take = [&](size_t b) { size_t o = tot; tot += (b + 255) & ~size_t(255); return o; };
     for (int f = 0; f < n_frames; ++f) {
         const FwdSplit fs_min = fwd_split_budget(P->T[f], P->g[f].nx, P->g[f].ny, bmin);
         const FwdSplit fs_single = forward_split(P->T[f], P->g[f].nx, P->g[f].ny, 4, forward_target_items());
         const AdjSplit as_min = adj_split_budget(P->T[f], P->g[f].nx, P->g[f].ny, bmin);
         const AdjSplit as_single = adjoint_split(P->T[f], P->g[f].nx, P->g[f].ny, default_target_items(), 4);
-        const int fch = std::max(fs_min.n_chunks, fs_single.n_chunks);
-        const int ach = std::max(as_min.n_chunks, as_single.n_chunks);
-        o_geo.push_back(take(geometry_bytes<float>(P->T[f], P->g[f].nx, P->g[f].ny)));
+        FieldPlan fp;
+        const bool gr = field_solve_plan(P->m[f], P->g[f], P->T[f], P->n_iter, P->n_cg,
+                                         !(flags & MPI_BATCH_MATCH_SINGLE), fp);
+        P->gridded.push_back(gr ? 1 : 0);
+        P->fld.push_back(fp);
+        o_keep.push_back(gr ? take(fp.keep_bytes) : 0);
+        if (gr) field_work = std::max(field_work, fp.work_bytes);
+        const int fch = gr ? 0 : std::max(fs_min.n_chunks, fs_single.n_chunks);
+        const int ach = gr ? 0 : std::max(as_min.n_chunks, as_single.n_chunks);
+        o_geo.push_back(take(gr ? 0 : geometry_bytes<float>(P->T[f], P->g[f].nx, P->g[f].ny)));
         o_fp.push_back(take(sizeof(float) * size_t(fch) * P->m[f].n_ch * P->T[f]));
         o_ap.push_back(take(sizeof(float) * size_t(ach) * P->N[f]));
-        o_sA.push_back(take(sizeof(float) * P->m[f].n_ch * P->T[f]));
-        P->npq.push_back((int)((P->N[f] + 31) / 32));
+        o_sA.push_back(take(gr ? 0 : sizeof(float) * P->m[f].n_ch * P->T[f]));
+        P->npq.push_back(gr ? field_dot_blocks(P->g[f].ny) : (int)((P->N[f] + 31) / 32));
         P->nvblk.push_back(vec_blocks(P->N[f]));
         o_pq.push_back(take(sizeof(double) * P->npq.back()));
         o_rr0.push_back(take(sizeof(double) * P->nvblk.back()));
@@ -759,6 +790,7 @@ int mpi_batch_plan_create(int n_frames, const mpi_model *models, const mpi_grid_
     const size_t o_b0 = take(vb), o_x = take(vb), o_r = take(vb), o_p = take(vb), o_q = take(vb);
     const size_t o_r1 = take(sizeof(float) * P->Ntot), o_r2 = take(sizeof(float) * P->Ntot);
     const size_t o_qu = take(sizeof(unsigned long long) * 4);
+    const size_t o_work = take(field_work);
     if (const char *fl = getenv("MPI_FAULT")) {
         if (strcmp(fl, "alloc") == 0) {
             set_error("plan allocation of %zu bytes failed (injected by MPI_FAULT=alloc)", tot);
@@ -785,6 +817,7 @@ int mpi_batch_plan_create(int n_frames, const mpi_model *models, const mpi_grid_
         P->rr1.push_back(reinterpret_cast<double *>(d + o_rr1[f]));
         P->scal.push_back(reinterpret_cast<double *>(d + o_sc[f]));
         P->done.push_back(reinterpret_cast<int *>(d + o_sc[f] + sizeof(double) * 8));
+        if (P->gridded[f]) field_carve(P->fld[f], d + o_keep[f], d + o_work);
     }
     P->b0 = reinterpret_cast<double *>(d + o_b0);
     P->x = reinterpret_cast<double *>(d + o_x);
@@ -852,7 +885,9 @@ int mpi_batch_pnp_run(mpi_batch_plan *P, const void *const *r, const void *const
             return MPI_ERR_INVALID;
         }
     const cudaStream_t st = as_stream(stream);
-    for (int f = 0; f < P->n; ++f) MPI_TRY(prepare_geometry<float>(P->m[f], P->g[f], P->T[f], r[f], v[f], P->geo[f], st));
+    for (int f = 0; f < P->n; ++f)
+        if (!P->gridded[f])
+            MPI_TRY(prepare_geometry<float>(P->m[f], P->g[f], P->T[f], r[f], v[f], P->geo[f], st));
     if (!P->tuned) {
         MPI_TRY(autotune(*P, st));
         if (P->exec) {  // the split changed: recapture
@@ -868,8 +903,17 @@ int mpi_batch_pnp_run(mpi_batch_plan *P, const void *const *r, const void *const
     MPI_TRY(launch_adj_kernel(*P, Bs, st));
     RedTab Rb = P->red_adj[0];
     for (int f = 0; f < P->n; ++f) Rb.f[f].out = P->b0 + P->voff[f];
-    k_reduce_batch<double, false><<<(unsigned)red_blocks(Rb), 256, 0, st>>>(Rb);
-    MPI_CHECK_LAUNCH();
+    if (P->adj_items > 0) {
+        k_reduce_batch<double, false><<<(unsigned)red_blocks(Rb), 256, 0, st>>>(Rb);
+        MPI_CHECK_LAUNCH();
+    }
+    for (int f = 0; f < P->n; ++f) {
+        if (!P->gridded[f]) continue;
+        const float *rf = static_cast<const float *>(r[f]), *vf = static_cast<const float *>(v[f]);
+        MPI_TRY(field_prepare(P->fld[f], nullptr, rf, vf, st));
+        MPI_TRY(field_order(P->fld[f], rf, vf, static_cast<const float *>(s[f]), st));
+        MPI_TRY(field_adjoint<double>(P->fld[f], P->b0 + P->voff[f], nullptr, nullptr, nullptr, st));
+    }
     MPI_TRY_CUDA(cudaMemsetAsync(P->rho2, 0, sizeof(float) * P->Ntot, st));
     k_init_b<<<(P->n + 63) / 64, 64, 0, st>>>(P->stat);
     MPI_CHECK_LAUNCH();

@@ -148,8 +148,10 @@ __device__ __forceinline__ df row_times(const float (&B0)[2], const float (&B1)[
     return df_add(u, w);
 }
 
-__device__ __forceinline__ SampleRec make_sample(const FieldDev &d, float2 r, float2 v)
+__device__ __forceinline__ SampleRec make_sample(const FieldDev &d, const float *__restrict__ rp, const float *__restrict__ vp,
+                                                 int64_t t)
 {
+    const float2 r = make_float2(rp[2 * t], rp[2 * t + 1]), v = make_float2(vp[2 * t], vp[2 * t + 1]);
     SampleRec q;
     const bool bx = node_coord(d.x, r.x, q.ix, q.fx);
     const bool by = node_coord(d.y, r.y, q.iy, q.fy);
@@ -223,7 +225,7 @@ __device__ __forceinline__ int sample_tile(const FieldDev &d, const SampleRec &q
 
 // Tile of every sample of run `run` and the run's tile counts, by one warp;
 // cnt: tx ty + 1 ints of shared memory.
-__device__ void bin_run(const FieldDev &d, int run, int *cnt, const float2 *__restrict__ r, const float2 *__restrict__ v)
+__device__ void bin_run(const FieldDev &d, int run, int *cnt, const float *__restrict__ r, const float *__restrict__ v)
 {
     const int nt = d.tx * d.ty + 1, lane = threadIdx.x & 31;
     for (int k = lane; k < nt; k += 32) cnt[k] = 0;
@@ -234,7 +236,7 @@ __device__ void bin_run(const FieldDev &d, int run, int *cnt, const float2 *__re
         const int64_t t = t0 + u + lane;
         int k = -1;
         if (t < d.T) {
-            k = sample_tile(d, make_sample(d, r[t], v[t]));
+            k = sample_tile(d, make_sample(d, r, v, t));
             d.b.key[t] = k;
         }
         const unsigned peers = __match_any_sync(0xffffffffu, k);
@@ -335,8 +337,8 @@ __device__ __forceinline__ float4 operand(const FieldDev &d, const float *__rest
 
 // Places each run's samples: position = the tile's first + its samples in
 // earlier runs + the rank within the run.
-__global__ void __launch_bounds__(128) k_field_place(const __grid_constant__ FieldDev d, const float2 *__restrict__ r,
-                                                     const float2 *__restrict__ v, const float *__restrict__ s)
+__global__ void __launch_bounds__(128) k_field_place(const __grid_constant__ FieldDev d, const float *__restrict__ r,
+                                                     const float *__restrict__ v, const float *__restrict__ s)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int nt = d.tx * d.ty + 1, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -351,7 +353,7 @@ __global__ void __launch_bounds__(128) k_field_place(const __grid_constant__ Fie
         const bool valid = t < d.T;
         const int k = valid ? d.b.key[t] : -1;
         SampleRec q{};
-        if (valid) q = make_sample(d, r[t], v[t]);
+        if (valid) q = make_sample(d, r, v, t);
         const unsigned peers = __match_any_sync(0xffffffffu, k);
         const int lead = __ffs(peers) - 1;
         int first = 0;
@@ -386,8 +388,8 @@ __global__ void __launch_bounds__(256) k_field_load(const __grid_constant__ Fiel
 
 // Tables (32 entries per block: FP64 functions, spread over the SMs) and, in
 // the blocks behind them, the samples' tiles.
-__global__ void __launch_bounds__(128) k_field_setup(const __grid_constant__ FieldDev d, int n_table, const float2 *__restrict__ r,
-                                                     const float2 *__restrict__ v)
+__global__ void __launch_bounds__(128) k_field_setup(const __grid_constant__ FieldDev d, int n_table, const float *__restrict__ r,
+                                                     const float *__restrict__ v)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     if (int(blockIdx.x) < n_table) {
@@ -806,6 +808,7 @@ __global__ void __launch_bounds__(512) k_field_cols_fwd(const __grid_constant__ 
 __global__ void __launch_bounds__(512) k_field_rows_inv(const __grid_constant__ FieldDev d)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ float4 s_low[3][kFieldLow];  // (re, im) of both rows' lowest modes
     const int P = d.x.P, J = d.x.J, J1 = J + 1;
     V2<float> *a = reinterpret_cast<V2<float> *>(smem_raw);
     V2<float> *b = a + (smem_fft_pad(P - 1) + 1) * 3;
@@ -829,7 +832,11 @@ __global__ void __launch_bounds__(512) k_field_rows_inv(const __grid_constant__ 
         V2<float> *o = a + smem_fft_pad(k) * 3, *n = a + smem_fft_pad(P - k) * 3;
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-            if (k == 0) A[c].y = B[c].y = 0.0f;  // the mean of a real row
+            if (k < kFieldLow) {  // added at the end (the mean of a real row is real)
+                const float f = k ? 2.0f : 1.0f;
+                s_low[c][k] = make_float4(f * A[c].x, k ? f * A[c].y : 0.0f, f * B[c].x, k ? f * B[c].y : 0.0f);
+                A[c] = B[c] = z0;
+            }
             o[c] = V2<float>{A[c].x - B[c].y, A[c].y + B[c].x};
             if (k > 0 && 2 * k < P) n[c] = V2<float>{A[c].x + B[c].y, B[c].x - A[c].y};
         }
@@ -841,10 +848,25 @@ __global__ void __launch_bounds__(512) k_field_rows_inv(const __grid_constant__ 
     for (int i = threadIdx.x; i < d.x.w; i += blockDim.x) {
         int l = l0 + i;
         l -= l >= P ? P : 0;
-        const V2<float> *e = z + smem_fft_pad(l) * 3;
-        const V2<float> q2 = e[2];
-        N[i] = make_float4(e[0].x, e[0].y, q2.x, 0.0f);
-        if (two) N[d.x.w + i] = make_float4(e[1].x, e[1].y, q2.y, 0.0f);
+        V2<float> q[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) q[c] = z[smem_fft_pad(l) * 3 + c];
+        int at = l * (kFieldLow - 1) % P;
+#pragma unroll
+        for (int k = kFieldLow - 1; k >= 0; --k) {  // the mean last: one rounding at full size
+            const float2 w = d.b.twPx[at];          // exp(-2 pi i k l / P)
+            at -= l;
+            at += at < 0 ? P : 0;
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                const float4 s = s_low[c][k];
+                if (k) q[c].x = fmaf(s.y, w.y, q[c].x), q[c].y = fmaf(s.w, w.y, q[c].y);
+                q[c].x = fmaf(s.x, w.x, q[c].x);
+                q[c].y = fmaf(s.z, w.x, q[c].y);
+            }
+        }
+        N[i] = make_float4(q[0].x, q[0].y, q[2].x, 0.0f);
+        if (two) N[d.x.w + i] = make_float4(q[1].x, q[1].y, q[2].y, 0.0f);
     }
 }
 
@@ -886,7 +908,7 @@ __device__ float2 outside_sum(const FieldDev &d, const CIN *__restrict__ cin, fl
 enum { kInterpForward = 0, kInterpOrdered = 1 };
 
 struct InterpArgs {
-    const float2 *r, *v;  // unordered trajectory
+    const float *r, *v;   // unordered trajectory
     float *s;             // [n_ch][T]
 };
 
@@ -919,7 +941,7 @@ __global__ void __launch_bounds__(256) k_field_interp(const __grid_constant__ Fi
             q.Wx = make_float2(w.x, w.z);
             q.Wy = make_float2(w.y, w.w);
         } else {
-            q = make_sample(d, A.r[t], A.v[t]);
+            q = make_sample(d, A.r, A.v, t);
         }
     }
     const bool in = valid && q.in;
@@ -1513,6 +1535,69 @@ template <typename K> int allow_smem(K k, size_t bytes)
     return MPI_OK;
 }
 
+// Shared memory above 48 KB is granted per kernel; asked for outside any
+// stream capture (field_prepare), so the launches only launch.
+int allow_all(const FieldDev &d, bool forward, bool adjoint)
+{
+    const bool four = cols_nc(d) == 4;
+    MPI_TRY(allow_smem(k_field_rows, rows_smem(d)));
+    MPI_TRY(allow_smem(four ? k_field_kcols<4> : k_field_kcols<2>, cols_smem(d)));
+    if (forward) {
+        MPI_TRY(allow_smem(k_field_image<double>, image_smem(d)));
+        MPI_TRY(allow_smem(four ? k_field_cols_fwd<4> : k_field_cols_fwd<2>, cols_smem(d)));
+        MPI_TRY(allow_smem(k_field_rows_inv, rows_smem(d)));
+    }
+    if (adjoint) {
+        MPI_TRY(allow_smem(k_field_setup, order_smem(d)));
+        MPI_TRY(allow_smem(k_field_place, order_smem(d)));
+        MPI_TRY(allow_smem(k_field_rows_fwd, rows_smem(d)));
+        MPI_TRY(allow_smem(four ? k_field_cols_adj<4> : k_field_cols_adj<2>, cols_smem(d)));
+        MPI_TRY(allow_smem(k_field_out<float, false>, image_smem(d)));
+        MPI_TRY(allow_smem(k_field_out<double, false>, image_smem(d)));
+        MPI_TRY(allow_smem(k_field_out<double, true>, image_smem(d)));
+    }
+    return MPI_OK;
+}
+
+// The plan's buffers: `keep` holds what a prepared plan needs between
+// applications, `work` what one preparation or application uses.
+void lay_out(FieldPlan &plan, char *keep, char *work, size_t &keep_bytes, size_t &work_bytes)
+{
+    FieldDev &d = plan.d;
+    FieldBuf &b = d.b;
+    size_t tot[2] = {0, 0};
+    auto take = [&](int which, auto *&ptr, size_t n) {
+        char *base = which ? work : keep;
+        ptr = base ? reinterpret_cast<std::remove_reference_t<decltype(ptr)>>(base + tot[which]) : nullptr;
+        tot[which] += up256(sizeof(*ptr) * n);
+    };
+    const size_t J1 = d.x.J + 1, T1 = size_t(d.T), ny = d.y.n, nt = size_t(d.tx) * d.ty, nh = (nt + 1) * d.n_run;
+    take(0, b.twPx, d.x.P); take(0, b.twPy, d.y.P); take(0, b.twQy, d.y.Q); take(0, b.twQx, d.x.Q);
+    take(0, b.iphx, J1); take(0, b.iphy, d.y.J + 1);
+    take(0, b.xcol, d.x.n); take(0, b.yrow, ny);
+    take(0, b.KH, size_t(3) * d.n_grp * cols_nc(d) * (2 * d.y.J + 1));
+    take(0, b.KL, 3 * kFieldLow * kLowY);
+    take(1, b.KR, 3 * size_t(d.y.P / 2 + 1) * J1);
+    take(1, b.FC, size_t(3) * d.y.w * J1);
+    if (plan.forward) {
+        take(1, b.CR, ny * (d.x.Q / 2 + 1));
+        take(1, b.CL, ny * kFieldLow);
+        take(1, b.FN, size_t(d.y.w) * d.x.w);
+    }
+    if (plan.adjoint) {
+        take(1, b.key, T1); take(1, b.hist, nh); take(1, b.pos, nh); take(1, b.tcnt, nt + 1);
+        take(0, b.list, T1); take(0, b.toff, nt + 1); take(0, b.uoff, nt + 1); take(0, b.unit_tile, d.n_unit_max);
+        take(0, b.rec, T1); take(0, b.wv, T1);
+        take(1, b.q4, T1);
+        take(1, b.upart, size_t(3) * kPatchSize * d.n_unit_max);
+        take(1, b.opart, size_t(d.out_chunks) * d.x.n * ny);
+        take(1, b.AC, 3 * ny * J1);
+        take(1, b.AL, 3 * ny * kFieldLow);
+    }
+    keep_bytes = tot[0];
+    work_bytes = tot[1];
+}
+
 }  // namespace
 
 int field_plan(const ModelH &m, const GridH &g, int64_t T, bool forward, bool adjoint, FieldPlan &plan)
@@ -1563,92 +1648,32 @@ int field_plan(const ModelH &m, const GridH &g, int64_t T, bool forward, bool ad
     d.magQy = unsigned((int64_t(1) << 32) / d.y.Q + 1);
     if (std::max({rows_smem(d), cols_smem(d), order_smem(d)}) > 227 * 1024 - 2048)
         return MPI_ERR_UNSUPPORTED;
-    size_t tot = 0;
-    auto add = [&](size_t b) { tot += up256(b); };
-    const size_t J1 = d.x.J + 1, T1 = size_t(T);
-    add(sizeof(float2) * d.x.P); add(sizeof(float2) * d.y.P); add(sizeof(float2) * d.y.Q); add(sizeof(float2) * d.x.Q);
-    add(sizeof(double) * J1); add(sizeof(double) * (d.y.J + 1));
-    add(sizeof(float2) * g.nx); add(sizeof(float2) * g.ny);
-    add(sizeof(float2) * 3 * (d.y.P / 2 + 1) * J1);
-    add(sizeof(float) * 3 * d.n_grp * cols_nc(d) * (2 * d.y.J + 1));
-    add(sizeof(double) * 3 * kFieldLow * kLowY);
-    add(sizeof(float2) * 3 * d.y.w * J1);
-    if (forward) {
-        add(sizeof(float2) * g.ny * (d.x.Q / 2 + 1));
-        add(sizeof(float4) * g.ny * kFieldLow);
-        add(sizeof(float4) * size_t(d.y.w) * d.x.w);
-    }
-    if (adjoint) {
-        const size_t nh = size_t(nt + 1) * d.n_run;
-        add(sizeof(int) * T1); add(sizeof(int) * nh); add(sizeof(int) * nh); add(sizeof(int) * (nt + 1));
-        add(sizeof(int) * T1); add(sizeof(int) * (nt + 1)); add(sizeof(int) * (nt + 1)); add(sizeof(int) * d.n_unit_max);
-        add(sizeof(float4) * T1); add(sizeof(float4) * T1); add(sizeof(float4) * T1);
-        add(sizeof(float) * 3 * kPatchSize * size_t(d.n_unit_max));
-        add(sizeof(float) * size_t(d.out_chunks) * N);
-        add(sizeof(float2) * 3 * g.ny * J1);
-        add(sizeof(float4) * 3 * g.ny * kFieldLow);
-    }
-    plan.bytes = tot;
     plan.forward = forward;
     plan.adjoint = adjoint;
+    lay_out(plan, nullptr, nullptr, plan.keep_bytes, plan.work_bytes);
     return MPI_OK;
 }
 
-void field_carve(FieldPlan &plan, void *scratch)
+void field_carve(FieldPlan &plan, void *keep, void *work)
 {
-    FieldDev &d = plan.d;
-    FieldBuf &b = d.b;
-    char *p = static_cast<char *>(scratch);
-    auto take = [&](auto *&ptr, size_t bytes) {
-        ptr = reinterpret_cast<std::remove_reference_t<decltype(ptr)>>(p);
-        p += up256(bytes);
-    };
-    const size_t J1 = d.x.J + 1, T1 = size_t(d.T);
-    const int nx = d.x.n, ny = d.y.n, nt = d.tx * d.ty;
-    take(b.twPx, sizeof(float2) * d.x.P); take(b.twPy, sizeof(float2) * d.y.P); take(b.twQy, sizeof(float2) * d.y.Q);
-    take(b.twQx, sizeof(float2) * d.x.Q);
-    take(b.iphx, sizeof(double) * J1); take(b.iphy, sizeof(double) * (d.y.J + 1));
-    take(b.xcol, sizeof(float2) * nx); take(b.yrow, sizeof(float2) * ny);
-    take(b.KR, sizeof(float2) * 3 * (d.y.P / 2 + 1) * J1);
-    take(b.KH, sizeof(float) * 3 * d.n_grp * cols_nc(d) * (2 * d.y.J + 1));
-    take(b.KL, sizeof(double) * 3 * kFieldLow * kLowY);
-    take(b.FC, sizeof(float2) * 3 * d.y.w * J1);
-    if (plan.forward) {
-        take(b.CR, sizeof(float2) * ny * (d.x.Q / 2 + 1));
-        take(b.CL, sizeof(float4) * ny * kFieldLow);
-        take(b.FN, sizeof(float4) * size_t(d.y.w) * d.x.w);
-    }
-    if (plan.adjoint) {
-        const size_t nh = size_t(nt + 1) * d.n_run;
-        take(b.key, sizeof(int) * T1); take(b.hist, sizeof(int) * nh); take(b.pos, sizeof(int) * nh);
-        take(b.tcnt, sizeof(int) * (nt + 1));
-        take(b.list, sizeof(int) * T1); take(b.toff, sizeof(int) * (nt + 1)); take(b.uoff, sizeof(int) * (nt + 1));
-        take(b.unit_tile, sizeof(int) * d.n_unit_max);
-        take(b.rec, sizeof(float4) * T1); take(b.wv, sizeof(float4) * T1); take(b.q4, sizeof(float4) * T1);
-        take(b.upart, sizeof(float) * 3 * kPatchSize * size_t(d.n_unit_max));
-        take(b.opart, sizeof(float) * size_t(d.out_chunks) * nx * ny);
-        take(b.AC, sizeof(float2) * 3 * ny * J1);
-        take(b.AL, sizeof(float4) * 3 * ny * kFieldLow);
-    }
+    size_t k, w;
+    lay_out(plan, static_cast<char *>(keep), static_cast<char *>(work), k, w);
 }
 
 int field_prepare(const FieldPlan &plan, const float *c, const float *r, const float *v, cudaStream_t st)
 {
     const FieldDev &d = plan.d;
-    const float2 *r2 = reinterpret_cast<const float2 *>(r), *v2 = reinterpret_cast<const float2 *>(v);
+    MPI_TRY(allow_all(d, plan.forward, plan.adjoint));
     const int n_table = (table_entries(d) + 31) / 32, ow = order_warps(d);
     const int n_bin = plan.adjoint ? (d.n_run + ow - 1) / ow : 0;
     const size_t osm = plan.adjoint ? order_smem(d) : 0;
-    MPI_TRY(allow_smem(k_field_setup, osm));
-    k_field_setup<<<n_table + n_bin, 32 * ow, osm, st>>>(d, n_table, r2, v2);
+    k_field_setup<<<n_table + n_bin, 32 * ow, osm, st>>>(d, n_table, r, v);
     MPI_CHECK_LAUNCH();
     const int kr = (d.y.P / 2 + 2) / 2, tr = fft_threads(3, d.x.P);
     const int more = c ? (d.y.n + 1) / 2 : plan.adjoint ? (d.tx * d.ty + 1 + tr / 32 - 1) / (tr / 32) : 0;
-    MPI_TRY(allow_smem(k_field_rows, rows_smem(d)));
     k_field_rows<<<kr + more, tr, rows_smem(d), st>>>(d, kr, c);
     MPI_CHECK_LAUNCH();
     auto cols = cols_nc(d) == 4 ? k_field_kcols<4> : k_field_kcols<2>;
-    MPI_TRY(allow_smem(cols, cols_smem(d)));
     cols<<<3 * d.n_grp + (plan.adjoint ? 1 : 0), fft_threads(cols_nc(d), d.y.P), cols_smem(d), st>>>(d);
     MPI_CHECK_LAUNCH();
     return MPI_OK;
@@ -1658,9 +1683,7 @@ int field_order(const FieldPlan &plan, const float *r, const float *v, const flo
 {
     const FieldDev &d = plan.d;
     const int ow = order_warps(d);
-    MPI_TRY(allow_smem(k_field_place, order_smem(d)));
-    k_field_place<<<(d.n_run + ow - 1) / ow, 32 * ow, order_smem(d), st>>>(d, reinterpret_cast<const float2 *>(r),
-                                                                           reinterpret_cast<const float2 *>(v), s);
+    k_field_place<<<(d.n_run + ow - 1) / ow, 32 * ow, order_smem(d), st>>>(d, r, v, s);
     MPI_CHECK_LAUNCH();
     return MPI_OK;
 }
@@ -1678,10 +1701,8 @@ namespace {
 int field_nodes(const FieldDev &d, cudaStream_t st)
 {
     auto cols = cols_nc(d) == 4 ? k_field_cols_fwd<4> : k_field_cols_fwd<2>;
-    MPI_TRY(allow_smem(cols, cols_smem(d)));
     cols<<<3 * d.n_grp, fft_threads(cols_nc(d), std::max(d.y.P, d.y.Q)), cols_smem(d), st>>>(d);
     MPI_CHECK_LAUNCH();
-    MPI_TRY(allow_smem(k_field_rows_inv, rows_smem(d)));
     k_field_rows_inv<<<(d.y.w + 1) / 2, fft_threads(3, d.x.P), rows_smem(d), st>>>(d);
     MPI_CHECK_LAUNCH();
     return MPI_OK;
@@ -1696,7 +1717,7 @@ int field_forward(const FieldPlan &plan, const float *c, const float *r, const f
     ProfScope prof(kProfForward, st);
     MPI_TRY(field_prepare(plan, c, r, v, st));
     MPI_TRY(field_nodes(plan.d, st));
-    InterpArgs A{reinterpret_cast<const float2 *>(r), reinterpret_cast<const float2 *>(v), s};
+    const InterpArgs A{r, v, s};
     k_field_interp<kInterpForward, float><<<interp_blocks(plan.d.T), 256, 0, st>>>(plan.d, A, c);
     MPI_CHECK_LAUNCH();
     return MPI_OK;
@@ -1707,7 +1728,6 @@ int field_forward_ordered(const FieldPlan &plan, const CIN *c, cudaStream_t st)
 {
     const FieldDev &d = plan.d;
     ProfScope prof(kProfForward, st);
-    MPI_TRY(allow_smem(k_field_image<CIN>, image_smem(d)));
     k_field_image<CIN><<<(d.y.n + 1) / 2, 128, image_smem(d), st>>>(d, c);
     MPI_CHECK_LAUNCH();
     MPI_TRY(field_nodes(d, st));
@@ -1726,18 +1746,15 @@ int field_adjoint(const FieldPlan &plan, OUT *out, const double *cg_p, const dou
     ProfScope prof(kProfAdjoint, st);
     k_field_spread<<<d.n_unit_max + d.out_tiles * d.out_chunks, kSpreadThreads, 0, st>>>(d);
     MPI_CHECK_LAUNCH();
-    MPI_TRY(allow_smem(k_field_rows_fwd, rows_smem(d)));
     k_field_rows_fwd<<<(d.y.w + 1) / 2, fft_threads(3, d.x.P), rows_smem(d), st>>>(d);
     MPI_CHECK_LAUNCH();
     auto cols = cols_nc(d) == 4 ? k_field_cols_adj<4> : k_field_cols_adj<2>;
-    MPI_TRY(allow_smem(cols, cols_smem(d)));
     cols<<<3 * d.n_grp, fft_threads(cols_nc(d), std::max(d.y.P, d.y.Q)), cols_smem(d), st>>>(d);
     MPI_CHECK_LAUNCH();
     const unsigned nb = (unsigned)field_dot_blocks(d.y.n);
     if constexpr (sizeof(OUT) == sizeof(double)) {
         if (cg_p) {
-            MPI_TRY(allow_smem(k_field_out<double, true>, image_smem(d)));
-            k_field_out<double, true><<<nb, 128, image_smem(d), st>>>(d, out, cg_p, nu_dev, dot_part);
+                    k_field_out<double, true><<<nb, 128, image_smem(d), st>>>(d, out, cg_p, nu_dev, dot_part);
             MPI_CHECK_LAUNCH();
             return MPI_OK;
         }
@@ -1745,7 +1762,6 @@ int field_adjoint(const FieldPlan &plan, OUT *out, const double *cg_p, const dou
         set_error("internal: CG epilogue needs FP64 output");
         return MPI_ERR_INVALID;
     }
-    MPI_TRY(allow_smem(k_field_out<OUT, false>, image_smem(d)));
     k_field_out<OUT, false><<<nb, 128, image_smem(d), st>>>(d, out, nullptr, nullptr, nullptr);
     MPI_CHECK_LAUNCH();
     return MPI_OK;
@@ -1757,14 +1773,33 @@ bool field_worth(const GridH &g, int64_t T) { return double(T) * g.nx * g.ny >= 
 // 2.3e6 pairs/us (1.05e6 with a general G, whose pairs are all checked).
 // Gridded, per 768 x 768 nodes and per sample: forward 25 + 55 + 0.00019,
 // A^T with the ordering of the samples 40 + 75 + 0.0003.
-bool field_route(const FieldPlan &plan, bool adjoint)
+bool field_route(const FieldPlan &plan)
 {
     const FieldDev &d = plan.d;
     const double T = double(d.T), pairs = T * d.x.n * d.y.n;
     const double nodes = double(d.x.P) * d.y.P / (768.0 * 768.0);
     const double direct = 25.0 + pairs / (d.diag ? 2.3e6 : 1.05e6);
-    const double field = adjoint ? 40.0 + 75.0 * nodes + 0.0003 * T : 25.0 + 55.0 * nodes + 0.00019 * T;
+    const double field = plan.adjoint ? 40.0 + 75.0 * nodes + 0.0003 * T : 25.0 + 55.0 * nodes + 0.00019 * T;
     return field < direct;
+}
+
+// A solve prepares once (60 + 60 and 0.0004 per sample) and applies A^T A:
+// 15 + 75 and 0.0005 per sample against twice 2.4e6 pairs/us and, unless the
+// launches of many frames are shared, 30.
+static bool field_route_solve(const FieldPlan &plan, int64_t products, bool shared)
+{
+    const FieldDev &d = plan.d;
+    const double T = double(d.T), pairs = T * d.x.n * d.y.n;
+    const double nodes = double(d.x.P) * d.y.P / (768.0 * 768.0);
+    const double direct = (shared ? 0.0 : 30.0) + 2.0 * pairs / (d.diag ? 2.4e6 : 1.05e6);
+    const double field = 15.0 + 75.0 * nodes + 0.0005 * T;
+    return double(products) * (direct - field) > 60.0 + 60.0 * nodes + 0.0004 * T;
+}
+
+bool field_solve_plan(const ModelH &m, const GridH &g, int64_t T, int n_iter, int n_cg, bool shared, FieldPlan &plan)
+{
+    return T > 0 && field_worth(g, T) && field_plan(m, g, T, true, true, plan) == MPI_OK &&
+           field_route_solve(plan, (int64_t)n_iter * (n_cg + 1), shared);
 }
 
 template int field_forward_ordered<double>(const FieldPlan &, const double *, cudaStream_t);

@@ -73,16 +73,22 @@ bool field_worth(const GridH &g, int64_t T);
 
 struct FieldPlan {
     FieldDev d;
-    size_t bytes = 0;
+    size_t keep_bytes = 0, work_bytes = 0;
     bool forward = false, adjoint = false;  // which buffers it lays out
 };
-// Fills plan.d's sizes and the bytes of scratch it needs (adjoint: also the
-// sample order); MPI_ERR_UNSUPPORTED when the box or its transforms would be
-// too large.  field_carve then points the buffers into the scratch.
+// Fills plan.d's sizes and the bytes of scratch it needs (adjoint: also for
+// the sample order); MPI_ERR_UNSUPPORTED when the box or its transforms would
+// be too large.  field_carve points the buffers into the scratch: keep_bytes
+// hold a prepared plan, work_bytes serve one preparation or application (plans
+// used one after another on one stream may share them).  Both 256-aligned.
 int field_plan(const ModelH &m, const GridH &g, int64_t T, bool forward, bool adjoint, FieldPlan &plan);
-void field_carve(FieldPlan &plan, void *scratch);
+void field_carve(FieldPlan &plan, void *keep, void *work);
 // Whether one call on this plan costs less than the direct sums.
-bool field_route(const FieldPlan &plan, bool adjoint);
+bool field_route(const FieldPlan &plan);
+// The plan (both directions) of a PnP solve with A, if it costs less than the
+// direct sums over the solve's n_iter (n_cg + 1) products A^T A (shared: sums
+// whose launches serve many frames).
+bool field_solve_plan(const ModelH &m, const GridH &g, int64_t T, int n_iter, int n_cg, bool shared, FieldPlan &plan);
 
 // Tables and the kernel spectrum; with an adjoint plan also the first half of the sample order (r, v); c: the
 // rows of an image for the forward operator (plans without adjoint).

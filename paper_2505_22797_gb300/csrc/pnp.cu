@@ -12,6 +12,7 @@
 
 #include "graph.cuh"
 #include "conv_ops.cuh"
+#include "field_ops.cuh"
 #include "pnp_device.cuh"
 
 namespace mpi {
@@ -299,6 +300,9 @@ struct PnPOp2D final : PnPOperator<R> {
     FwdSplit fs{};
     AdjSplit as{};
     R *fwd_part = nullptr, *adj_part = nullptr, *sA = nullptr;
+    // FP32: A and A^T by the gridded operators, on the samples ordered by tile
+    bool gridded = false;
+    FieldPlan fld;
     ConvPlan<R> C;
     R *tmp1 = nullptr, *tmp2 = nullptr;
     int64_t N = 0;
@@ -321,6 +325,12 @@ struct PnPOp2D final : PnPOperator<R> {
     }
     int rhs(const R *data, double *b0, cudaStream_t st) override
     {
+        if constexpr (sizeof(R) == 4)
+            if (gridded) {
+                MPI_TRY(field_load(fld, data, st));
+                MPI_TRY(field_adjoint<double>(fld, b0, nullptr, nullptr, nullptr, st));
+                return ar ? reduce(b0, st) : MPI_OK;
+            }
         if (op == MPI_OP_FORWARD) {
             MPI_TRY((launch_adjoint<R, double>(m, g, T, geo, as, data, adj_part, b0, nullptr, nullptr,
                                                nullptr, st)));
@@ -331,6 +341,13 @@ struct PnPOp2D final : PnPOperator<R> {
     int apply_normal(const double *v, double *q, const double *nu_dev, double *pq_part,
                      cudaStream_t st) override
     {
+        if (gridded) {
+            MPI_TRY(field_forward_ordered<double>(fld, v, st));
+            if (!ar) return field_adjoint<double>(fld, q, v, nu_dev, pq_part, st);
+            MPI_TRY(field_adjoint<double>(fld, red, nullptr, nullptr, nullptr, st));
+            MPI_TRY(reduce(red, st));
+            return axpy_dot_launch<double>(N, red, v, nu_dev, q, pq_part, st);
+        }
         if (op == MPI_OP_FORWARD) {
             MPI_TRY((launch_forward<R, double, R>(m, g, T, geo, fs, v, fwd_part, sA, st)));
             if (!ar)
@@ -348,6 +365,7 @@ struct PnPOp2D final : PnPOperator<R> {
     }
     int n_pq() const override
     {
+        if (gridded && !ar) return field_dot_blocks(g.ny);
         return (op == MPI_OP_FORWARD && !ar) ? adjoint_dot_blocks(g.nx, g.ny) : vec_blocks(N);
     }
     int denoise(const R *in, R *out, const double *sigma_dev, cudaStream_t st) override
@@ -376,6 +394,24 @@ static int pnp_impl(const ModelH &m, const GridH &g, const mpi_traj *tr, const v
     S.ar = ar;
     S.ar_user = ar_user;
     const int target = default_target_items();
+
+    if constexpr (sizeof(R) == 4) {
+        Scratch fscr(st);
+        if (o.op == MPI_OP_FORWARD && field_solve_plan(m, g, S.T, o.n_iter, o.n_cg, false, S.fld)) {
+            const size_t o_keep = fscr.reserve(S.fld.keep_bytes), o_work = fscr.reserve(S.fld.work_bytes);
+            const size_t o_sum = ar ? fscr.reserve(sizeof(double) * size_t(S.N)) : 0;
+            if (fscr.allocate() == MPI_OK) {
+                S.gridded = true;
+                if (ar) S.red = fscr.at<double>(o_sum);
+                field_carve(S.fld, fscr.at<char>(o_keep), fscr.at<char>(o_work));
+                const float *r = static_cast<const float *>(tr->r), *v = static_cast<const float *>(tr->v);
+                MPI_TRY(field_prepare(S.fld, nullptr, r, v, st));
+                MPI_TRY(field_order(S.fld, r, v, nullptr, st));
+                return pnp_run<R>(S, S.N, data, o, rho_out, info, st);
+            }
+            (void)cudaGetLastError();  // the pair sums need less
+        }
+    }
 
     Scratch scr(st);
     size_t o_geo = 0, o_fp = 0, o_ap = 0, o_sA = 0, o_K = 0, o_t1 = 0, o_t2 = 0, o_ord = 0, o_red = 0;

@@ -1,7 +1,7 @@
 """The gridded FP32 route of the 2-D pair operators (large problems) against
 the FP64 oracle: odd sizes, thin and one-column grids, general and negative
 axes, one channel, dwelling and repeated positions, samples beyond the node
-window, non-finite positions, and the calls that stay with the direct sums.
+window, non-finite positions, unaligned arrays.
 
 Tolerance 1e-6: the transforms have about 25 butterfly levels and the
 interpolation 6 more, each rounding by 2^-24; if all of them added up the
@@ -90,12 +90,43 @@ def test_field_non_finite_positions(orc):
     assert np.isnan(host(api.mpi_adjoint(m, g, dev(bad, F32), dev(v, F32), dev(s, F32)))).all()
 
 
-def test_field_and_direct_routes_agree_on_alignment(orc):
-    """A trajectory that is not 8-byte aligned runs the direct sums."""
+def test_field_unaligned_trajectory(orc):
+    """Arrays that are aligned to single floats only."""
     m, g, r, v, c, s = _case(128, 128, 16384, 8)
-    buf = torch.empty(2 * r.size + 2, dtype=F32, device="cuda")
-    R = buf[1:1 + r.size].view(-1, 2)
+    buf = torch.empty((2, 2 * r.size + 2), dtype=F32, device="cuda")
+    R, V = (buf[k, 1:1 + r.size].view(-1, 2) for k in range(2))
     R.copy_(dev(r, F32))
-    assert R.data_ptr() % 8 == 4
-    got = host(api.mpi_forward(m, g, R, dev(v, F32), dev(c, F32)))
-    assert rel_l2(got, orc.forward(m, g, r, v, c)) <= TOL
+    V.copy_(dev(v, F32))
+    assert R.data_ptr() % 8 == 4 and V.data_ptr() % 8 == 4
+    assert rel_l2(host(api.mpi_forward(m, g, R, V, dev(c, F32))), orc.forward(m, g, r, v, c)) <= TOL
+    assert rel_l2(host(api.mpi_adjoint(m, g, R, V, dev(s, F32))), orc.adjoint(m, g, r, v, s)) <= TOL
+
+
+def test_field_solve_single_batch_and_sharded(orc):
+    """Algorithm 1 on the gridded operators (64 x 60, 40 001 samples: the
+    smallest frames that take them) against the oracle, held to the FP32 bar
+    of the well-posed solves; the matched batch (beside a frame that keeps the
+    pair sums) bit for bit, and the sharded solve."""
+    big, small = _case(64, 60, 40001, 11), _case(20, 24, 900, 12)
+    nu0 = []
+    for m, g, r, v, c, s in (big, small):
+        nu0.append(orc.nu0_from_frob2(orc.frob2(m, g, r, v), g["nx"] * g["ny"]))
+    data = [rounded(orc.forward(m, g, r, v, c), F32) for m, g, r, v, c, _ in (big, small)]
+    single = []
+    for (m, g, r, v, c, _), s, nu in zip((big, small), data, nu0):
+        single.append(host(api.mpi_pnp_solve(m, g, dev(r, F32), dev(v, F32), dev(s, F32), 3, 4, nu)))
+    m, g, r, v = big[:4]
+    want = orc.pnp(lambda x: orc.forward(m, g, r, v, x), lambda y: orc.adjoint(m, g, r, v, y), data[0],
+                   (g["ny"], g["nx"]), 3, 4, nu0[0])
+    assert rel_l2(single[0], want) <= 1e-5
+    plan = api.BatchPlan([(q[0], q[1], q[2].shape[0]) for q in (big, small)], nu0, 3, 4,
+                         flags=api.MPI_BATCH_MATCH_SINGLE)
+    assert plan.info()["forward_items"] > 0  # the small frame's pair items
+    arrays = [[dev(x, F32) for x in xs] for xs in ([big[2], small[2]], [big[3], small[3]], data)]
+    for _ in range(2):
+        got = [host(x) for x in plan.run(*arrays)]
+        for a, b in zip(got, single):
+            assert np.array_equal(a, b)
+    sharded = host(api.mpi_pnp_solve_sharded(m, g, dev(r, F32), dev(v, F32), dev(data[0], F32), 3, 4, nu0[0],
+                                             lambda t: None))
+    assert rel_l2(sharded, want) <= 1e-5
