@@ -57,9 +57,9 @@ constexpr int kPatch = kTile + kWin - 1;        // a tile's stencils reach 23 x 
 // apart, start 0, 24, 16, 8 banks in.
 constexpr int kPatchPitch = 28;
 constexpr int kPatchSize = kPatch * kPatch;
-constexpr int kFieldUnit = 128;                 // samples per spreading unit
-constexpr int kSpreadThreads = 192;             // warp = (entry of K, row parity)
-constexpr int kRunMin = 256, kRunMax = 512;     // samples per run at least, runs at most
+constexpr int kFieldUnit = 224;                 // samples per spreading unit
+constexpr int kSpreadThreads = 384;             // warp = (half of the unit, entry of K, row parity)
+constexpr int kRunMin = 128, kRunMax = 512;     // samples per run at least, runs at most
 constexpr int kOutThreads = kSpreadThreads;
 constexpr int kOutVox = 4;                      // voxels per thread of the outside sums
 
@@ -538,36 +538,80 @@ __device__ void kernel_rows(const FieldDev &d, int l0, unsigned char *smem)
     store_rows(z, P, d.x.J + 1, l0, half + 1, s_low, d.b.KR);
 }
 
-// sum_e get(e) exp(-2 pi i m e / n), e < n_e, by one warp in pairs of floats
-// (get: (re, im) hi and lo); result in every lane.
+// The modes +-m of a sequence (get(e): (re, im) hi and lo, e < n_e) of period
+// n by one warp: four terms in FP32, then in pairs (the rounding errors of
+// many small sums average out, those of a few large ones do not).  Valid in
+// every lane.
+struct LowPair {
+    F2Sum rp, ip, rm, im;  // mode m, mode -m
+};
 template <typename F>
-__device__ __forceinline__ void low_mode(int n_e, int n, int m, const float2 *__restrict__ tw, F get, F2Sum &re, F2Sum &im)
+__device__ __forceinline__ LowPair low_modes(int n_e, int n, int m, const float2 *__restrict__ tw, F get)
 {
-    re = F2Sum{};
-    im = F2Sum{};
     const int lane = threadIdx.x & 31;
-    const int mm = m < 0 ? n + m % n : m % n;
-    int at = int(unsigned(lane * mm) % unsigned(n));
-    const int step = int(unsigned(32 * mm) % unsigned(n));
-#pragma unroll 4
-    for (int e = lane; e < n_e; e += 32) {
-        const float2 w = tw[at];
-        at += step;
-        at -= at >= n ? n : 0;
-        const float4 q = get(e);
-        f2_fma(re, q.x, w.x);
-        f2_fma(re, -q.y, w.y);
-        f2_fma(im, q.x, w.y);
-        f2_fma(im, q.y, w.x);
-        re.lo += fmaf(q.z, w.x, -q.w * w.y);
-        im.lo += fmaf(q.z, w.y, q.w * w.x);
+    int at = (lane * m) % n;
+    const int step = (32 * m) % n;
+    F2Sum xc{}, xd{}, yc{}, yd{};
+#pragma unroll 1
+    for (int e0 = lane; e0 < n_e; e0 += 128) {
+        float4 s = make_float4(0.0f, 0.0f, 0.0f, 0.0f), l = s;  // x c, x d, y c, y d of four terms
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int e = e0 + 32 * u;
+            const float2 w = tw[at];
+            at += step;
+            at -= at >= n ? n : 0;
+            if (e < n_e) {
+                const float4 q = get(e);
+                s.x = fmaf(q.x, w.x, s.x);
+                s.y = fmaf(q.x, w.y, s.y);
+                s.z = fmaf(q.y, w.x, s.z);
+                s.w = fmaf(q.y, w.y, s.w);
+                l.x = fmaf(q.z, w.x, l.x);
+                l.y = fmaf(q.z, w.y, l.y);
+                l.z = fmaf(q.w, w.x, l.z);
+                l.w = fmaf(q.w, w.y, l.w);
+            }
+        }
+        xc.add(s.x); xc.lo += l.x;
+        xd.add(s.y); xd.lo += l.y;
+        yc.add(s.z); yc.lo += l.z;
+        yd.add(s.w); yd.lo += l.w;
     }
-    re = f2_warp(re);
-    im = f2_warp(im);
+    xc = f2_warp(xc);
+    xd = f2_warp(xd);
+    yc = f2_warp(yc);
+    yd = f2_warp(yd);
+    LowPair r{xc, yc, xc, yc};
+    r.rm.add(yd);
+    r.ip.add(xd);
+    yd.hi = -yd.hi, yd.lo = -yd.lo;
+    xd.hi = -xd.hi, xd.lo = -xd.lo;
+    r.rp.add(yd);
+    r.im.add(xd);
+    return r;
+}
+
+// The coefficients of a column's lowest modes, mode sums times the kernel's
+// (pairs): out[ky + kFieldLow - 1].
+template <typename F>
+__device__ __forceinline__ void low_coefs(int n_e, int n, int ky, const float2 *__restrict__ tw, const float2 *__restrict__ K,
+                                          float4 *out, F get)
+{
+    const LowPair s = low_modes(n_e, n, ky, tw, get);
+    if ((threadIdx.x & 31) == 0) {
+#pragma unroll
+        for (int sg = 0; sg < 2; ++sg) {
+            const int q = kFieldLow - 1 + (sg ? -ky : ky);
+            const F2Sum re = sg ? s.rm : s.rp, im = sg ? s.im : s.ip;
+            const df r = df_mul(df_fast_two_sum(re.hi, re.lo), K[q]), i = df_mul(df_fast_two_sum(im.hi, im.lo), K[q]);
+            out[q] = make_float4(r.x, i.x, r.y, i.y);
+        }
+    }
 }
 
 // Adds the lowest modes' part of element e: sum over ky of the pair
-// coefficient co[ky] times exp(2 pi i ky e / n).
+// coefficient co[ky] times exp(2 pi i ky e / n), as pairs.
 __device__ __forceinline__ void low_add(const float4 *co, int e, int n, const float2 *__restrict__ tw, F2Sum &re, F2Sum &im)
 {
     int at = 0;
@@ -589,6 +633,25 @@ __device__ __forceinline__ void low_add(const float4 *co, int e, int n, const fl
             im.lo += fmaf(v.z, ty, v.w * t.x);
         }
     }
+}
+// The same rounded to FP32 as it goes, the mean last (one rounding at full
+// size): for values that many others average.
+__device__ __forceinline__ void low_add32(const float4 *co, int e, int n, const float2 *__restrict__ tw, V2<float> &q)
+{
+    int at = int(unsigned(e * (kFieldLow - 1)) % unsigned(n));
+#pragma unroll
+    for (int k = kFieldLow - 1; k > 0; --k) {
+        const float2 t = tw[at];
+        at -= e;
+        at += at < 0 ? n : 0;
+        const float4 v = co[kFieldLow - 1 + k], u = co[kFieldLow - 1 - k];
+        // v (t.x - i t.y) + u (t.x + i t.y)
+        q.x = fmaf(v.x + u.x, t.x, fmaf(v.y - u.y, t.y, q.x));
+        q.y = fmaf(v.y + u.y, t.x, fmaf(u.x - v.x, t.y, q.y));
+    }
+    const float4 v = co[kFieldLow - 1];
+    q.x = (q.x + v.z) + v.x;
+    q.y = (q.y + v.w) + v.y;
 }
 
 // Columns of the kernel's spectrum: NC adjacent kx (group g) of entry m.  The
@@ -612,18 +675,19 @@ template <int NC> __device__ void kernel_cols(const FieldDev &d, int g, int m, u
     __syncthreads();
     if (g * NC < kFieldLow) {
         const int nw = blockDim.x >> 5, w = threadIdx.x >> 5;
-        for (int q = w; q < NC * kLowY; q += nw) {
-            const int cc = q % NC, ky = q / NC - (kFieldLow - 1), kk = g * NC + cc;
+        for (int q = w; q < NC * kFieldLow; q += nw) {
+            const int cc = q % NC, ky = q / NC, kk = g * NC + cc;
             if (kk >= kFieldLow) continue;
-            F2Sum re, im;
-            low_mode(P, P, ky, d.b.twPy,
-                     [&](int e) {
-                         const V2<float> z = a[smem_fft_pad(e) * NC + cc];
-                         return make_float4(z.x, z.y, 0.0f, 0.0f);
-                     },
-                     re, im);
-            if ((threadIdx.x & 31) == 0)
-                d.b.KL[(m * kFieldLow + kk) * kLowY + ky + kFieldLow - 1] = re.value() * d.b.iphx[kk] * d.b.iphy[abs(ky)];
+            const LowPair s = low_modes(P, P, ky, d.b.twPy, [&](int e) {
+                const V2<float> z = a[smem_fft_pad(e) * NC + cc];
+                return make_float4(z.x, z.y, 0.0f, 0.0f);
+            });
+            if ((threadIdx.x & 31) == 0) {
+                const double f = d.b.iphx[kk] * d.b.iphy[ky];
+                float2 *K = d.b.KL + (m * kFieldLow + kk) * kLowY + kFieldLow - 1;
+                K[ky] = df_from_double(s.rp.value() * f);
+                K[-ky] = df_from_double(s.rm.value() * f);
+            }
         }
         __syncthreads();
     }
@@ -658,15 +722,12 @@ template <typename CIN> __device__ void image_rows(const FieldDev &d, int j0, co
     for (int q = w; q < 2 * kFieldLow; q += nw) {
         const int kx = q >> 1, rr = q & 1;
         if (rr && !two) continue;
-        F2Sum re, im;
-        low_mode(nx, Q, kx, d.b.twQx,
-                 [&](int e) {
-                     const V2<float> z = a[smem_fft_pad(e)];
-                     return make_float4(rr ? z.y : z.x, 0.0f, 0.0f, 0.0f);
-                 },
-                 re, im);
+        const LowPair s = low_modes(nx, Q, kx, d.b.twQx, [&](int e) {
+            const V2<float> z = a[smem_fft_pad(e)];
+            return make_float4(rr ? z.y : z.x, 0.0f, 0.0f, 0.0f);
+        });
         if ((threadIdx.x & 31) == 0) {
-            const float2 r = df_fast_two_sum(re.hi, re.lo), i = df_fast_two_sum(im.hi, im.lo);
+            const float2 r = df_fast_two_sum(s.rp.hi, s.rp.lo), i = df_fast_two_sum(s.ip.hi, s.ip.lo);
             d.b.CL[int64_t(j0 + rr) * kFieldLow + kx] = make_float4(r.x, i.x, r.y, i.y);
         }
     }
@@ -755,16 +816,11 @@ __global__ void __launch_bounds__(512) k_field_cols_fwd(const __grid_constant__ 
     const bool low = g * NC < kFieldLow;
     if (low) {
         const int nw = blockDim.x >> 5, w = threadIdx.x >> 5;
-        for (int q = w; q < NC * kLowY; q += nw) {
-            const int cc = q % NC, ky = q / NC - (kFieldLow - 1), kk = g * NC + cc;
-            if (kk >= kFieldLow) continue;
-            F2Sum re, im;
-            low_mode(ny, Q, ky, d.b.twQy, [&](int e) { return d.b.CL[int64_t(e) * kFieldLow + kk]; }, re, im);
-            if ((threadIdx.x & 31) == 0) {
-                const double h = d.b.KL[(m * kFieldLow + kk) * kLowY + ky + kFieldLow - 1];
-                const df r = df_from_double(re.value() * h), i = df_from_double(im.value() * h);
-                s_low[cc][q / NC] = make_float4(r.x, i.x, r.y, i.y);
-            }
+        for (int q = w; q < NC * kFieldLow; q += nw) {
+            const int cc = q % NC, kk = g * NC + cc;
+            if (kk < kFieldLow)
+                low_coefs(ny, Q, q / NC, d.b.twQy, d.b.KL + (m * kFieldLow + kk) * kLowY, s_low[cc],
+                          [&](int e) { return d.b.CL[int64_t(e) * kFieldLow + kk]; });
         }
     }
     V2<float> *z = smem_fft<NC, -1, float>(a, b, d.fQy, reinterpret_cast<const V2<float> *>(d.b.twQy));
@@ -773,16 +829,14 @@ __global__ void __launch_bounds__(512) k_field_cols_fwd(const __grid_constant__ 
     const float *KH = d.b.KH + ((int64_t(m) * d.n_grp + g) * JY + J) * NC + c;
     const int lift = (J / Q + 1) * Q;
     const int skip = kx < kFieldLow ? kFieldLow : 0;  // modes carried in pairs
+    for (int l = J + 1 + j0; l < P - J; l += dj) o[smem_fft_pad(l) * NC + c] = V2<float>{0.0f, 0.0f};
 #pragma unroll 4
-    for (int l = j0; l < P; l += dj) {
-        const int ky = l <= P / 2 ? l : l - P;
+    for (int ky = j0 - J; ky <= J; ky += dj) {
         V2<float> q{0.0f, 0.0f};
-        if (ky >= -J && ky <= J && abs(ky) >= skip) {
-            const V2<float> u = z[smem_fft_pad(fast_mod(ky, Q, d.magQy, lift)) * NC + c];
-            const float h = KH[ky * NC];
-            q = V2<float>{u.x * h, u.y * h};
-        }
-        o[smem_fft_pad(l) * NC + c] = q;
+        const V2<float> u = z[smem_fft_pad(fast_mod(ky, Q, d.magQy, lift)) * NC + c];
+        const float h = KH[ky * NC];
+        if (abs(ky) >= skip) q = V2<float>{u.x * h, u.y * h};
+        o[smem_fft_pad(ky < 0 ? ky + P : ky) * NC + c] = q;
     }
     __syncthreads();
     z = smem_fft<NC, 1, float>(o, o == a ? b : a, d.fPy, reinterpret_cast<const V2<float> *>(d.b.twPy));
@@ -794,11 +848,7 @@ __global__ void __launch_bounds__(512) k_field_cols_fwd(const __grid_constant__ 
         int l = l0 + i;
         l -= l >= P ? P : 0;
         V2<float> q = z[smem_fft_pad(l) * NC + c];
-        if (low && kx < kFieldLow) {
-            F2Sum re{q.x, 0.0f}, im{q.y, 0.0f};
-            low_add(s_low[c], l, P, d.b.twPy, re, im);
-            q = V2<float>{re.hi + re.lo, im.hi + im.lo};
-        }
+        if (low && kx < kFieldLow) low_add32(s_low[c], l, P, d.b.twPy, q);
         F[int64_t(i) * J1] = f2c(q);
     }
 }
@@ -983,20 +1033,25 @@ __global__ void __launch_bounds__(256) k_field_interp(const __grid_constant__ Fi
                 s1 = fmaf(wy, f[b].y, s1);
                 s2 = fmaf(wy, f[b].z, s2);
             }
+            // Products as pairs, then the sums over the eight lanes: the lane
+            // bits 0 and 1 also choose which entry a lane goes on with (0: xx,
+            // 1: xy, 2: yy, 3: none), so three levels take four additions.
             F2Sum p0{}, p1{}, p2{};
             p0.hi = s0 * wx; p0.lo = fmaf(s0, wx, -p0.hi);
             p1.hi = s1 * wx; p1.lo = fmaf(s1, wx, -p1.hi);
             p2.hi = s2 * wx; p2.lo = fmaf(s2, wx, -p2.hi);
-#pragma unroll
-            for (int o = 1; o < 8; o <<= 1) {
-                p0.add(f2_shfl_xor(p0, o));
-                p1.add(f2_shfl_xor(p1, o));
-                p2.add(f2_shfl_xor(p2, o));
-            }
+            const bool up = lane & 2;  // keeps yy, sends xx and xy
+            F2Sum a = up ? p2 : p0, e = up ? F2Sum{} : p1;
+            const F2Sum sa = up ? p0 : p2, se = up ? p1 : F2Sum{};
+            a.add(f2_shfl_xor(sa, 2));
+            e.add(f2_shfl_xor(se, 2));
+            F2Sum v = (lane & 1) ? e : a;
+            v.add(f2_shfl_xor((lane & 1) ? a : e, 1));
+            v.add(f2_shfl_xor(v, 4));
             const int back = 8 * (lane & 3);
-            const float h0 = __shfl_sync(0xffffffffu, p0.hi, back), l0 = __shfl_sync(0xffffffffu, p0.lo, back);
-            const float h1 = __shfl_sync(0xffffffffu, p1.hi, back), l1 = __shfl_sync(0xffffffffu, p1.lo, back);
-            const float h2 = __shfl_sync(0xffffffffu, p2.hi, back), l2 = __shfl_sync(0xffffffffu, p2.lo, back);
+            const float h0 = __shfl_sync(0xffffffffu, v.hi, back), l0 = __shfl_sync(0xffffffffu, v.lo, back);
+            const float h1 = __shfl_sync(0xffffffffu, v.hi, back + 1), l1 = __shfl_sync(0xffffffffu, v.lo, back + 1);
+            const float h2 = __shfl_sync(0xffffffffu, v.hi, back + 2), l2 = __shfl_sync(0xffffffffu, v.lo, back + 2);
             if ((lane >> 2) == g) {
                 phi[0] = df_fast_two_sum(h0, l0);
                 phi[1] = df_fast_two_sum(h1, l1);
@@ -1059,15 +1114,16 @@ __global__ void __launch_bounds__(256) k_field_interp(const __grid_constant__ Fi
 // tile, summed over its samples in order.  A warp owns one entry of K on the
 // patch rows of one parity: a sample's stencil has four such rows of eight
 // points, one per lane, so no two lanes share a node and the order of the
-// additions is the samples' order.  What bounds it is the shared-memory
-// pipe: per sample and warp one load and one store of the patch, and a
+// additions is the samples' order.  The unit's two halves go to two copies of
+// the patch, added at the end: twice the independent chains of load, FMA and
+// store.  What bounds it is the shared-memory pipe: per sample and warp one load and one store of the patch, and a
 // quarter of three 16-byte loads (weights and addresses of four samples,
 // fetched one step ahead).  The other blocks: partial images of the samples
 // outside the window (none: they return).
 constexpr int kUnitPitch = kFieldUnit + 4;
 __global__ void __launch_bounds__(kSpreadThreads) k_field_spread(const __grid_constant__ FieldDev d)
 {
-    __shared__ float s_patch[3][kPatch * kPatchPitch];
+    __shared__ float s_patch[2][3][kPatch * kPatchPitch];
     __shared__ __align__(16) float s_wx[kWin][kUnitPitch];
     __shared__ __align__(16) float s_c[3][kWin][kUnitPitch];  // entry x row weight, rows by parity
     __shared__ __align__(16) int s_at[kUnitPitch];
@@ -1093,7 +1149,7 @@ __global__ void __launch_bounds__(kSpreadThreads) k_field_spread(const __grid_co
             vy[k] = xc.y + yr.y;
             acc[k] = comp[k] = 0.0f;
         }
-        float *s_p = &s_patch[0][0];  // six values per staged sample
+        float *s_p = &s_patch[0][0][0];  // six values per staged sample
         for (int cb = c0; cb < c1; cb += kOutThreads) {
             const int nb = min(kOutThreads, c1 - cb);
             __syncthreads();
@@ -1146,7 +1202,7 @@ __global__ void __launch_bounds__(kSpreadThreads) k_field_spread(const __grid_co
     const int len = (t1 - t0 + nu - 1) / nu;  // the tile's units share its samples evenly
     const int q0 = t0 + (u - u0) * len;
     const int n = max(0, min(len, t1 - q0)), n4 = (n + 3) & ~3;
-    for (int k = threadIdx.x; k < 3 * kPatch * kPatchPitch; k += kSpreadThreads) (&s_patch[0][0])[k] = 0.0f;
+    for (int k = threadIdx.x; k < 6 * kPatch * kPatchPitch; k += kSpreadThreads) (&s_patch[0][0][0])[k] = 0.0f;
     const int ox = (tile % d.tx) * kTile, oy = (tile / d.tx) * kTile;
     for (int k = threadIdx.x; k < n4; k += kSpreadThreads) {
         float wx[kWin] = {}, wy[kWin] = {};
@@ -1185,23 +1241,25 @@ __global__ void __launch_bounds__(kSpreadThreads) k_field_spread(const __grid_co
         }
     }
     __syncthreads();
-    if (n > 0) {
-        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-        const int m = warp >> 1, par = warp & 1;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int half = warp / 6, mid = (n4 / 4 + 1) / 2 * 4;
+    const int k0 = half ? mid : 0, k1 = half ? n4 : mid;
+    if (k0 < k1) {
+        const int m = (warp % 6) >> 1, par = warp & 1;
         const int col = lane & 7, p = 2 * (lane >> 3) + par;
         const float4 *wp = reinterpret_cast<const float4 *>(s_wx[col]), *cp = reinterpret_cast<const float4 *>(s_c[m][p]);
         const int4 *ap = reinterpret_cast<const int4 *>(s_at);
         // this lane's offset in the stencil for an even / odd first row
-        float *P0 = s_patch[m] + p * kPatchPitch + col, *P1 = s_patch[m] + (p ^ 1) * kPatchPitch + col;
+        float *P0 = s_patch[half][m] + p * kPatchPitch + col, *P1 = s_patch[half][m] + (p ^ 1) * kPatchPitch + col;
         auto add = [&](int at, float c, float w) {
             float *o = ((at >> 16) ? P1 : P0) + (at & 0xffff);
             *o = fmaf(c, w, *o);
             __syncwarp();
         };
-        int4 at = ap[0];
-        float4 w = wp[0], c = cp[0];
-        for (int k = 0; k < n4; k += 4) {
-            const int nx = min(k + 4, n4 - 4) >> 2;
+        int4 at = ap[k0 >> 2];
+        float4 w = wp[k0 >> 2], c = cp[k0 >> 2];
+        for (int k = k0; k < k1; k += 4) {
+            const int nx = min(k + 4, k1 - 4) >> 2;
             const int4 at2 = ap[nx];
             const float4 w2 = wp[nx], c2 = cp[nx];
             add(at.x, c.x, w.x);
@@ -1217,7 +1275,8 @@ __global__ void __launch_bounds__(kSpreadThreads) k_field_spread(const __grid_co
     float *out = d.b.upart + int64_t(u) * 3 * kPatchSize;
     for (int k = threadIdx.x; k < 3 * kPatchSize; k += kSpreadThreads) {
         const int mm = k / kPatchSize, e = k % kPatchSize;
-        out[k] = s_patch[mm][(e / kPatch) * kPatchPitch + e % kPatch];
+        const int at = (e / kPatch) * kPatchPitch + e % kPatch;
+        out[k] = s_patch[0][mm][at] + s_patch[1][mm][at];
     }
 }
 
@@ -1300,21 +1359,13 @@ __global__ void __launch_bounds__(512) k_field_cols_adj(const __grid_constant__ 
     const bool low = g * NC < kFieldLow;
     if (low) {
         const int nw = blockDim.x >> 5, w = threadIdx.x >> 5;
-        for (int q = w; q < NC * kLowY; q += nw) {
-            const int cc = q % NC, ky = q / NC - (kFieldLow - 1), kk = g * NC + cc;
-            if (kk >= kFieldLow) continue;
-            F2Sum re, im;
-            low_mode(P, P, ky, d.b.twPy,
-                     [&](int e) {
-                         const V2<float> z = a[smem_fft_pad(e) * NC + cc];
-                         return make_float4(z.x, z.y, 0.0f, 0.0f);
-                     },
-                     re, im);
-            if ((threadIdx.x & 31) == 0) {
-                const double h = d.b.KL[(m * kFieldLow + kk) * kLowY + ky + kFieldLow - 1];
-                const df r = df_from_double(re.value() * h), i = df_from_double(im.value() * h);
-                s_low[cc][q / NC] = make_float4(r.x, i.x, r.y, i.y);
-            }
+        for (int q = w; q < NC * kFieldLow; q += nw) {
+            const int cc = q % NC, kk = g * NC + cc;
+            if (kk < kFieldLow)
+                low_coefs(P, P, q / NC, d.b.twPy, d.b.KL + (m * kFieldLow + kk) * kLowY, s_low[cc], [&](int e) {
+                    const V2<float> z = a[smem_fft_pad(e) * NC + cc];
+                    return make_float4(z.x, z.y, 0.0f, 0.0f);
+                });
         }
         __syncthreads();
     }
@@ -1323,10 +1374,11 @@ __global__ void __launch_bounds__(512) k_field_cols_adj(const __grid_constant__ 
     const int J = d.y.J, JY = 2 * J + 1;
     const float *KH = d.b.KH + ((int64_t(m) * d.n_grp + g) * JY + J) * NC + c;
     const int skip = kx < kFieldLow ? kFieldLow : 0;  // modes carried in pairs
+#pragma unroll 2
     for (int k = j0; k < Q; k += dj) {
         V2<float> s{0.0f, 0.0f};
         // modes ky = k mod Q
-        for (int ky = k - ((J + k) / Q) * Q; ky <= J; ky += Q) {
+        for (int ky = k - int(__umulhi(unsigned(J + k), d.magQy)) * Q; ky <= J; ky += Q) {
             if (abs(ky) < skip) continue;
             const V2<float> u = z[smem_fft_pad(ky < 0 ? ky + P : ky) * NC + c];
             const float h = KH[ky * NC];
@@ -1515,7 +1567,8 @@ bool plan_axis(int n, double pitch, double p0, double h, FieldAxis &a)
 }
 
 int cols_nc(const FieldDev &d) { return std::max(d.y.P, d.y.Q) <= 2048 ? 4 : 2; }
-// One radix-8 butterfly per thread and pass, up to 512 threads.
+// One radix-8 butterfly per thread and pass, up to 512 threads (384 at 4 x 768
+// points; 512 or 256 threads were 10 and 7 % slower over a whole A).
 int fft_threads(int nc, int n)
 {
     const int b = (nc * n + 7) / 8, per = (b + 511) / 512;

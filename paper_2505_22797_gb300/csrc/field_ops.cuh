@@ -30,7 +30,7 @@ struct FieldBuf {
     V2<float> *xcol, *yrow;  // voxel positions (samples outside the window)
     float2 *KR;      // kernel rows' half spectra [3][Py/2 + 1][Jx + 1]
     float *KH;       // kernel spectrum, scaled: [3][groups of adjacent kx][2 Jy + 1][kx in the group]
-    double *KL;      // its lowest modes [3][kFieldLow][2 kFieldLow - 1]
+    float2 *KL;      // its lowest modes in pairs [3][kFieldLow][2 kFieldLow - 1]
     float2 *CR;      // image rows' half spectra [ny][Qx/2 + 1]
     float4 *CL;      // their lowest modes in pairs [ny][kFieldLow]
     float2 *FC;      // column-transformed half spectra [3][wy][Jx + 1]

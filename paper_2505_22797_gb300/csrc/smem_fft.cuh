@@ -3,7 +3,7 @@
 //
 // NC sequences lie interleaved, element e of sequence c at
 // [smem_fft_pad(e) * NC + c], and move between two buffers, one Stockham pass
-// per radix (8, 5, 4, 3, 2; a length is a product of these).  One element of
+// per radix (16, 8, 5, 4, 3, 2; a length is a product of these).  One element of
 // padding per eight keeps the first pass's stride-8 writes off one bank: for
 // FP32 pairs and NC = 4, consecutive butterflies are then 36 words apart in
 // 8-byte units instead of 32.
@@ -28,7 +28,13 @@ inline SmemFft smem_fft_plan(int n)
     p.n = n;
     int m = n, two = 0, r[kFftMaxPasses], k = 0;
     while (m % 2 == 0) m /= 2, ++two;
-    while (two >= 5 || two == 3) r[k++] = 8, two -= 3;
+    // 2^two as 16s and 8s, as few as possible (4 or 2 where that leaves a rest)
+    int n16 = two / 4;
+    while (n16 > 0 && (two - 4 * n16) % 3 != 0) --n16;
+    if ((two - 4 * n16) % 3 != 0) n16 = 0;
+    two -= 4 * n16;
+    while (n16-- > 0) r[k++] = 16;
+    while (two >= 3 && two != 4) r[k++] = 8, two -= 3;
     while (two >= 2) r[k++] = 4, two -= 2;
     int one2 = two;
     while (m % 5 == 0 && k < kFftMaxPasses) r[k++] = 5, m /= 5;
@@ -104,6 +110,33 @@ template <int RAD, int SGN, typename R> __device__ __forceinline__ void dft(V2<R
         v[4] = csub(m1, n1);
         v[2] = cadd(m2, n2);
         v[3] = csub(m2, n2);
+    } else if constexpr (RAD == 16) {
+        // 4 x 4: DFTs over n1 of v[4 n1 + n2], twiddles w16^(n2 k1), DFTs over n2
+        const R c1 = R(0.92387953251128675613), s1 = R(0.38268343236508977173), h = R(0.70710678118654752440);
+#pragma unroll
+        for (int n2 = 0; n2 < 4; ++n2) dft4<SGN>(v[n2], v[4 + n2], v[8 + n2], v[12 + n2]);
+        // v[4 k1 + n2]
+        const R S = R(SGN);
+        v[5] = cmul(v[5], V2<R>{c1, S * s1});
+        v[6] = cmul(v[6], V2<R>{h, S * h});
+        v[7] = cmul(v[7], V2<R>{s1, S * c1});
+        v[9] = cmul(v[9], V2<R>{h, S * h});
+        v[10] = cmuli<SGN>(v[10]);
+        v[11] = cmul(v[11], V2<R>{-h, S * h});
+        v[13] = cmul(v[13], V2<R>{s1, S * c1});
+        v[14] = cmul(v[14], V2<R>{-h, S * h});
+        v[15] = cmul(v[15], V2<R>{-c1, -S * s1});
+#pragma unroll
+        for (int k1 = 0; k1 < 4; ++k1) dft4<SGN>(v[4 * k1], v[4 * k1 + 1], v[4 * k1 + 2], v[4 * k1 + 3]);
+        // v[4 k1 + k2] is output k1 + 4 k2: transpose
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = i + 1; j < 4; ++j) {
+                const V2<R> t = v[4 * i + j];
+                v[4 * i + j] = v[4 * j + i];
+                v[4 * j + i] = t;
+            }
     } else {
         static_assert(RAD == 8, "radix");
         const R h = R(0.70710678118654752440);
@@ -156,11 +189,14 @@ __device__ __forceinline__ void smem_fft_pass(const V2<R> *__restrict__ a, V2<R>
         }
         dft<RAD, SGN>(v);
         const int base = q * ns * RAD + k;
-        if ((ns & 7) == 0 || (ns == 1 && RAD == 8)) {
-            V2<R> *o = b + smem_fft_pad(base) * NC + c;
+        V2<R> *o = b + smem_fft_pad(base) * NC + c;
+        if ((ns & 7) == 0) {
             const int os = (ns + (ns >> 3)) * NC;
 #pragma unroll
             for (int r = 0; r < RAD; ++r) o[r * os] = v[r];
+        } else if (RAD % 8 == 0 && ns == 1) {
+#pragma unroll
+            for (int r = 0; r < RAD; ++r) o[(r + (r >> 3)) * NC] = v[r];
         } else {
 #pragma unroll
             for (int r = 0; r < RAD; ++r) b[smem_fft_pad(base + r * ns) * NC + c] = v[r];
@@ -180,7 +216,8 @@ __device__ V2<R> *smem_fft(V2<R> *a, V2<R> *b, const SmemFft &p, const V2<R> *__
     for (int q = 0; q < p.np; ++q) {
         const int r = p.rad[q];
         const unsigned mag = p.mag[q];
-        if (r == 8) smem_fft_pass<8, NC, SGN, R>(a, b, p.n, ns, mag, tw);
+        if (r == 16) smem_fft_pass<16, NC, SGN, R>(a, b, p.n, ns, mag, tw);
+        else if (r == 8) smem_fft_pass<8, NC, SGN, R>(a, b, p.n, ns, mag, tw);
         else if (r == 4) smem_fft_pass<4, NC, SGN, R>(a, b, p.n, ns, mag, tw);
         else if (r == 5) smem_fft_pass<5, NC, SGN, R>(a, b, p.n, ns, mag, tw);
         else if (r == 3) smem_fft_pass<3, NC, SGN, R>(a, b, p.n, ns, mag, tw);
