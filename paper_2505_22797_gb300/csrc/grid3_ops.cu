@@ -11,7 +11,7 @@
 // work units of at most kUnitLen samples and combined per node in a fixed
 // order (no float atomics, run-to-run identical), CG vectors and inner
 // products in FP64.
-#include "grid_common.cuh"
+#include "core_resident.cuh"
 
 namespace mpi {
 
@@ -58,13 +58,13 @@ __device__ __forceinline__ InterpRec3<R> make_rec3(R px, R py, R pz, const Axes3
 // records precomputed): the field is node-interleaved, A4[node K + k] =
 // (A_{3k}, A_{3k+1}, A_{3k+2}, 0) with K rows, so a corner's three
 // components are one 16-byte load.
-template <typename R, typename AT, int CH, bool PRE, bool IL = false>
-__global__ void __launch_bounds__(256)
-k_interp3(int64_t T, const R *__restrict__ r, const InterpRec3<R> *__restrict__ rec,
-          const R *__restrict__ v, const AT *__restrict__ A, Axes3 ax, R *__restrict__ s)
+// COH: the field is written during the launch.
+template <typename R, typename AT, int CH, bool PRE, bool IL, bool COH>
+__device__ __forceinline__ void interp3_outputs(int64_t T, const R *__restrict__ r, const InterpRec3<R> *__restrict__ rec,
+                                                const R *__restrict__ v, const AT *A, int nx, int ny, int nz,
+                                                const Axes3 &ax, R *s)
 {
-    const int nx = ax.x.n, ny = ax.y.n;
-    const int64_t N = (int64_t)nx * ny * ax.z.n;
+    const int64_t N = (int64_t)nx * ny * nz;
     constexpr int K = CH < 0 ? 3 : 1;
     for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < K * T;
          e += (int64_t)gridDim.x * blockDim.x) {
@@ -75,7 +75,7 @@ k_interp3(int64_t T, const R *__restrict__ r, const InterpRec3<R> *__restrict__ 
         else q = make_rec3<R>(r[3 * t], r[3 * t + 1], r[3 * t + 2], ax);
         const R vv[3] = {v[3 * t], v[3 * t + 1], v[3 * t + 2]};
         const int i0 = q.i0, j0 = q.j0, l0 = q.l0;
-        const int i1 = nx > 1 ? i0 + 1 : i0, j1 = ny > 1 ? j0 + 1 : j0, l1 = ax.z.n > 1 ? l0 + 1 : l0;
+        const int i1 = nx > 1 ? i0 + 1 : i0, j1 = ny > 1 ? j0 + 1 : j0, l1 = nz > 1 ? l0 + 1 : l0;
         const R wx1 = q.wx1, wy1 = q.wy1, wz1 = q.wz1;
         const R wx0 = R(1) - wx1, wy0 = R(1) - wy1, wz0 = R(1) - wz1;
         const int64_t r00 = ((int64_t)l0 * ny + j0) * nx, r01 = ((int64_t)l0 * ny + j1) * nx;
@@ -83,10 +83,9 @@ k_interp3(int64_t T, const R *__restrict__ r, const InterpRec3<R> *__restrict__ 
         R acc = R(0);
         if constexpr (IL) {
             const float4 *A4 = reinterpret_cast<const float4 *>(A);
-            const float4 a000 = A4[(r00 + i0) * K + k], a100 = A4[(r00 + i1) * K + k];
-            const float4 a010 = A4[(r01 + i0) * K + k], a110 = A4[(r01 + i1) * K + k];
-            const float4 a001 = A4[(r10 + i0) * K + k], a101 = A4[(r10 + i1) * K + k];
-            const float4 a011 = A4[(r11 + i0) * K + k], a111 = A4[(r11 + i1) * K + k];
+            auto ld = [&](int64_t node) { return ld_shared_by_blocks<COH>(A4 + node * K + k); };
+            const float4 a000 = ld(r00 + i0), a100 = ld(r00 + i1), a010 = ld(r01 + i0), a110 = ld(r01 + i1);
+            const float4 a001 = ld(r10 + i0), a101 = ld(r10 + i1), a011 = ld(r11 + i0), a111 = ld(r11 + i1);
             auto tri = [&](float c000, float c100, float c010, float c110, float c001, float c101, float c011,
                            float c111) {
                 const R lo = wy0 * (wx0 * c000 + wx1 * c100) + wy1 * (wx0 * c010 + wx1 * c110);
@@ -109,6 +108,14 @@ k_interp3(int64_t T, const R *__restrict__ r, const InterpRec3<R> *__restrict__ 
         }
         s[e] = acc;
     }
+}
+
+template <typename R, typename AT, int CH, bool PRE, bool IL = false>
+__global__ void __launch_bounds__(256)
+k_interp3(int64_t T, const R *__restrict__ r, const InterpRec3<R> *__restrict__ rec,
+          const R *__restrict__ v, const AT *__restrict__ A, Axes3 ax, R *__restrict__ s)
+{
+    interp3_outputs<R, AT, CH, PRE, IL, false>(T, r, rec, v, A, ax.x.n, ax.y.n, ax.z.n, ax, s);
 }
 
 template <typename R>
@@ -173,18 +180,17 @@ __device__ __forceinline__ V2<double> cell_pair(const SumAcc<double> &a) { retur
 // the cell's corner-`corner` sum of w_dx w_dy w_dz v_m s_k (CH < 0: 9 sums,
 // component 3k + m; CH = k: channel k only, 3 sums).  cell_cnt: zero on entry
 // and on exit.
-template <typename R, int CH>
-__global__ void __launch_bounds__(kUnitThreads)
-k_interp3_T_cells(const InterpRec3<R> *__restrict__ rec, const R *__restrict__ vs, const R *__restrict__ s,
-                  int64_t T, const int *__restrict__ offset, const int *__restrict__ cunit_off,
-                  const int *__restrict__ unit_cell, const int *__restrict__ n_units_dev, int n_iter,
-                  R *__restrict__ unit_part, V2<R> *__restrict__ cell_part, unsigned *__restrict__ cell_cnt)
+// COH: s is written during the launch.
+template <typename R, int CH, bool COH>
+__device__ __forceinline__ void T3_units(const InterpRec3<R> *__restrict__ rec, const R *__restrict__ vs, const R *s,
+                                         int64_t T, const int *__restrict__ offset, const int *__restrict__ cunit_off,
+                                         const int *__restrict__ unit_cell, int n_units, R *unit_part, V2<R> *cell_part,
+                                         unsigned *cell_cnt)
 {
     constexpr int NC = CH < 0 ? 9 : 3;
     const int lane = threadIdx.x & 31, corner = lane & 7, g = lane >> 3;
     const int dx = corner & 1, dy = (corner >> 1) & 1, dz = corner >> 2;
-    const int n_units = *n_units_dev;
-    for (int base = blockIdx.x * kT3UnitsPerBlock; base < n_iter; base += gridDim.x * kT3UnitsPerBlock) {
+    for (int base = blockIdx.x * kT3UnitsPerBlock; base < n_units; base += gridDim.x * kT3UnitsPerBlock) {
         const int w = base + (int)(threadIdx.x >> 5);  // warp-uniform
         if (w >= n_units) continue;
         R acc[NC];
@@ -205,13 +211,13 @@ k_interp3_T_cells(const InterpRec3<R> *__restrict__ rec, const R *__restrict__ v
             if constexpr (CH < 0) {
 #pragma unroll
                 for (int kk = 0; kk < 3; ++kk) {
-                    const R sk = wt * s[(int64_t)kk * T + q];
+                    const R sk = wt * ld_shared_by_blocks<COH>(s + (int64_t)kk * T + q);
                     acc[3 * kk] += v0 * sk;
                     acc[3 * kk + 1] += v1 * sk;
                     acc[3 * kk + 2] += v2 * sk;
                 }
             } else {
-                const R sk = wt * s[q];
+                const R sk = wt * ld_shared_by_blocks<COH>(s + q);
                 acc[0] += v0 * sk;
                 acc[1] += v1 * sk;
                 acc[2] += v2 * sk;
@@ -251,13 +257,28 @@ k_interp3_T_cells(const InterpRec3<R> *__restrict__ rec, const R *__restrict__ v
     }
 }
 
+template <typename R, int CH>
+__global__ void __launch_bounds__(kUnitThreads)
+k_interp3_T_cells(const InterpRec3<R> *__restrict__ rec, const R *__restrict__ vs, const R *__restrict__ s,
+                  int64_t T, const int *__restrict__ offset, const int *__restrict__ cunit_off,
+                  const int *__restrict__ unit_cell, const int *__restrict__ n_units_dev,
+                  R *__restrict__ unit_part, V2<R> *__restrict__ cell_part, unsigned *__restrict__ cell_cnt)
+{
+    T3_units<R, CH, false>(rec, vs, s, T, offset, cunit_off, unit_cell, *n_units_dev, unit_part, cell_part, cell_cnt);
+}
+
 // The combine of one node (at i, j, l), all NC components: the sums, over
 // the node's adjacent non-empty cells in ascending cell order, of the cell
 // sums of the corner the node is in that cell.
-template <typename R, int NC>
+__device__ __forceinline__ V2<float> ld_pair_cg(const V2<float> *p)
+{
+    const float2 q = __ldcg(reinterpret_cast<const float2 *>(p));
+    return V2<float>{q.x, q.y};
+}
+template <typename R, int NC, bool COH = false>
 __device__ __forceinline__ void node_combine3(int i, int j, int l, int ncx, int ncy, int ncz,
                                               const int *__restrict__ cunit_off,
-                                              const V2<R> *__restrict__ cell_part, SumAcc<R> (&sum)[NC])
+                                              const V2<R> *cell_part, SumAcc<R> (&sum)[NC])
 {
 #pragma unroll
     for (int dz = 1; dz >= 0; --dz)
@@ -272,7 +293,10 @@ __device__ __forceinline__ void node_combine3(int i, int j, int l, int ncx, int 
                 if (cunit_off[cc + 1] == u0) continue;
                 const V2<R> *cp = cell_part + ((int64_t)u0 * 8 + dx + 2 * dy + 4 * dz) * NC;
 #pragma unroll
-                for (int m = 0; m < NC; ++m) cell_add(sum[m], cp[m]);
+                for (int m = 0; m < NC; ++m) {
+                    if constexpr (COH) cell_add(sum[m], ld_pair_cg(cp + m));
+                    else cell_add(sum[m], cp[m]);
+                }
             }
 }
 
@@ -312,15 +336,17 @@ __device__ __forceinline__ double lap3_at(const double *__restrict__ f, int64_t 
     return f[k + xm] + f[k + xp] + f[k + ym] + f[k + yp] + f[k + zm] + f[k + zp] - 6.0 * f[k];
 }
 // The same in double-float arithmetic (coefficients as double-float pairs).
-__device__ __forceinline__ df lap3_at(const df *__restrict__ f, int64_t k, int i, int j, int l, int nx, int ny,
+template <bool COH = false>
+__device__ __forceinline__ df lap3_at(const df *f, int64_t k, int i, int j, int l, int nx, int ny,
                                       int nz, bool scaled, Coef3<df> c)
 {
+    auto at = [&](int64_t e) { return ld_shared_by_blocks<COH>(f + e); };
     const int64_t sx = 1, sy = nx, sz = (int64_t)nx * ny;
     const int64_t xm = i > 0 ? -sx : 0, xp = i < nx - 1 ? sx : 0;
     const int64_t ym = j > 0 ? -sy : 0, yp = j < ny - 1 ? sy : 0;
     const int64_t zm = l > 0 ? -sz : 0, zp = l < nz - 1 ? sz : 0;
-    const df c0 = f[k];
-    const df ax = df_add(f[k + xm], f[k + xp]), ay = df_add(f[k + ym], f[k + yp]), az = df_add(f[k + zm], f[k + zp]);
+    const df c0 = at(k);
+    const df ax = df_add(at(k + xm), at(k + xp)), ay = df_add(at(k + ym), at(k + yp)), az = df_add(at(k + zm), at(k + zp));
     if (scaled) {
         const df m2 = make_float2(-2.0f, 0.0f);
         return df_add(df_add(df_mul(df_axpy(ax, m2, c0), c.x), df_mul(df_axpy(ay, m2, c0), c.y)),
@@ -403,8 +429,7 @@ struct Bins3 {
     void *unit_part;  // 8 corners x (9 or 3) sums per unit
     void *cell_part;  // V2<R>: the cell's corner sums, at its first unit's slot
     unsigned *cell_cnt;  // per-cell arrival counters of the units
-    int n_units_max;  // bound on the units (allocation)
-    int n_units = -1;  // the exact count when read back to the host, else -1
+    int n_units_max;  // bound on the units (allocation); the count is on the device, cunit_off[n_cells]
     int ncx, ncy, ncz;
 };
 
@@ -527,12 +552,7 @@ int launch_interp3_T_units(int64_t T, const R *s_sorted, const Bins3 &b, cudaStr
 {
     const int nc = b.ncx * b.ncy * b.ncz;
     constexpr int per_block = kT3UnitsPerBlock;
-    // Blocks for the exact unit count where the host has it, else for the
-    // bound (the real count is on the device, cunit_off[nc], and surplus
-    // blocks exit at once).
-    const int units = b.n_units >= 0 ? b.n_units : b.n_units_max;
-    const int n_iter = (units + per_block - 1) / per_block * per_block;
-    const unsigned blocks = (unsigned)std::max(1, std::min(n_iter / per_block, 65535));
+    const unsigned blocks = unit_blocks(b.n_units_max, per_block);
     const InterpRec3<R> *rec = static_cast<const InterpRec3<R> *>(b.rec);
     const R *vs = static_cast<const R *>(b.vs);
     R *part = static_cast<R *>(b.unit_part);
@@ -540,11 +560,11 @@ int launch_interp3_T_units(int64_t T, const R *s_sorted, const Bins3 &b, cudaStr
     const int *n_units = b.cunit_off + nc;
     if (ch < 0)
         k_interp3_T_cells<R, -1><<<blocks, kUnitThreads, 0, st>>>(rec, vs, s_sorted, T, b.offset, b.cunit_off,
-                                                                  b.unit_cell, n_units, n_iter, part, cpart,
+                                                                  b.unit_cell, n_units, part, cpart,
                                                                   b.cell_cnt);
     else
         k_interp3_T_cells<R, 0><<<blocks, kUnitThreads, 0, st>>>(rec, vs, s_sorted, T, b.offset, b.cunit_off,
-                                                                 b.unit_cell, n_units, n_iter, part, cpart,
+                                                                 b.unit_cell, n_units, part, cpart,
                                                                  b.cell_cnt);
     MPI_CHECK_LAUNCH();
     return MPI_OK;
@@ -567,6 +587,45 @@ int launch_interp3_T(const G3 &g, int64_t T, const R *s_sorted, const Bins3 &b, 
     MPI_CHECK_LAUNCH();
     return MPI_OK;
 }
+
+// The 3-D operator of the one-launch solve (core_resident.cuh).
+template <int CH>
+struct Resident3 {
+    static constexpr int kNC = CH < 0 ? 9 : 3, kPhases = 2, kRows = CH < 0 ? 3 : 1;
+    int nx, ny, nz, ncx, ncy, ncz;
+    bool scaled;
+    Coef3<df> c;
+    df scale, gamma;
+    int64_t T;
+    const InterpRec3<float> *rec;
+    const float *vs;
+    const int *offset, *cunit_off, *unit_cell;
+    float *s, *unit_part, *p32;
+    V2<float> *cell_part;
+    unsigned *cell_cnt;
+
+    __device__ __forceinline__ void phase(int k) const
+    {
+        if (k == 0)
+            interp3_outputs<float, float, CH, true, true, true>(T, nullptr, rec, vs, p32, nx, ny, nz, Axes3{}, s);
+        else
+            T3_units<float, CH, true>(rec, vs, s, T, offset, cunit_off, unit_cell, cunit_off[ncx * ncy * ncz], unit_part,
+                                      cell_part, cell_cnt);
+    }
+    __device__ __forceinline__ void combine(int node, SumAcc<float> (&sum)[kNC]) const
+    {
+        node_combine3<float, kNC, true>(node % nx, (node / nx) % ny, node / (nx * ny), ncx, ncy, ncz, cunit_off,
+                                        cell_part, sum);
+    }
+    __device__ __forceinline__ df lap(const df *f, int node) const
+    {
+        return lap3_at<true>(f, node, node % nx, (node / nx) % ny, node / (nx * ny), nx, ny, nz, scaled, c);
+    }
+    __device__ __forceinline__ void store_p32(int node, const float *v) const
+    {
+        p32_store<kRows == 3 ? kP32Rows3x4 : kP32Rows1x4>(p32, node, v);
+    }
+};
 
 // The 3-D Core Stage operator: (1/T) M^T M through the binned records and
 // the 7-point Laplacian of each component.  A step: l2 = gamma Lap Lap p on
@@ -598,6 +657,23 @@ struct GridOp3 final : CoreStageOp<typename CsElem<R>::type> {
         if constexpr (sizeof(R) == 4)
             return P32{reinterpret_cast<float *>(p_il), ch < 0 ? kP32Rows3x4 : kP32Rows1x4, g.n()};
         return P32{};
+    }
+    template <int CH>
+    int resident_as(const E *b, const mpi_grid_opts &o, E *x, CsScal *sc, cudaStream_t st, bool &taken)
+    {
+        E *tag = nullptr;
+        Resident3<CH> d{g.nx, g.ny, g.nz, bins.ncx, bins.ncy, bins.ncz, scaled, lap_coef(), cs_host_scalar(invT, tag),
+                        cs_host_scalar(o.gamma, tag), T, static_cast<const InterpRec3<float> *>(bins.rec),
+                        static_cast<const float *>(bins.vs), bins.offset, bins.cunit_off, bins.unit_cell, s_tmp,
+                        static_cast<float *>(bins.unit_part), reinterpret_cast<float *>(p_il),
+                        static_cast<V2<float> *>(bins.cell_part), bins.cell_cnt};
+        return launch_resident(d, g.n(), T / 8, b, o, x, sc, st, taken);
+    }
+    int resident(const E *b, const mpi_grid_opts &o, E *x, CsScal *sc, cudaStream_t st, bool &taken) override
+    {
+        if constexpr (sizeof(R) == 4)
+            return ch < 0 ? resident_as<-1>(b, o, x, sc, st, taken) : resident_as<0>(b, o, x, sc, st, taken);
+        return MPI_OK;
     }
     int pq_blocks(int64_t) const override { return (int)((g.n() + kQThreads3 - 1) / kQThreads3); }
     int step_q(const E *p, double gamma, E *q, double *pq_part, CsScal *sc, E *l1, E *l2, const StepFork &fk,
@@ -663,19 +739,6 @@ int grid3_impl(const G3 &g, const mpi_traj *tr, const void *s_in, const mpi_grid
 
     MPI_TRY(build_bins3<R>(g, T, r, v, bins, st));
     MPI_TRY(gather_rows<R>(T, rows, bins.list, s, s_data, st));
-    // The transpose runs a few thousand times with the same units: read their
-    // count once, so every launch covers exactly them.
-    {
-        const int n_cells = bins.ncx * bins.ncy * bins.ncz;
-        int n_units = 0;
-        MPI_TRY_CUDA(cudaMemcpyAsync(&n_units, bins.cunit_off + n_cells, sizeof(int), cudaMemcpyDeviceToHost, st));
-        MPI_TRY_CUDA(cudaStreamSynchronize(st));
-        if (n_units < 0 || n_units > bins.n_units_max) {
-            set_error("3-D Core Stage: %d work units exceed the bound %d", n_units, bins.n_units_max);
-            return MPI_ERR_CUDA;
-        }
-        bins.n_units = n_units;
-    }
     GridOp3<R> op(g, T, ch, bins, scr.at<R>(o_s), scr.at<float4>(o_pr), o.lap_scaled != 0);
     MPI_TRY((launch_interp3_T<R, E>(g, T, s_data, bins, b, op.invT, st, ch)));
     MPI_TRY(core_stage_cg<E>(op, nv, b, o, x, n_iter_out, st));

@@ -56,6 +56,9 @@ constexpr int kUnitLen = 128;
 constexpr int kUnitLanes = 8;     // lanes per unit
 constexpr int kUnitThreads = 256;
 
+// Blocks of a pass over at most n_units_max work units (grid_ops.cu).
+unsigned unit_blocks(int n_units_max, int per_block);
+
 inline int grid_blocks(int64_t n) { return (int)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, 8192)); }
 
 // count[c] += 1 for each lane's cell c (c < 0: none); lanes that hold the
@@ -260,6 +263,29 @@ struct P32 {
     int64_t N = 0;
 };
 
+#ifdef __CUDACC__
+// Components per node, and the store of one node's.
+template <int L>
+constexpr int p32_nc()
+{
+    return L == kP32Node4 ? 4 : L == kP32Node2 ? 2 : L == kP32Rows3x4 ? 9 : 3;
+}
+template <int L>
+__device__ __forceinline__ void p32_store(float *buf, int64_t node, const float *v)
+{
+    if constexpr (L == kP32Node4) {
+        reinterpret_cast<float4 *>(buf)[node] = make_float4(v[0], v[1], v[2], v[3]);
+    } else if constexpr (L == kP32Node2) {
+        reinterpret_cast<float2 *>(buf)[node] = make_float2(v[0], v[1]);
+    } else {
+        constexpr int K = p32_nc<L>() / 3;
+#pragma unroll
+        for (int k = 0; k < K; ++k)
+            reinterpret_cast<float4 *>(buf)[node * K + k] = make_float4(v[3 * k], v[3 * k + 1], v[3 * k + 2], 0.0f);
+    }
+}
+#endif
+
 // A side stream for work of a step that is independent of its main chain:
 // forked from and joined back into the step's stream with the two events
 // (inside a graph capture this makes parallel branches).
@@ -282,6 +308,13 @@ struct CoreStageOp {
     // pq_blocks(nv) fixed blocks, finished by the producing kernel with
     // cs_finish_pq on sc.  l1, l2: work vectors of nv values.
     virtual int pq_blocks(int64_t nv) const = 0;
+    // The whole solve in one cooperative launch, if the problem is small
+    // enough for the device to hold (taken); sc receives the update count.
+    virtual int resident(const E *, const mpi_grid_opts &, E *, CsScal *, cudaStream_t, bool &taken)
+    {
+        taken = false;
+        return MPI_OK;
+    }
     virtual int step_q(const E *p, double gamma, E *q, double *pq_part, CsScal *sc, E *l1, E *l2,
                        const StepFork &fk, cudaStream_t st) = 0;
 };

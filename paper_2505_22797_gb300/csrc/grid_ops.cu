@@ -8,6 +8,7 @@
 // per-cell sort by sample index give every cell a fixed sample order), and
 // each node gathers from its (up to) four adjacent cells.  All of it is
 // memory/latency bound.
+#include "core_resident.cuh"
 #include "graph.cuh"
 #include "grid_common.cuh"
 
@@ -50,10 +51,11 @@ template <typename R, int NCOMP> struct NodeVec;
 template <> struct NodeVec<float, 4> { using T = float4; };
 template <> struct NodeVec<float, 2> { using T = float2; };
 
-template <typename R, int NCOMP>
-__device__ __forceinline__ void load_node(const R *__restrict__ A, int64_t node, R (&out)[NCOMP])
+template <typename R, int NCOMP, bool COH = false>
+__device__ __forceinline__ void load_node(const R *A, int64_t node, R (&out)[NCOMP])
 {
-    const typename NodeVec<R, NCOMP>::T q = reinterpret_cast<const typename NodeVec<R, NCOMP>::T *>(A)[node];
+    using V = typename NodeVec<R, NCOMP>::T;
+    const V q = ld_shared_by_blocks<COH>(reinterpret_cast<const V *>(A) + node);
     if constexpr (NCOMP == 4) { out[0] = q.x; out[1] = q.y; out[2] = q.z; out[3] = q.w; }
     else { out[0] = q.x; out[1] = q.y; }
 }
@@ -165,14 +167,14 @@ __global__ void k_cunit_fill(int n_cells, const int *__restrict__ cunit_off, int
 // Corner sums of one unit: for the corners (dx, dy) of the unit's cell
 // (corner index dx + 2 dy) and the NC components, the sum over the unit's
 // entries of w_dx w_dy v_m s_k, with rec, vs and s in list (cell) order.
-// CH = k: only channel k (s one row, two components).  n_iter: the unit
-// bound rounded up to whole blocks, so every warp runs the same iterations
-// and its shuffles see full warps.
+// CH = k: only channel k (s one row, two components).  The units are rounded
+// up to whole blocks, so every warp runs the same iterations and its shuffles
+// see full warps.
 template <typename R, int CH>
 __global__ void __launch_bounds__(kUnitThreads)
 k_interp_T_cells(const InterpRec<R> *__restrict__ rec, const R *__restrict__ vs, const R *__restrict__ s,
                  int64_t T, const int *__restrict__ offset, const int *__restrict__ cunit_off,
-                 const int *__restrict__ unit_cell, const int *__restrict__ n_units_dev, int n_iter,
+                 const int *__restrict__ unit_cell, const int *__restrict__ n_units_dev,
                  R *__restrict__ unit_part)
 {
     constexpr int NC = CH < 0 ? 4 : 2;
@@ -180,6 +182,7 @@ k_interp_T_cells(const InterpRec<R> *__restrict__ rec, const R *__restrict__ vs,
     constexpr int per_block = kUnitThreads / G;
     const int sub = threadIdx.x % G;
     const int n_units = *n_units_dev;
+    const int n_iter = (n_units + per_block - 1) / per_block * per_block;
     for (int base = blockIdx.x * per_block; base < n_iter; base += gridDim.x * per_block) {
         const int w = base + (int)threadIdx.x / G;
         R acc[4][NC];
@@ -236,20 +239,20 @@ k_interp_T_cells(const InterpRec<R> *__restrict__ rec, const R *__restrict__ vs,
 // once (record and velocity) instead of gathered, stored and read again.
 // IL: the field node-interleaved in R (NC components per node), else
 // component-major in AT; CH = k: only channel k (two components).
-template <typename R, typename AT, int CH, bool IL>
-__global__ void __launch_bounds__(kUnitThreads)
-k_interp_normal_cells(const InterpRec<R> *__restrict__ rec, const R *__restrict__ vs, const AT *__restrict__ A,
-                      int nx, int ny, int ncx, const int *__restrict__ offset, const int *__restrict__ cunit_off,
-                      const int *__restrict__ unit_cell, const int *__restrict__ n_units_dev, int n_iter,
-                      R *__restrict__ unit_part)
+// COH: the field is written during the launch.
+template <typename R, typename AT, int CH, bool IL, bool COH>
+__device__ __forceinline__ void
+normal_units(const InterpRec<R> *__restrict__ rec, const R *__restrict__ vs, const AT *A, int nx, int ny, int ncx,
+             const int *__restrict__ offset, const int *__restrict__ cunit_off, const int *__restrict__ unit_cell,
+             int n_units, R *unit_part)
 {
     constexpr int K = CH < 0 ? 2 : 1;
     constexpr int NC = 2 * K;
     constexpr int G = kUnitLanes;
     constexpr int per_block = kUnitThreads / G;
     const int sub = threadIdx.x % G;
-    const int n_units = *n_units_dev;
     const int64_t N = (int64_t)nx * ny;
+    const int n_iter = (n_units + per_block - 1) / per_block * per_block;
     for (int base = blockIdx.x * per_block; base < n_iter; base += gridDim.x * per_block) {
         const int w = base + (int)threadIdx.x / G;
         R acc[4][NC];
@@ -268,7 +271,7 @@ k_interp_normal_cells(const InterpRec<R> *__restrict__ rec, const R *__restrict_
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 if constexpr (IL) {
-                    load_node<R, NC>(reinterpret_cast<const R *>(A), nodes[k], f[k]);
+                    load_node<R, NC, COH>(reinterpret_cast<const R *>(A), nodes[k], f[k]);
                 } else {
 #pragma unroll
                     for (int e = 0; e < NC; ++e) f[k][e] = R(A[(int64_t)e * N + nodes[k]]);
@@ -316,13 +319,23 @@ k_interp_normal_cells(const InterpRec<R> *__restrict__ rec, const R *__restrict_
     }
 }
 
+template <typename R, typename AT, int CH, bool IL>
+__global__ void __launch_bounds__(kUnitThreads)
+k_interp_normal_cells(const InterpRec<R> *__restrict__ rec, const R *__restrict__ vs, const AT *__restrict__ A,
+                      int nx, int ny, int ncx, const int *__restrict__ offset, const int *__restrict__ cunit_off,
+                      const int *__restrict__ unit_cell, const int *__restrict__ n_units_dev,
+                      R *__restrict__ unit_part)
+{
+    normal_units<R, AT, CH, IL, false>(rec, vs, A, nx, ny, ncx, offset, cunit_off, unit_cell, *n_units_dev, unit_part);
+}
+
 // sum[m] += the unit sums of `corner` of units w0 .. w1 - 1, in unit order.
 // Four units' values are loaded before they are added: the additions depend
 // on one another, the loads do not, and a node beside a dense cell adds tens
 // of units (one L2 round trip each when every load waits for the previous
 // addition).
-template <typename R, int NC>
-__device__ __forceinline__ void add_unit_sums(const R *__restrict__ unit_part, int w0, int w1, int corner,
+template <typename R, int NC, bool COH = false>
+__device__ __forceinline__ void add_unit_sums(const R *unit_part, int w0, int w1, int corner,
                                               SumAcc<R> (&sum)[NC])
 {
     int w = w0;
@@ -331,7 +344,7 @@ __device__ __forceinline__ void add_unit_sums(const R *__restrict__ unit_part, i
 #pragma unroll
         for (int u = 0; u < 4; ++u)
 #pragma unroll
-            for (int m = 0; m < NC; ++m) v[u][m] = unit_part[((int64_t)(w + u) * 4 + corner) * NC + m];
+            for (int m = 0; m < NC; ++m) v[u][m] = ld_shared_by_blocks<COH>(unit_part + ((int64_t)(w + u) * 4 + corner) * NC + m);
 #pragma unroll
         for (int u = 0; u < 4; ++u)
 #pragma unroll
@@ -339,7 +352,7 @@ __device__ __forceinline__ void add_unit_sums(const R *__restrict__ unit_part, i
     }
     for (; w < w1; ++w)
 #pragma unroll
-        for (int m = 0; m < NC; ++m) sum[m].add(unit_part[((int64_t)w * 4 + corner) * NC + m]);
+        for (int m = 0; m < NC; ++m) sum[m].add(ld_shared_by_blocks<COH>(unit_part + ((int64_t)w * 4 + corner) * NC + m));
 }
 
 // Ahat_m(node) = scale * the sum, over the node's adjacent cells (row-major
@@ -384,8 +397,7 @@ struct Bins {
     // of each unit; 4 corners x 4 partial sums per unit.
     int *cunit_cnt, *cunit_off, *unit_cell;
     void *unit_part;
-    int n_units_max;   // bound on the units (allocation)
-    int n_units = -1;  // the exact count when read back to the host, else -1
+    int n_units_max;   // bound on the units (allocation); the count is on the device, cunit_off[n_cells]
     int ncx, ncy;
 };
 
@@ -493,6 +505,14 @@ static int launch_interp(const GridH &g, int64_t T, const R *r, const R *v, cons
     return MPI_OK;
 }
 
+// Blocks of a pass over the units: the bound counts every cell non-empty, so
+// beyond 16 per SM the blocks stride (the count itself is on the device, and
+// reading it back would leave the GPU idle for the round trip).
+unsigned unit_blocks(int n_units_max, int per_block)
+{
+    return (unsigned)std::max(1, std::min((n_units_max + per_block - 1) / per_block, 16 * device_sm_count()));
+}
+
 // The transpose's unit sums (k_interp_T_cells) into b.unit_part.
 // s_sorted: the samples' values in list order ([rows][T]).
 template <typename R>
@@ -500,22 +520,17 @@ static int launch_interp_T_units(int64_t T, const R *s_sorted, const Bins &b, cu
 {
     const int nc = b.ncx * b.ncy;
     constexpr int per_block = kUnitThreads / kUnitLanes;
-    // Blocks for the exact unit count where the host has it, else for the
-    // bound (every cell counted non-empty): the real count is on the device
-    // and the surplus blocks exit at once.
-    const int units = b.n_units >= 0 ? b.n_units : b.n_units_max;
-    const int n_iter = (units + per_block - 1) / per_block * per_block;
-    const unsigned blocks = (unsigned)std::max(1, std::min(n_iter / per_block, 65535));
+    const unsigned blocks = unit_blocks(b.n_units_max, per_block);
     const InterpRec<R> *rec = static_cast<const InterpRec<R> *>(b.rec);
     const R *vs = static_cast<const R *>(b.vs);
     R *part = static_cast<R *>(b.unit_part);
     const int *n_units = b.cunit_off + nc;
     if (ch < 0)
         k_interp_T_cells<R, -1><<<blocks, kUnitThreads, 0, st>>>(rec, vs, s_sorted, T, b.offset, b.cunit_off,
-                                                                 b.unit_cell, n_units, n_iter, part);
+                                                                 b.unit_cell, n_units, part);
     else
         k_interp_T_cells<R, 0><<<blocks, kUnitThreads, 0, st>>>(rec, vs, s_sorted, T, b.offset, b.cunit_off,
-                                                                b.unit_cell, n_units, n_iter, part);
+                                                                b.unit_cell, n_units, part);
     MPI_CHECK_LAUNCH();
     return MPI_OK;
 }
@@ -544,19 +559,17 @@ static int launch_normal_units(const GridH &g, const Bins &b, const AT *A, int c
 {
     const int nc = b.ncx * b.ncy;
     constexpr int per_block = kUnitThreads / kUnitLanes;
-    const int units = b.n_units >= 0 ? b.n_units : b.n_units_max;
-    const int n_iter = (units + per_block - 1) / per_block * per_block;
-    const unsigned blocks = (unsigned)std::max(1, std::min(n_iter / per_block, 65535));
+    const unsigned blocks = unit_blocks(b.n_units_max, per_block);
     const InterpRec<R> *rec = static_cast<const InterpRec<R> *>(b.rec);
     const R *vs = static_cast<const R *>(b.vs);
     R *part = static_cast<R *>(b.unit_part);
     const int *n_units = b.cunit_off + nc;
     if (ch < 0)
         k_interp_normal_cells<R, AT, -1, IL><<<blocks, kUnitThreads, 0, st>>>(
-            rec, vs, A, g.nx, g.ny, b.ncx, b.offset, b.cunit_off, b.unit_cell, n_units, n_iter, part);
+            rec, vs, A, g.nx, g.ny, b.ncx, b.offset, b.cunit_off, b.unit_cell, n_units, part);
     else
         k_interp_normal_cells<R, AT, 0, IL><<<blocks, kUnitThreads, 0, st>>>(
-            rec, vs, A, g.nx, g.ny, b.ncx, b.offset, b.cunit_off, b.unit_cell, n_units, n_iter, part);
+            rec, vs, A, g.nx, g.ny, b.ncx, b.offset, b.cunit_off, b.unit_cell, n_units, part);
     MPI_CHECK_LAUNCH();
     return MPI_OK;
 }
@@ -578,13 +591,14 @@ __device__ __forceinline__ double lap2_at(const double *__restrict__ f, int k, i
     return f[j * nx + im] + f[j * nx + ip] + f[jm * nx + i] + f[jp * nx + i] - 4.0 * f[k];
 }
 // The same in double-float arithmetic (cx, cy as double-float pairs).
-__device__ __forceinline__ df lap2_at(const df *__restrict__ f, int k, int i, int j, int nx, int ny, bool scaled,
-                                      df cx, df cy)
+template <bool COH = false>
+__device__ __forceinline__ df lap2_at(const df *f, int k, int i, int j, int nx, int ny, bool scaled, df cx, df cy)
 {
+    auto at = [&](int e) { return ld_shared_by_blocks<COH>(f + e); };
     const int im = i > 0 ? i - 1 : 0, ip = i < nx - 1 ? i + 1 : nx - 1;
     const int jm = j > 0 ? j - 1 : 0, jp = j < ny - 1 ? j + 1 : ny - 1;
-    const df c0 = f[k];
-    const df sx = df_add(f[j * nx + im], f[j * nx + ip]), sy = df_add(f[jm * nx + i], f[jp * nx + i]);
+    const df c0 = at(k);
+    const df sx = df_add(at(j * nx + im), at(j * nx + ip)), sy = df_add(at(jm * nx + i), at(jp * nx + i));
     if (scaled) {
         const df m2 = make_float2(-2.0f, 0.0f);
         return df_add(df_mul(df_axpy(sx, m2, c0), cx), df_mul(df_axpy(sy, m2, c0), cy));
@@ -757,26 +771,7 @@ k_cs_step2(int64_t n, const E *__restrict__ r, E *__restrict__ p, const CsScal *
 // Stage gathers FP32 values in its interpolation (GB300 converts FP64 at a
 // small fraction of the FP32 rate; a gather converting 16 or 72 values per
 // sample was bound by that conversion), and the direction update writes the
-// copy as it forms p.  Components per node:
-template <int L>
-constexpr int p32_nc()
-{
-    return L == kP32Node4 ? 4 : L == kP32Node2 ? 2 : L == kP32Rows3x4 ? 9 : 3;
-}
-template <int L>
-__device__ __forceinline__ void p32_store(float *buf, int64_t node, const float *v)
-{
-    if constexpr (L == kP32Node4) {
-        reinterpret_cast<float4 *>(buf)[node] = make_float4(v[0], v[1], v[2], v[3]);
-    } else if constexpr (L == kP32Node2) {
-        reinterpret_cast<float2 *>(buf)[node] = make_float2(v[0], v[1]);
-    } else {
-        constexpr int K = p32_nc<L>() / 3;
-#pragma unroll
-        for (int k = 0; k < K; ++k)
-            reinterpret_cast<float4 *>(buf)[node * K + k] = make_float4(v[3 * k], v[3 * k + 1], v[3 * k + 2], 0.0f);
-    }
-}
+// copy as it forms p (p32_store).
 
 // buf = p rounded to FP32 (one thread per node, all its components).
 template <typename E, int L>
@@ -873,6 +868,45 @@ __global__ void k_grid_output(int64_t N, int ch, const E *__restrict__ x, R *__r
     }
 }
 
+// The 2-D operator of the one-launch solve (core_resident.cuh).
+template <int CH>
+struct Resident2 {
+    static constexpr int kNC = CH < 0 ? 4 : 2, kPhases = 1;
+    int nx, ny, ncx, ncy;
+    bool scaled;
+    df cx, cy, scale, gamma;
+    const InterpRec<float> *rec;
+    const float *vs;
+    const int *offset, *cunit_off, *unit_cell;
+    float *unit_part, *p32;
+
+    __device__ __forceinline__ void phase(int) const
+    {
+        normal_units<float, float, CH, true, true>(rec, vs, p32, nx, ny, ncx, offset, cunit_off, unit_cell,
+                                                   cunit_off[ncx * ncy], unit_part);
+    }
+    __device__ __forceinline__ void combine(int node, SumAcc<float> (&sum)[kNC]) const
+    {
+        const int i = node % nx, j = node / nx;
+        for (int cj = j - 1; cj <= j; ++cj) {
+            if (cj < 0 || cj >= ncy) continue;
+            for (int ci = i - 1; ci <= i; ++ci) {
+                if (ci < 0 || ci >= ncx) continue;
+                const int c = cj * ncx + ci;
+                add_unit_sums<float, kNC, true>(unit_part, cunit_off[c], cunit_off[c + 1], (i - ci) + 2 * (j - cj), sum);
+            }
+        }
+    }
+    __device__ __forceinline__ df lap(const df *f, int node) const
+    {
+        return lap2_at<true>(f, node, node % nx, node / nx, nx, ny, scaled, cx, cy);
+    }
+    __device__ __forceinline__ void store_p32(int node, const float *v) const
+    {
+        p32_store<kNC == 4 ? kP32Node4 : kP32Node2>(p32, node, v);
+    }
+};
+
 // The 2-D Core Stage operator: (1/T) M^T M through the binned records and
 // the 5-point Laplacian of each component.  A step: l2 = gamma Lap Lap p on
 // the side stream (two passes) while the main chain runs M p (through the
@@ -897,6 +931,22 @@ struct GridOp2 final : CoreStageOp<typename CsElem<R>::type> {
         if constexpr (sizeof(R) == 4)
             return P32{reinterpret_cast<float *>(p_r), nc == 4 ? kP32Node4 : kP32Node2, int64_t(g.nx) * g.ny};
         return P32{};
+    }
+    template <int CH>
+    int resident_as(const E *b, const mpi_grid_opts &o, E *x, CsScal *sc, cudaStream_t st, bool &taken)
+    {
+        E *tag = nullptr;
+        Resident2<CH> d{g.nx, g.ny, bins.ncx, bins.ncy, scaled, cs_host_scalar(1.0 / (g.dx * g.dx), tag),
+                        cs_host_scalar(1.0 / (g.dy * g.dy), tag), cs_host_scalar(invT, tag), cs_host_scalar(o.gamma, tag),
+                        static_cast<const InterpRec<float> *>(bins.rec), static_cast<const float *>(bins.vs),
+                        bins.offset, bins.cunit_off, bins.unit_cell, static_cast<float *>(bins.unit_part), p_r};
+        return launch_resident(d, int64_t(g.nx) * g.ny, T / 4, b, o, x, sc, st, taken);
+    }
+    int resident(const E *b, const mpi_grid_opts &o, E *x, CsScal *sc, cudaStream_t st, bool &taken) override
+    {
+        if constexpr (sizeof(R) == 4)
+            return ch < 0 ? resident_as<-1>(b, o, x, sc, st, taken) : resident_as<0>(b, o, x, sc, st, taken);
+        return MPI_OK;
     }
     int pq_blocks(int64_t) const override { return (int)((int64_t(g.nx) * g.ny + kQThreads - 1) / kQThreads); }
     int step_q(const E *p, double gamma, E *q, double *pq_part, CsScal *sc, E *l1, E *l2, const StepFork &fk,
@@ -955,19 +1005,6 @@ static int grid_impl(const GridH &g, const mpi_traj *tr, const void *s_in, const
     MPI_TRY(build_bins<R>(g, T, r, v, bins, st));
     // The sample vectors of the solve live in list (cell) order.
     MPI_TRY(gather_rows<R>(T, rows, bins.list, s, s_data, st));
-    // The transpose runs up to thousands of times with the same units: read
-    // their count once, so every launch covers exactly them.
-    {
-        int n_units = 0;
-        MPI_TRY_CUDA(cudaMemcpyAsync(&n_units, bins.cunit_off + bins.ncx * bins.ncy, sizeof(int),
-                                     cudaMemcpyDeviceToHost, st));
-        MPI_TRY_CUDA(cudaStreamSynchronize(st));
-        if (n_units < 0 || n_units > bins.n_units_max) {
-            set_error("Core Stage: %d work units exceed the bound %d", n_units, bins.n_units_max);
-            return MPI_ERR_CUDA;
-        }
-        bins.n_units = n_units;
-    }
     GridOp2<R> op(g, T, ch, bins, scr.at<R>(o_pr), o.lap_scaled != 0);
     // b = (1/T) M^T s
     MPI_TRY((launch_interp_T<R, E>(g, T, s_data, bins, b, op.invT, st, ch)));
@@ -1015,6 +1052,21 @@ template <typename E>
 int core_stage_cg(CoreStageOp<E> &op, int64_t nv, const E *b, const mpi_grid_opts &o, E *x, int *n_iter_out,
                   cudaStream_t st)
 {
+    // Small problems: the whole solve in one launch.
+    {
+        Scratch scr(st);
+        const size_t o_sc = scr.reserve(sizeof(CsScal));
+        MPI_TRY(scr.allocate());
+        bool taken = false;
+        MPI_TRY(op.resident(b, o, x, scr.at<CsScal>(o_sc), st, taken));
+        if (taken) {
+            if (n_iter_out) {
+                MPI_TRY_CUDA(cudaMemcpyAsync(n_iter_out, &scr.at<CsScal>(o_sc)->iters, sizeof(int), cudaMemcpyDeviceToHost, st));
+                MPI_TRY_CUDA(cudaStreamSynchronize(st));
+            }
+            return MPI_OK;
+        }
+    }
     const int ncs = cs_blocks(nv);
     const int npq = op.pq_blocks(nv);
     const P32 p32 = op.p32();
@@ -1034,10 +1086,13 @@ int core_stage_cg(CoreStageOp<E> &op, int64_t nv, const E *b, const mpi_grid_opt
     // solve returns; the stream's work is joined into st by then).
     struct Fork {
         StepFork f{nullptr, nullptr, nullptr};
+        bool joined = false;
         ~Fork()
         {
             if (f.side) {
-                cudaStreamSynchronize(f.side);  // (an error path may have left a fork unjoined)
+                // (an error path may have left a fork unjoined; work that is
+                // joined into st need not be waited for here)
+                if (!joined) cudaStreamSynchronize(f.side);
                 cudaStreamDestroy(f.side);
             }
             if (f.fork) cudaEventDestroy(f.fork);
@@ -1055,12 +1110,7 @@ int core_stage_cg(CoreStageOp<E> &op, int64_t nv, const E *b, const mpi_grid_opt
     MPI_CHECK_LAUNCH();
     if (p32.buf) MPI_TRY(cs_round_launch(p32, p, st));
 
-    int *h_done = nullptr;
-    MPI_TRY_CUDA(cudaMallocHost(reinterpret_cast<void **>(&h_done), sizeof(int)));
-    struct PinnedFree {
-        int *p;
-        ~PinnedFree() { cudaFreeHost(p); }
-    } guard{h_done};
+    int h_done = 0;  // (pageable: page-locking it on each call takes longer than its copies)
     int *done = &sc->done, *iters = &sc->iters;
     const bool thresh = o.rel_tol > 0.0;
 
@@ -1074,9 +1124,9 @@ int core_stage_cg(CoreStageOp<E> &op, int64_t nv, const E *b, const mpi_grid_opt
         return cs_step2_launch(p32, nv, rr, p, sc, s);
     };
     auto poll_done = [&](bool &stop) -> int {
-        MPI_TRY_CUDA(cudaMemcpyAsync(h_done, done, sizeof(int), cudaMemcpyDeviceToHost, st));
+        MPI_TRY_CUDA(cudaMemcpyAsync(&h_done, done, sizeof(int), cudaMemcpyDeviceToHost, st));
         MPI_TRY_CUDA(cudaStreamSynchronize(st));
-        stop = *h_done != 0;
+        stop = h_done != 0;
         return MPI_OK;
     };
 
@@ -1106,10 +1156,11 @@ int core_stage_cg(CoreStageOp<E> &op, int64_t nv, const E *b, const mpi_grid_opt
         if (thresh && (it + 1) % poll == 0 && it + 1 < o.max_iter) MPI_TRY(poll_done(stop));
     }
     if (n_iter_out) {
-        MPI_TRY_CUDA(cudaMemcpyAsync(h_done, iters, sizeof(int), cudaMemcpyDeviceToHost, st));
+        MPI_TRY_CUDA(cudaMemcpyAsync(&h_done, iters, sizeof(int), cudaMemcpyDeviceToHost, st));
         MPI_TRY_CUDA(cudaStreamSynchronize(st));
-        *n_iter_out = *h_done;
+        *n_iter_out = h_done;
     }
+    fk.joined = true;
     return MPI_OK;
 }
 template int core_stage_cg<double>(CoreStageOp<double> &, int64_t, const double *, const mpi_grid_opts &, double *,
