@@ -34,14 +34,15 @@ template <bool COH, typename T> __device__ __forceinline__ T ld_shared_by_blocks
     else return *p;
 }
 
-// All threads call it; false once a wait has given up.
+// All threads call it; false once a wait has given up.  The block's writes
+// are ordered before its arrival (bar.sync, then a release by thread 0), the
+// others' after the wait (an acquire by thread 0, then bar.sync).
 __device__ __forceinline__ bool res_barrier(ResBarrier *b, unsigned long long &target, int *s_ok)
 {
     target += gridDim.x;
     __syncthreads();
     if (threadIdx.x == 0) {
-        __threadfence();
-        atomicAdd(&b->arrived, 1ull);
+        asm volatile("red.release.gpu.global.add.u64 [%0], 1;" ::"l"(&b->arrived) : "memory");
         int ok = 1, n = 0;
         unsigned long long seen;
         for (;;) {
@@ -53,7 +54,6 @@ __device__ __forceinline__ bool res_barrier(ResBarrier *b, unsigned long long &t
                 break;
             }
         }
-        __threadfence();
         *s_ok = ok;
     }
     __syncthreads();
@@ -72,14 +72,17 @@ k_cs_resident(const __grid_constant__ Op op, int N, const float2 *__restrict__ b
 {
     constexpr int NC = Op::kNC;
     __shared__ double sh[kResThreads / 32];
-    __shared__ double s_val;
-    __shared__ int s_ok;
+    __shared__ df s_coef;
+    __shared__ int s_ok, s_stop;
     unsigned long long target = 0;
     const int node = blockIdx.x * kResThreads + threadIdx.x;
     const bool in = node < N;
     bool ok = true;
-    // Sum over all threads in a fixed order, known to every thread; a barrier.
-    auto grid_sum = [&](const CsDot<df> &acc, int slot) -> double {
+    // Sum over all threads in a fixed order; a barrier.  The sum is known to
+    // thread 0 of every block, which calls then(sum): FP64 arithmetic takes a
+    // whole warp 19 clocks an instruction here, so one thread forms the
+    // step's scalars.
+    auto grid_sum = [&](const CsDot<df> &acc, int slot, auto then) {
         const double t = acc.template block_total<kResThreads>(sh);
         double *mine = part + slot * gridDim.x;
         if (threadIdx.x == 0) mine[blockIdx.x] = t;
@@ -88,13 +91,11 @@ k_cs_resident(const __grid_constant__ Op op, int N, const float2 *__restrict__ b
             double a = 0.0;
             for (int k = threadIdx.x; k < int(gridDim.x); k += 32) a += __ldcg(mine + k);
             a = warp_sum(a);
-            if (threadIdx.x == 0) s_val = a;
+            if (threadIdx.x == 0) then(a);
         }
         __syncthreads();
-        const double v = s_val;
-        __syncthreads();
-        return v;
     };
+    double rr = 0.0, tol = -1.0;  // thread 0's
     df r[NC], d[NC];
     CsDot<df> acc{};
     if (in) {
@@ -110,8 +111,10 @@ k_cs_resident(const __grid_constant__ Op op, int N, const float2 *__restrict__ b
         }
         op.store_p32(node, v);
     }
-    double rr = grid_sum(acc, 0);
-    const double tol = rel_tol > 0.0 ? rel_tol * sqrt(rr) : -1.0;
+    grid_sum(acc, 0, [&](double v) {
+        rr = v;
+        tol = rel_tol > 0.0 ? rel_tol * sqrt(v) : -1.0;
+    });
     int it = 0;
     for (; ok && it < max_iter; ++it) {
         if (in) {
@@ -135,10 +138,12 @@ k_cs_resident(const __grid_constant__ Op op, int N, const float2 *__restrict__ b
                 pq_acc.add(d[m], q[m]);
             }
         }
-        const double pq = grid_sum(pq_acc, 1);
-        if (!ok || rr == 0.0 || pq == 0.0 || (tol >= 0.0 && sqrt(rr) <= tol)) break;
-        const double alpha = rr / pq;
-        const df al = df_from_double(alpha), nal = df_neg(al);
+        grid_sum(pq_acc, 1, [&](double pq) {
+            s_stop = rr == 0.0 || pq == 0.0 || (tol >= 0.0 && sqrt(rr) <= tol);
+            s_coef = df_from_double(rr / pq);
+        });
+        if (!ok || s_stop) break;
+        const df al = s_coef, nal = df_neg(al);
         CsDot<df> rr_acc{};
         if (in) {
 #pragma unroll
@@ -149,9 +154,11 @@ k_cs_resident(const __grid_constant__ Op op, int N, const float2 *__restrict__ b
                 rr_acc.add(r[m], r[m]);
             }
         }
-        const double rr_new = grid_sum(rr_acc, 0);
-        const df be = df_from_double(rr_new / rr);
-        rr = rr_new;
+        grid_sum(rr_acc, 0, [&](double v) {
+            s_coef = df_from_double(v / rr);
+            rr = v;
+        });
+        const df be = s_coef;
         if (in) {
             float v[NC];
 #pragma unroll
