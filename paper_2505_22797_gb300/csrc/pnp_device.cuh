@@ -3,6 +3,8 @@
 // percentile/variance block and the 5-tap Gaussian tile.
 #pragma once
 
+#include <cooperative_groups.h>
+
 #include <cmath>
 
 #include "pnp_ops.cuh"
@@ -48,47 +50,6 @@ __device__ __forceinline__ double key_f64(uint64_t k)
     return __longlong_as_double((long long)b);
 }
 
-template <int NT>
-__device__ double block_select(const double *__restrict__ x, int64_t N, int64_t rank,
-                               unsigned *hist, unsigned long long *sh_u)
-{
-    uint64_t prefix = 0, mask = 0;
-    int64_t krem = rank;
-    const int lane = threadIdx.x & 31;
-    for (int shift = 56; shift >= 0; shift -= 8) {
-        for (int b = threadIdx.x; b < 256; b += NT) hist[b] = 0;
-        __syncthreads();
-        for (int64_t i0 = 0; i0 < N; i0 += NT) {
-            const int64_t i = i0 + threadIdx.x;
-            unsigned digit = 256;  // no bin
-            if (i < N) {
-                const uint64_t key = f64_key(x[i]);
-                if ((key & mask) == prefix) digit = (unsigned)((key >> shift) & 255u);
-            }
-            const unsigned peers = __match_any_sync(0xffffffffu, digit);
-            if (digit < 256 && lane == __ffs(peers) - 1) atomicAdd(&hist[digit], (unsigned)__popc(peers));
-        }
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            int64_t cum = 0;
-            unsigned d = 0;
-            for (; d < 255; ++d) {
-                if (cum + hist[d] > krem) break;
-                cum += hist[d];
-            }
-            krem -= cum;
-            sh_u[0] = prefix | ((uint64_t)d << shift);
-            sh_u[1] = (unsigned long long)krem;
-        }
-        __syncthreads();
-        prefix = sh_u[0];
-        krem = (int64_t)sh_u[1];
-        mask |= (uint64_t)255 << shift;
-        __syncthreads();
-    }
-    return key_f64(prefix);
-}
-
 // Minimum over the block (order-independent), returned to every thread.
 template <int NT>
 __device__ __forceinline__ double block_min(double v, double *sh /* >= NT/32 + 1 */)
@@ -110,7 +71,98 @@ __device__ __forceinline__ double block_min(double v, double *sh /* >= NT/32 + 1
     return r;
 }
 
-// One block computes, for the N values x: the clip value P (the pct-th
+// The percentile step runs on a cluster of kStatBlocks blocks per image
+// (distributed shared memory, cluster barriers): FP64 additions and
+// comparisons take a block's SM 19 clocks per warp, so one block alone was
+// bound by them (80 us at 100 x 100 values, a third of it one thread's walk
+// over the digit counts).  The cluster takes 53 us less there.
+constexpr int kStatBlocks = 8;
+
+struct StatShared {
+    unsigned hist[256];
+    double part[2];            // this block's partial sums / minimum, read by the others
+    unsigned long long cnt;    // this block's count, read by the others
+    double sh[kStatThreads / 32 + 1];
+    unsigned long long sel[2]; // prefix, remaining rank
+};
+
+// The values of rank `rank` (0-based) among the N: an 8-pass radix select on
+// the order-preserving integer image; every block ends with the same value.
+__device__ inline double cluster_select(const double *__restrict__ x, int64_t N, int64_t rank, StatShared &S)
+{
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int64_t first = (int64_t)cl.block_rank() * kStatThreads, stride = (int64_t)kStatBlocks * kStatThreads;
+    uint64_t prefix = 0, mask = 0;
+    int64_t krem = rank;
+    for (int shift = 56; shift >= 0; shift -= 8) {
+        if (tid < 256) S.hist[tid] = 0;
+        __syncthreads();
+        for (int64_t i0 = first; i0 < N; i0 += stride) {
+            const int64_t i = i0 + tid;
+            unsigned digit = 256;  // no bin
+            if (i < N) {
+                const uint64_t key = f64_key(x[i]);
+                if ((key & mask) == prefix) digit = (unsigned)((key >> shift) & 255u);
+            }
+            const unsigned peers = __match_any_sync(0xffffffffu, digit);
+            if (digit < 256 && lane == __ffs(peers) - 1) atomicAdd(&S.hist[digit], (unsigned)__popc(peers));
+        }
+        cl.sync();
+        if (tid < 32) {  // eight digits per lane: the digit that holds the rank
+            unsigned long long c[8], sum = 0;
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                unsigned long long n = 0;
+                for (int b = 0; b < kStatBlocks; ++b) n += *cl.map_shared_rank(&S.hist[8 * lane + q], b);
+                c[q] = n;
+                sum += n;
+            }
+            unsigned long long pre = sum;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const unsigned long long y = __shfl_up_sync(0xffffffffu, pre, o);
+                if (lane >= o) pre += y;
+            }
+            pre -= sum;
+            const unsigned long long k = (unsigned long long)krem;
+            if ((k >= pre && k < pre + sum) || (lane == 31 && k >= pre + sum)) {
+                int q = 0;
+                while (q < 7 && pre + c[q] <= k) pre += c[q++];
+                S.sel[0] = prefix | ((uint64_t)(8 * lane + q) << shift);
+                S.sel[1] = k - pre;
+            }
+        }
+        cl.sync();  // the counts are read; sel is written
+        prefix = S.sel[0];
+        krem = (int64_t)S.sel[1];
+        mask |= (uint64_t)255 << shift;
+    }
+    return key_f64(prefix);
+}
+
+// Sum of v over the cluster in a fixed order, for every thread; slot: which of
+// the two partials it uses (alternate, so no barrier is needed to reuse one).
+__device__ inline double cluster_sum(double v, int slot, StatShared &S)
+{
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    const double t = block_sum<double, kStatThreads>(v, S.sh);
+    if (threadIdx.x == 0) S.part[slot] = t;
+    cl.sync();
+    if (threadIdx.x == 0) {
+        double a = 0.0;
+        for (int b = 0; b < kStatBlocks; ++b) a += *cl.map_shared_rank(&S.part[slot], b);
+        S.sh[kStatThreads / 32] = a;
+    }
+    __syncthreads();
+    const double r = S.sh[kStatThreads / 32];
+    __syncthreads();
+    return r;
+}
+
+// One cluster computes, for the N values x: the clip value P (the pct-th
 // percentile, linear interpolation between order statistics; -inf when
 // do_clip is 0), rho1 = max(x, P) rounded to R, the population variance of
 // rho1 in two FP64 passes, and updates the PnP scalars: sigma, lambda = nu0
@@ -118,75 +170,82 @@ __device__ __forceinline__ double block_min(double v, double *sh /* >= NT/32 + 1
 // rr_part/nblk: partial sums of the final CG residual for info_row (sigma,
 // nu, residual norm, clip value: kInfoCols values).
 template <typename R>
-__device__ void outer_stats_block(int64_t N, const double *__restrict__ x, int do_clip, double pct,
-                                  bool first, double nu0, double *__restrict__ scal,
-                                  const double *__restrict__ rr_part, int nblk,
-                                  double *__restrict__ info_row, R *__restrict__ rho1)
+__device__ void outer_stats_cluster(int64_t N, const double *__restrict__ x, int do_clip, double pct,
+                                    bool first, double nu0, double *__restrict__ scal,
+                                    const double *__restrict__ rr_part, int nblk,
+                                    double *__restrict__ info_row, R *__restrict__ rho1)
 {
-    __shared__ unsigned hist[256];
-    __shared__ unsigned long long sh_u[2];
-    __shared__ double sh[kStatThreads / 32 + 1];
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    __shared__ StatShared S;
+    const int64_t i0 = (int64_t)cl.block_rank() * kStatThreads + threadIdx.x;
+    const int64_t stride = (int64_t)kStatBlocks * kStatThreads;
     double P = -INFINITY;
     if (do_clip) {
         const double h = double(N - 1) * pct / 100.0;
         const int64_t lo = (int64_t)floor(h);
         const int64_t hi = min(lo + 1, N - 1);
-        const double xlo = block_select<kStatThreads>(x, N, lo, hist, sh_u);
+        const double xlo = cluster_select(x, N, lo, S);
         // The next order statistic in one pass instead of a second select:
         // x(lo + 1) is xlo itself when more than lo + 1 values are <= xlo,
         // else the smallest value above xlo (exact, order-independent).
         double xhi = xlo;
         if (hi != lo) {
-            int64_t le = 0;
+            long long le = 0;
             double gt = INFINITY;
-            for (int64_t i = threadIdx.x; i < N; i += kStatThreads) {
+            for (int64_t i = i0; i < N; i += stride) {
                 const double v = x[i];
                 if (v <= xlo) ++le;
                 else gt = fmin(gt, v);
             }
-            le = block_sum<int64_t, kStatThreads>(le, reinterpret_cast<int64_t *>(sh));
-            if (threadIdx.x == 0) sh_u[0] = (unsigned long long)le;
-            __syncthreads();
-            le = (int64_t)sh_u[0];
-            __syncthreads();
-            gt = block_min<kStatThreads>(gt, sh);
+            le = block_sum<long long, kStatThreads>(le, reinterpret_cast<long long *>(S.sh));
+            gt = block_min<kStatThreads>(gt, S.sh);
+            if (threadIdx.x == 0) {
+                S.cnt = (unsigned long long)le;
+                S.part[1] = gt;
+            }
+            cl.sync();
+            le = 0;
+            for (int b = 0; b < kStatBlocks; ++b) {
+                le += (long long)*cl.map_shared_rank(&S.cnt, b);
+                gt = fmin(gt, *cl.map_shared_rank(&S.part[1], b));
+            }
             xhi = le > hi ? xlo : gt;
         }
         P = xlo + (h - double(lo)) * (xhi - xlo);
     }
     double s = 0.0;
-    for (int64_t i = threadIdx.x; i < N; i += kStatThreads) {
+    for (int64_t i = i0; i < N; i += stride) {
         const double v = fmax(x[i], P);
         rho1[i] = R(v);
         s += v;
     }
-    s = block_sum<double, kStatThreads>(s, sh);
-    if (threadIdx.x == 0) sh[kStatThreads / 32] = s;
-    __syncthreads();
-    const double mean = sh[kStatThreads / 32] / double(N);
-    __syncthreads();
+    const double mean = cluster_sum(s, 0, S) / double(N);
     double q = 0.0;
-    for (int64_t i = threadIdx.x; i < N; i += kStatThreads) {
+    for (int64_t i = i0; i < N; i += stride) {
         const double dv = fmax(x[i], P) - mean;
         q += dv * dv;
     }
-    q = block_sum<double, kStatThreads>(q, sh);
-    if (threadIdx.x == 0) {
+    q = cluster_sum(q, 1, S);
+    if (cl.block_rank() == 0 && threadIdx.x < 32) {
         double rr = 0.0;
-        for (int b = 0; b < nblk; ++b) rr += rr_part[b];
-        const double sigma = sqrt(q / double(N));
-        if (first) scal[kScalLambda] = nu0 * sigma * sigma;
-        if (sigma > 0.0) scal[kScalNu] = scal[kScalLambda] / (sigma * sigma);
-        scal[kScalSigma] = sigma;
-        scal[kScalPct] = P;
-        if (info_row) {
-            info_row[0] = sigma;
-            info_row[1] = scal[kScalNu];
-            info_row[2] = sqrt(rr);
-            info_row[3] = P;
+        for (int b = threadIdx.x; b < nblk; b += 32) rr += rr_part[b];
+        rr = warp_sum(rr);
+        if (threadIdx.x == 0) {
+            const double sigma = sqrt(q / double(N));
+            if (first) scal[kScalLambda] = nu0 * sigma * sigma;
+            if (sigma > 0.0) scal[kScalNu] = scal[kScalLambda] / (sigma * sigma);
+            scal[kScalSigma] = sigma;
+            scal[kScalPct] = P;
+            if (info_row) {
+                info_row[0] = sigma;
+                info_row[1] = scal[kScalNu];
+                info_row[2] = sqrt(rr);
+                info_row[3] = P;
+            }
         }
     }
-    __syncthreads();
+    cl.sync();  // no block leaves while another reads its shared memory
 }
 
 // ---------------------------------------------------------------------------
