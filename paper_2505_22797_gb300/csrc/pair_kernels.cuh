@@ -628,6 +628,7 @@ __device__ __forceinline__ void adjoint_item(const PairBatch<R, MAXF> &B, int64_
     const int st_id = MPI_ADJ_WSTAGE ? lane : (int)threadIdx.x;
     constexpr int st_n = MPI_ADJ_WSTAGE ? 32 : kAdjThreads;
     const int ic = min(i, F.nx - 1);
+    const bool warp_in = __any_sync(0xffffffffu, i < F.nx && jb < F.ny);
 
     const V2<R> xc = F.xcol[ic];
     R yrow_y[kAdjV], yrow_x[kAdjV];
@@ -705,6 +706,9 @@ __device__ __forceinline__ void adjoint_item(const PairBatch<R, MAXF> &B, int64_
         }
         if (MPI_ADJ_WSTAGE) __syncwarp();
         else __syncthreads();
+        // A warp whose box lies wholly outside the grid only stages (at 64 x 48
+        // voxels the second tile row holds 16 rows of 32).
+        if (!warp_in) continue;
         // Far / very-far flags of this warp for the staged samples.
         for (int m = 0; m < kAdjBlock / 32; ++m) {
             const int k = m * 32 + lane;
