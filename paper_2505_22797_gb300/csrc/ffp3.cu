@@ -16,7 +16,9 @@
 //   k_adjoint3   one work item = 1024 voxels (8 per thread) x a chunk of
 //                samples; each staged sample carries (B r, B v, U = sum_k s_k
 //                p_k, U.B v) so a pair costs two dot products.
-//   Both test the near field once per staged pass: the gap between the
+//   k_forward3_rows / k_adjoint3_lines   the same sums for a diagonal G, along
+//                grid lines (below); the two kernels above serve a general G.
+//   Those two test the near field once per staged pass: the gap between the
 //   bounding box of the pass's prescaled voxel positions and that of the
 //   samples (precomputed per 512 voxels / 256 samples) decides whether every
 //   pair of the pass is in the asymptotic range (one rsqrt per pair), in the
@@ -34,6 +36,7 @@
 
 #include "conv_ops.cuh"
 #include "langevin.cuh"
+#include "pair_kernels.cuh"
 #include "pnp_device.cuh"
 #include "pnp_ops.cuh"
 
@@ -517,6 +520,351 @@ k_adjoint3(const __grid_constant__ Adj3Args<R> a)
 }
 
 // ---------------------------------------------------------------------------
+// Diagonal G: the row forms.
+//
+// With a diagonal G the prescaled offset y = B (x_v - r) varies in one
+// component only along a grid line, so the other two (and what they contribute
+// to u, y.W and y.U) are formed once per line and sample instead of once per
+// pair: 12 packed FP32 operations per pair of pairs instead of 19 (forward),
+// 10 instead of 18 (adjoint).  And the regime is decided where it changes:
+// per row of the warp's 64 samples by the columns within the asymptotic radius
+// (forward), per sample and 8 x 8 x 4 voxel box of a warp (adjoint), not per
+// 512 voxels x 256 samples.  Bound by FP32 issue and the special-function
+// unit as the 2-D sums; A then A^T at 48 x 48 x 24 / 65 536 samples: 3.18 ms,
+// with the general kernels 5.08 ms.
+
+template <typename R, typename CIN>
+struct Fwd3RowArgs {
+    const V4<R> *rs, *ws, *vox;
+    const CIN *c;
+    R *part;
+    int64_t T;
+    int nx, rows;                // columns; rows = ny nz
+    int n_tiles, chunk_rows, rows_staged, near_cols, n_ch;
+    R inv_h;                     // 1 / (prescaled column pitch, signed)
+    R p[9];
+};
+
+#ifndef MPI_FWD3R_MINB
+#define MPI_FWD3R_MINB 5
+#endif
+constexpr int k3RowFold = 8;  // rows summed plainly before a compensated add
+
+template <typename R, typename CIN>
+__global__ void __launch_bounds__(kFwdThreads, sizeof(R) == 4 ? MPI_FWD3R_MINB : 2)
+k_forward3_rows(const __grid_constant__ Fwd3RowArgs<R, CIN> a)
+{
+    extern __shared__ __align__(16) unsigned char smem3[];
+    const int nx = a.nx, RB = a.rows_staged;
+    V2<R> *s_y = reinterpret_cast<V2<R> *>(smem3);  // (y, z) of the staged rows
+    V2<R> *s_xc = s_y + RB;                          // their (x_i, c_i)
+    const int tile = (int)(blockIdx.x % a.n_tiles);
+    const int chunk = (int)(blockIdx.x / a.n_tiles);
+    const int j0 = chunk * a.chunk_rows;
+    const int nr = min(a.chunk_rows, a.rows - j0);
+
+    R Rx[kFwdS], Ry[kFwdS], Rz[kFwdS], Wx[kFwdS], Wy[kFwdS], Wz[kFwdS];
+    int64_t t[kFwdS];
+#pragma unroll
+    for (int s = 0; s < kFwdS; ++s) {
+        // a warp's samples are one run of the trajectory (a compact extent)
+        t[s] = (int64_t)tile * kFwdTile + (threadIdx.x >> 5) * (32 * kFwdS) + s * 32 + (threadIdx.x & 31);
+        const int64_t tt = t[s] < a.T ? t[s] : a.T - 1;
+        const V4<R> r = a.rs[tt], w = a.ws[tt];
+        Rx[s] = r.x, Ry[s] = r.y, Rz[s] = r.z;
+        Wx[s] = w.x, Wy[s] = w.y, Wz[s] = w.z;
+    }
+    R wl[3] = {Rx[0], Ry[0], Rz[0]}, wh[3] = {Rx[0], Ry[0], Rz[0]};
+#pragma unroll
+    for (int s = 1; s < kFwdS; ++s) {
+        const R q[3] = {Rx[s], Ry[s], Rz[s]};
+#pragma unroll
+        for (int k = 0; k < 3; ++k) wl[k] = min(wl[k], q[k]), wh[k] = max(wh[k], q[k]);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            wl[k] = min(wl[k], __shfl_xor_sync(0xffffffffu, wl[k], o));
+            wh[k] = max(wh[k], __shfl_xor_sync(0xffffffffu, wh[k], o));
+        }
+    constexpr R kUv = vfar_threshold<R, false>();
+    R A1, D1;  // the closed form at u = near_u (what clamped pairs received)
+    Lang<R>::ad_far(Lang<R>::near_u, A1, D1);
+    const R x0c = a.vox[0].x;
+    const R ax_lo = wl[0] - x0c, ax_hi = wh[0] - x0c;
+
+    R Sa[kFwdS], Vx[kFwdS], Vy[kFwdS], Vz[kFwdS], cSa[kFwdS], cVx[kFwdS], cVy[kFwdS], cVz[kFwdS];
+    R sa[kFwdS], vx[kFwdS], vy[kFwdS], vz[kFwdS];
+#pragma unroll
+    for (int s = 0; s < kFwdS; ++s) {
+        Sa[s] = Vx[s] = Vy[s] = Vz[s] = cSa[s] = cVx[s] = cVy[s] = cVz[s] = R(0);
+        sa[s] = vx[s] = vy[s] = vz[s] = R(0);
+    }
+#pragma unroll 1
+    for (int jb = j0; jb < j0 + nr; jb += RB) {
+        const int nrb = min(RB, j0 + nr - jb);
+        __syncthreads();
+        for (int k = threadIdx.x; k < nrb * nx; k += kFwdThreads)
+            s_xc[k] = V2<R>{a.vox[k % nx].x, R(a.c[(int64_t)jb * nx + k])};
+        for (int k = threadIdx.x; k < nrb; k += kFwdThreads) {
+            const V4<R> q = a.vox[(int64_t)(jb + k) * nx];
+            s_y[k] = V2<R>{q.y, q.z};
+        }
+        __syncthreads();
+#pragma unroll 1
+        for (int r = 0; r < nrb; ++r) {
+            const V2<R> yr = s_y[r];
+            const V2<R> *xc = s_xc + r * nx;
+            R oy[kFwdS], oz[kFwdS], r2[kFwdS], rW[kFwdS], fr[kFwdS];
+            bool near = false;
+#pragma unroll
+            for (int s = 0; s < kFwdS; ++s) {
+                oy[s] = yr.x - Ry[s];
+                oz[s] = yr.y - Rz[s];
+                r2[s] = fmx(oz[s], oz[s], oy[s] * oy[s]);
+                rW[s] = fmx(oz[s], Wz[s], oy[s] * Wy[s]);
+                near |= r2[s] < Lang<R>::near_u;
+                fr[s] = R(0);
+            }
+            // Columns [lo, hi] may hold a pair of this warp with u < vfar_u
+            // (one column and 1e-4 to spare on each side).
+            int lo = 1, hi = 0;
+            const R gy = max(R(0), max(wl[1] - yr.x, yr.x - wh[1]));
+            const R gz = max(R(0), max(wl[2] - yr.y, yr.y - wh[2]));
+            const R g2 = fmx(gz, gz, gy * gy);
+            if (g2 < kUv) {
+                const R x = kUv - g2;
+                const R w = x * R(rsqrt_approx(float(x))) * R(1.0001);
+                const R ia = (ax_lo - w) * a.inv_h, ib = (ax_hi + w) * a.inv_h;
+                lo = (int)min(max(floor(min(ia, ib)) - R(1), R(0)), R(nx));
+                hi = (int)min(max(ceil(max(ia, ib)) + R(1), R(-1)), R(nx - 1));
+            }
+            if (lo > hi) {
+                fwd_row_vfar<R>(0, nx, xc, Rx, r2, Wx, rW, sa, vx, fr);
+            } else {
+                fwd_row_vfar<R>(0, lo, xc, Rx, r2, Wx, rW, sa, vx, fr);
+                if (!__any_sync(0xffffffffu, near)) {
+                    fwd_row_far<R, false>(lo, hi + 1, xc, Rx, r2, Wx, rW, sa, vx, fr);
+                } else {
+                    fwd_row_far<R, true>(lo, hi + 1, xc, Rx, r2, Wx, rW, sa, vx, fr);
+#pragma unroll
+                    for (int s = 0; s < kFwdS; ++s)
+                        if (r2[s] < Lang<R>::near_u)
+                            fwd_near_fix<R>(nx, xc, Rx[s], r2[s], Wx[s], rW[s], A1, D1, a.near_cols, sa[s],
+                                            vx[s], fr[s]);
+                }
+                fwd_row_vfar<R>(hi + 1, nx, xc, Rx, r2, Wx, rW, sa, vx, fr);
+            }
+            const bool fold = (r + 1) % k3RowFold == 0 || r + 1 == nrb;
+#pragma unroll
+            for (int s = 0; s < kFwdS; ++s) {
+                vy[s] = fmx(oy[s], fr[s], vy[s]);
+                vz[s] = fmx(oz[s], fr[s], vz[s]);
+                if (fold) {
+                    kahan_add(Sa[s], cSa[s], sa[s]);
+                    kahan_add(Vx[s], cVx[s], vx[s]);
+                    kahan_add(Vy[s], cVy[s], vy[s]);
+                    kahan_add(Vz[s], cVz[s], vz[s]);
+                    sa[s] = vx[s] = vy[s] = vz[s] = R(0);
+                }
+            }
+        }
+    }
+    // s_k = p_k^T (W sum c a + sum c d (y.W) y)
+#pragma unroll
+    for (int s = 0; s < kFwdS; ++s) {
+        if (t[s] >= a.T) continue;
+        const R ox = fmx(Wx[s], Sa[s], Vx[s]), oy = fmx(Wy[s], Sa[s], Vy[s]), oz = fmx(Wz[s], Sa[s], Vz[s]);
+        for (int k = 0; k < a.n_ch; ++k)
+            a.part[((int64_t)chunk * a.n_ch + k) * a.T + t[s]] =
+                fmx(a.p[3 * k + 2], oz, fmx(a.p[3 * k + 1], oy, a.p[3 * k] * ox));
+    }
+}
+
+template <typename R>
+struct Adj3LineArgs {
+    const V4<R> *rs, *ws, *vox;
+    const R *s;
+    R *part;
+    int64_t T, chunk_len;
+    int nx, ny, nz, bx, by, bz;  // voxels; warp boxes per axis
+    int n_groups, n_ch;          // groups of k3LineWarps boxes
+    R p[9];
+};
+
+constexpr int k3LineWarps = k3Threads / 32;
+constexpr int k3BoxX = 8, k3BoxY = k3AdjV, k3BoxZ = 4;  // a warp's voxel box: lanes 8 (x) x 4 (z), 8 rows per thread
+static_assert(k3BoxX * k3BoxZ == 32, "one lane per column");
+#ifndef MPI_ADJ3L_MINB
+#define MPI_ADJ3L_MINB 5
+#endif
+
+// One staged sample, Q = (B r, u.W), W = (B v, W_y U_y), U, against a thread's
+// line of voxels (x, Y[v], z): U^T K W = a (U.W) + d (y.U)(y.W), the product
+// expanded in y_y.
+template <typename R, int MODE>
+__device__ __forceinline__ void adj3_line(const V4<R> Q, const V4<R> W, const V4<R> U, R x, R z,
+                                          const R (&Y)[k3AdjV], R (&blk)[k3AdjV])
+{
+    const R yx = x - Q.x, yz = z - Q.z;
+    const R w2 = fmx(yz, yz, yx * yx);
+    const R aU = fmx(yz, U.z, yx * U.x), aW = fmx(yz, W.z, yx * W.x);
+    const R Q0 = aU * aW, Q1 = fmx(aU, W.y, aW * U.y);
+#pragma unroll
+    for (int v = 0; v < k3AdjV; ++v) {
+        const R yy = Y[v] - Q.y;
+        const R u = fmx(yy, yy, w2);
+        const R P = fmx(yy, fmx(W.w, yy, Q1), Q0);
+        if constexpr (MODE == 2) {
+            blk[v] = pair_acc_vfar<R, false>(u, Q.w, P, blk[v]);
+        } else {
+            R f1, f2;
+            lang_mode<R, false, MODE>(u, f1, f2);
+            blk[v] += fmx(f1, Q.w, f2 * P);
+        }
+    }
+}
+
+// Two staged samples in the two lanes of packed FP32 arithmetic, asymptotic
+// range.  pk: six float4, each entry (even, odd sample): (-Qx, -Qy), (-Qz, uW),
+// (Wx, Wy), (Wz, Wy Uy), (Ux, Uy), (Uz, -uW).
+__device__ __forceinline__ void adj3_line_packed(const float4 *pk, float x, float z, const float (&Y)[k3AdjV],
+                                                 float2 (&blk2)[k3AdjV])
+{
+    const float2 m1 = make_float2(-1.0f, -1.0f), two = make_float2(2.0f, 2.0f);
+    const float4 A = pk[0], B = pk[1], C = pk[2], D = pk[3], E = pk[4], F = pk[5];
+    const float2 nQy = make_float2(A.z, A.w), uW = make_float2(B.z, B.w), Wy = make_float2(C.z, C.w);
+    const float2 WUy = make_float2(D.z, D.w), Uy = make_float2(E.z, E.w), nuW = make_float2(F.z, F.w);
+    const float2 yx = __fadd2_rn(make_float2(x, x), make_float2(A.x, A.y));
+    const float2 yz = __fadd2_rn(make_float2(z, z), make_float2(B.x, B.y));
+    const float2 w2 = __ffma2_rn(yz, yz, __fmul2_rn(yx, yx));
+    const float2 aU = __ffma2_rn(yz, make_float2(F.x, F.y), __fmul2_rn(yx, make_float2(E.x, E.y)));
+    const float2 aW = __ffma2_rn(yz, make_float2(D.x, D.y), __fmul2_rn(yx, make_float2(C.x, C.y)));
+    const float2 Q0 = __fmul2_rn(aU, aW), Q1 = __ffma2_rn(aU, Wy, __fmul2_rn(aW, Uy));
+#pragma unroll
+    for (int v = 0; v < k3AdjV; ++v) {
+        const float2 yy = __fadd2_rn(make_float2(Y[v], Y[v]), nQy);
+        const float2 u = __ffma2_rn(yy, yy, w2);
+        const float2 P = __ffma2_rn(yy, __ffma2_rn(WUy, yy, Q1), Q0);
+        const float2 iz = make_float2(Lang<float>::iz_vfar(u.x), Lang<float>::iz_vfar(u.y));
+        // iz (uW + iz (iz (2 iz - 1) P - uW)), as pair_acc_vfar
+        const float2 w = __ffma2_rn(iz, __fmul2_rn(P, __ffma2_rn(iz, two, m1)), nuW);
+        blk2[v] = __ffma2_rn(iz, __ffma2_rn(iz, w, uW), blk2[v]);
+    }
+}
+
+template <typename R>
+__global__ void __launch_bounds__(k3Threads, sizeof(R) == 4 ? MPI_ADJ3L_MINB : 2)
+k_adjoint3_lines(const __grid_constant__ Adj3LineArgs<R> a)
+{
+    constexpr bool PACK = sizeof(R) == 4;
+    __shared__ V4<R> sQ[k3Batch], sW[k3Batch], sU[k3Batch];
+    __shared__ float4 sPk[PACK ? 6 * (k3Batch / 2) : 1];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t chunk = blockIdx.x / a.n_groups;
+    const int box = (int)(blockIdx.x % a.n_groups) * k3LineWarps + warp;
+    const int n_box = a.bx * a.by * a.bz;
+    const int bq = min(box, n_box - 1);
+    const int i = (bq % a.bx) * k3BoxX + (lane & 7), l = (bq / (a.bx * a.by)) * k3BoxZ + (lane >> 3);
+    const int jb = (bq / a.bx) % a.by * k3BoxY;
+    const int64_t plane = (int64_t)a.nx * a.ny;
+    const int64_t v0 = (int64_t)min(l, a.nz - 1) * plane + min(i, a.nx - 1);
+    const R x = a.vox[v0].x, z = a.vox[v0].z;
+    R Y[k3AdjV], acc[k3AdjV], comp[k3AdjV];
+#pragma unroll
+    for (int v = 0; v < k3AdjV; ++v) {
+        Y[v] = a.vox[v0 + (int64_t)min(jb + v, a.ny - 1) * a.nx].y;
+        acc[v] = comp[v] = R(0);
+    }
+    // the warp's voxel box
+    R lo[3] = {x, Y[0], z}, hi[3] = {x, Y[0], z};
+#pragma unroll
+    for (int v = 1; v < k3AdjV; ++v) lo[1] = min(lo[1], Y[v]), hi[1] = max(hi[1], Y[v]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        lo[0] = min(lo[0], __shfl_xor_sync(0xffffffffu, lo[0], o));
+        hi[0] = max(hi[0], __shfl_xor_sync(0xffffffffu, hi[0], o));
+        lo[2] = min(lo[2], __shfl_xor_sync(0xffffffffu, lo[2], o));
+        hi[2] = max(hi[2], __shfl_xor_sync(0xffffffffu, hi[2], o));
+    }
+    const int64_t t0 = chunk * a.chunk_len, t1 = std::min<int64_t>(a.T, t0 + a.chunk_len);
+#pragma unroll 1
+    for (int64_t tb = t0; tb < t1; tb += k3Batch) {
+        const int nb = (int)std::min<int64_t>(k3Batch, t1 - tb);
+        __syncthreads();
+        for (int e = threadIdx.x; e < nb; e += k3Threads) {
+            const int64_t t = tb + e;
+            const V4<R> q = a.rs[t], w = a.ws[t];
+            R ux = R(0), uy = R(0), uz = R(0);
+            for (int k = 0; k < a.n_ch; ++k) {
+                const R sk = a.s[k * a.T + t];
+                ux = fmx(sk, a.p[3 * k], ux);
+                uy = fmx(sk, a.p[3 * k + 1], uy);
+                uz = fmx(sk, a.p[3 * k + 2], uz);
+            }
+            const R uW = fmx(uz, w.z, fmx(uy, w.y, ux * w.x));
+            sQ[e] = V4<R>{q.x, q.y, q.z, uW};
+            sW[e] = V4<R>{w.x, w.y, w.z, w.y * uy};
+            sU[e] = V4<R>{ux, uy, uz, R(0)};
+            if constexpr (PACK) {
+                float *pb = reinterpret_cast<float *>(sPk + 6 * (e >> 1)) + (e & 1);
+                const float f[12] = {-float(q.x), -float(q.y), -float(q.z), float(uW), float(w.x), float(w.y),
+                                     float(w.z), float(w.y * uy), float(ux), float(uy), float(uz), -float(uW)};
+#pragma unroll
+                for (int j = 0; j < 12; ++j) pb[2 * j] = f[j];
+            }
+        }
+        __syncthreads();
+        if (box >= n_box) continue;  // (the whole warp; it only stages)
+        R blk[k3AdjV];
+#pragma unroll
+        for (int v = 0; v < k3AdjV; ++v) blk[v] = R(0);
+#pragma unroll 1
+        for (int k0 = 0; k0 < nb; k0 += 32) {
+            const int kn = min(32, nb - k0);
+            bool far = true, vfar = true;
+            if (lane < kn) {
+                const V4<R> q = sQ[k0 + lane];
+                const R gx = max(R(0), max(lo[0] - q.x, q.x - hi[0]));
+                const R gy = max(R(0), max(lo[1] - q.y, q.y - hi[1]));
+                const R gz = max(R(0), max(lo[2] - q.z, q.z - hi[2]));
+                const R d2 = fmx(gy, gy, fmx(gz, gz, gx * gx));
+                far = d2 >= Lang<R>::near_u;
+                vfar = d2 >= vfar_threshold<R, false>();
+            }
+            const uint32_t fm = __ballot_sync(0xffffffffu, far), vm = __ballot_sync(0xffffffffu, vfar);
+            if (PACK && kn == 32 && vm == 0xffffffffu) {
+                if constexpr (PACK) {
+                    float2 blk2[k3AdjV];
+#pragma unroll
+                    for (int v = 0; v < k3AdjV; ++v) blk2[v] = make_float2(0.0f, 0.0f);
+#pragma unroll 1
+                    for (int h = k0 >> 1; h < (k0 >> 1) + 16; ++h) adj3_line_packed(sPk + 6 * h, x, z, Y, blk2);
+#pragma unroll
+                    for (int v = 0; v < k3AdjV; ++v) blk[v] += blk2[v].x + blk2[v].y;
+                }
+            } else {
+#pragma unroll 1
+                for (int k = 0; k < kn; ++k) {
+                    const V4<R> q = sQ[k0 + k], w = sW[k0 + k], U = sU[k0 + k];
+                    if ((vm >> k) & 1u) adj3_line<R, 2>(q, w, U, x, z, Y, blk);
+                    else if ((fm >> k) & 1u) adj3_line<R, 1>(q, w, U, x, z, Y, blk);
+                    else adj3_line<R, 0>(q, w, U, x, z, Y, blk);
+                }
+            }
+        }
+#pragma unroll
+        for (int v = 0; v < k3AdjV; ++v) kahan_add(acc[v], comp[v], blk[v]);
+    }
+    if (box >= n_box || i >= a.nx || l >= a.nz) return;
+    R *part = a.part + chunk * plane * a.nz + (int64_t)l * plane + i;
+#pragma unroll
+    for (int v = 0; v < k3AdjV; ++v)
+        if (jb + v < a.ny) part[(int64_t)(jb + v) * a.nx] = acc[v];
+}
+
+// ---------------------------------------------------------------------------
 // Host side of the pair operators.
 
 struct Split3 {
@@ -545,6 +893,8 @@ struct Op3 {
     Geo3<R> geo{};
     Split3 fs{}, as{};
     R *fwd_part = nullptr, *adj_part = nullptr;
+    bool rows = false;  // the row forms (diagonal G)
+    int bx = 0, by = 0, bz = 0, rows_staged = 0;
 
     size_t scratch_bytes() const
     {
@@ -558,8 +908,36 @@ struct Op3 {
         T = TT;
         N = gg.n();
         const int target = default_target_items();
-        fs = split3(T, k3FwdTile, N, k3Piece, target);
-        as = split3(N, k3AdjTile, T, k3Batch, target);
+        rows = plan_rows();
+        if (rows) {
+            bx = (g.nx + k3BoxX - 1) / k3BoxX, by = (g.ny + k3BoxY - 1) / k3BoxY, bz = (g.nz + k3BoxZ - 1) / k3BoxZ;
+            fs = split3(T, kFwdTile, (int64_t)g.ny * g.nz, 1, target);
+            as = split3((int64_t)bx * by * bz, k3LineWarps, T, k3Batch, target);
+            rows_staged = fwd_rows_staged((int)fs.chunk_len, g.nx, sizeof(R));
+        } else {
+            fs = split3(T, k3FwdTile, N, k3Piece, target);
+            as = split3(N, k3AdjTile, T, k3Batch, target);
+        }
+    }
+    // The row forms serve a diagonal G whose columns R resolves evenly (the
+    // segment bounds and the near columns are indexed by distance: the
+    // rounding of a column's position times nx below a quarter of the pitch) and whose staged row fits the
+    // shared memory a block has without opting in for more.
+    bool plan_rows() const
+    {
+        for (int q = 0; q < 9; ++q)
+            if (q % 4 != 0 && m.G[q] != 0.0) return false;
+        const double h = m.beta * m.G[0] * g.dx;
+        const double far = std::fabs(m.beta * m.G[0]) * std::max(std::fabs(g.x0), std::fabs(g.x0 + g.nx * g.dx));
+        const int bits = sizeof(R) == 4 ? 21 : 50;
+        if (!(far * g.nx <= std::ldexp(std::fabs(h), bits)) || !std::isfinite(R(1.0 / h)) || R(1.0 / h) == R(0)) return false;
+        const int64_t boxes = (int64_t)((g.nx + 7) / 8) * ((g.ny + 7) / 8) * ((g.nz + 3) / 4);
+        return sizeof(R) * (2 + 2 * (int64_t)g.nx) <= 48 * 1024 && (int64_t)g.ny * g.nz < (1 << 30) && boxes < (1 << 30);
+    }
+    int near_cols() const
+    {
+        const double w = std::sqrt(double(Lang<R>::near_u)) / std::fabs(m.beta * m.G[0] * g.dx);
+        return (int)std::min(w + 2.0, double(g.nx) + 2.0);
     }
     void carve(char *base)
     {
@@ -598,6 +976,23 @@ struct Op3 {
     int forward(const CIN *c, OUT *s, cudaStream_t st)
     {
         if (T == 0) return MPI_OK;
+        if (rows) {
+            Fwd3RowArgs<R, CIN> a;
+            a.rs = geo.rs, a.ws = geo.ws, a.vox = geo.vox;
+            a.c = c;
+            a.part = fwd_part;
+            a.T = T, a.nx = g.nx, a.rows = g.ny * g.nz;
+            a.n_tiles = fs.n_tiles, a.chunk_rows = (int)fs.chunk_len, a.rows_staged = rows_staged;
+            a.near_cols = near_cols(), a.n_ch = m.n_ch;
+            a.inv_h = R(1.0 / (m.beta * m.G[0] * g.dx));
+            for (int q = 0; q < 9; ++q) a.p[q] = R(m.p[q]);
+            const size_t smem = sizeof(V2<R>) * (size_t(rows_staged) + size_t(rows_staged) * g.nx);
+            ProfScope prof(kProfForward, st);
+            k_forward3_rows<R, CIN><<<(unsigned)((int64_t)fs.n_tiles * fs.n_chunks), kFwdThreads, smem, st>>>(a);
+            MPI_CHECK_LAUNCH();
+            return reduce_chunks<R, OUT>(fwd_part, fs.n_chunks, (int64_t)m.n_ch * T, s, nullptr, nullptr,
+                                         nullptr, st);
+        }
         Fwd3Args<R, CIN> a;
         a.rs = geo.rs, a.ws = geo.ws, a.vox = geo.vox, a.sbox = geo.sbox, a.vbox = geo.vbox;
         a.c = c;
@@ -619,7 +1014,19 @@ struct Op3 {
                 cudaStream_t st)
     {
         int nch = as.n_chunks;
-        if (T > 0) {
+        if (T > 0 && rows) {
+            Adj3LineArgs<R> a;
+            a.rs = geo.rs, a.ws = geo.ws, a.vox = geo.vox;
+            a.s = s;
+            a.part = adj_part;
+            a.T = T, a.chunk_len = as.chunk_len;
+            a.nx = g.nx, a.ny = g.ny, a.nz = g.nz, a.bx = bx, a.by = by, a.bz = bz;
+            a.n_groups = as.n_tiles, a.n_ch = m.n_ch;
+            for (int q = 0; q < 9; ++q) a.p[q] = R(m.p[q]);
+            ProfScope prof(kProfAdjoint, st);
+            k_adjoint3_lines<R><<<(unsigned)((int64_t)as.n_tiles * as.n_chunks), k3Threads, 0, st>>>(a);
+            MPI_CHECK_LAUNCH();
+        } else if (T > 0) {
             Adj3Args<R> a;
             a.rs = geo.rs, a.ws = geo.ws, a.vox = geo.vox, a.sbox = geo.sbox, a.vbox = geo.vbox;
             a.s = s;
