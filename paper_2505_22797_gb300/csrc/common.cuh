@@ -37,6 +37,41 @@ const char *last_error();
 // also counts it (mpi_kernel_launches()).
 void note_launch();
 void note_launches(long long n);
+#ifdef __CUDACC__
+// Launches of one dependent chain: the next kernel's launch overlaps the end
+// of the one before (programmatic dependent launch), and every kernel of a
+// chain opens with chain_wait(), which returns once all work before it is
+// complete and visible.  A chained kernel's input pointers are not
+// __restrict__: loads the compiler may take for those of constant data could
+// move ahead of the wait.  The gridded operators' six to eight launches gain
+// 1.5 us each: A at 128 x 128 / 65 536 samples 79 -> 70 us, A^T 107 -> 94 us.
+// Inside a graph capture the edges are plain ones
+// (128 x 128 reconstruction, replayed graphs: 2.70 ms, with programmatic edges
+// 2.84 ms).
+__device__ __forceinline__ void chain_wait()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+template <typename... P, typename... A>
+inline void launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A &&...args)
+{
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = cudaStreamIsCapturing(st, &capture) == cudaSuccess && capture == cudaStreamCaptureStatusNone;
+    (void)cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);  // MPI_CHECK_LAUNCH reports
+}
+#endif
+
 #define MPI_CHECK_LAUNCH()                          \
     do {                                            \
         ::mpi::note_launch();                       \

@@ -337,9 +337,10 @@ __device__ __forceinline__ float4 operand(const FieldDev &d, const float *__rest
 
 // Places each run's samples: position = the tile's first + its samples in
 // earlier runs + the rank within the run.
-__global__ void __launch_bounds__(128) k_field_place(const __grid_constant__ FieldDev d, const float *__restrict__ r,
-                                                     const float *__restrict__ v, const float *__restrict__ s)
+__global__ void __launch_bounds__(128) k_field_place(const __grid_constant__ FieldDev d, const float *r,
+                                                     const float *v, const float *s)
 {
+    chain_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int nt = d.tx * d.ty + 1, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int run = blockIdx.x * (blockDim.x >> 5) + warp;
@@ -374,8 +375,9 @@ __global__ void __launch_bounds__(128) k_field_place(const __grid_constant__ Fie
     }
 }
 
-__global__ void __launch_bounds__(256) k_field_load(const __grid_constant__ FieldDev d, const float *__restrict__ s)
+__global__ void __launch_bounds__(256) k_field_load(const __grid_constant__ FieldDev d, const float *s)
 {
+    chain_wait();
     const int64_t p = int64_t(blockIdx.x) * 256 + threadIdx.x;
     if (p >= d.T) return;
     const float4 rc = d.b.rec[p], w = d.b.wv[p];
@@ -388,9 +390,10 @@ __global__ void __launch_bounds__(256) k_field_load(const __grid_constant__ Fiel
 
 // Tables (32 entries per block: FP64 functions, spread over the SMs) and, in
 // the blocks behind them, the samples' tiles.
-__global__ void __launch_bounds__(128) k_field_setup(const __grid_constant__ FieldDev d, int n_table, const float *__restrict__ r,
-                                                     const float *__restrict__ v)
+__global__ void __launch_bounds__(128) k_field_setup(const __grid_constant__ FieldDev d, int n_table, const float *r,
+                                                     const float *v)
 {
+    chain_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     if (int(blockIdx.x) < n_table) {
         if (threadIdx.x < 32) fill_table(d, blockIdx.x * 32 + threadIdx.x);
@@ -744,16 +747,18 @@ template <typename CIN> __device__ void image_rows(const FieldDev &d, int j0, co
 }
 
 template <typename CIN>
-__global__ void __launch_bounds__(128) k_field_image(const __grid_constant__ FieldDev d, const CIN *__restrict__ c)
+__global__ void __launch_bounds__(128) k_field_image(const __grid_constant__ FieldDev d, const CIN *c)
 {
+    chain_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     image_rows(d, 2 * blockIdx.x, c, smem_raw);
 }
 
 // The sampled kernel's rows and, behind them, what else needs only the
 // tables: the image's rows (c) or the tiles' prefix sums.
-__global__ void __launch_bounds__(512) k_field_rows(const __grid_constant__ FieldDev d, int n_kernel, const float *__restrict__ c)
+__global__ void __launch_bounds__(512) k_field_rows(const __grid_constant__ FieldDev d, int n_kernel, const float *c)
 {
+    chain_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int b = blockIdx.x;
     if (b < n_kernel) {
@@ -770,6 +775,7 @@ __global__ void __launch_bounds__(512) k_field_rows(const __grid_constant__ Fiel
 template <int NC>
 __global__ void __launch_bounds__(512) k_field_kcols(const __grid_constant__ FieldDev d)
 {
+    chain_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int s_w[32];
     const int g = blockIdx.x % d.n_grp, m = blockIdx.x / d.n_grp;
@@ -790,6 +796,7 @@ __device__ __forceinline__ int fast_mod(int k, int n, unsigned mag, int lift)
 template <int NC>
 __global__ void __launch_bounds__(512) k_field_cols_fwd(const __grid_constant__ FieldDev d)
 {
+    chain_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ float4 s_low[NC][kLowY];
     const int P = d.y.P, Q = d.y.Q, J1 = d.x.J + 1, ny = d.y.n, M = max(P, Q);
@@ -857,6 +864,7 @@ __global__ void __launch_bounds__(512) k_field_cols_fwd(const __grid_constant__ 
 // each row and yy of both as three complex sequences.
 __global__ void __launch_bounds__(512) k_field_rows_inv(const __grid_constant__ FieldDev d)
 {
+    chain_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ float4 s_low[3][kFieldLow];  // (re, im) of both rows' lowest modes
     const int P = d.x.P, J = d.x.J, J1 = J + 1;
@@ -969,8 +977,9 @@ struct InterpArgs {
 // lanes in pairs of floats.
 template <int MODE, typename CIN>
 __global__ void __launch_bounds__(256) k_field_interp(const __grid_constant__ FieldDev d, const __grid_constant__ InterpArgs A,
-                                                      const CIN *__restrict__ cin)
+                                                      const CIN *cin)
 {
+    chain_wait();
     __shared__ float4 s_out[256];
     __shared__ int s_id[256];
     __shared__ int s_n;
@@ -1123,6 +1132,7 @@ __global__ void __launch_bounds__(256) k_field_interp(const __grid_constant__ Fi
 constexpr int kUnitPitch = kFieldUnit + 4;
 __global__ void __launch_bounds__(kSpreadThreads) k_field_spread(const __grid_constant__ FieldDev d)
 {
+    chain_wait();
     __shared__ float s_patch[2][3][kPatch * kPatchPitch];
     __shared__ __align__(16) float s_wx[kWin][kUnitPitch];
     __shared__ __align__(16) float s_c[3][kWin][kUnitPitch];  // entry x row weight, rows by parity
@@ -1284,6 +1294,7 @@ __global__ void __launch_bounds__(kSpreadThreads) k_field_spread(const __grid_co
 // the up to four tiles that reach it, units in order.
 __global__ void __launch_bounds__(512) k_field_rows_fwd(const __grid_constant__ FieldDev d)
 {
+    chain_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int P = d.x.P, J1 = d.x.J + 1, wx = d.x.w;
     V2<float> *a = reinterpret_cast<V2<float> *>(smem_raw);
@@ -1334,6 +1345,7 @@ __global__ void __launch_bounds__(512) k_field_rows_fwd(const __grid_constant__ 
 template <int NC>
 __global__ void __launch_bounds__(512) k_field_cols_adj(const __grid_constant__ FieldDev d)
 {
+    chain_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ float4 s_low[NC][kLowY];
     const int P = d.y.P, Q = d.y.Q, J1 = d.x.J + 1, ny = d.y.n, M = max(P, Q), wy = d.y.w;
@@ -1409,9 +1421,10 @@ __global__ void __launch_bounds__(512) k_field_cols_adj(const __grid_constant__ 
 // added in pairs), plus the outside samples' partial images.
 template <typename OUT, bool CG>
 __global__ void __launch_bounds__(128) k_field_out(const __grid_constant__ FieldDev d, OUT *__restrict__ out,
-                                                   const double *__restrict__ p, const double *__restrict__ nu_dev,
+                                                   const double *p, const double *nu_dev,
                                                    double *__restrict__ dot_part)
 {
+    chain_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ double s_red[4];
     __shared__ float4 s_low[2][kFieldLow];
@@ -1720,14 +1733,14 @@ int field_prepare(const FieldPlan &plan, const float *c, const float *r, const f
     const int n_table = (table_entries(d) + 31) / 32, ow = order_warps(d);
     const int n_bin = plan.adjoint ? (d.n_run + ow - 1) / ow : 0;
     const size_t osm = plan.adjoint ? order_smem(d) : 0;
-    k_field_setup<<<n_table + n_bin, 32 * ow, osm, st>>>(d, n_table, r, v);
+    launch_chained(k_field_setup, n_table + n_bin, 32 * ow, osm, st, d, n_table, r, v);
     MPI_CHECK_LAUNCH();
     const int kr = (d.y.P / 2 + 2) / 2, tr = fft_threads(3, d.x.P);
     const int more = c ? (d.y.n + 1) / 2 : plan.adjoint ? (d.tx * d.ty + 1 + tr / 32 - 1) / (tr / 32) : 0;
-    k_field_rows<<<kr + more, tr, rows_smem(d), st>>>(d, kr, c);
+    launch_chained(k_field_rows, kr + more, tr, rows_smem(d), st, d, kr, c);
     MPI_CHECK_LAUNCH();
     auto cols = cols_nc(d) == 4 ? k_field_kcols<4> : k_field_kcols<2>;
-    cols<<<3 * d.n_grp + (plan.adjoint ? 1 : 0), fft_threads(cols_nc(d), d.y.P), cols_smem(d), st>>>(d);
+    launch_chained(cols, 3 * d.n_grp + (plan.adjoint ? 1 : 0), fft_threads(cols_nc(d), d.y.P), cols_smem(d), st, d);
     MPI_CHECK_LAUNCH();
     return MPI_OK;
 }
@@ -1736,14 +1749,14 @@ int field_order(const FieldPlan &plan, const float *r, const float *v, const flo
 {
     const FieldDev &d = plan.d;
     const int ow = order_warps(d);
-    k_field_place<<<(d.n_run + ow - 1) / ow, 32 * ow, order_smem(d), st>>>(d, r, v, s);
+    launch_chained(k_field_place, (d.n_run + ow - 1) / ow, 32 * ow, order_smem(d), st, d, r, v, s);
     MPI_CHECK_LAUNCH();
     return MPI_OK;
 }
 
 int field_load(const FieldPlan &plan, const float *s, cudaStream_t st)
 {
-    k_field_load<<<(unsigned)((plan.d.T + 255) / 256), 256, 0, st>>>(plan.d, s);
+    launch_chained(k_field_load, (unsigned)((plan.d.T + 255) / 256), 256, 0, st, plan.d, s);
     MPI_CHECK_LAUNCH();
     return MPI_OK;
 }
@@ -1754,9 +1767,9 @@ namespace {
 int field_nodes(const FieldDev &d, cudaStream_t st)
 {
     auto cols = cols_nc(d) == 4 ? k_field_cols_fwd<4> : k_field_cols_fwd<2>;
-    cols<<<3 * d.n_grp, fft_threads(cols_nc(d), std::max(d.y.P, d.y.Q)), cols_smem(d), st>>>(d);
+    launch_chained(cols, 3 * d.n_grp, fft_threads(cols_nc(d), std::max(d.y.P, d.y.Q)), cols_smem(d), st, d);
     MPI_CHECK_LAUNCH();
-    k_field_rows_inv<<<(d.y.w + 1) / 2, fft_threads(3, d.x.P), rows_smem(d), st>>>(d);
+    launch_chained(k_field_rows_inv, (d.y.w + 1) / 2, fft_threads(3, d.x.P), rows_smem(d), st, d);
     MPI_CHECK_LAUNCH();
     return MPI_OK;
 }
@@ -1771,7 +1784,7 @@ int field_forward(const FieldPlan &plan, const float *c, const float *r, const f
     MPI_TRY(field_prepare(plan, c, r, v, st));
     MPI_TRY(field_nodes(plan.d, st));
     const InterpArgs A{r, v, s};
-    k_field_interp<kInterpForward, float><<<interp_blocks(plan.d.T), 256, 0, st>>>(plan.d, A, c);
+    launch_chained(k_field_interp<kInterpForward, float>, interp_blocks(plan.d.T), 256, 0, st, plan.d, A, c);
     MPI_CHECK_LAUNCH();
     return MPI_OK;
 }
@@ -1781,10 +1794,10 @@ int field_forward_ordered(const FieldPlan &plan, const CIN *c, cudaStream_t st)
 {
     const FieldDev &d = plan.d;
     ProfScope prof(kProfForward, st);
-    k_field_image<CIN><<<(d.y.n + 1) / 2, 128, image_smem(d), st>>>(d, c);
+    launch_chained(k_field_image<CIN>, (d.y.n + 1) / 2, 128, image_smem(d), st, d, c);
     MPI_CHECK_LAUNCH();
     MPI_TRY(field_nodes(d, st));
-    k_field_interp<kInterpOrdered, CIN><<<interp_blocks(plan.d.T), 256, 0, st>>>(plan.d, InterpArgs{}, c);
+    launch_chained(k_field_interp<kInterpOrdered, CIN>, interp_blocks(plan.d.T), 256, 0, st, plan.d, InterpArgs{}, c);
     MPI_CHECK_LAUNCH();
     return MPI_OK;
 }
@@ -1797,17 +1810,17 @@ int field_adjoint(const FieldPlan &plan, OUT *out, const double *cg_p, const dou
 {
     const FieldDev &d = plan.d;
     ProfScope prof(kProfAdjoint, st);
-    k_field_spread<<<d.n_unit_max + d.out_tiles * d.out_chunks, kSpreadThreads, 0, st>>>(d);
+    launch_chained(k_field_spread, d.n_unit_max + d.out_tiles * d.out_chunks, kSpreadThreads, 0, st, d);
     MPI_CHECK_LAUNCH();
-    k_field_rows_fwd<<<(d.y.w + 1) / 2, fft_threads(3, d.x.P), rows_smem(d), st>>>(d);
+    launch_chained(k_field_rows_fwd, (d.y.w + 1) / 2, fft_threads(3, d.x.P), rows_smem(d), st, d);
     MPI_CHECK_LAUNCH();
     auto cols = cols_nc(d) == 4 ? k_field_cols_adj<4> : k_field_cols_adj<2>;
-    cols<<<3 * d.n_grp, fft_threads(cols_nc(d), std::max(d.y.P, d.y.Q)), cols_smem(d), st>>>(d);
+    launch_chained(cols, 3 * d.n_grp, fft_threads(cols_nc(d), std::max(d.y.P, d.y.Q)), cols_smem(d), st, d);
     MPI_CHECK_LAUNCH();
     const unsigned nb = (unsigned)field_dot_blocks(d.y.n);
     if constexpr (sizeof(OUT) == sizeof(double)) {
         if (cg_p) {
-                    k_field_out<double, true><<<nb, 128, image_smem(d), st>>>(d, out, cg_p, nu_dev, dot_part);
+                    launch_chained(k_field_out<double, true>, nb, 128, image_smem(d), st, d, out, cg_p, nu_dev, dot_part);
             MPI_CHECK_LAUNCH();
             return MPI_OK;
         }
@@ -1815,7 +1828,7 @@ int field_adjoint(const FieldPlan &plan, OUT *out, const double *cg_p, const dou
         set_error("internal: CG epilogue needs FP64 output");
         return MPI_ERR_INVALID;
     }
-    k_field_out<OUT, false><<<nb, 128, image_smem(d), st>>>(d, out, nullptr, nullptr, nullptr);
+    launch_chained(k_field_out<OUT, false>, nb, 128, image_smem(d), st, d, out, nullptr, nullptr, nullptr);
     MPI_CHECK_LAUNCH();
     return MPI_OK;
 }
