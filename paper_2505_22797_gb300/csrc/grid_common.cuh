@@ -315,6 +315,8 @@ struct CoreStageOp {
         taken = false;
         return MPI_OK;
     }
+    // Whether step_q uses the fork (else its events and stream are not made).
+    virtual bool forks() const { return true; }
     virtual int step_q(const E *p, double gamma, E *q, double *pq_part, CsScal *sc, E *l1, E *l2,
                        const StepFork &fk, cudaStream_t st) = 0;
 };

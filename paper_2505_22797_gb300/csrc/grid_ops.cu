@@ -244,7 +244,7 @@ template <typename R, typename AT, int CH, bool IL, bool COH>
 __device__ __forceinline__ void
 normal_units(const InterpRec<R> *__restrict__ rec, const R *__restrict__ vs, const AT *A, int nx, int ny, int ncx,
              const int *__restrict__ offset, const int *__restrict__ cunit_off, const int *__restrict__ unit_cell,
-             int n_units, R *unit_part)
+             int n_units, R *unit_part, int n_blocks)
 {
     constexpr int K = CH < 0 ? 2 : 1;
     constexpr int NC = 2 * K;
@@ -253,7 +253,7 @@ normal_units(const InterpRec<R> *__restrict__ rec, const R *__restrict__ vs, con
     const int sub = threadIdx.x % G;
     const int64_t N = (int64_t)nx * ny;
     const int n_iter = (n_units + per_block - 1) / per_block * per_block;
-    for (int base = blockIdx.x * per_block; base < n_iter; base += gridDim.x * per_block) {
+    for (int base = blockIdx.x * per_block; base < n_iter; base += n_blocks * per_block) {
         const int w = base + (int)threadIdx.x / G;
         R acc[4][NC];
 #pragma unroll
@@ -317,16 +317,6 @@ normal_units(const InterpRec<R> *__restrict__ rec, const R *__restrict__ vs, con
                 for (int m = 0; m < NC; ++m) unit_part[((int64_t)w * 4 + k) * NC + m] = acc[k][m];
         }
     }
-}
-
-template <typename R, typename AT, int CH, bool IL>
-__global__ void __launch_bounds__(kUnitThreads)
-k_interp_normal_cells(const InterpRec<R> *__restrict__ rec, const R *__restrict__ vs, const AT *__restrict__ A,
-                      int nx, int ny, int ncx, const int *__restrict__ offset, const int *__restrict__ cunit_off,
-                      const int *__restrict__ unit_cell, const int *__restrict__ n_units_dev,
-                      R *__restrict__ unit_part)
-{
-    normal_units<R, AT, CH, IL, false>(rec, vs, A, nx, ny, ncx, offset, cunit_off, unit_cell, *n_units_dev, unit_part);
 }
 
 // sum[m] += the unit sums of `corner` of units w0 .. w1 - 1, in unit order.
@@ -553,27 +543,6 @@ static int launch_interp_T(const GridH &g, int64_t T, const R *s_sorted, const B
     return MPI_OK;
 }
 
-// Unit sums of M^T M p (k_interp_normal_cells) for the Core Stage step.
-template <typename R, typename AT, bool IL>
-static int launch_normal_units(const GridH &g, const Bins &b, const AT *A, int ch, cudaStream_t st)
-{
-    const int nc = b.ncx * b.ncy;
-    constexpr int per_block = kUnitThreads / kUnitLanes;
-    const unsigned blocks = unit_blocks(b.n_units_max, per_block);
-    const InterpRec<R> *rec = static_cast<const InterpRec<R> *>(b.rec);
-    const R *vs = static_cast<const R *>(b.vs);
-    R *part = static_cast<R *>(b.unit_part);
-    const int *n_units = b.cunit_off + nc;
-    if (ch < 0)
-        k_interp_normal_cells<R, AT, -1, IL><<<blocks, kUnitThreads, 0, st>>>(
-            rec, vs, A, g.nx, g.ny, b.ncx, b.offset, b.cunit_off, b.unit_cell, n_units, part);
-    else
-        k_interp_normal_cells<R, AT, 0, IL><<<blocks, kUnitThreads, 0, st>>>(
-            rec, vs, A, g.nx, g.ny, b.ncx, b.offset, b.cunit_off, b.unit_cell, n_units, part);
-    MPI_CHECK_LAUNCH();
-    return MPI_OK;
-}
-
 // --- Laplacian and the Core Stage operator ---------------------------------
 
 // (Lap f)(node k at i, j): 5-point, replicated boundary (a missing
@@ -606,33 +575,44 @@ __device__ __forceinline__ df lap2_at(const df *f, int k, int i, int j, int nx, 
     return df_axpy(df_add(sx, sy), make_float2(-4.0f, 0.0f), c0);
 }
 
-// out_m = Lap x_m for the nc components (SCALE: w Lap x_m); E: FP64 or
-// double-float elements (and scalars).
-template <typename E, bool SCALE>
-__global__ void k_lap(int nx, int ny, int nc, bool scaled, E cx, E cy, const E *__restrict__ x, E *__restrict__ out,
-                      E w)
+// The first launch of a 2-D Core Stage step: the unit sums of M^T M p by the
+// first n_unit_blocks blocks, l1 = Lap p by the others.  Both read the
+// direction only, and neither fills the memory system alone.
+template <typename R, typename AT, int CH, bool IL, typename E>
+__global__ void __launch_bounds__(kUnitThreads)
+k_step_units(const InterpRec<R> *rec, const R *vs, const AT *A, int nx, int ny,
+             int ncx, const int *offset, const int *cunit_off,
+             const int *unit_cell, const int *n_units_dev, R *__restrict__ unit_part,
+             int n_unit_blocks, int nc, bool scaled, E cx, E cy, const E *p, E *__restrict__ l1)
 {
+    chain_wait();
+    if (int(blockIdx.x) < n_unit_blocks) {
+        normal_units<R, AT, CH, IL, false>(rec, vs, A, nx, ny, ncx, offset, cunit_off, unit_cell, *n_units_dev,
+                                           unit_part, n_unit_blocks);
+        return;
+    }
     const int N = nx * ny;  // nc N < 2^31 (grids of at most 2^28 nodes)
-    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < nc * N; e += gridDim.x * blockDim.x) {
-        const int m = e / N, k = e - m * N;
-        const E L = lap2_at(x + (int64_t)m * N, k, k % nx, k / nx, nx, ny, scaled, cx, cy);
-        out[e] = SCALE ? cs_scale(L, w) : L;
+    const int stride = (gridDim.x - n_unit_blocks) * kUnitThreads;
+    for (int64_t e = (blockIdx.x - n_unit_blocks) * kUnitThreads + threadIdx.x; e < (int64_t)nc * N; e += stride) {
+        const int m = int(e / N), k = int(e - (int64_t)m * N);
+        l1[e] = lap2_at(p + (int64_t)m * N, k, k % nx, k / nx, nx, ny, scaled, cx, cy);
     }
 }
 
 // One 2-D Core Stage step after the transpose's unit sums, one thread per
 // node and all its components m: q = scale * (the node's combine, as
-// k_interp_T_cell_combine forms it) + l2 with l2 = gamma Lap Lap p (formed
-// on the side stream), written to q, and the partial sums of <p, q> over
+// k_interp_T_cell_combine forms it) + gamma Lap l1 with l1 = Lap p, written to
+// q, and the partial sums of <p, q> over
 // blocks of kQThreads consecutive nodes, finished into alpha by the last
 // block.
 constexpr int kQThreads = 256;
 template <typename R, int NC, typename E>
 __global__ void __launch_bounds__(kQThreads)
-k_grid_q(int nx, int ny, int ncx, int ncy, const int *__restrict__ cunit_off, const R *__restrict__ unit_part,
-         E scale, const E *__restrict__ l2, const E *__restrict__ p, E *__restrict__ q, double *__restrict__ pq_part,
-         CsScal *sc)
+k_grid_q(int nx, int ny, int ncx, int ncy, const int *cunit_off, const R *unit_part,
+         E scale, bool scaled, E cx, E cy, E gamma, const E *l1, const E *p,
+         E *__restrict__ q, double *__restrict__ pq_part, CsScal *sc)
 {
+    chain_wait();
     __shared__ double sh[kQThreads / 32];
     __shared__ bool last;
     const int N = nx * ny;  // <= 2^28
@@ -653,7 +633,8 @@ k_grid_q(int nx, int ny, int ncx, int ncy, const int *__restrict__ cunit_off, co
 #pragma unroll
         for (int m = 0; m < NC; ++m) {
             const int64_t e = (int64_t)m * N + node;
-            const E qe = cs_sum_scale_add(sum[m], scale, l2[e]);
+            const E lap = lap2_at(l1 + (int64_t)m * N, node, i, j, nx, ny, scaled, cx, cy);
+            const E qe = cs_sum_scale_add(sum[m], scale, cs_scale(lap, gamma));
             q[e] = qe;
             acc.add(p[e], qe);
         }
@@ -708,9 +689,10 @@ k_cs_init(int64_t n, const E *__restrict__ b, E *__restrict__ r, E *__restrict__
 // counts the update.  Nothing once the solve has stopped.
 template <typename E>
 __global__ void __launch_bounds__(kCsThreads)
-k_cs_step1(int64_t n, E *__restrict__ x, E *__restrict__ r, const E *__restrict__ p, const E *__restrict__ q,
+k_cs_step1(int64_t n, E *__restrict__ x, E *__restrict__ r, const E *p, const E *q,
            double *__restrict__ rr_part, CsScal *sc)
 {
+    chain_wait();
     __shared__ double sh[kCsThreads / 32];
     __shared__ bool last;
     constexpr int U = kCsPer / kCsThreads;
@@ -755,8 +737,9 @@ k_cs_step1(int64_t n, E *__restrict__ x, E *__restrict__ r, const E *__restrict_
 // p = r + beta p.
 template <typename E>
 __global__ void __launch_bounds__(kCsThreads)
-k_cs_step2(int64_t n, const E *__restrict__ r, E *__restrict__ p, const CsScal *sc)
+k_cs_step2(int64_t n, const E *r, E *__restrict__ p, const CsScal *sc)
 {
+    chain_wait();
     if (sc->done) return;
     const E beta = cs_beta<E>(sc);
     const int64_t e0 = (int64_t)blockIdx.x * kCsPer;
@@ -790,8 +773,9 @@ __global__ void __launch_bounds__(kCsThreads) k_cs_round(int64_t N, const E *__r
 // p = r + beta p and its FP32 copy (one thread per node, all its components).
 template <typename E, int L>
 __global__ void __launch_bounds__(kCsThreads)
-k_cs_step2_p32(int64_t N, const E *__restrict__ r, E *__restrict__ p, const CsScal *sc, float *buf)
+k_cs_step2_p32(int64_t N, const E *r, E *__restrict__ p, const CsScal *sc, float *buf)
 {
+    chain_wait();
     constexpr int NC = p32_nc<L>();
     for (int64_t node = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; node < N;
          node += (int64_t)gridDim.x * blockDim.x) {
@@ -832,21 +816,21 @@ template <typename E>
 static int cs_step2_launch(const P32 &d, int64_t nv, const E *r, E *p, const CsScal *sc, cudaStream_t st)
 {
     if (!d.buf) {
-        k_cs_step2<E><<<cs_blocks(nv), kCsThreads, 0, st>>>(nv, r, p, sc);
+        launch_chained(k_cs_step2<E>, cs_blocks(nv), kCsThreads, 0, st, nv, r, p, sc);
     } else {
         const int blocks = grid_blocks(d.N);
         switch (d.layout) {
             case kP32Node4:
-                k_cs_step2_p32<E, kP32Node4><<<blocks, kCsThreads, 0, st>>>(d.N, r, p, sc, d.buf);
+                launch_chained(k_cs_step2_p32<E, kP32Node4>, blocks, kCsThreads, 0, st, d.N, r, p, sc, d.buf);
                 break;
             case kP32Node2:
-                k_cs_step2_p32<E, kP32Node2><<<blocks, kCsThreads, 0, st>>>(d.N, r, p, sc, d.buf);
+                launch_chained(k_cs_step2_p32<E, kP32Node2>, blocks, kCsThreads, 0, st, d.N, r, p, sc, d.buf);
                 break;
             case kP32Rows3x4:
-                k_cs_step2_p32<E, kP32Rows3x4><<<blocks, kCsThreads, 0, st>>>(d.N, r, p, sc, d.buf);
+                launch_chained(k_cs_step2_p32<E, kP32Rows3x4>, blocks, kCsThreads, 0, st, d.N, r, p, sc, d.buf);
                 break;
             default:
-                k_cs_step2_p32<E, kP32Rows1x4><<<blocks, kCsThreads, 0, st>>>(d.N, r, p, sc, d.buf);
+                launch_chained(k_cs_step2_p32<E, kP32Rows1x4>, blocks, kCsThreads, 0, st, d.N, r, p, sc, d.buf);
                 break;
         }
     }
@@ -883,7 +867,7 @@ struct Resident2 {
     __device__ __forceinline__ void phase(int) const
     {
         normal_units<float, float, CH, true, true>(rec, vs, p32, nx, ny, ncx, offset, cunit_off, unit_cell,
-                                                   cunit_off[ncx * ncy], unit_part);
+                                                   cunit_off[ncx * ncy], unit_part, gridDim.x);
     }
     __device__ __forceinline__ void combine(int node, SumAcc<float> (&sum)[kNC]) const
     {
@@ -908,10 +892,9 @@ struct Resident2 {
 };
 
 // The 2-D Core Stage operator: (1/T) M^T M through the binned records and
-// the 5-point Laplacian of each component.  A step: l2 = gamma Lap Lap p on
-// the side stream (two passes) while the main chain runs M p (through the
-// FP32 copy of p on the FP32 path) and the transpose's unit sums; then one
-// pass forms q and the <p, q> partials (k_grid_q).  The CG vectors are FP64
+// the 5-point Laplacian of each component.  A step is two launches: the unit
+// sums of M^T M p (from the FP32 copy of p on the FP32 path) beside l1 = Lap p,
+// then q with gamma Lap l1 and the <p, q> partials.  The CG vectors are FP64
 // (FP64 path) or double-float pairs (FP32 path: E = float2).
 template <typename R>
 struct GridOp2 final : CoreStageOp<typename CsElem<R>::type> {
@@ -948,33 +931,41 @@ struct GridOp2 final : CoreStageOp<typename CsElem<R>::type> {
             return ch < 0 ? resident_as<-1>(b, o, x, sc, st, taken) : resident_as<0>(b, o, x, sc, st, taken);
         return MPI_OK;
     }
+    bool forks() const override { return false; }
     int pq_blocks(int64_t) const override { return (int)((int64_t(g.nx) * g.ny + kQThreads - 1) / kQThreads); }
     int step_q(const E *p, double gamma, E *q, double *pq_part, CsScal *sc, E *l1, E *l2, const StepFork &fk,
                cudaStream_t st) override
     {
         E *tag = nullptr;
         const E cx = cs_host_scalar(1.0 / (g.dx * g.dx), tag), cy = cs_host_scalar(1.0 / (g.dy * g.dy), tag);
-        const int lb = grid_blocks(int64_t(nc) * g.nx * g.ny);
-        MPI_TRY_CUDA(cudaEventRecord(fk.fork, st));
-        MPI_TRY_CUDA(cudaStreamWaitEvent(fk.side, fk.fork, 0));
-        k_lap<E, false><<<lb, 256, 0, fk.side>>>(g.nx, g.ny, nc, scaled, cx, cy, p, l1, cs_host_scalar(1.0, tag));
+        const int64_t n = int64_t(nc) * g.nx * g.ny;
+        (void)l2;
+        (void)fk;
+        constexpr bool IL = sizeof(R) == 4;
+        using AT = std::conditional_t<IL, R, double>;
+        const AT *A;
+        if constexpr (IL) A = p_r;
+        else A = p;
+        const InterpRec<R> *rec = static_cast<const InterpRec<R> *>(bins.rec);
+        const R *vs = static_cast<const R *>(bins.vs);
+        R *part = static_cast<R *>(bins.unit_part);
+        const unsigned nu = unit_blocks(bins.n_units_max, kUnitThreads / kUnitLanes);
+        const unsigned nl = (unsigned)std::min<int64_t>((n + kUnitThreads - 1) / kUnitThreads, 8192);
+        auto units = [&](auto kernel) {
+            launch_chained(kernel, nu + nl, kUnitThreads, 0, st, rec, vs, A, g.nx, g.ny, bins.ncx, bins.offset,
+                           bins.cunit_off, bins.unit_cell, bins.cunit_off + bins.ncx * bins.ncy, part, (int)nu, nc, scaled,
+                           cx, cy, p, l1);
+        };
+        auto form_q = [&](auto kernel) {
+            launch_chained(kernel, (unsigned)pq_blocks(0), kQThreads, 0, st, g.nx, g.ny, bins.ncx, bins.ncy,
+                           bins.cunit_off, part, cs_host_scalar(invT, tag), scaled, cx, cy, cs_host_scalar(gamma, tag), l1,
+                           p, q, pq_part, sc);
+        };
+        if (ch < 0) units(k_step_units<R, AT, -1, IL, E>);
+        else units(k_step_units<R, AT, 0, IL, E>);
         MPI_CHECK_LAUNCH();
-        k_lap<E, true><<<lb, 256, 0, fk.side>>>(g.nx, g.ny, nc, scaled, cx, cy, l1, l2, cs_host_scalar(gamma, tag));
-        MPI_CHECK_LAUNCH();
-        MPI_TRY_CUDA(cudaEventRecord(fk.join, fk.side));
-        // main branch: the unit sums of M^T M p, one pass over the samples
-        if constexpr (sizeof(R) == 4) MPI_TRY((launch_normal_units<R, R, true>(g, bins, p_r, ch, st)));
-        else MPI_TRY((launch_normal_units<R, double, false>(g, bins, reinterpret_cast<const double *>(p), ch, st)));
-        MPI_TRY_CUDA(cudaStreamWaitEvent(st, fk.join, 0));
-        const unsigned blocks = (unsigned)pq_blocks(0);
-        const R *part = static_cast<const R *>(bins.unit_part);
-        const E sc_T = cs_host_scalar(invT, tag);
-        if (ch < 0)
-            k_grid_q<R, 4, E><<<blocks, kQThreads, 0, st>>>(g.nx, g.ny, bins.ncx, bins.ncy, bins.cunit_off, part,
-                                                           sc_T, l2, p, q, pq_part, sc);
-        else
-            k_grid_q<R, 2, E><<<blocks, kQThreads, 0, st>>>(g.nx, g.ny, bins.ncx, bins.ncy, bins.cunit_off, part,
-                                                           sc_T, l2, p, q, pq_part, sc);
+        if (ch < 0) form_q(k_grid_q<R, 4, E>);
+        else form_q(k_grid_q<R, 2, E>);
         MPI_CHECK_LAUNCH();
         return MPI_OK;
     }
@@ -1099,9 +1090,11 @@ int core_stage_cg(CoreStageOp<E> &op, int64_t nv, const E *b, const mpi_grid_opt
             if (f.join) cudaEventDestroy(f.join);
         }
     } fk;
-    MPI_TRY_CUDA(cudaStreamCreateWithFlags(&fk.f.side, cudaStreamNonBlocking));
-    MPI_TRY_CUDA(cudaEventCreateWithFlags(&fk.f.fork, cudaEventDisableTiming));
-    MPI_TRY_CUDA(cudaEventCreateWithFlags(&fk.f.join, cudaEventDisableTiming));
+    if (op.forks()) {
+        MPI_TRY_CUDA(cudaStreamCreateWithFlags(&fk.f.side, cudaStreamNonBlocking));
+        MPI_TRY_CUDA(cudaEventCreateWithFlags(&fk.f.fork, cudaEventDisableTiming));
+        MPI_TRY_CUDA(cudaEventCreateWithFlags(&fk.f.join, cudaEventDisableTiming));
+    }
 
     MPI_TRY_CUDA(cudaMemsetAsync(x, 0, vb, st));
     MPI_TRY_CUDA(cudaMemsetAsync(sc, 0, sizeof(CsScal), st));
@@ -1119,7 +1112,7 @@ int core_stage_cg(CoreStageOp<E> &op, int64_t nv, const E *b, const mpi_grid_opt
     // FP32 copy).
     auto enqueue_step = [&](int, cudaStream_t s) -> int {
         MPI_TRY(op.step_q(p, o.gamma, q, pq_part, sc, l1, l2, fk.f, s));
-        k_cs_step1<E><<<ncs, kCsThreads, 0, s>>>(nv, x, rr, p, q, rr_part, sc);
+        launch_chained(k_cs_step1<E>, ncs, kCsThreads, 0, s, nv, x, rr, p, q, rr_part, sc);
         MPI_CHECK_LAUNCH();
         return cs_step2_launch(p32, nv, rr, p, sc, s);
     };
