@@ -5,7 +5,7 @@
 // the solve has a fixed order.
 //
 // The ordering is a least-significant-digit radix sort of the cell indices
-// (8-bit digits, as many passes as the largest cell index has digits).  Each
+// (9-bit digits, as many passes as the largest cell index has digits).  Each
 // pass is stable, so a cell's samples keep their ascending order and no
 // per-cell sort follows.  One pass is three launches: a digit histogram per
 // tile of kSortTile samples, an exclusive scan of the histograms in
@@ -19,11 +19,11 @@ namespace mpi {
 
 namespace {
 
-constexpr int kSortThreads = 256;                      // 8 warps
+constexpr int kSortThreads = 512;                      // 16 warps
 constexpr int kSortWarps = kSortThreads / 32;
-constexpr int kSortRounds = 8;                         // items per thread and tile
+constexpr int kSortRounds = 4;                         // items per thread and tile
 constexpr int kSortTile = kSortThreads * kSortRounds;  // 2048 samples
-constexpr int kDigitBits = 8;
+constexpr int kDigitBits = 9;                          // 512 x 512 grids in two passes
 constexpr int kDigits = 1 << kDigitBits;
 static_assert(kSortThreads == kDigits, "the tile bookkeeping runs one thread per digit");
 
@@ -40,8 +40,9 @@ inline int scan_tiles(int64_t n) { return (int)std::max<int64_t>(1, (n + kScanTi
 // Per-tile digit counts, hist[d * n_tiles + tile].  Lanes holding the same
 // digit add once (the trajectory keeps consecutive samples in one cell).
 __global__ void __launch_bounds__(kSortThreads)
-k_digit_hist(const int *__restrict__ key, int64_t n, int shift, int n_tiles, int *__restrict__ hist)
+k_digit_hist(const int *key, int64_t n, int shift, int n_tiles, int *__restrict__ hist)
 {
+    chain_wait();
     __shared__ int h[kDigits];
     h[threadIdx.x] = 0;
     __syncthreads();
@@ -64,10 +65,11 @@ k_digit_hist(const int *__restrict__ key, int64_t n, int shift, int n_tiles, int
 // formed from the histogram of the same digits, so it lies in [0, n) whatever
 // the keys hold.
 __global__ void __launch_bounds__(kSortThreads)
-k_digit_scatter(const int *__restrict__ key_in, const int *__restrict__ val_in, int64_t n, int shift,
-                int n_tiles, const int *__restrict__ pos, int *__restrict__ key_out,
+k_digit_scatter(const int *key_in, const int *val_in, int64_t n, int shift,
+                int n_tiles, const int *pos, int *__restrict__ key_out,
                 int *__restrict__ val_out)
 {
+    chain_wait();
     __shared__ int s_next[kDigits];              // next position of each digit for this tile
     __shared__ int s_warp[kSortWarps][kDigits];  // a round's items per warp and digit, then their prefix
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -109,6 +111,7 @@ k_digit_scatter(const int *__restrict__ key_in, const int *__restrict__ val_in, 
 
 __global__ void k_iota(int64_t n, int *__restrict__ out)
 {
+    chain_wait();
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
         out[i] = int(i);
 }
@@ -142,8 +145,9 @@ __device__ __forceinline__ int block_scan_excl(int v, int *s_w, int *total)
 
 // Sum of each tile of kScanTile entries.
 __global__ void __launch_bounds__(kScanBlock)
-k_scan_reduce(const int *__restrict__ in, int64_t n, int *__restrict__ part)
+k_scan_reduce(const int *in, int64_t n, int *__restrict__ part)
 {
+    chain_wait();
     __shared__ int s_w[32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t i0 = int64_t(blockIdx.x) * kScanTile + int64_t(threadIdx.x) * kScanPer;
@@ -163,6 +167,7 @@ k_scan_reduce(const int *__restrict__ in, int64_t n, int *__restrict__ part)
 // Exclusive scan of the nb tile sums in place; part[nb] = the total.
 __global__ void __launch_bounds__(kScanBlock) k_scan_top(int nb, int *__restrict__ part)
 {
+    chain_wait();
     __shared__ int s_w[32];
     const int per = (nb + kScanBlock - 1) / kScanBlock;
     const int b0 = threadIdx.x * per, b1 = min(nb, b0 + per);
@@ -181,8 +186,9 @@ __global__ void __launch_bounds__(kScanBlock) k_scan_top(int nb, int *__restrict
 // out[i] = part[tile] + the exclusive prefix of in within the tile; out[n] =
 // the total.  in and out are distinct arrays.
 __global__ void __launch_bounds__(kScanBlock)
-k_scan_tiles(const int *__restrict__ in, int64_t n, const int *__restrict__ part, int nb, int *__restrict__ out)
+k_scan_tiles(const int *in, int64_t n, const int *part, int nb, int *__restrict__ out)
 {
+    chain_wait();
     __shared__ int s_w[32];
     const int64_t i0 = int64_t(blockIdx.x) * kScanTile + int64_t(threadIdx.x) * kScanPer;
     int c[kScanPer];
@@ -204,8 +210,9 @@ k_scan_tiles(const int *__restrict__ in, int64_t n, const int *__restrict__ part
 
 // count[c] = the number of samples with cell_of[t] = c; values outside
 // [0, n_cells) are not counted.
-__global__ void k_cell_hist(const int *__restrict__ cell_of, int64_t T, int n_cells, int *__restrict__ count)
+__global__ void k_cell_hist(const int *cell_of, int64_t T, int n_cells, int *__restrict__ count)
 {
+    chain_wait();
     for (int64_t t0 = int64_t(blockIdx.x) * blockDim.x; t0 < T; t0 += int64_t(gridDim.x) * blockDim.x) {
         const int64_t t = t0 + threadIdx.x;
         int c = t < T ? cell_of[t] : -1;
@@ -233,11 +240,11 @@ int cell_scan_launch(const int *count, int64_t n, int *offset, void *tmp, cudaSt
     }
     int *part = static_cast<int *>(tmp);
     const int nb = scan_tiles(n);
-    k_scan_reduce<<<nb, kScanBlock, 0, st>>>(count, n, part);
+    launch_chained(k_scan_reduce, nb, kScanBlock, 0, st, count, n, part);
     MPI_CHECK_LAUNCH();
-    k_scan_top<<<1, kScanBlock, 0, st>>>(nb, part);
+    launch_chained(k_scan_top, 1, kScanBlock, 0, st, nb, part);
     MPI_CHECK_LAUNCH();
-    k_scan_tiles<<<nb, kScanBlock, 0, st>>>(count, n, part, nb, offset);
+    launch_chained(k_scan_tiles, nb, kScanBlock, 0, st, count, n, part, nb, offset);
     MPI_CHECK_LAUNCH();
     return MPI_OK;
 }
@@ -248,7 +255,7 @@ int cell_order_launch(int64_t T, const int *cell_of, int n_cells, int *list, voi
     const int bits = n_cells > 1 ? 32 - __builtin_clz(unsigned(n_cells - 1)) : 0;
     const int passes = (bits + kDigitBits - 1) / kDigitBits;
     if (passes == 0) {  // one cell: the identity order
-        k_iota<<<grid_blocks(T), 256, 0, st>>>(T, list);
+        launch_chained(k_iota, grid_blocks(T), 256, 0, st, T, list);
         MPI_CHECK_LAUNCH();
         return MPI_OK;
     }
@@ -268,10 +275,10 @@ int cell_order_launch(int64_t T, const int *cell_of, int n_cells, int *list, voi
         const bool last = q == passes - 1;
         int *kout = last ? nullptr : kbuf[q & 1];
         int *vout = last ? list : vbuf[q & 1];
-        k_digit_hist<<<nt, kSortThreads, 0, st>>>(kin, T, q * kDigitBits, nt, hist);
+        launch_chained(k_digit_hist, nt, kSortThreads, 0, st, kin, T, q * kDigitBits, nt, hist);
         MPI_CHECK_LAUNCH();
         MPI_TRY(cell_scan_launch(hist, nh, pos, p, st));
-        k_digit_scatter<<<nt, kSortThreads, 0, st>>>(kin, vin, T, q * kDigitBits, nt, pos, kout, vout);
+        launch_chained(k_digit_scatter, nt, kSortThreads, 0, st, kin, vin, T, q * kDigitBits, nt, pos, kout, vout);
         MPI_CHECK_LAUNCH();
         kin = kout;
         vin = vout;
@@ -299,7 +306,7 @@ extern "C" int mpi_cell_order(int64_t T, const int *cell_of, int n_cells, int *l
         int *count = scr.at<int>(o_cnt);
         MPI_TRY_CUDA(cudaMemsetAsync(count, 0, sizeof(int) * size_t(n_cells), st));
         if (T > 0) {
-            k_cell_hist<<<grid_blocks(T), 256, 0, st>>>(cell_of, T, n_cells, count);
+            launch_chained(k_cell_hist, grid_blocks(T), 256, 0, st, cell_of, T, n_cells, count);
             MPI_CHECK_LAUNCH();
         }
         MPI_TRY(cell_scan_launch(count, n_cells, offset, scr.at<char>(o_tmp), st));

@@ -5,8 +5,16 @@
 // the work.  Here one thread owns one node for the whole solve, with the
 // residual and the direction of all its components in registers; a step is
 // its phases with a grid barrier between them, and the stop test runs on the
-// device (the host polls nothing).  Blocks read one another's vectors
-// through L2 (__ldcg).
+// device (the host polls nothing).  The barrier's release and acquire order
+// the blocks' vectors for one another, so these are read by ordinary loads
+// (from L1 where a neighbour in the block has read the line: the two
+// Laplacians read each node seven times in 3-D); their pointers must not be
+// __restrict__, which would let them take the path for constant data.
+//
+// Measured on GB300: 48 x 48 x 24 / 65 536 samples, 20 steps with the setup
+// 1.02 ms (by launches 1.33 ms); 100 x 100 / 1632 samples to the tolerance,
+// 65 steps, 34 us a step (by launches 48 us).  Four (2-D) or five (3-D)
+// barriers and the L2 latency of what crosses them bound a step.
 #pragma once
 
 #include "grid_common.cuh"
@@ -15,6 +23,7 @@ namespace mpi {
 
 constexpr int kResThreads = 256;
 constexpr int kResMinBlocks = 2;
+constexpr int kResFlat = 2048;  // unknowns per partial sum of r.r
 
 // Barrier of all blocks of a cooperative launch: `arrived` counts up for the
 // life of the launch.  A wait gives up after kResSpin polls (seconds) and
@@ -26,13 +35,6 @@ struct ResBarrier {
 constexpr int kResSpin = 1 << 22;
 
 #ifdef __CUDACC__
-
-// Loads of data that other blocks write during the launch (COH) or before it.
-template <bool COH, typename T> __device__ __forceinline__ T ld_shared_by_blocks(const T *p)
-{
-    if constexpr (COH) return __ldcg(p);
-    else return *p;
-}
 
 // All threads call it; false once a wait has given up.  The block's writes
 // are ordered before its arrival (bar.sync, then a release by thread 0), the
@@ -60,44 +62,93 @@ __device__ __forceinline__ bool res_barrier(ResBarrier *b, unsigned long long &t
     return *s_ok != 0;
 }
 
+// The block's partial sums of v over groups of PT consecutive threads, as
+// CsDot::block_total<PT> forms them; part[group] for the first n_part groups.
+template <int PT>
+__device__ __forceinline__ void res_partials(F2Sum v, F2Sum *w, double *part, int n_part)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        F2Sum t;
+        t.hi = __shfl_xor_sync(0xffffffffu, v.hi, o);
+        t.lo = __shfl_xor_sync(0xffffffffu, v.lo, o);
+        v.add(t);
+    }
+    __syncthreads();  // (w may still be read)
+    if ((threadIdx.x & 31) == 0) w[threadIdx.x >> 5] = v;
+    __syncthreads();
+    constexpr int G = kResThreads / PT, W = PT / 32;
+    const int group = blockIdx.x * G + threadIdx.x;
+    if (threadIdx.x < G && group < n_part) {
+        F2Sum s = w[threadIdx.x * W];
+#pragma unroll
+        for (int k = 1; k < W; ++k) s.add(w[threadIdx.x * W + k]);
+        part[group] = s.value();
+    }
+}
+
+// Their sum as cs_sum_parts<PT> forms it, in thread 0.  (FP64 additions take
+// a warp 19 clocks: warps without a partial leave them out.)
+template <int PT>
+__device__ __forceinline__ double res_sum(const double *part, int n, double *sh)
+{
+    const int warp = threadIdx.x >> 5;
+    if (threadIdx.x < PT && 32 * warp < n) {
+        double a = 0.0;
+        for (int k = threadIdx.x; k < n; k += PT) a += part[k];
+        a = warp_sum(a);
+        if ((threadIdx.x & 31) == 0) sh[warp] = a;
+    }
+    __syncthreads();
+    double t = 0.0;
+    if (threadIdx.x == 0)
+        for (int w = 0; w < PT / 32 && 32 * w < n; ++w) t += sh[w];
+    return t;
+}
+
 // One solve.  Op: kNC components; kPhases phases of M^T M p (phase(k) by all
 // threads, a barrier after each); combine(node, sum), the node's sums of the
 // transpose; lap(f, node); store_p32(node, v), the FP32 copy of the direction
-// that phase(0) reads; scalars scale = 1/T and gamma.  p, l1: kNC N elements;
-// part: 2 gridDim.x doubles; bar zeroed before the launch.
+// that phase(0) reads; kPqThreads; scalars scale = 1/T and gamma.  p, l1, q:
+// kNC N elements; pq_part, rr_part: their partial sums; bar zeroed before the
+// launch.
+//
+// Every sum is taken in the order of the step by launches, so that both give
+// the same bits (a solve to a tolerance on a badly conditioned system carries
+// a last-bit difference into the fourth digit of the field): <p, q> over
+// groups of kPqThreads nodes, r.r over blocks of kResFlat unknowns in memory
+// order.  For the latter the first blocks also keep the residual in that
+// order and update it from q, which the owners of the nodes leave in memory.
 template <class Op>
 __global__ void __launch_bounds__(kResThreads, kResMinBlocks)
 k_cs_resident(const __grid_constant__ Op op, int N, const float2 *__restrict__ b, float2 *x, float2 *p, float2 *l1,
-              double rel_tol, int max_iter, double *part, CsScal *sc, ResBarrier *bar)
+              float2 *qv, double rel_tol, int max_iter, double *pq_part, double *rr_part, CsScal *sc, ResBarrier *bar)
 {
-    constexpr int NC = Op::kNC;
+    constexpr int NC = Op::kNC, PT = Op::kPqThreads, U = kResFlat / kResThreads;
     __shared__ double sh[kResThreads / 32];
+    __shared__ F2Sum sw[kResThreads / 32];
     __shared__ df s_coef;
     __shared__ int s_ok, s_stop;
     unsigned long long target = 0;
     const int node = blockIdx.x * kResThreads + threadIdx.x;
     const bool in = node < N;
+    const int n_pq = (N + PT - 1) / PT;
+    const int64_t n = (int64_t)NC * N, flat0 = (int64_t)blockIdx.x * kResFlat + threadIdx.x;
+    const int n_rr = (int)((n + kResFlat - 1) / kResFlat);
+    const bool flat = int(blockIdx.x) < n_rr;
     bool ok = true;
-    // Sum over all threads in a fixed order; a barrier.  The sum is known to
-    // thread 0 of every block, which calls then(sum): FP64 arithmetic takes a
-    // whole warp 19 clocks an instruction here, so one thread forms the
-    // step's scalars.
-    auto grid_sum = [&](const CsDot<df> &acc, int slot, auto then) {
-        const double t = acc.template block_total<kResThreads>(sh);
-        double *mine = part + slot * gridDim.x;
-        if (threadIdx.x == 0) mine[blockIdx.x] = t;
-        ok = res_barrier(bar, target, &s_ok) && ok;
-        if (threadIdx.x < 32) {
-            double a = 0.0;
-            for (int k = threadIdx.x; k < int(gridDim.x); k += 32) a += __ldcg(mine + k);
-            a = warp_sum(a);
-            if (threadIdx.x == 0) then(a);
-        }
-        __syncthreads();
-    };
     double rr = 0.0, tol = -1.0;  // thread 0's
-    df r[NC], d[NC];
-    CsDot<df> acc{};
+    df r[NC], d[NC], rf[U];
+    if (flat) {
+        CsDot<df> acc{};
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int64_t e = flat0 + u * kResThreads;
+            rf[u] = e < n ? b[e] : make_float2(0.0f, 0.0f);
+            if (e < n) acc.add(rf[u], rf[u]);
+        }
+        res_partials<kResThreads>(acc.s, sw, rr_part, n_rr);
+    }
     if (in) {
         float v[NC];
 #pragma unroll
@@ -106,15 +157,16 @@ k_cs_resident(const __grid_constant__ Op op, int N, const float2 *__restrict__ b
             r[m] = d[m] = b[e];
             x[e] = make_float2(0.0f, 0.0f);
             p[e] = d[m];
-            acc.add(r[m], r[m]);
             v[m] = cs_to_float(d[m]);
         }
         op.store_p32(node, v);
     }
-    grid_sum(acc, 0, [&](double v) {
+    ok = res_barrier(bar, target, &s_ok);
+    {
+        const double v = res_sum<kResThreads>(rr_part, n_rr, sh);
         rr = v;
         tol = rel_tol > 0.0 ? rel_tol * sqrt(v) : -1.0;
-    });
+    }
     int it = 0;
     for (; ok && it < max_iter; ++it) {
         if (in) {
@@ -135,29 +187,51 @@ k_cs_resident(const __grid_constant__ Op op, int N, const float2 *__restrict__ b
 #pragma unroll
             for (int m = 0; m < NC; ++m) {
                 q[m] = cs_sum_scale_add(sum[m], op.scale, df_mul(op.lap(l1 + (int64_t)m * N, node), op.gamma));
+                qv[(int64_t)m * N + node] = q[m];
                 pq_acc.add(d[m], q[m]);
             }
         }
-        grid_sum(pq_acc, 1, [&](double pq) {
-            s_stop = rr == 0.0 || pq == 0.0 || (tol >= 0.0 && sqrt(rr) <= tol);
-            s_coef = df_from_double(rr / pq);
-        });
+        res_partials<PT>(pq_acc.s, sw, pq_part, n_pq);
+        ok = res_barrier(bar, target, &s_ok) && ok;
+        {
+            const double pq = res_sum<PT>(pq_part, n_pq, sh);
+            if (threadIdx.x == 0) {
+                s_stop = rr == 0.0 || pq == 0.0 || (tol >= 0.0 && sqrt(rr) <= tol);
+                s_coef = df_from_double(rr / pq);
+            }
+            __syncthreads();
+        }
         if (!ok || s_stop) break;
         const df al = s_coef, nal = df_neg(al);
-        CsDot<df> rr_acc{};
+        if (flat) {
+            CsDot<df> acc{};
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int64_t e = flat0 + u * kResThreads;
+                if (e < n) {
+                    rf[u] = df_axpy(rf[u], nal, qv[e]);
+                    acc.add(rf[u], rf[u]);
+                }
+            }
+            res_partials<kResThreads>(acc.s, sw, rr_part, n_rr);
+        }
         if (in) {
 #pragma unroll
             for (int m = 0; m < NC; ++m) {
                 const int64_t e = (int64_t)m * N + node;
                 x[e] = df_axpy(x[e], al, d[m]);
                 r[m] = df_axpy(r[m], nal, q[m]);
-                rr_acc.add(r[m], r[m]);
             }
         }
-        grid_sum(rr_acc, 0, [&](double v) {
-            s_coef = df_from_double(v / rr);
-            rr = v;
-        });
+        ok = res_barrier(bar, target, &s_ok) && ok;
+        {
+            const double v = res_sum<kResThreads>(rr_part, n_rr, sh);
+            if (threadIdx.x == 0) {
+                s_coef = df_from_double(v / rr);
+                rr = v;
+            }
+            __syncthreads();
+        }
         const df be = s_coef;
         if (in) {
             float v[NC];
@@ -193,21 +267,23 @@ int launch_resident(const Op &op, int64_t N, int64_t work, const float2 *b, cons
     int per_sm = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kResThreads, 0) != cudaSuccess) return MPI_OK;
     const int64_t most = (int64_t)std::min(per_sm, kResMinBlocks) * device_sm_count();
-    const int64_t need = (N + kResThreads - 1) / kResThreads;
+    const int64_t n_rr = (Op::kNC * N + kResFlat - 1) / kResFlat, n_pq = (N + Op::kPqThreads - 1) / Op::kPqThreads;
+    const int64_t need = std::max((N + kResThreads - 1) / kResThreads, n_rr);
     if (need > most) return MPI_OK;
     int grid = (int)std::min(most, std::max(need, work * 32 / kResThreads));
     Scratch scr(st);
     const size_t vb = sizeof(float2) * Op::kNC * N;
-    const size_t o_p = scr.reserve(vb), o_l = scr.reserve(vb), o_part = scr.reserve(sizeof(double) * 2 * grid),
+    const size_t o_p = scr.reserve(vb), o_l = scr.reserve(vb), o_q = scr.reserve(vb),
+                 o_pq = scr.reserve(sizeof(double) * n_pq), o_rr = scr.reserve(sizeof(double) * n_rr),
                  o_bar = scr.reserve(sizeof(ResBarrier));
     MPI_TRY(scr.allocate());
-    float2 *p = scr.at<float2>(o_p), *l1 = scr.at<float2>(o_l);
-    double *part = scr.at<double>(o_part), rel_tol = o.rel_tol;
+    float2 *p = scr.at<float2>(o_p), *l1 = scr.at<float2>(o_l), *q = scr.at<float2>(o_q);
+    double *pq_part = scr.at<double>(o_pq), *rr_part = scr.at<double>(o_rr), rel_tol = o.rel_tol;
     ResBarrier *bar = scr.at<ResBarrier>(o_bar);
     int n = (int)N, max_iter = o.max_iter;
     Op arg = op;
     MPI_TRY_CUDA(cudaMemsetAsync(bar, 0, sizeof(ResBarrier), st));
-    void *args[] = {&arg, &n, &b, &x, &p, &l1, &rel_tol, &max_iter, &part, &sc, &bar};
+    void *args[] = {&arg, &n, &b, &x, &p, &l1, &q, &rel_tol, &max_iter, &pq_part, &rr_part, &sc, &bar};
     if (cudaLaunchCooperativeKernel(kern, dim3(grid), dim3(kResThreads), args, 0, st) != cudaSuccess) {
         (void)cudaGetLastError();  // the launches do the same
         return MPI_OK;

@@ -44,9 +44,9 @@ __device__ __forceinline__ InterpRec3<R> make_rec3(R px, R py, R pz, const Axes3
 {
     InterpRec3<R> q;
     R w0;
-    axis_weights<R>(px, a.x, q.i0, w0, q.wx1);
-    axis_weights<R>(py, a.y, q.j0, w0, q.wy1);
-    axis_weights<R>(pz, a.z, q.l0, w0, q.wz1);
+    axis_weights(px, a.x, q.i0, w0, q.wx1);
+    axis_weights(py, a.y, q.j0, w0, q.wy1);
+    axis_weights(pz, a.z, q.l0, w0, q.wz1);
     return q;
 }
 
@@ -58,8 +58,8 @@ __device__ __forceinline__ InterpRec3<R> make_rec3(R px, R py, R pz, const Axes3
 // records precomputed): the field is node-interleaved, A4[node K + k] =
 // (A_{3k}, A_{3k+1}, A_{3k+2}, 0) with K rows, so a corner's three
 // components are one 16-byte load.
-// COH: the field is written during the launch.
-template <typename R, typename AT, int CH, bool PRE, bool IL, bool COH>
+// (The field may be written during the launch: it is not __restrict__.)
+template <typename R, typename AT, int CH, bool PRE, bool IL>
 __device__ __forceinline__ void interp3_outputs(int64_t T, const R *__restrict__ r, const InterpRec3<R> *__restrict__ rec,
                                                 const R *__restrict__ v, const AT *A, int nx, int ny, int nz,
                                                 const Axes3 &ax, R *s)
@@ -83,7 +83,7 @@ __device__ __forceinline__ void interp3_outputs(int64_t T, const R *__restrict__
         R acc = R(0);
         if constexpr (IL) {
             const float4 *A4 = reinterpret_cast<const float4 *>(A);
-            auto ld = [&](int64_t node) { return ld_shared_by_blocks<COH>(A4 + node * K + k); };
+            auto ld = [&](int64_t node) { return A4[node * K + k]; };
             const float4 a000 = ld(r00 + i0), a100 = ld(r00 + i1), a010 = ld(r01 + i0), a110 = ld(r01 + i1);
             const float4 a001 = ld(r10 + i0), a101 = ld(r10 + i1), a011 = ld(r11 + i0), a111 = ld(r11 + i1);
             auto tri = [&](float c000, float c100, float c010, float c110, float c001, float c101, float c011,
@@ -115,13 +115,14 @@ __global__ void __launch_bounds__(256)
 k_interp3(int64_t T, const R *__restrict__ r, const InterpRec3<R> *__restrict__ rec,
           const R *__restrict__ v, const AT *__restrict__ A, Axes3 ax, R *__restrict__ s)
 {
-    interp3_outputs<R, AT, CH, PRE, IL, false>(T, r, rec, v, A, ax.x.n, ax.y.n, ax.z.n, ax, s);
+    interp3_outputs<R, AT, CH, PRE, IL>(T, r, rec, v, A, ax.x.n, ax.y.n, ax.z.n, ax, s);
 }
 
 template <typename R>
-__global__ void k_cell_count3(int64_t T, const R *__restrict__ r, Axes3 ax, int ncx, int ncy,
+__global__ void k_cell_count3(int64_t T, const R *r, Axes3 ax, int ncx, int ncy,
                               int *__restrict__ cell_of, int *__restrict__ count, InterpRec3<R> *__restrict__ rec)
 {
+    chain_wait();
     // every lane of a warp runs the same iterations (warp_count_add)
     for (int64_t t0 = int64_t(blockIdx.x) * blockDim.x; t0 < T; t0 += int64_t(gridDim.x) * blockDim.x) {
         const int64_t t = t0 + threadIdx.x;
@@ -180,8 +181,8 @@ __device__ __forceinline__ V2<double> cell_pair(const SumAcc<double> &a) { retur
 // the cell's corner-`corner` sum of w_dx w_dy w_dz v_m s_k (CH < 0: 9 sums,
 // component 3k + m; CH = k: channel k only, 3 sums).  cell_cnt: zero on entry
 // and on exit.
-// COH: s is written during the launch.
-template <typename R, int CH, bool COH>
+// (s may be written during the launch: it is not __restrict__.)
+template <typename R, int CH>
 __device__ __forceinline__ void T3_units(const InterpRec3<R> *__restrict__ rec, const R *__restrict__ vs, const R *s,
                                          int64_t T, const int *__restrict__ offset, const int *__restrict__ cunit_off,
                                          const int *__restrict__ unit_cell, int n_units, R *unit_part, V2<R> *cell_part,
@@ -211,13 +212,13 @@ __device__ __forceinline__ void T3_units(const InterpRec3<R> *__restrict__ rec, 
             if constexpr (CH < 0) {
 #pragma unroll
                 for (int kk = 0; kk < 3; ++kk) {
-                    const R sk = wt * ld_shared_by_blocks<COH>(s + (int64_t)kk * T + q);
+                    const R sk = wt * s[(int64_t)kk * T + q];
                     acc[3 * kk] += v0 * sk;
                     acc[3 * kk + 1] += v1 * sk;
                     acc[3 * kk + 2] += v2 * sk;
                 }
             } else {
-                const R sk = wt * ld_shared_by_blocks<COH>(s + q);
+                const R sk = wt * s[q];
                 acc[0] += v0 * sk;
                 acc[1] += v1 * sk;
                 acc[2] += v2 * sk;
@@ -264,18 +265,13 @@ k_interp3_T_cells(const InterpRec3<R> *__restrict__ rec, const R *__restrict__ v
                   const int *__restrict__ unit_cell, const int *__restrict__ n_units_dev,
                   R *__restrict__ unit_part, V2<R> *__restrict__ cell_part, unsigned *__restrict__ cell_cnt)
 {
-    T3_units<R, CH, false>(rec, vs, s, T, offset, cunit_off, unit_cell, *n_units_dev, unit_part, cell_part, cell_cnt);
+    T3_units<R, CH>(rec, vs, s, T, offset, cunit_off, unit_cell, *n_units_dev, unit_part, cell_part, cell_cnt);
 }
 
 // The combine of one node (at i, j, l), all NC components: the sums, over
 // the node's adjacent non-empty cells in ascending cell order, of the cell
 // sums of the corner the node is in that cell.
-__device__ __forceinline__ V2<float> ld_pair_cg(const V2<float> *p)
-{
-    const float2 q = __ldcg(reinterpret_cast<const float2 *>(p));
-    return V2<float>{q.x, q.y};
-}
-template <typename R, int NC, bool COH = false>
+template <typename R, int NC>
 __device__ __forceinline__ void node_combine3(int i, int j, int l, int ncx, int ncy, int ncz,
                                               const int *__restrict__ cunit_off,
                                               const V2<R> *cell_part, SumAcc<R> (&sum)[NC])
@@ -293,10 +289,7 @@ __device__ __forceinline__ void node_combine3(int i, int j, int l, int ncx, int 
                 if (cunit_off[cc + 1] == u0) continue;
                 const V2<R> *cp = cell_part + ((int64_t)u0 * 8 + dx + 2 * dy + 4 * dz) * NC;
 #pragma unroll
-                for (int m = 0; m < NC; ++m) {
-                    if constexpr (COH) cell_add(sum[m], ld_pair_cg(cp + m));
-                    else cell_add(sum[m], cp[m]);
-                }
+                for (int m = 0; m < NC; ++m) cell_add(sum[m], cp[m]);
             }
 }
 
@@ -336,11 +329,10 @@ __device__ __forceinline__ double lap3_at(const double *__restrict__ f, int64_t 
     return f[k + xm] + f[k + xp] + f[k + ym] + f[k + yp] + f[k + zm] + f[k + zp] - 6.0 * f[k];
 }
 // The same in double-float arithmetic (coefficients as double-float pairs).
-template <bool COH = false>
 __device__ __forceinline__ df lap3_at(const df *f, int64_t k, int i, int j, int l, int nx, int ny,
                                       int nz, bool scaled, Coef3<df> c)
 {
-    auto at = [&](int64_t e) { return ld_shared_by_blocks<COH>(f + e); };
+    auto at = [&](int64_t e) { return f[e]; };
     const int64_t sx = 1, sy = nx, sz = (int64_t)nx * ny;
     const int64_t xm = i > 0 ? -sx : 0, xp = i < nx - 1 ? sx : 0;
     const int64_t ym = j > 0 ? -sy : 0, yp = j < ny - 1 ? sy : 0;
@@ -495,15 +487,14 @@ int build_bins3(const G3 &g, int64_t T, const R *r, const R *v, const Bins3 &b, 
     MPI_TRY_CUDA(cudaMemsetAsync(b.count, 0, sizeof(int) * nc, st));
     MPI_TRY_CUDA(cudaMemsetAsync(b.cell_cnt, 0, sizeof(unsigned) * nc, st));
     if (T > 0) {
-        k_cell_count3<R><<<grid_blocks(T), 256, 0, st>>>(T, r, ax, b.ncx, b.ncy, b.cell_of, b.count,
+        launch_chained(k_cell_count3<R>, grid_blocks(T), 256, 0, st, T, r, ax, b.ncx, b.ncy, b.cell_of, b.count,
                                                           static_cast<InterpRec3<R> *>(b.rec_t));
         MPI_CHECK_LAUNCH();
     }
     MPI_TRY(cell_scan_launch(b.count, nc, b.offset, b.sort_tmp, st));
     if (T > 0) {
         MPI_TRY(cell_order_launch(T, b.cell_of, nc, b.list, b.sort_tmp, st));
-        k_sort_records<InterpRec3<R>, R, 3><<<grid_blocks(T), 256, 0, st>>>(
-            T, b.list, static_cast<const InterpRec3<R> *>(b.rec_t), v, static_cast<InterpRec3<R> *>(b.rec),
+        launch_chained(k_sort_records<InterpRec3<R>, R, 3>, grid_blocks(T), 256, 0, st, T, b.list, static_cast<const InterpRec3<R> *>(b.rec_t), v, static_cast<InterpRec3<R> *>(b.rec),
             static_cast<R *>(b.vs));
         MPI_CHECK_LAUNCH();
     }
@@ -591,7 +582,7 @@ int launch_interp3_T(const G3 &g, int64_t T, const R *s_sorted, const Bins3 &b, 
 // The 3-D operator of the one-launch solve (core_resident.cuh).
 template <int CH>
 struct Resident3 {
-    static constexpr int kNC = CH < 0 ? 9 : 3, kPhases = 2, kRows = CH < 0 ? 3 : 1;
+    static constexpr int kNC = CH < 0 ? 9 : 3, kPhases = 2, kPqThreads = kQThreads3, kRows = CH < 0 ? 3 : 1;
     int nx, ny, nz, ncx, ncy, ncz;
     bool scaled;
     Coef3<df> c;
@@ -607,19 +598,19 @@ struct Resident3 {
     __device__ __forceinline__ void phase(int k) const
     {
         if (k == 0)
-            interp3_outputs<float, float, CH, true, true, true>(T, nullptr, rec, vs, p32, nx, ny, nz, Axes3{}, s);
+            interp3_outputs<float, float, CH, true, true>(T, nullptr, rec, vs, p32, nx, ny, nz, Axes3{}, s);
         else
-            T3_units<float, CH, true>(rec, vs, s, T, offset, cunit_off, unit_cell, cunit_off[ncx * ncy * ncz], unit_part,
+            T3_units<float, CH>(rec, vs, s, T, offset, cunit_off, unit_cell, cunit_off[ncx * ncy * ncz], unit_part,
                                       cell_part, cell_cnt);
     }
     __device__ __forceinline__ void combine(int node, SumAcc<float> (&sum)[kNC]) const
     {
-        node_combine3<float, kNC, true>(node % nx, (node / nx) % ny, node / (nx * ny), ncx, ncy, ncz, cunit_off,
+        node_combine3<float, kNC>(node % nx, (node / nx) % ny, node / (nx * ny), ncx, ncy, ncz, cunit_off,
                                         cell_part, sum);
     }
     __device__ __forceinline__ df lap(const df *f, int node) const
     {
-        return lap3_at<true>(f, node, node % nx, (node / nx) % ny, node / (nx * ny), nx, ny, nz, scaled, c);
+        return lap3_at(f, node, node % nx, (node / nx) % ny, node / (nx * ny), nx, ny, nz, scaled, c);
     }
     __device__ __forceinline__ void store_p32(int node, const float *v) const
     {

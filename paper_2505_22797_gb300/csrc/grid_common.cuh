@@ -18,32 +18,74 @@ struct AxisMap {
     double inv_h;   // 1/h
     double off;     // -p0/h - 1/2: continuous node index = p inv_h + off
     int n;
+    float inv_hi, inv_lo, off_hi, off_lo;  // inv_h and off as sums of two floats,
+    bool pair;                             // where FP32 holds them
 };
 
-// Node interval and cosine weights of a position along one axis: between
-// nodes k and k+1 at fraction f, node k+1 weighs (1 - cos(pi f))/2.  Outside
-// the node hull the position clamps to the edge node.
+// Cosine weights at fraction f between two nodes: the second weighs
+// (1 - cos(pi f))/2.
 template <typename R>
-__device__ __forceinline__ void axis_weights(R pos, const AxisMap &a, int &k0, R &w0, R &w1)
+__device__ __forceinline__ void cosine_weights(R f, R &w0, R &w1)
 {
-    if (a.n == 1) { k0 = 0; w0 = R(1); w1 = R(0); return; }
-    // The node index is formed in FP64: in FP32 its rounding (~1e-5 of a cell
-    // on 100+ node grids) would already be visible in the weights.
-    const double fi = double(pos) * a.inv_h + a.off;
-    if (!(fi > 0.0)) { k0 = 0; w0 = R(1); w1 = R(0); return; }
-    if (fi >= double(a.n - 1)) { k0 = a.n - 2; w0 = R(0); w1 = R(1); return; }
-    int k = (int)floor(fi);
-    k = min(k, a.n - 2);
-    const R f = R(fi - double(k));
-    k0 = k;
     if constexpr (sizeof(R) == 4) w1 = 0.5f * (1.0f - cospif(f));
     else w1 = 0.5 * (1.0 - cospi(f));
     w0 = R(1) - w1;
 }
 
+// Node interval and cosine weights of a position along one axis.  Outside
+// the node hull the position clamps to the edge node.  The node index needs
+// more than FP32: its rounding (~1e-5 of a cell on 100+ node grids) would
+// already be visible in the weights.
+__device__ __forceinline__ void axis_weights(double pos, const AxisMap &a, int &k0, double &w0, double &w1)
+{
+    if (a.n == 1) { k0 = 0; w0 = 1.0; w1 = 0.0; return; }
+    const double fi = pos * a.inv_h + a.off;
+    if (!(fi > 0.0)) { k0 = 0; w0 = 1.0; w1 = 0.0; return; }
+    if (fi >= double(a.n - 1)) { k0 = a.n - 2; w0 = 0.0; w1 = 1.0; return; }
+    const int k = min((int)floor(fi), a.n - 2);
+    k0 = k;
+    cosine_weights(fi - double(k), w0, w1);
+}
+
+// FP32 positions: the same values, bit for bit, without FP64 arithmetic (eight
+// FP64 operations per axis bound the pass over the samples: 38 us for 2^20 of
+// them).  The index is formed as a sum of two floats s + lo (the product and
+// the sum error-free, Dekker and Knuth) to within delta of both the exact and
+// the FP64 one; where delta could change the interval or the rounded fraction
+// (a thousandth of the samples), the FP64 form decides.
+__device__ __forceinline__ void axis_weights(float pos, const AxisMap &a, int &k0, float &w0, float &w1)
+{
+    if (a.n == 1) { k0 = 0; w0 = 1.0f; w1 = 0.0f; return; }
+    const float p = __fmul_rn(pos, a.inv_hi), pe = __fmaf_rn(pos, a.inv_hi, -p);
+    const float s = __fadd_rn(p, a.off_hi), bb = __fadd_rn(s, -p);
+    const float se = __fadd_rn(__fadd_rn(p, -__fadd_rn(s, -bb)), __fadd_rn(a.off_hi, -bb));
+    const float lo = __fadd_rn(__fadd_rn(pe, se), __fmaf_rn(pos, a.inv_lo, a.off_lo));
+    const float delta = (fabsf(p) + fabsf(a.off_hi) + 1.0f) * 5.7e-14f;  // 2^-44
+    const float k = floorf(s), t = __fadd_rn(s, -k);
+    const float f = __fadd_rn(t, __fadd_rn(lo, -delta)), g = __fadd_rn(t, __fadd_rn(lo, delta));
+    if (a.pair && fabsf(s) < 1e6f && f == g && f >= 0.0f && f < 1.0f) {
+        if (k < 0.0f) { k0 = 0; w0 = 1.0f; w1 = 0.0f; return; }
+        if (k >= float(a.n - 1)) { k0 = a.n - 2; w0 = 0.0f; w1 = 1.0f; return; }
+        k0 = (int)k;
+        cosine_weights(f, w0, w1);
+        return;
+    }
+    const double fi = double(pos) * a.inv_h + a.off;
+    if (!(fi > 0.0)) { k0 = 0; w0 = 1.0f; w1 = 0.0f; return; }
+    if (fi >= double(a.n - 1)) { k0 = a.n - 2; w0 = 0.0f; w1 = 1.0f; return; }
+    const int k64 = min((int)floor(fi), a.n - 2);
+    k0 = k64;
+    cosine_weights(float(fi - double(k64)), w0, w1);
+}
+
 inline AxisMap make_axis(double p0, double h, int n)
 {
-    return AxisMap{1.0 / h, -p0 / h - 0.5, n};
+    AxisMap a{1.0 / h, -p0 / h - 0.5, n};
+    a.inv_hi = float(a.inv_h), a.inv_lo = float(a.inv_h - double(a.inv_hi));
+    a.off_hi = float(a.off), a.off_lo = float(a.off - double(a.off_hi));
+    const double m = std::fabs(a.inv_h);
+    a.pair = m > 1e-25 && m < 1e25 && std::fabs(a.off) < 1e25;  // (no part under- or overflows)
+    return a;
 }
 
 constexpr int kInterpSPT = 4;     // samples per thread of the interpolation (gathers in flight)
@@ -334,9 +376,10 @@ int core_stage_cg(CoreStageOp<E> &op, int64_t nv, const E *b, const mpi_grid_opt
 // rec[q] = rec_t[list[q]] and vs[q] = v[list[q]] (D velocity components):
 // the records and velocities of the samples in list (cell) order.
 template <typename Rec, typename R, int D>
-__global__ void k_sort_records(int64_t T, const int *__restrict__ list, const Rec *__restrict__ rec_t,
-                               const R *__restrict__ v, Rec *__restrict__ rec, R *__restrict__ vs)
+__global__ void k_sort_records(int64_t T, const int *list, const Rec *rec_t,
+                               const R *v, Rec *__restrict__ rec, R *__restrict__ vs)
 {
+    chain_wait();
     for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < T;
          q += (int64_t)gridDim.x * blockDim.x) {
         const int64_t t = list[q];
@@ -348,9 +391,10 @@ __global__ void k_sort_records(int64_t T, const int *__restrict__ list, const Re
 
 // out[k][q] = in[k][list[q]] for the n_rows rows of a [n_rows][T] array.
 template <typename R>
-__global__ void k_gather_rows(int64_t T, int n_rows, const int *__restrict__ list, const R *__restrict__ in,
+__global__ void k_gather_rows(int64_t T, int n_rows, const int *list, const R *in,
                               R *__restrict__ out)
 {
+    chain_wait();
     for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < T;
          q += (int64_t)gridDim.x * blockDim.x) {
         const int64_t t = list[q];
@@ -362,7 +406,7 @@ template <typename R>
 int gather_rows(int64_t T, int n_rows, const int *list, const R *in, R *out, cudaStream_t st)
 {
     if (T == 0) return MPI_OK;
-    k_gather_rows<R><<<grid_blocks(T), 256, 0, st>>>(T, n_rows, list, in, out);
+    launch_chained(k_gather_rows<R>, grid_blocks(T), 256, 0, st, T, n_rows, list, in, out);
     MPI_CHECK_LAUNCH();
     return MPI_OK;
 }

@@ -33,8 +33,8 @@ __device__ __forceinline__ InterpRec<R> make_rec(R px, R py, const AxisMap &ax, 
 {
     InterpRec<R> q;
     R w0;
-    axis_weights<R>(px, ax, q.i0, w0, q.wx1);
-    axis_weights<R>(py, ay, q.j0, w0, q.wy1);
+    axis_weights(px, ax, q.i0, w0, q.wx1);
+    axis_weights(py, ay, q.j0, w0, q.wy1);
     return q;
 }
 
@@ -51,11 +51,11 @@ template <typename R, int NCOMP> struct NodeVec;
 template <> struct NodeVec<float, 4> { using T = float4; };
 template <> struct NodeVec<float, 2> { using T = float2; };
 
-template <typename R, int NCOMP, bool COH = false>
+template <typename R, int NCOMP>
 __device__ __forceinline__ void load_node(const R *A, int64_t node, R (&out)[NCOMP])
 {
     using V = typename NodeVec<R, NCOMP>::T;
-    const V q = ld_shared_by_blocks<COH>(reinterpret_cast<const V *>(A) + node);
+    const V q = reinterpret_cast<const V *>(A)[node];
     if constexpr (NCOMP == 4) { out[0] = q.x; out[1] = q.y; out[2] = q.z; out[3] = q.w; }
     else { out[0] = q.x; out[1] = q.y; }
 }
@@ -124,10 +124,11 @@ k_interp(int64_t T, const R *__restrict__ r, const InterpRec<R> *__restrict__ re
 // --- binning of samples by interpolation cell -------------------------------
 
 template <typename R>
-__global__ void k_cell_count(int64_t T, const R *__restrict__ r, AxisMap ax, AxisMap ay, int ncx,
+__global__ void k_cell_count(int64_t T, const R *r, AxisMap ax, AxisMap ay, int ncx,
                              int *__restrict__ cell_of, int *__restrict__ count,
                              InterpRec<R> *__restrict__ rec)
 {
+    chain_wait();
     // every lane of a warp runs the same iterations (warp_count_add)
     for (int64_t t0 = int64_t(blockIdx.x) * blockDim.x; t0 < T; t0 += int64_t(gridDim.x) * blockDim.x) {
         const int64_t t = t0 + threadIdx.x;
@@ -152,14 +153,16 @@ __global__ void k_cell_count(int64_t T, const R *__restrict__ r, AxisMap ax, Axi
 // read once instead of once per corner node, and a cell where the trajectory
 // dwells (thousands of samples) spreads over many units.
 
-__global__ void k_cunit_count(int n_cells, const int *__restrict__ offset, int *__restrict__ cunit_cnt)
+__global__ void k_cunit_count(int n_cells, const int *offset, int *__restrict__ cunit_cnt)
 {
+    chain_wait();
     for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < n_cells; c += gridDim.x * blockDim.x)
         cunit_cnt[c] = (offset[c + 1] - offset[c] + kUnitLen - 1) / kUnitLen;
 }
 
-__global__ void k_cunit_fill(int n_cells, const int *__restrict__ cunit_off, int *__restrict__ unit_cell)
+__global__ void k_cunit_fill(int n_cells, const int *cunit_off, int *__restrict__ unit_cell)
 {
+    chain_wait();
     for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < n_cells; c += gridDim.x * blockDim.x)
         for (int w = cunit_off[c]; w < cunit_off[c + 1]; ++w) unit_cell[w] = c;
 }
@@ -172,11 +175,12 @@ __global__ void k_cunit_fill(int n_cells, const int *__restrict__ cunit_off, int
 // see full warps.
 template <typename R, int CH>
 __global__ void __launch_bounds__(kUnitThreads)
-k_interp_T_cells(const InterpRec<R> *__restrict__ rec, const R *__restrict__ vs, const R *__restrict__ s,
-                 int64_t T, const int *__restrict__ offset, const int *__restrict__ cunit_off,
-                 const int *__restrict__ unit_cell, const int *__restrict__ n_units_dev,
+k_interp_T_cells(const InterpRec<R> *rec, const R *vs, const R *s,
+                 int64_t T, const int *offset, const int *cunit_off,
+                 const int *unit_cell, const int *n_units_dev,
                  R *__restrict__ unit_part)
 {
+    chain_wait();
     constexpr int NC = CH < 0 ? 4 : 2;
     constexpr int G = kUnitLanes;
     constexpr int per_block = kUnitThreads / G;
@@ -239,8 +243,8 @@ k_interp_T_cells(const InterpRec<R> *__restrict__ rec, const R *__restrict__ vs,
 // once (record and velocity) instead of gathered, stored and read again.
 // IL: the field node-interleaved in R (NC components per node), else
 // component-major in AT; CH = k: only channel k (two components).
-// COH: the field is written during the launch.
-template <typename R, typename AT, int CH, bool IL, bool COH>
+// (The field may be written during the launch: it is not __restrict__.)
+template <typename R, typename AT, int CH, bool IL>
 __device__ __forceinline__ void
 normal_units(const InterpRec<R> *__restrict__ rec, const R *__restrict__ vs, const AT *A, int nx, int ny, int ncx,
              const int *__restrict__ offset, const int *__restrict__ cunit_off, const int *__restrict__ unit_cell,
@@ -271,7 +275,7 @@ normal_units(const InterpRec<R> *__restrict__ rec, const R *__restrict__ vs, con
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 if constexpr (IL) {
-                    load_node<R, NC, COH>(reinterpret_cast<const R *>(A), nodes[k], f[k]);
+                    load_node<R, NC>(reinterpret_cast<const R *>(A), nodes[k], f[k]);
                 } else {
 #pragma unroll
                     for (int e = 0; e < NC; ++e) f[k][e] = R(A[(int64_t)e * N + nodes[k]]);
@@ -324,7 +328,7 @@ normal_units(const InterpRec<R> *__restrict__ rec, const R *__restrict__ vs, con
 // on one another, the loads do not, and a node beside a dense cell adds tens
 // of units (one L2 round trip each when every load waits for the previous
 // addition).
-template <typename R, int NC, bool COH = false>
+template <typename R, int NC>
 __device__ __forceinline__ void add_unit_sums(const R *unit_part, int w0, int w1, int corner,
                                               SumAcc<R> (&sum)[NC])
 {
@@ -334,7 +338,7 @@ __device__ __forceinline__ void add_unit_sums(const R *unit_part, int w0, int w1
 #pragma unroll
         for (int u = 0; u < 4; ++u)
 #pragma unroll
-            for (int m = 0; m < NC; ++m) v[u][m] = ld_shared_by_blocks<COH>(unit_part + ((int64_t)(w + u) * 4 + corner) * NC + m);
+            for (int m = 0; m < NC; ++m) v[u][m] = unit_part[((int64_t)(w + u) * 4 + corner) * NC + m];
 #pragma unroll
         for (int u = 0; u < 4; ++u)
 #pragma unroll
@@ -342,16 +346,17 @@ __device__ __forceinline__ void add_unit_sums(const R *unit_part, int w0, int w1
     }
     for (; w < w1; ++w)
 #pragma unroll
-        for (int m = 0; m < NC; ++m) sum[m].add(ld_shared_by_blocks<COH>(unit_part + ((int64_t)w * 4 + corner) * NC + m));
+        for (int m = 0; m < NC; ++m) sum[m].add(unit_part[((int64_t)w * 4 + corner) * NC + m]);
 }
 
 // Ahat_m(node) = scale * the sum, over the node's adjacent cells (row-major
 // cell order) and their units in order, of the unit sums of the corner the
 // node is in that cell (FP32 unit sums as error-free double-float pairs).
 template <typename R, typename OUT, int NC>
-__global__ void k_interp_T_cell_combine(int nx, int ny, int ncx, int ncy, const int *__restrict__ cunit_off,
-                                        const R *__restrict__ unit_part, OUT *__restrict__ A, double scale)
+__global__ void k_interp_T_cell_combine(int nx, int ny, int ncx, int ncy, const int *cunit_off,
+                                        const R *unit_part, OUT *__restrict__ A, double scale)
 {
+    chain_wait();
     const int N = nx * ny;
     for (int node = blockIdx.x * blockDim.x + threadIdx.x; node < N; node += gridDim.x * blockDim.x) {
         const int i = node % nx, j = node / nx;
@@ -444,23 +449,23 @@ static int build_bins(const GridH &g, int64_t T, const R *r, const R *v, const B
     const int nc = b.ncx * b.ncy;
     MPI_TRY_CUDA(cudaMemsetAsync(b.count, 0, sizeof(int) * nc, st));
     if (T > 0) {
-        k_cell_count<R><<<grid_blocks(T), 256, 0, st>>>(T, r, ax, ay, b.ncx, b.cell_of, b.count,
+        launch_chained(k_cell_count<R>, grid_blocks(T), 256, 0, st, T, r, ax, ay, b.ncx, b.cell_of, b.count,
                                                          static_cast<InterpRec<R> *>(b.rec_t));
         MPI_CHECK_LAUNCH();
     }
     MPI_TRY(cell_scan_launch(b.count, nc, b.offset, b.sort_tmp, st));
     if (T > 0) {
         MPI_TRY(cell_order_launch(T, b.cell_of, nc, b.list, b.sort_tmp, st));
-        k_sort_records<InterpRec<R>, R, 2><<<grid_blocks(T), 256, 0, st>>>(T, b.list, static_cast<const InterpRec<R> *>(b.rec_t),
+        launch_chained(k_sort_records<InterpRec<R>, R, 2>, grid_blocks(T), 256, 0, st, T, b.list, static_cast<const InterpRec<R> *>(b.rec_t),
                                                           v, static_cast<InterpRec<R> *>(b.rec),
                                                           static_cast<R *>(b.vs));
         MPI_CHECK_LAUNCH();
     }
     // Work units of the transpose.
-    k_cunit_count<<<grid_blocks(nc), 256, 0, st>>>(nc, b.offset, b.cunit_cnt);
+    launch_chained(k_cunit_count, grid_blocks(nc), 256, 0, st, nc, b.offset, b.cunit_cnt);
     MPI_CHECK_LAUNCH();
     MPI_TRY(cell_scan_launch(b.cunit_cnt, nc, b.cunit_off, b.sort_tmp, st));
-    k_cunit_fill<<<grid_blocks(nc), 256, 0, st>>>(nc, b.cunit_off, b.unit_cell);
+    launch_chained(k_cunit_fill, grid_blocks(nc), 256, 0, st, nc, b.cunit_off, b.unit_cell);
     MPI_CHECK_LAUNCH();
     return MPI_OK;
 }
@@ -516,10 +521,10 @@ static int launch_interp_T_units(int64_t T, const R *s_sorted, const Bins &b, cu
     R *part = static_cast<R *>(b.unit_part);
     const int *n_units = b.cunit_off + nc;
     if (ch < 0)
-        k_interp_T_cells<R, -1><<<blocks, kUnitThreads, 0, st>>>(rec, vs, s_sorted, T, b.offset, b.cunit_off,
+        launch_chained(k_interp_T_cells<R, -1>, blocks, kUnitThreads, 0, st, rec, vs, s_sorted, T, b.offset, b.cunit_off,
                                                                  b.unit_cell, n_units, part);
     else
-        k_interp_T_cells<R, 0><<<blocks, kUnitThreads, 0, st>>>(rec, vs, s_sorted, T, b.offset, b.cunit_off,
+        launch_chained(k_interp_T_cells<R, 0>, blocks, kUnitThreads, 0, st, rec, vs, s_sorted, T, b.offset, b.cunit_off,
                                                                 b.unit_cell, n_units, part);
     MPI_CHECK_LAUNCH();
     return MPI_OK;
@@ -534,10 +539,10 @@ static int launch_interp_T(const GridH &g, int64_t T, const R *s_sorted, const B
     const int N = g.nx * g.ny;
     const R *part = static_cast<const R *>(b.unit_part);
     if (ch < 0)
-        k_interp_T_cell_combine<R, OUT, 4><<<grid_blocks(N), 256, 0, st>>>(g.nx, g.ny, b.ncx, b.ncy, b.cunit_off,
+        launch_chained(k_interp_T_cell_combine<R, OUT, 4>, grid_blocks(N), 256, 0, st, g.nx, g.ny, b.ncx, b.ncy, b.cunit_off,
                                                                           part, A, scale);
     else
-        k_interp_T_cell_combine<R, OUT, 2><<<grid_blocks(N), 256, 0, st>>>(g.nx, g.ny, b.ncx, b.ncy, b.cunit_off,
+        launch_chained(k_interp_T_cell_combine<R, OUT, 2>, grid_blocks(N), 256, 0, st, g.nx, g.ny, b.ncx, b.ncy, b.cunit_off,
                                                                           part, A, scale);
     MPI_CHECK_LAUNCH();
     return MPI_OK;
@@ -560,10 +565,9 @@ __device__ __forceinline__ double lap2_at(const double *__restrict__ f, int k, i
     return f[j * nx + im] + f[j * nx + ip] + f[jm * nx + i] + f[jp * nx + i] - 4.0 * f[k];
 }
 // The same in double-float arithmetic (cx, cy as double-float pairs).
-template <bool COH = false>
 __device__ __forceinline__ df lap2_at(const df *f, int k, int i, int j, int nx, int ny, bool scaled, df cx, df cy)
 {
-    auto at = [&](int e) { return ld_shared_by_blocks<COH>(f + e); };
+    auto at = [&](int e) { return f[e]; };
     const int im = i > 0 ? i - 1 : 0, ip = i < nx - 1 ? i + 1 : nx - 1;
     const int jm = j > 0 ? j - 1 : 0, jp = j < ny - 1 ? j + 1 : ny - 1;
     const df c0 = at(k);
@@ -587,7 +591,7 @@ k_step_units(const InterpRec<R> *rec, const R *vs, const AT *A, int nx, int ny,
 {
     chain_wait();
     if (int(blockIdx.x) < n_unit_blocks) {
-        normal_units<R, AT, CH, IL, false>(rec, vs, A, nx, ny, ncx, offset, cunit_off, unit_cell, *n_units_dev,
+        normal_units<R, AT, CH, IL>(rec, vs, A, nx, ny, ncx, offset, cunit_off, unit_cell, *n_units_dev,
                                            unit_part, n_unit_blocks);
         return;
     }
@@ -655,9 +659,10 @@ inline int cs_blocks(int64_t n) { return (int)std::max<int64_t>(1, (n + kCsPer -
 // E: the element type of the vectors (double, or double-float pairs).
 template <typename E>
 __global__ void __launch_bounds__(kCsThreads)
-k_cs_init(int64_t n, const E *__restrict__ b, E *__restrict__ r, E *__restrict__ p, double *__restrict__ rr_part,
+k_cs_init(int64_t n, const E *b, E *__restrict__ r, E *__restrict__ p, double *__restrict__ rr_part,
           double rel_tol, CsScal *sc)
 {
+    chain_wait();
     __shared__ double sh[kCsThreads / 32];
     __shared__ bool last;
     const int64_t e0 = (int64_t)blockIdx.x * kCsPer;
@@ -758,8 +763,9 @@ k_cs_step2(int64_t n, const E *r, E *__restrict__ p, const CsScal *sc)
 
 // buf = p rounded to FP32 (one thread per node, all its components).
 template <typename E, int L>
-__global__ void __launch_bounds__(kCsThreads) k_cs_round(int64_t N, const E *__restrict__ p, float *buf)
+__global__ void __launch_bounds__(kCsThreads) k_cs_round(int64_t N, const E *p, float *buf)
 {
+    chain_wait();
     constexpr int NC = p32_nc<L>();
     for (int64_t node = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; node < N;
          node += (int64_t)gridDim.x * blockDim.x) {
@@ -803,10 +809,10 @@ static int cs_round_launch(const P32 &d, const E *p, cudaStream_t st)
 {
     const int blocks = grid_blocks(d.N);
     switch (d.layout) {
-        case kP32Node4: k_cs_round<E, kP32Node4><<<blocks, kCsThreads, 0, st>>>(d.N, p, d.buf); break;
-        case kP32Node2: k_cs_round<E, kP32Node2><<<blocks, kCsThreads, 0, st>>>(d.N, p, d.buf); break;
-        case kP32Rows3x4: k_cs_round<E, kP32Rows3x4><<<blocks, kCsThreads, 0, st>>>(d.N, p, d.buf); break;
-        default: k_cs_round<E, kP32Rows1x4><<<blocks, kCsThreads, 0, st>>>(d.N, p, d.buf); break;
+        case kP32Node4: launch_chained(k_cs_round<E, kP32Node4>, blocks, kCsThreads, 0, st, d.N, p, d.buf); break;
+        case kP32Node2: launch_chained(k_cs_round<E, kP32Node2>, blocks, kCsThreads, 0, st, d.N, p, d.buf); break;
+        case kP32Rows3x4: launch_chained(k_cs_round<E, kP32Rows3x4>, blocks, kCsThreads, 0, st, d.N, p, d.buf); break;
+        default: launch_chained(k_cs_round<E, kP32Rows1x4>, blocks, kCsThreads, 0, st, d.N, p, d.buf); break;
     }
     MPI_CHECK_LAUNCH();
     return MPI_OK;
@@ -855,7 +861,7 @@ __global__ void k_grid_output(int64_t N, int ch, const E *__restrict__ x, R *__r
 // The 2-D operator of the one-launch solve (core_resident.cuh).
 template <int CH>
 struct Resident2 {
-    static constexpr int kNC = CH < 0 ? 4 : 2, kPhases = 1;
+    static constexpr int kNC = CH < 0 ? 4 : 2, kPhases = 1, kPqThreads = kQThreads;
     int nx, ny, ncx, ncy;
     bool scaled;
     df cx, cy, scale, gamma;
@@ -866,7 +872,7 @@ struct Resident2 {
 
     __device__ __forceinline__ void phase(int) const
     {
-        normal_units<float, float, CH, true, true>(rec, vs, p32, nx, ny, ncx, offset, cunit_off, unit_cell,
+        normal_units<float, float, CH, true>(rec, vs, p32, nx, ny, ncx, offset, cunit_off, unit_cell,
                                                    cunit_off[ncx * ncy], unit_part, gridDim.x);
     }
     __device__ __forceinline__ void combine(int node, SumAcc<float> (&sum)[kNC]) const
@@ -877,13 +883,13 @@ struct Resident2 {
             for (int ci = i - 1; ci <= i; ++ci) {
                 if (ci < 0 || ci >= ncx) continue;
                 const int c = cj * ncx + ci;
-                add_unit_sums<float, kNC, true>(unit_part, cunit_off[c], cunit_off[c + 1], (i - ci) + 2 * (j - cj), sum);
+                add_unit_sums<float, kNC>(unit_part, cunit_off[c], cunit_off[c + 1], (i - ci) + 2 * (j - cj), sum);
             }
         }
     }
     __device__ __forceinline__ df lap(const df *f, int node) const
     {
-        return lap2_at<true>(f, node, node % nx, node / nx, nx, ny, scaled, cx, cy);
+        return lap2_at(f, node, node % nx, node / nx, nx, ny, scaled, cx, cy);
     }
     __device__ __forceinline__ void store_p32(int node, const float *v) const
     {
@@ -1099,7 +1105,7 @@ int core_stage_cg(CoreStageOp<E> &op, int64_t nv, const E *b, const mpi_grid_opt
     MPI_TRY_CUDA(cudaMemsetAsync(x, 0, vb, st));
     MPI_TRY_CUDA(cudaMemsetAsync(sc, 0, sizeof(CsScal), st));
     // r = b, p = b, r.r, ||b|| and the threshold
-    k_cs_init<E><<<ncs, kCsThreads, 0, st>>>(nv, b, rr, p, rr_part, o.rel_tol, sc);
+    launch_chained(k_cs_init<E>, ncs, kCsThreads, 0, st, nv, b, rr, p, rr_part, o.rel_tol, sc);
     MPI_CHECK_LAUNCH();
     if (p32.buf) MPI_TRY(cs_round_launch(p32, p, st));
 
