@@ -78,10 +78,16 @@ __device__ __forceinline__ double block_min(double v, double *sh /* >= NT/32 + 1
 // over the digit counts).  The cluster takes 53 us less there.
 constexpr int kStatBlocks = 8;
 
+// The sums run in the order of one block of kStatThreads threads (thread t
+// over the values t, t + kStatThreads, ...; its warps in order): each block
+// takes kStatSumWarps of that block's warps.
+constexpr int kStatSumWarps = kStatThreads / 32 / kStatBlocks;
+
 struct StatShared {
     unsigned hist[256];
-    double part[2];            // this block's partial sums / minimum, read by the others
-    unsigned long long cnt;    // this block's count, read by the others
+    double part[kStatSumWarps];  // this block's partial sums, minimum and count,
+    double least;                // read by the others
+    unsigned long long cnt;
     double sh[kStatThreads / 32 + 1];
     unsigned long long sel[2]; // prefix, remaining rank
 };
@@ -142,24 +148,28 @@ __device__ inline double cluster_select(const double *__restrict__ x, int64_t N,
     return key_f64(prefix);
 }
 
-// Sum of v over the cluster in a fixed order, for every thread; slot: which of
-// the two partials it uses (alternate, so no barrier is needed to reuse one).
-__device__ inline double cluster_sum(double v, int slot, StatShared &S)
+// Sum of f(i) over the N values in the order of one block, for every thread.
+template <typename F>
+__device__ inline double cluster_sum(int64_t N, F f, StatShared &S)
 {
     namespace cg = cooperative_groups;
     cg::cluster_group cl = cg::this_cluster();
-    const double t = block_sum<double, kStatThreads>(v, S.sh);
-    if (threadIdx.x == 0) S.part[slot] = t;
-    cl.sync();
-    if (threadIdx.x == 0) {
-        double a = 0.0;
-        for (int b = 0; b < kStatBlocks; ++b) a += *cl.map_shared_rank(&S.part[slot], b);
-        S.sh[kStatThreads / 32] = a;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (warp < kStatSumWarps) {
+        double s = 0.0;
+        for (int64_t i = ((int)cl.block_rank() * kStatSumWarps + warp) * 32 + lane; i < N; i += kStatThreads) s += f(i);
+        s = warp_sum(s);
+        if (lane == 0) S.part[warp] = s;
     }
-    __syncthreads();
-    const double r = S.sh[kStatThreads / 32];
-    __syncthreads();
-    return r;
+    cl.sync();
+    if (warp == 0) {
+        double t = *cl.map_shared_rank(&S.part[lane % kStatSumWarps], lane / kStatSumWarps);
+        double a = 0.0;
+        for (int w = 0; w < kStatThreads / 32; ++w) a += __shfl_sync(0xffffffffu, t, w);
+        if (lane == 0) S.sh[kStatThreads / 32] = a;
+    }
+    cl.sync();  // (the partials are read)
+    return S.sh[kStatThreads / 32];
 }
 
 // One cluster computes, for the N values x: the clip value P (the pct-th
@@ -202,31 +212,24 @@ __device__ void outer_stats_cluster(int64_t N, const double *__restrict__ x, int
             gt = block_min<kStatThreads>(gt, S.sh);
             if (threadIdx.x == 0) {
                 S.cnt = (unsigned long long)le;
-                S.part[1] = gt;
+                S.least = gt;
             }
             cl.sync();
             le = 0;
             for (int b = 0; b < kStatBlocks; ++b) {
                 le += (long long)*cl.map_shared_rank(&S.cnt, b);
-                gt = fmin(gt, *cl.map_shared_rank(&S.part[1], b));
+                gt = fmin(gt, *cl.map_shared_rank(&S.least, b));
             }
             xhi = le > hi ? xlo : gt;
         }
         P = xlo + (h - double(lo)) * (xhi - xlo);
     }
-    double s = 0.0;
-    for (int64_t i = i0; i < N; i += stride) {
-        const double v = fmax(x[i], P);
-        rho1[i] = R(v);
-        s += v;
-    }
-    const double mean = cluster_sum(s, 0, S) / double(N);
-    double q = 0.0;
-    for (int64_t i = i0; i < N; i += stride) {
+    for (int64_t i = i0; i < N; i += stride) rho1[i] = R(fmax(x[i], P));
+    const double mean = cluster_sum(N, [&](int64_t i) { return fmax(x[i], P); }, S) / double(N);
+    const double q = cluster_sum(N, [&](int64_t i) {
         const double dv = fmax(x[i], P) - mean;
-        q += dv * dv;
-    }
-    q = cluster_sum(q, 1, S);
+        return dv * dv;
+    }, S);
     if (cl.block_rank() == 0 && threadIdx.x < 32) {
         double rr = 0.0;
         for (int b = threadIdx.x; b < nblk; b += 32) rr += rr_part[b];
