@@ -24,6 +24,7 @@
 // route (full complex grid, two transposes) up to round-off: the parts the
 // three launches skip are zeros or conjugates.
 #include "conv_ops.cuh"
+#include "pnp_device.cuh"
 
 namespace mpi {
 
@@ -93,6 +94,30 @@ __device__ C *smem_dft(C *A, C *B, int lg_n, int lg_c, const C *__restrict__ W)
     return src;
 }
 
+// The two rows' half spectra of each pair from the pair's DFT Z.
+template <typename C>
+__device__ __forceinline__ void rows_split(const C *Z, int ny, int lg_nx, int lg_rp, int LD, int pair0,
+                                           C *__restrict__ X1)
+{
+    using R = decltype(C{}.x);
+    const int NX = 1 << lg_nx, rp = 1 << lg_rp;
+    const int half = NX >> 1;
+    for (int q = threadIdx.x; q < LD * rp; q += blockDim.x) {
+        const int s = q / LD, k = q - s * LD;
+        const int ja = 2 * (pair0 + s), jb = ja + 1;
+        if (ja >= ny) continue;
+        C a = cxv(R(0), R(0)), b = cxv(R(0), R(0));
+        if (k <= half) {
+            const C zk = Z[(k << lg_rp) + s];
+            const C zm = Z[(((NX - k) & (NX - 1)) << lg_rp) + s];  // Z[-k]
+            a = cxv(R(0.5) * (zk.x + zm.x), R(0.5) * (zk.y - zm.y));
+            b = cxv(R(0.5) * (zk.y + zm.y), R(0.5) * (zm.x - zk.x));
+        }
+        X1[(int64_t)ja * LD + k] = a;
+        if (jb < ny) X1[(int64_t)jb * LD + k] = b;
+    }
+}
+
 // Launch 1: the half spectra X1[j][k], k < LD (k > NX/2: zero), of the input
 // rows j < ny.  A block takes 2^lg_rp row pairs.
 template <typename C, typename IN>
@@ -118,21 +143,7 @@ k_cf_rows_fwd(int nx, int ny, int lg_nx, int lg_rp, int LD, const IN *__restrict
     }
     __syncthreads();
     const C *Z = smem_dft(A, B, lg_nx, lg_rp, W);
-    const int half = NX >> 1;
-    for (int q = threadIdx.x; q < LD * rp; q += blockDim.x) {
-        const int s = q / LD, k = q - s * LD;
-        const int ja = 2 * (pair0 + s), jb = ja + 1;
-        if (ja >= ny) continue;
-        C a = cxv(R(0), R(0)), b = cxv(R(0), R(0));
-        if (k <= half) {
-            const C zk = Z[(k << lg_rp) + s];
-            const C zm = Z[(((NX - k) & (NX - 1)) << lg_rp) + s];  // Z[-k]
-            a = cxv(R(0.5) * (zk.x + zm.x), R(0.5) * (zk.y - zm.y));
-            b = cxv(R(0.5) * (zk.y + zm.y), R(0.5) * (zm.x - zk.x));
-        }
-        X1[(int64_t)ja * LD + k] = a;
-        if (jb < ny) X1[(int64_t)jb * LD + k] = b;
-    }
+    rows_split(Z, ny, lg_nx, lg_rp, LD, pair0, X1);
 }
 
 // Column pass (launch 2 in 2-D; the y and z passes in 3-D): a block takes
@@ -223,6 +234,25 @@ __device__ __forceinline__ C herm_at(const C *__restrict__ row, int k, int half)
     return cxv(v.x, -v.y);
 }
 
+// conj(a + i b) of each row pair, both rows real: the inverse DFT of the
+// product's inverse column transforms, unscaled.
+template <typename C>
+__device__ __forceinline__ C *rows_inverse(C *A, C *B, int ny, int lg_nx, int lg_rp, int LD, int pair0,
+                                           const C *__restrict__ Y2, const C *__restrict__ W)
+{
+    using R = decltype(C{}.x);
+    const int NX = 1 << lg_nx, half = NX >> 1;
+    for (int q = threadIdx.x; q < (NX << lg_rp); q += blockDim.x) {
+        const int s = q >> lg_nx, k = q & (NX - 1);
+        const int ja = 2 * (pair0 + s), jb = ja + 1;
+        const C a = ja < ny ? herm_at(Y2 + (int64_t)ja * LD, k, half) : cxv(R(0), R(0));
+        const C b = jb < ny ? herm_at(Y2 + (int64_t)jb * LD, k, half) : cxv(R(0), R(0));
+        A[(k << lg_rp) + s] = cxv(a.x - b.y, -(a.y + b.x));  // conj(a + i b)
+    }
+    __syncthreads();
+    return smem_dft(A, B, lg_nx, lg_rp, W);
+}
+
 // Launch 3: pairs of rows j < ny of the product's inverse column transforms,
 // Z = A + i B over the full length NX, IDFT(Z) = conj(DFT(conj Z)) = a + i b;
 // out[j][i] = scale a[i] (row 2p) and scale b[i] (row 2p + 1), i < nx.
@@ -233,19 +263,11 @@ k_cf_rows_inv(int nx, int ny, int lg_nx, int lg_rp, int LD, const C *__restrict_
 {
     using R = decltype(C{}.x);
     extern __shared__ __align__(16) unsigned char cf_smem[];
-    const int NX = 1 << lg_nx, rp = 1 << lg_rp, half = NX >> 1;
+    const int NX = 1 << lg_nx, rp = 1 << lg_rp;
     C *A = reinterpret_cast<C *>(cf_smem);
     C *B = A + (NX << lg_rp);
     const int pair0 = blockIdx.x * rp;
-    for (int q = threadIdx.x; q < (NX << lg_rp); q += blockDim.x) {
-        const int s = q >> lg_nx, k = q & (NX - 1);
-        const int ja = 2 * (pair0 + s), jb = ja + 1;
-        const C a = ja < ny ? herm_at(Y2 + (int64_t)ja * LD, k, half) : cxv(R(0), R(0));
-        const C b = jb < ny ? herm_at(Y2 + (int64_t)jb * LD, k, half) : cxv(R(0), R(0));
-        A[(k << lg_rp) + s] = cxv(a.x - b.y, -(a.y + b.x));  // conj(a + i b)
-    }
-    __syncthreads();
-    const C *V = smem_dft(A, B, lg_nx, lg_rp, W);
+    const C *V = rows_inverse(A, B, ny, lg_nx, lg_rp, LD, pair0, Y2, W);
     const R sc = R(scale);
     for (int q = threadIdx.x; q < nx * rp; q += blockDim.x) {
         const int s = q / nx, i = q - s * nx;
@@ -255,6 +277,91 @@ k_cf_rows_inv(int nx, int ny, int lg_nx, int lg_rp, int LD, const C *__restrict_
         out[(int64_t)ja * nx + i] = OUT(v.x * sc);
         if (jb < ny) out[(int64_t)jb * nx + i] = OUT(-v.y * sc);
     }
+}
+
+// Launch 1 on the CG direction p as it is updated: p = r + beta p with beta =
+// r.r(new) / r.r(old) (the arithmetic of k_cg_step2, whose launch this saves;
+// the partial sums are added as sum_parts<kVecThreads> adds them), each value
+// by the one thread that loads it.  A row launch has at least kVecThreads
+// threads.
+template <typename C>
+__global__ void __launch_bounds__(kCfMaxThreads)
+k_cf_rows_direction(int nx, int ny, int lg_nx, int lg_rp, int LD, const CgDirection dir,
+                    const C *__restrict__ W, C *__restrict__ X1)
+{
+    using R = decltype(C{}.x);
+    extern __shared__ __align__(16) unsigned char cf_smem[];
+    __shared__ double sh[2][kVecThreads / 32], s_beta;
+    __shared__ bool s_update;
+    const int NX = 1 << lg_nx, rp = 1 << lg_rp;
+    C *A = reinterpret_cast<C *>(cf_smem);
+    C *B = A + (NX << lg_rp);
+    const int pair0 = blockIdx.x * rp;
+    const int warp = threadIdx.x >> 5;
+    if (threadIdx.x < kVecThreads) {
+        double ro = 0.0, rn = 0.0;
+        if (32 * warp < dir.n_part) {
+            for (int k = threadIdx.x; k < dir.n_part; k += kVecThreads) ro += dir.rr_old[k], rn += dir.rr_new[k];
+            ro = warp_sum(ro);
+            rn = warp_sum(rn);
+        }
+        if ((threadIdx.x & 31) == 0) sh[0][warp] = ro, sh[1][warp] = rn;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {  // (FP64: one thread, not every warp)
+        double ro = 0.0, rn = 0.0;
+        for (int w = 0; w < kVecThreads / 32 && 32 * w < dir.n_part; ++w) ro += sh[0][w], rn += sh[1][w];
+        s_beta = rn / ro;
+        s_update = *dir.done == 0;
+    }
+    __syncthreads();
+    const bool update = s_update;
+    const double beta = s_beta;
+    auto next = [&](int64_t e) {
+        double v = dir.p[e];
+        if (update) dir.p[e] = v = dir.r[e] + beta * v;
+        return R(v);
+    };
+    for (int q = threadIdx.x; q < (NX << lg_rp); q += blockDim.x) {
+        const int s = q >> lg_nx, e = q & (NX - 1);
+        const int ja = 2 * (pair0 + s), jb = ja + 1;
+        R xa = R(0), xb = R(0);
+        if (e < nx) {
+            if (ja < ny) xa = next((int64_t)ja * nx + e);
+            if (jb < ny) xb = next((int64_t)jb * nx + e);
+        }
+        A[(e << lg_rp) + s] = cxv(xa, xb);
+    }
+    __syncthreads();
+    const C *Z = smem_dft(A, B, lg_nx, lg_rp, W);
+    rows_split(Z, ny, lg_nx, lg_rp, LD, pair0, X1);
+}
+
+// Between the two convolutions of C C v: launch 3 of the first and launch 1 of
+// the second on the same row pairs, the real rows staying in shared memory
+// (rounded to the call's precision as if stored).
+template <typename C>
+__global__ void __launch_bounds__(kCfMaxThreads)
+k_cf_rows_mid(int nx, int ny, int lg_nx, int lg_rp, int LD, const C *__restrict__ Y2, const C *__restrict__ W,
+              double scale, C *__restrict__ X1)
+{
+    using R = decltype(C{}.x);
+    extern __shared__ __align__(16) unsigned char cf_smem[];
+    const int NX = 1 << lg_nx, rp = 1 << lg_rp;
+    C *A = reinterpret_cast<C *>(cf_smem);
+    C *B = A + (NX << lg_rp);
+    const int pair0 = blockIdx.x * rp;
+    C *V = rows_inverse(A, B, ny, lg_nx, lg_rp, LD, pair0, Y2, W);
+    const R sc = R(scale);
+    for (int q = threadIdx.x; q < (NX << lg_rp); q += blockDim.x) {
+        const int s = q & (rp - 1), i = q >> lg_rp;
+        const int ja = 2 * (pair0 + s);
+        const C v = V[q];
+        V[q] = cxv(i < nx && ja < ny ? v.x * sc : R(0), i < nx && ja + 1 < ny ? -v.y * sc : R(0));
+    }
+    __syncthreads();
+    const C *Z = smem_dft(V, V == A ? B : A, lg_nx, lg_rp, W);
+    rows_split(Z, ny, lg_nx, lg_rp, LD, pair0, X1);
 }
 
 // Kh2[ky][kx] = Kh[kx][ky], kx < LD: the columns of the (transposed) kernel
@@ -401,6 +508,40 @@ int conv_apply_fused(const ConvPlan<R> &P, const IN *in, OUT *out, cudaStream_t 
     MPI_TRY(cf_cols<C>(c, P.a, P.Kh, P.WY, P.t, st));
     return cf_rows_inv<C, OUT>(P.nx, P.ny, P.NX, P.LD, P.t, P.WX, 1.0 / (double(P.NX) * double(P.NY)), out, st);
 }
+
+// out = C C v.  Five launches instead of six; at 100 x 100 each launch of the
+// chain costs 4 to 5 us whatever it does.
+template <typename R>
+int conv_twice_fused(const ConvPlan<R> &P, const double *v, const CgDirection *dir, R *out, cudaStream_t st)
+{
+    using C = typename ConvPlan<R>::C2;
+    const int lg_nx = ilog2(P.NX), lg_rp = rows_lg_rp(P.NX);
+    const unsigned blocks = (unsigned)(((P.ny + 1) / 2 + (1 << lg_rp) - 1) >> lg_rp), threads = block_threads(lg_nx, lg_rp);
+    const size_t smem = 2 * sizeof(C) * (size_t(P.NX) << lg_rp);
+    const double scale = 1.0 / (double(P.NX) * double(P.NY));
+    CfCols c{};
+    c.mode = kCfFused;
+    c.n = P.NY;
+    c.n_in = c.n_out = P.ny;
+    c.n_outer = 1;
+    c.LD = P.LD;
+    c.in_stride = c.out_stride = c.k_stride = P.LD;
+    if (dir) {
+        MPI_TRY(allow_smem(k_cf_rows_direction<C>, smem));
+        k_cf_rows_direction<C><<<blocks, threads, smem, st>>>(P.nx, P.ny, lg_nx, lg_rp, P.LD, *dir, P.WX, P.a);
+        MPI_CHECK_LAUNCH();
+    } else {
+        MPI_TRY((cf_rows_fwd<C, double>(P.nx, P.ny, P.NX, P.LD, v, P.WX, P.a, st)));
+    }
+    MPI_TRY(cf_cols<C>(c, P.a, P.Kh, P.WY, P.t, st));
+    MPI_TRY(allow_smem(k_cf_rows_mid<C>, smem));
+    k_cf_rows_mid<C><<<blocks, threads, smem, st>>>(P.nx, P.ny, lg_nx, lg_rp, P.LD, P.t, P.WX, scale, P.a);
+    MPI_CHECK_LAUNCH();
+    MPI_TRY(cf_cols<C>(c, P.a, P.Kh, P.WY, P.t, st));
+    return cf_rows_inv(P.nx, P.ny, P.NX, P.LD, P.t, P.WX, scale, out, st);
+}
+template int conv_twice_fused(const ConvPlan<float> &, const double *, const CgDirection *, float *, cudaStream_t);
+template int conv_twice_fused(const ConvPlan<double> &, const double *, const CgDirection *, double *, cudaStream_t);
 
 template int cf_rows_fwd<float2, float>(int, int, int, int, const float *, const float2 *, float2 *, cudaStream_t);
 template int cf_rows_fwd<float2, double>(int, int, int, int, const double *, const float2 *, float2 *, cudaStream_t);

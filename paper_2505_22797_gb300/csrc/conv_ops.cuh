@@ -60,6 +60,12 @@ int conv_fused_kernel(int NX, int NY, int LD, C *Kh, C *tmp, cudaStream_t st);
 template <typename R, typename IN, typename OUT>
 int conv_apply_fused(const ConvPlan<R> &P, const IN *in, OUT *out, cudaStream_t st);
 
+// out = C C v for a plan of the three-launch form, after the update of v that
+// dir (nullable) describes; five launches.
+struct CgDirection;
+template <typename R>
+int conv_twice_fused(const ConvPlan<R> &P, const double *v, const CgDirection *dir, R *out, cudaStream_t st);
+
 // Pieces of the shared-memory FFT routes (conv_fft2.cu), shared by the 2-D
 // and 3-D convolutions.  Row launches: n_rows real rows of nx values (row r
 // at in + r nx) <-> their half spectra (row r at X + r LD, LD entries, bins

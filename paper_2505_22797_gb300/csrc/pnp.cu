@@ -160,14 +160,23 @@ int cg_init_launch(int64_t N, const double *b0, const double *x, const double *q
     return MPI_OK;
 }
 
-int cg_step_launch(int64_t N, double *x, double *r, double *p, const double *q,
-                   const double *pq_part, int n_pq, const double *rr_in, double *rr_out, int *done,
-                   const double *thresh, int *iters, cudaStream_t st)
+int cg_update_launch(int64_t N, double *x, double *r, const double *p, const double *q,
+                     const double *pq_part, int n_pq, const double *rr_in, double *rr_out, int *done,
+                     const double *thresh, int *iters, cudaStream_t st)
 {
     const int nblk = vec_blocks(N);
     k_cg_step1<<<nblk, kVecThreads, 0, st>>>(N, nblk, x, r, p, q, pq_part, n_pq, rr_in, rr_out,
                                             done, thresh, iters);
     MPI_CHECK_LAUNCH();
+    return MPI_OK;
+}
+
+int cg_step_launch(int64_t N, double *x, double *r, double *p, const double *q,
+                   const double *pq_part, int n_pq, const double *rr_in, double *rr_out, int *done,
+                   const double *thresh, int *iters, cudaStream_t st)
+{
+    const int nblk = vec_blocks(N);
+    MPI_TRY(cg_update_launch(N, x, r, p, q, pq_part, n_pq, rr_in, rr_out, done, thresh, iters, st));
     k_cg_step2<<<nblk, kVecThreads, 0, st>>>(N, nblk, r, p, rr_in, rr_out, done);
     MPI_CHECK_LAUNCH();
     return MPI_OK;
@@ -240,9 +249,15 @@ int pnp_run(PnPOperator<R> &op, int64_t N, const void *data, const mpi_pnp_opts 
         MPI_TRY(op.apply_normal(x, q, scal + kScalNu, pq_part, s));
         MPI_TRY(cg_init_launch(N, b0, x, q, scal + kScalNu, r, p, rr_part[0], done, s));
         for (int i = 0; i < o.n_cg; ++i) {
-            MPI_TRY(op.apply_normal(p, q, scal + kScalNu, pq_part, s));
-            MPI_TRY(cg_step_launch(N, x, r, p, q, pq_part, n_pq, rr_part[i & 1], rr_part[(i + 1) & 1],
-                                   done, nullptr, nullptr, s));
+            double *const rr_in = rr_part[i & 1], *const rr_out = rr_part[(i + 1) & 1];
+            const bool dir = op.takes_direction();
+            if (dir && i > 0)
+                MPI_TRY(op.apply_direction(CgDirection{p, r, rr_out, rr_in, nblk, done}, q, scal + kScalNu, pq_part, s));
+            else MPI_TRY(op.apply_normal(p, q, scal + kScalNu, pq_part, s));
+            if (dir)
+                MPI_TRY(cg_update_launch(N, x, r, p, q, pq_part, n_pq, rr_in, rr_out, done, nullptr, nullptr, s));
+            else
+                MPI_TRY(cg_step_launch(N, x, r, p, q, pq_part, n_pq, rr_in, rr_out, done, nullptr, nullptr, s));
         }
         return MPI_OK;
     };
@@ -359,9 +374,26 @@ struct PnPOp2D final : PnPOperator<R> {
             MPI_TRY(reduce(red, st));
             return axpy_dot_launch<double>(N, red, v, nu_dev, q, pq_part, st);
         }
-        MPI_TRY((conv_apply<R, double, R>(C, v, tmp1, st)));
-        MPI_TRY((conv_apply<R, R, R>(C, tmp1, tmp2, st)));
+        if (C.fused) {
+            MPI_TRY(conv_twice(v, nullptr, st));
+        } else {
+            MPI_TRY((conv_apply<R, double, R>(C, v, tmp1, st)));
+            MPI_TRY((conv_apply<R, R, R>(C, tmp1, tmp2, st)));
+        }
         return axpy_dot_launch<R>(N, tmp2, v, nu_dev, q, pq_part, st);
+    }
+    int conv_twice(const double *v, const CgDirection *dir, cudaStream_t st)  // tmp2 = C C v
+    {
+        ProfScope prof(kProfConv, st);
+        return conv_twice_fused<R>(C, v, dir, tmp2, st);
+    }
+    // (the trace-kernel convolution's first row launch loads every value of p once)
+    bool takes_direction() const override { return op != MPI_OP_FORWARD && C.fused; }
+    int apply_direction(const CgDirection &dir, double *q, const double *nu_dev, double *pq_part,
+                        cudaStream_t st) override
+    {
+        MPI_TRY(conv_twice(dir.p, &dir, st));
+        return axpy_dot_launch<R>(N, tmp2, dir.p, nu_dev, q, pq_part, st);
     }
     int n_pq() const override
     {

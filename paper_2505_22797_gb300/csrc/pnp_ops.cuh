@@ -25,6 +25,10 @@ int cg_init_launch(int64_t N, const double *b0, const double *x, const double *q
 // partial sums of r.r alternate between rr_in and rr_out.  thresh (device,
 // nullable): stop once ||r|| <= *thresh.  iters (device, nullable): counts
 // the updates performed.
+int cg_update_launch(int64_t N, double *x, double *r, const double *p, const double *q,
+                     const double *pq_part, int n_pq, const double *rr_in, double *rr_out, int *done,
+                     const double *thresh, int *iters, cudaStream_t st);
+// The update and the new direction p.
 int cg_step_launch(int64_t N, double *x, double *r, double *p, const double *q,
                    const double *pq_part, int n_pq, const double *rr_in, double *rr_out, int *done,
                    const double *thresh, int *iters, cudaStream_t st);
@@ -37,6 +41,15 @@ int launch_gauss5(const R *in, R *out, int nx, int ny, cudaStream_t st);
 template <typename R>
 int axpy_dot_launch(int64_t N, const R *y, const double *v, const double *nu_dev, double *q,
                     double *dot_part, cudaStream_t st);
+
+// A pending update of the CG direction p: p = r + beta p with beta = r.r(new)
+// / r.r(old) from their n_part partial sums; nothing once *done is set.
+struct CgDirection {
+    double *p;
+    const double *r, *rr_old, *rr_new;
+    int n_part;
+    const int *done;
+};
 
 // The data-fidelity operator O of one ZeroShot-PnP solve (Algorithm 1): the
 // solve driver below is written against this interface, so the 2-D operators
@@ -51,6 +64,13 @@ struct PnPOperator {
     virtual int apply_normal(const double *v, double *q, const double *nu_dev, double *pq_part,
                              cudaStream_t st) = 0;
     virtual int n_pq() const = 0;
+    // The same after the pending update of p, for operators whose first
+    // launch can form it.
+    virtual bool takes_direction() const { return false; }
+    virtual int apply_direction(const CgDirection &, double *, const double *, double *, cudaStream_t)
+    {
+        return MPI_ERR_INVALID;
+    }
     // The denoiser step (Algorithm 1, "Denoise"): the built-in Gaussian or a
     // user callback; returns the callback's status (nonzero = failure).
     virtual int denoise(const R *in, R *out, const double *sigma_dev, cudaStream_t st) = 0;
