@@ -36,15 +36,20 @@ constexpr int kResSpin = 1 << 22;
 
 #ifdef __CUDACC__
 
-// All threads call it; false once a wait has given up.  The block's writes
-// are ordered before its arrival (bar.sync, then a release by thread 0), the
-// others' after the wait (an acquire by thread 0, then bar.sync).
-__device__ __forceinline__ bool res_barrier(ResBarrier *b, unsigned long long &target, int *s_ok)
+// The barrier in two halves.  All threads call both; work of a block's own
+// may stand between them.  The block's writes before res_arrive are ordered
+// before its arrival (bar.sync, then a release by thread 0), the others'
+// after the wait (an acquire by thread 0, then bar.sync).  res_wait is false
+// once a wait has given up.
+__device__ __forceinline__ void res_arrive(ResBarrier *b)
+{
+    __syncthreads();
+    if (threadIdx.x == 0) asm volatile("red.release.gpu.global.add.u64 [%0], 1;" ::"l"(&b->arrived) : "memory");
+}
+__device__ __forceinline__ bool res_wait(ResBarrier *b, unsigned long long &target, int *s_ok)
 {
     target += gridDim.x;
-    __syncthreads();
     if (threadIdx.x == 0) {
-        asm volatile("red.release.gpu.global.add.u64 [%0], 1;" ::"l"(&b->arrived) : "memory");
         int ok = 1, n = 0;
         unsigned long long seen;
         for (;;) {
@@ -60,6 +65,11 @@ __device__ __forceinline__ bool res_barrier(ResBarrier *b, unsigned long long &t
     }
     __syncthreads();
     return *s_ok != 0;
+}
+__device__ __forceinline__ bool res_barrier(ResBarrier *b, unsigned long long &target, int *s_ok)
+{
+    res_arrive(b);
+    return res_wait(b, target, s_ok);
 }
 
 // The block's partial sums of v over groups of PT consecutive threads, as
@@ -128,7 +138,8 @@ k_cs_resident(const __grid_constant__ Op op, int N, const float2 *__restrict__ b
     __shared__ double sh[kResThreads / 32];
     __shared__ F2Sum sw[kResThreads / 32];
     __shared__ df s_coef;
-    __shared__ int s_ok, s_stop;
+    __shared__ int s_ok, s_stop, s_zero;
+    __shared__ double s_rr, s_tol;
     unsigned long long target = 0;
     const int node = blockIdx.x * kResThreads + threadIdx.x;
     const bool in = node < N;
@@ -137,7 +148,7 @@ k_cs_resident(const __grid_constant__ Op op, int N, const float2 *__restrict__ b
     const int n_rr = (int)((n + kResFlat - 1) / kResFlat);
     const bool flat = int(blockIdx.x) < n_rr;
     bool ok = true;
-    double rr = 0.0, tol = -1.0;  // thread 0's
+    double rr = 0.0;  // thread 0's
     df r[NC], d[NC], rf[U];
     if (flat) {
         CsDot<df> acc{};
@@ -164,8 +175,10 @@ k_cs_resident(const __grid_constant__ Op op, int N, const float2 *__restrict__ b
     ok = res_barrier(bar, target, &s_ok);
     {
         const double v = res_sum<kResThreads>(rr_part, n_rr, sh);
-        rr = v;
-        tol = rel_tol > 0.0 ? rel_tol * sqrt(v) : -1.0;
+        if (threadIdx.x == 0) {
+            rr = s_rr = v;
+            s_tol = rel_tol > 0.0 ? rel_tol * sqrt(v) : -1.0;
+        }
     }
     int it = 0;
     for (; ok && it < max_iter; ++it) {
@@ -196,12 +209,14 @@ k_cs_resident(const __grid_constant__ Op op, int N, const float2 *__restrict__ b
         {
             const double pq = res_sum<PT>(pq_part, n_pq, sh);
             if (threadIdx.x == 0) {
-                s_stop = rr == 0.0 || pq == 0.0 || (tol >= 0.0 && sqrt(rr) <= tol);
+                s_zero = pq == 0.0;
                 s_coef = df_from_double(rr / pq);
+            } else if (threadIdx.x == 32) {  // (beside the division)
+                s_stop = s_rr == 0.0 || (s_tol >= 0.0 && sqrt(s_rr) <= s_tol);
             }
             __syncthreads();
         }
-        if (!ok || s_stop) break;
+        if (!ok || s_stop || s_zero) break;
         const df al = s_coef, nal = df_neg(al);
         if (flat) {
             CsDot<df> acc{};
@@ -215,6 +230,7 @@ k_cs_resident(const __grid_constant__ Op op, int N, const float2 *__restrict__ b
             }
             res_partials<kResThreads>(acc.s, sw, rr_part, n_rr);
         }
+        res_arrive(bar);
         if (in) {
 #pragma unroll
             for (int m = 0; m < NC; ++m) {
@@ -223,12 +239,12 @@ k_cs_resident(const __grid_constant__ Op op, int N, const float2 *__restrict__ b
                 r[m] = df_axpy(r[m], nal, q[m]);
             }
         }
-        ok = res_barrier(bar, target, &s_ok) && ok;
+        ok = res_wait(bar, target, &s_ok) && ok;
         {
             const double v = res_sum<kResThreads>(rr_part, n_rr, sh);
             if (threadIdx.x == 0) {
                 s_coef = df_from_double(v / rr);
-                rr = v;
+                rr = s_rr = v;
             }
             __syncthreads();
         }
