@@ -205,16 +205,17 @@ struct StatTab {
 };
 
 // One cluster per frame: percentile trimming, noise estimate and PnP scalars.
-__global__ void __cluster_dims__(kStatBlocks, 1, 1) __launch_bounds__(kStatThreads)
+__global__ void __launch_bounds__(kStatThreads)
 k_stats_b(const __grid_constant__ StatTab B, const double *__restrict__ x, float *__restrict__ rho1)
 {
-    const int f = blockIdx.x / kStatBlocks;
+    const int blocks = cooperative_groups::this_cluster().num_blocks();
+    const int f = blockIdx.x / blocks;
     const VecFrame &F = B.f[f];
     const bool first = F.scal[kScalIter] == 0.0;
     outer_stats_cluster<float>(F.N, x + F.off, B.do_clip, B.pct, first, B.nu0[f], F.scal,
                                F.rr[B.final_parity], F.nblk, nullptr, rho1 + F.off);
     // (behind the cluster's last barrier: every block has read the count)
-    if (blockIdx.x % kStatBlocks == 0 && threadIdx.x == 0) F.scal[kScalIter] += 1.0;
+    if (blockIdx.x % blocks == 0 && threadIdx.x == 0) F.scal[kScalIter] += 1.0;
 }
 
 struct GaussFrame {
@@ -553,7 +554,8 @@ static int enqueue_iteration(mpi_batch_plan &P, cudaStream_t st)
         k_cg_step2_b<<<vb, kVecThreads, 0, st>>>(P.vec, i & 1, P.r, P.p);
         MPI_CHECK_LAUNCH();
     }
-    k_stats_b<<<P.n * kStatBlocks, kStatThreads, 0, st>>>(P.stat, P.x, P.rho1);
+    const int cluster = stat_blocks(*std::max_element(P.N.begin(), P.N.end()));
+    launch_cluster(k_stats_b, cluster, P.n * cluster, kStatThreads, st, P.stat, P.x, P.rho1);
     MPI_CHECK_LAUNCH();
     int mtx = 1, mty = 1;
     for (int f = 0; f < P.n; ++f) {

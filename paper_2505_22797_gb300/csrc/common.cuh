@@ -70,6 +70,23 @@ inline void launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t s
     cfg.numAttrs = cudaStreamIsCapturing(st, &capture) == cudaSuccess && capture == cudaStreamCaptureStatusNone;
     (void)cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);  // MPI_CHECK_LAUNCH reports
 }
+
+// A launch in clusters of `cluster` blocks.
+template <typename... P, typename... A>
+inline void launch_cluster(void (*kernel)(P...), int cluster, dim3 grid, dim3 block, cudaStream_t st, A &&...args)
+{
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = cluster;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    (void)cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);  // MPI_CHECK_LAUNCH reports
+}
 #endif
 
 #define MPI_CHECK_LAUNCH()                          \

@@ -183,7 +183,7 @@ int cg_step_launch(int64_t N, double *x, double *r, double *p, const double *q,
 }
 
 template <typename R>
-__global__ void __cluster_dims__(kStatBlocks, 1, 1) __launch_bounds__(kStatThreads)
+__global__ void __launch_bounds__(kStatThreads)
 k_outer_stats(int64_t N, const double *__restrict__ x, int do_clip, double pct, int k, double nu0,
               double *__restrict__ scal, const double *__restrict__ rr_part, int nblk,
               double *__restrict__ info_row, R *__restrict__ rho1)
@@ -273,7 +273,7 @@ int pnp_run(PnPOperator<R> &op, int64_t N, const void *data, const mpi_pnp_opts 
         if (cg_graph.ready()) MPI_TRY(cg_graph.launch(st));
         else MPI_TRY(enqueue_cg(st));
         // trimming, sigma, lambda (k = 0), nu
-        k_outer_stats<R><<<kStatBlocks, kStatThreads, 0, st>>>(N, x, o.clip_pct >= 0.0 ? 1 : 0, o.clip_pct, k,
+        launch_cluster(k_outer_stats<R>, stat_blocks(N), stat_blocks(N), kStatThreads, st, N, x, o.clip_pct >= 0.0 ? 1 : 0, o.clip_pct, k,
                                                     o.nu0, scal, rr_part[o.n_cg & 1], nblk,
                                                     inf + kInfoCols * k, rho1);
         MPI_CHECK_LAUNCH();

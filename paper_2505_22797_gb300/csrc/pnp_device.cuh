@@ -71,22 +71,23 @@ __device__ __forceinline__ double block_min(double v, double *sh /* >= NT/32 + 1
     return r;
 }
 
-// The percentile step runs on a cluster of kStatBlocks blocks per image
+// The percentile step runs on a cluster of up to kStatBlocks blocks per image
 // (distributed shared memory, cluster barriers): FP64 additions and
-// comparisons take a block's SM 19 clocks per warp, so one block alone was
-// bound by them (80 us at 100 x 100 values, a third of it one thread's walk
-// over the digit counts).  The cluster takes 53 us less there.
+// comparisons take a block's SM 19 clocks per warp, so one block alone is
+// bound by them (80 us at 100 x 100 values), while on few values the 20
+// barriers of a cluster cost more than they save.  Four iterations of a small
+// reconstruction with one block / with eight: 60 x 50 values 1040 / 1070 us,
+// 70 x 60 1120 / 1123 us, 80 x 70 1195 / 1175 us, 100 x 100 1463 / 1363 us.
 constexpr int kStatBlocks = 8;
+inline int stat_blocks(int64_t N) { return N <= 4096 ? 1 : kStatBlocks; }
 
 // The sums run in the order of one block of kStatThreads threads (thread t
 // over the values t, t + kStatThreads, ...; its warps in order): each block
-// takes kStatSumWarps of that block's warps.
-constexpr int kStatSumWarps = kStatThreads / 32 / kStatBlocks;
-
+// takes its share of that block's warps.
 struct StatShared {
     unsigned hist[256];
-    double part[kStatSumWarps];  // this block's partial sums, minimum and count,
-    double least;                // read by the others
+    double part[kStatThreads / 32];  // this block's partial sums, minimum and count,
+    double least;                    // read by the others
     unsigned long long cnt;
     double sh[kStatThreads / 32 + 1];
     unsigned long long sel[2]; // prefix, remaining rank
@@ -99,7 +100,8 @@ __device__ inline double cluster_select(const double *__restrict__ x, int64_t N,
     namespace cg = cooperative_groups;
     cg::cluster_group cl = cg::this_cluster();
     const int tid = threadIdx.x, lane = tid & 31;
-    const int64_t first = (int64_t)cl.block_rank() * kStatThreads, stride = (int64_t)kStatBlocks * kStatThreads;
+    const int nb = cl.num_blocks();
+    const int64_t first = (int64_t)cl.block_rank() * kStatThreads, stride = (int64_t)nb * kStatThreads;
     uint64_t prefix = 0, mask = 0;
     int64_t krem = rank;
     for (int shift = 56; shift >= 0; shift -= 8) {
@@ -121,7 +123,7 @@ __device__ inline double cluster_select(const double *__restrict__ x, int64_t N,
 #pragma unroll
             for (int q = 0; q < 8; ++q) {
                 unsigned long long n = 0;
-                for (int b = 0; b < kStatBlocks; ++b) n += *cl.map_shared_rank(&S.hist[8 * lane + q], b);
+                for (int b = 0; b < nb; ++b) n += *cl.map_shared_rank(&S.hist[8 * lane + q], b);
                 c[q] = n;
                 sum += n;
             }
@@ -154,16 +156,16 @@ __device__ inline double cluster_sum(int64_t N, F f, StatShared &S)
 {
     namespace cg = cooperative_groups;
     cg::cluster_group cl = cg::this_cluster();
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (warp < kStatSumWarps) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, share = kStatThreads / 32 / cl.num_blocks();
+    if (warp < share) {
         double s = 0.0;
-        for (int64_t i = ((int)cl.block_rank() * kStatSumWarps + warp) * 32 + lane; i < N; i += kStatThreads) s += f(i);
+        for (int64_t i = ((int)cl.block_rank() * share + warp) * 32 + lane; i < N; i += kStatThreads) s += f(i);
         s = warp_sum(s);
         if (lane == 0) S.part[warp] = s;
     }
     cl.sync();
     if (warp == 0) {
-        double t = *cl.map_shared_rank(&S.part[lane % kStatSumWarps], lane / kStatSumWarps);
+        double t = *cl.map_shared_rank(&S.part[lane % share], lane / share);
         double a = 0.0;
         for (int w = 0; w < kStatThreads / 32; ++w) a += __shfl_sync(0xffffffffu, t, w);
         if (lane == 0) S.sh[kStatThreads / 32] = a;
@@ -189,7 +191,7 @@ __device__ void outer_stats_cluster(int64_t N, const double *__restrict__ x, int
     cg::cluster_group cl = cg::this_cluster();
     __shared__ StatShared S;
     const int64_t i0 = (int64_t)cl.block_rank() * kStatThreads + threadIdx.x;
-    const int64_t stride = (int64_t)kStatBlocks * kStatThreads;
+    const int64_t stride = (int64_t)cl.num_blocks() * kStatThreads;
     double P = -INFINITY;
     if (do_clip) {
         const double h = double(N - 1) * pct / 100.0;
@@ -216,7 +218,7 @@ __device__ void outer_stats_cluster(int64_t N, const double *__restrict__ x, int
             }
             cl.sync();
             le = 0;
-            for (int b = 0; b < kStatBlocks; ++b) {
+            for (int b = 0; b < (int)cl.num_blocks(); ++b) {
                 le += (long long)*cl.map_shared_rank(&S.cnt, b);
                 gt = fmin(gt, *cl.map_shared_rank(&S.least, b));
             }
