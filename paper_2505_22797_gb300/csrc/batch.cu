@@ -110,6 +110,7 @@ struct VecFrame {
     double *rr[2];
     int *done;
     double *scal;
+    bool residual;  // q holds the initial residual itself (gridded frames)
 };
 struct VecTab {
     int n;
@@ -136,7 +137,7 @@ k_cg_init_b(const __grid_constant__ VecTab B, const double *__restrict__ b0, con
     const int64_t e0 = lb * kVecPerBlock, e1 = min(F.N, e0 + kVecPerBlock);
     double acc = 0.0;
     for (int64_t e = F.off + e0 + threadIdx.x; e < F.off + e1; e += kVecThreads) {
-        const double re = (b0[e] + nu * x[e]) - q[e];
+        const double re = F.residual ? q[e] : (b0[e] + nu * x[e]) - q[e];
         r[e] = re;
         p[e] = re;
         acc += re * re;
@@ -521,7 +522,8 @@ static int launch_adj_kernel(mpi_batch_plan &P, const PairTab &B, cudaStream_t s
     return MPI_OK;
 }
 
-// q = (A^T A + nu I) v for every frame (v = x for which = 0, p for 1).
+// q = (A^T A + nu I) v for every frame (v = x for which = 0, p for 1); for
+// which = 0 a gridded frame's q is the residual A^T (s - A x).
 static int apply_normal_b(mpi_batch_plan &P, int which, cudaStream_t st)
 {
     MPI_TRY(launch_fwd(P, which, st));
@@ -533,8 +535,10 @@ static int apply_normal_b(mpi_batch_plan &P, int which, cudaStream_t st)
     for (int f = 0; f < P.n; ++f) {
         if (!P.gridded[f]) continue;
         const double *v = (which == 0 ? P.x : P.p) + P.voff[f];
-        MPI_TRY(field_forward_ordered<double>(P.fld[f], v, st));
-        MPI_TRY(field_adjoint<double>(P.fld[f], P.q + P.voff[f], v, P.scal[f] + kScalNu, P.pq[f], st));
+        MPI_TRY(field_forward_ordered<double>(P.fld[f], v, which == 0, st));
+        const double *cg_p = which == 0 ? nullptr : v;
+        MPI_TRY(field_adjoint<double>(P.fld[f], P.q + P.voff[f], cg_p, cg_p ? P.scal[f] + kScalNu : nullptr,
+                                      cg_p ? P.pq[f] : nullptr, st));
     }
     return MPI_OK;
 }
@@ -861,6 +865,7 @@ int mpi_batch_plan_create(int n_frames, const mpi_model *models, const mpi_grid_
         V.rr[1] = P->rr1[f];
         V.done = P->done[f];
         V.scal = P->scal[f];
+        V.residual = P->gridded[f] != 0;
         P->vec.f[f] = V;
         P->stat.f[f] = V;
         P->stat.nu0[f] = P->nu0[f];
@@ -915,8 +920,8 @@ int mpi_batch_pnp_run(mpi_batch_plan *P, const void *const *r, const void *const
         if (!P->gridded[f]) continue;
         const float *rf = static_cast<const float *>(r[f]), *vf = static_cast<const float *>(v[f]);
         MPI_TRY(field_prepare(P->fld[f], nullptr, rf, vf, st));
-        MPI_TRY(field_order(P->fld[f], rf, vf, static_cast<const float *>(s[f]), st));
-        MPI_TRY(field_adjoint<double>(P->fld[f], P->b0 + P->voff[f], nullptr, nullptr, nullptr, st));
+        MPI_TRY(field_order(P->fld[f], rf, vf, nullptr, st));
+        MPI_TRY(field_load(P->fld[f], static_cast<const float *>(s[f]), st));
     }
     MPI_TRY_CUDA(cudaMemsetAsync(P->rho2, 0, sizeof(float) * P->Ntot, st));
     k_init_b<<<(P->n + 63) / 64, 64, 0, st>>>(P->stat);

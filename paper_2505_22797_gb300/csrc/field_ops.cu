@@ -21,8 +21,10 @@
 //
 // Rounding: FP32 transforms leave errors of about one rounding of the
 // largest modes, which for images are the few lowest ones.  So the modes |kx|, |ky| <
-// kFieldLow are summed directly in pairs of floats at every stage that they
-// would dominate, the kernel is sampled with correctly rounded functions, and
+// kFieldLow are carried in pairs of floats from the image (or the nodes) to
+// the nodes (or the voxels); one rounding of the columns between the two axes
+// alone left 5e-9 in the lowest modes, which the CG of a solve turned into 2e-6
+// of the image (now 4e-7, the direct sums' own error 1.7e-6); the kernel is sampled with correctly rounded functions, and
 // the interpolation's outer sum and the product with W are carried in pairs.
 //
 // Samples beyond the node window (more than 12 z units outside the voxels)
@@ -380,12 +382,8 @@ __global__ void __launch_bounds__(256) k_field_load(const __grid_constant__ Fiel
     chain_wait();
     const int64_t p = int64_t(blockIdx.x) * 256 + threadIdx.x;
     if (p >= d.T) return;
-    const float4 rc = d.b.rec[p], w = d.b.wv[p];
-    SampleRec q{};
-    q.in = __float_as_int(rc.z) >= 0;
-    q.Wx = make_float2(w.x, w.z);
-    q.Wy = make_float2(w.y, w.w);
-    d.b.q4[p] = operand(d, s, d.b.list[p], q);
+    const int64_t t = d.b.list[p];
+    d.b.sd[p] = make_float2(s[t], d.n_ch > 1 ? s[d.T + t] : 0.0f);
 }
 
 // Tables (32 entries per block: FP64 functions, spread over the SMs) and, in
@@ -637,26 +635,6 @@ __device__ __forceinline__ void low_add(const float4 *co, int e, int n, const fl
         }
     }
 }
-// The same rounded to FP32 as it goes, the mean last (one rounding at full
-// size): for values that many others average.
-__device__ __forceinline__ void low_add32(const float4 *co, int e, int n, const float2 *__restrict__ tw, V2<float> &q)
-{
-    int at = int(unsigned(e * (kFieldLow - 1)) % unsigned(n));
-#pragma unroll
-    for (int k = kFieldLow - 1; k > 0; --k) {
-        const float2 t = tw[at];
-        at -= e;
-        at += at < 0 ? n : 0;
-        const float4 v = co[kFieldLow - 1 + k], u = co[kFieldLow - 1 - k];
-        // v (t.x - i t.y) + u (t.x + i t.y)
-        q.x = fmaf(v.x + u.x, t.x, fmaf(v.y - u.y, t.y, q.x));
-        q.y = fmaf(v.y + u.y, t.x, fmaf(u.x - v.x, t.y, q.y));
-    }
-    const float4 v = co[kFieldLow - 1];
-    q.x = (q.x + v.z) + v.x;
-    q.y = (q.y + v.w) + v.y;
-}
-
 // Columns of the kernel's spectrum: NC adjacent kx (group g) of entry m.  The
 // spectrum of a real kernel that is even under (x, y) -> (-x, -y) is real;
 // the rows l > Py/2 are the conjugates of rows Py - l.
@@ -855,7 +833,15 @@ __global__ void __launch_bounds__(512) k_field_cols_fwd(const __grid_constant__ 
         int l = l0 + i;
         l -= l >= P ? P : 0;
         V2<float> q = z[smem_fft_pad(l) * NC + c];
-        if (low && kx < kFieldLow) low_add32(s_low[c], l, P, d.b.twPy, q);
+        if (low && kx < kFieldLow) {
+            F2Sum re{}, im{};
+            low_add(s_low[c], l, P, d.b.twPy, re, im);
+            re.add(q.x);
+            im.add(q.y);
+            const df r = df_fast_two_sum(re.hi, re.lo), s = df_fast_two_sum(im.hi, im.lo);
+            q = V2<float>{r.x, s.x};
+            d.b.FL[(int64_t(m) * d.y.w + i) * kFieldLow + kx] = make_float2(r.y, s.y);
+        }
         F[int64_t(i) * J1] = f2c(q);
     }
 }
@@ -867,6 +853,7 @@ __global__ void __launch_bounds__(512) k_field_rows_inv(const __grid_constant__ 
     chain_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ float4 s_low[3][kFieldLow];  // (re, im) of both rows' lowest modes
+    __shared__ float4 s_lo[3][kFieldLow];   // what those round off
     const int P = d.x.P, J = d.x.J, J1 = J + 1;
     V2<float> *a = reinterpret_cast<V2<float> *>(smem_raw);
     V2<float> *b = a + (smem_fft_pad(P - 1) + 1) * 3;
@@ -893,6 +880,12 @@ __global__ void __launch_bounds__(512) k_field_rows_inv(const __grid_constant__ 
             if (k < kFieldLow) {  // added at the end (the mean of a real row is real)
                 const float f = k ? 2.0f : 1.0f;
                 s_low[c][k] = make_float4(f * A[c].x, k ? f * A[c].y : 0.0f, f * B[c].x, k ? f * B[c].y : 0.0f);
+                // entry c of A: xx of row 0, xx of row 1, yy of row 0; of B: xy, xy, yy of row 1
+                const int64_t lp = int64_t(d.y.w) * kFieldLow, r0 = int64_t(i0) * kFieldLow + k, r1 = r0 + (two ? kFieldLow : 0);
+                const float2 *L = d.b.FL;
+                const float2 la = L[c == 0 ? r0 : c == 1 ? r1 : 2 * lp + r0];
+                const float2 lb = L[c == 0 ? lp + r0 : c == 1 ? lp + r1 : 2 * lp + r1];
+                s_lo[c][k] = make_float4(f * la.x, k ? f * la.y : 0.0f, f * lb.x, k ? f * lb.y : 0.0f);
                 A[c] = B[c] = z0;
             }
             o[c] = V2<float>{A[c].x - B[c].y, A[c].y + B[c].x};
@@ -909,6 +902,7 @@ __global__ void __launch_bounds__(512) k_field_rows_inv(const __grid_constant__ 
         V2<float> q[3];
 #pragma unroll
         for (int c = 0; c < 3; ++c) q[c] = z[smem_fft_pad(l) * 3 + c];
+        V2<float> h[3] = {};
         int at = l * (kFieldLow - 1) % P;
 #pragma unroll
         for (int k = kFieldLow - 1; k >= 0; --k) {  // the mean last: one rounding at full size
@@ -917,10 +911,16 @@ __global__ void __launch_bounds__(512) k_field_rows_inv(const __grid_constant__ 
             at += at < 0 ? P : 0;
 #pragma unroll
             for (int c = 0; c < 3; ++c) {
-                const float4 s = s_low[c][k];
-                if (k) q[c].x = fmaf(s.y, w.y, q[c].x), q[c].y = fmaf(s.w, w.y, q[c].y);
-                q[c].x = fmaf(s.x, w.x, q[c].x);
-                q[c].y = fmaf(s.z, w.x, q[c].y);
+                const float4 s = s_low[c][k], u = s_lo[c][k];
+                if (k) {
+                    h[c].x = fmaf(s.x, w.x, fmaf(s.y, w.y, h[c].x));
+                    h[c].y = fmaf(s.z, w.x, fmaf(s.w, w.y, h[c].y));
+                    q[c].x = fmaf(u.x, w.x, fmaf(u.y, w.y, q[c].x));
+                    q[c].y = fmaf(u.z, w.x, fmaf(u.w, w.y, q[c].y));
+                } else {
+                    q[c].x = ((q[c].x + u.x) + h[c].x) + s.x;
+                    q[c].y = ((q[c].y + u.z) + h[c].y) + s.z;
+                }
             }
         }
         N[i] = make_float4(q[0].x, q[0].y, q[2].x, 0.0f);
@@ -968,6 +968,7 @@ enum { kInterpForward = 0, kInterpOrdered = 1 };
 struct InterpArgs {
     const float *r, *v;   // unordered trajectory
     float *s;             // [n_ch][T]
+    bool residual;        // ordered: the data minus A c
 };
 
 // The field at the samples and its product with W.  A warp takes 32 samples,
@@ -1069,11 +1070,13 @@ __global__ void __launch_bounds__(256) k_field_interp(const __grid_constant__ Fi
         }
     }
     float sk[2] = {0.0f, 0.0f};
+    const bool residual = MODE == kInterpOrdered && A.residual;
     auto channels = [&](df Ox, df Oy) {
+        const float2 data = residual ? d.b.sd[t] : make_float2(0.0f, 0.0f);
         for (int k = 0; k < d.n_ch; ++k) {
             const float p0 = d.p[2 * k], p1 = d.p[2 * k + 1];
             const df o = df_add(df_mul(Ox, make_float2(p0, 0.0f)), df_mul(Oy, make_float2(p1, 0.0f)));
-            sk[k] = o.x + o.y;
+            sk[k] = residual ? ((k ? data.y : data.x) - o.x) - o.y : o.x + o.y;
         }
     };
     auto finish = [&](int64_t tt, float2 W, bool inside) {
@@ -1648,12 +1651,14 @@ void lay_out(FieldPlan &plan, char *keep, char *work, size_t &keep_bytes, size_t
     if (plan.forward) {
         take(1, b.CR, ny * (d.x.Q / 2 + 1));
         take(1, b.CL, ny * kFieldLow);
+        take(1, b.FL, size_t(3) * d.y.w * kFieldLow);
         take(1, b.FN, size_t(d.y.w) * d.x.w);
     }
     if (plan.adjoint) {
         take(1, b.key, T1); take(1, b.hist, nh); take(1, b.pos, nh); take(1, b.tcnt, nt + 1);
         take(0, b.list, T1); take(0, b.toff, nt + 1); take(0, b.uoff, nt + 1); take(0, b.unit_tile, d.n_unit_max);
         take(0, b.rec, T1); take(0, b.wv, T1);
+        if (plan.forward) take(0, b.sd, T1);
         take(1, b.q4, T1);
         take(1, b.upart, size_t(3) * kPatchSize * d.n_unit_max);
         take(1, b.opart, size_t(d.out_chunks) * d.x.n * ny);
@@ -1783,21 +1788,21 @@ int field_forward(const FieldPlan &plan, const float *c, const float *r, const f
     ProfScope prof(kProfForward, st);
     MPI_TRY(field_prepare(plan, c, r, v, st));
     MPI_TRY(field_nodes(plan.d, st));
-    const InterpArgs A{r, v, s};
+    const InterpArgs A{r, v, s, false};
     launch_chained(k_field_interp<kInterpForward, float>, interp_blocks(plan.d.T), 256, 0, st, plan.d, A, c);
     MPI_CHECK_LAUNCH();
     return MPI_OK;
 }
 
 template <typename CIN>
-int field_forward_ordered(const FieldPlan &plan, const CIN *c, cudaStream_t st)
+int field_forward_ordered(const FieldPlan &plan, const CIN *c, bool residual, cudaStream_t st)
 {
     const FieldDev &d = plan.d;
     ProfScope prof(kProfForward, st);
     launch_chained(k_field_image<CIN>, (d.y.n + 1) / 2, 128, image_smem(d), st, d, c);
     MPI_CHECK_LAUNCH();
     MPI_TRY(field_nodes(d, st));
-    launch_chained(k_field_interp<kInterpOrdered, CIN>, interp_blocks(plan.d.T), 256, 0, st, plan.d, InterpArgs{}, c);
+    launch_chained(k_field_interp<kInterpOrdered, CIN>, interp_blocks(plan.d.T), 256, 0, st, plan.d, InterpArgs{nullptr, nullptr, nullptr, residual}, c);
     MPI_CHECK_LAUNCH();
     return MPI_OK;
 }
@@ -1868,7 +1873,7 @@ bool field_solve_plan(const ModelH &m, const GridH &g, int64_t T, int n_iter, in
            field_route_solve(plan, (int64_t)n_iter * (n_cg + 1), shared);
 }
 
-template int field_forward_ordered<double>(const FieldPlan &, const double *, cudaStream_t);
+template int field_forward_ordered<double>(const FieldPlan &, const double *, bool, cudaStream_t);
 template int field_adjoint<float>(const FieldPlan &, float *, const double *, const double *, double *, cudaStream_t);
 template int field_adjoint<double>(const FieldPlan &, double *, const double *, const double *, double *, cudaStream_t);
 

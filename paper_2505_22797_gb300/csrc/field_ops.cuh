@@ -34,6 +34,7 @@ struct FieldBuf {
     float2 *CR;      // image rows' half spectra [ny][Qx/2 + 1]
     float4 *CL;      // their lowest modes in pairs [ny][kFieldLow]
     float2 *FC;      // column-transformed half spectra [3][wy][Jx + 1]
+    float2 *FL;      // what FC rounds off of its lowest modes [3][wy][kFieldLow]
     float4 *FN;      // node values (xx, xy, yy, 0) [wy][wx]
     // samples by tile (A^T and the solves)
     int *key, *hist, *pos, *tcnt;
@@ -41,6 +42,7 @@ struct FieldBuf {
     float4 *rec;     // inside: (fx, fy, node column | row << 16, 0); outside: (beta G r)
     float4 *wv;      // beta G v as pairs (hi x, hi y, lo x, lo y)
     float4 *q4;      // inside: (ux Wx, ux Wy + uy Wx, uy Wy, 0); outside: (ux, uy, 0, 0)
+    float2 *sd;      // the data of a solve, both channels, in the samples' order
     float *upart;    // unit patches
     float *opart;    // outside samples' partial images
     float2 *AC;      // [3][ny][Jx + 1]
@@ -96,13 +98,14 @@ int field_prepare(const FieldPlan &plan, const float *c, const float *r, const f
 // The second half of the sample order, after field_prepare; with s
 // ([n_ch][T]) also loads it as the operand of field_adjoint.
 int field_order(const FieldPlan &plan, const float *r, const float *v, const float *s, cudaStream_t st);
-// Loads s ([n_ch][T]) as the operand of field_adjoint.
+// Keeps s ([n_ch][T]) as the data of a solve (plans with both directions).
 int field_load(const FieldPlan &plan, const float *s, cudaStream_t st);
 // One call: s = A c on the unordered trajectory (a forward plan, not prepared).
 int field_forward(const FieldPlan &plan, const float *c, const float *r, const float *v, float *s, cudaStream_t st);
-// The operand of field_adjoint set to A c on the ordered samples.
+// The operand of field_adjoint set to A c on the ordered samples, or with
+// residual to the solve's data minus A c.
 template <typename CIN>
-int field_forward_ordered(const FieldPlan &plan, const CIN *c, cudaStream_t st);
+int field_forward_ordered(const FieldPlan &plan, const CIN *c, bool residual, cudaStream_t st);
 // out = A^T of the loaded operand (OUT float or double); with cg_p: out +=
 // nu cg_p (OUT double) and field_dot_blocks partial sums of <cg_p, out>.
 template <typename OUT>

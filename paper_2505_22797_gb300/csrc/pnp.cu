@@ -57,6 +57,27 @@ k_cg_init(int64_t N, const double *__restrict__ b0, const double *__restrict__ x
     }
 }
 
+// p = r and the partial sums of r.r, for a residual that is already there;
+// clears the stop flag.
+__global__ void __launch_bounds__(kVecThreads)
+k_cg_start(int64_t N, const double *__restrict__ r, double *__restrict__ p, double *__restrict__ rr_part,
+           int *__restrict__ done)
+{
+    __shared__ double sh[kVecThreads / 32 + 1];
+    const int64_t e0 = (int64_t)blockIdx.x * kVecPerBlock, e1 = min(N, e0 + kVecPerBlock);
+    double acc = 0.0;
+    for (int64_t e = e0 + threadIdx.x; e < e1; e += kVecThreads) {
+        const double re = r[e];
+        p[e] = re;
+        acc += re * re;
+    }
+    acc = block_sum<double, kVecThreads>(acc, sh);
+    if (threadIdx.x == 0) {
+        rr_part[blockIdx.x] = acc;
+        if (blockIdx.x == 0) *done = 0;
+    }
+}
+
 // alpha = r.r / p.q;  x += alpha p;  r -= alpha q;  partial sums of the new r.r.
 // Once r.r or p.q is exactly 0 the solve has converged to round-off: the stop
 // flag is set and the remaining steps leave x, r and p untouched.  With a
@@ -236,7 +257,8 @@ int pnp_run(PnPOperator<R> &op, int64_t N, const void *data, const mpi_pnp_opts 
     R *rho1 = scr.at<R>(o_r1), *rho2 = scr.at<R>(o_r2);
 
     // b0 = O^T data
-    MPI_TRY(op.rhs(static_cast<const R *>(data), b0, st));
+    const bool from_data = op.residual_from_data();
+    if (!from_data) MPI_TRY(op.rhs(static_cast<const R *>(data), b0, st));
     k_init_scalars<<<1, 32, 0, st>>>(scal, o.nu0);
     MPI_CHECK_LAUNCH();
 
@@ -246,8 +268,14 @@ int pnp_run(PnPOperator<R> &op, int64_t N, const void *data, const mpi_pnp_opts 
     // initial residual and n_cg steps -- the same launches with the same
     // arguments every iteration (nu is read on the device).
     auto enqueue_cg = [&](cudaStream_t s) -> int {
-        MPI_TRY(op.apply_normal(x, q, scal + kScalNu, pq_part, s));
-        MPI_TRY(cg_init_launch(N, b0, x, q, scal + kScalNu, r, p, rr_part[0], done, s));
+        if (from_data) {
+            MPI_TRY(op.residual(x, r, s));
+            k_cg_start<<<nblk, kVecThreads, 0, s>>>(N, r, p, rr_part[0], done);
+            MPI_CHECK_LAUNCH();
+        } else {
+            MPI_TRY(op.apply_normal(x, q, scal + kScalNu, pq_part, s));
+            MPI_TRY(cg_init_launch(N, b0, x, q, scal + kScalNu, r, p, rr_part[0], done, s));
+        }
         for (int i = 0; i < o.n_cg; ++i) {
             double *const rr_in = rr_part[i & 1], *const rr_out = rr_part[(i + 1) & 1];
             const bool dir = op.takes_direction();
@@ -340,12 +368,6 @@ struct PnPOp2D final : PnPOperator<R> {
     }
     int rhs(const R *data, double *b0, cudaStream_t st) override
     {
-        if constexpr (sizeof(R) == 4)
-            if (gridded) {
-                MPI_TRY(field_load(fld, data, st));
-                MPI_TRY(field_adjoint<double>(fld, b0, nullptr, nullptr, nullptr, st));
-                return ar ? reduce(b0, st) : MPI_OK;
-            }
         if (op == MPI_OP_FORWARD) {
             MPI_TRY((launch_adjoint<R, double>(m, g, T, geo, as, data, adj_part, b0, nullptr, nullptr,
                                                nullptr, st)));
@@ -357,7 +379,7 @@ struct PnPOp2D final : PnPOperator<R> {
                      cudaStream_t st) override
     {
         if (gridded) {
-            MPI_TRY(field_forward_ordered<double>(fld, v, st));
+            MPI_TRY(field_forward_ordered<double>(fld, v, false, st));
             if (!ar) return field_adjoint<double>(fld, q, v, nu_dev, pq_part, st);
             MPI_TRY(field_adjoint<double>(fld, red, nullptr, nullptr, nullptr, st));
             MPI_TRY(reduce(red, st));
@@ -394,6 +416,14 @@ struct PnPOp2D final : PnPOperator<R> {
     {
         MPI_TRY(conv_twice(dir.p, &dir, st));
         return axpy_dot_launch<R>(N, tmp2, dir.p, nu_dev, q, pq_part, st);
+    }
+    // (the gridded plan holds the data in its samples' order)
+    bool residual_from_data() const override { return gridded; }
+    int residual(const double *v, double *r, cudaStream_t st) override
+    {
+        MPI_TRY(field_forward_ordered<double>(fld, v, true, st));
+        MPI_TRY(field_adjoint<double>(fld, r, nullptr, nullptr, nullptr, st));
+        return ar ? reduce(r, st) : MPI_OK;
     }
     int n_pq() const override
     {
@@ -439,6 +469,7 @@ static int pnp_impl(const ModelH &m, const GridH &g, const mpi_traj *tr, const v
                 const float *r = static_cast<const float *>(tr->r), *v = static_cast<const float *>(tr->v);
                 MPI_TRY(field_prepare(S.fld, nullptr, r, v, st));
                 MPI_TRY(field_order(S.fld, r, v, nullptr, st));
+                MPI_TRY(field_load(S.fld, static_cast<const float *>(data), st));
                 return pnp_run<R>(S, S.N, data, o, rho_out, info, st);
             }
             (void)cudaGetLastError();  // the pair sums need less

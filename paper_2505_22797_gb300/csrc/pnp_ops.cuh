@@ -64,7 +64,14 @@ struct PnPOperator {
     virtual int apply_normal(const double *v, double *q, const double *nu_dev, double *pq_part,
                              cudaStream_t st) = 0;
     virtual int n_pq() const = 0;
-    // The same after the pending update of p, for operators whose first
+    // r = O^T (data - O v), the residual of the normal equations from x0 = v,
+    // for operators that form it this way (they hold the data; rhs is not
+    // called).  In exact arithmetic it is b0 + nu v - (O^T O + nu I) v; here the
+    // rounding of O v meets O^T before it reaches the residual, instead of
+    // that of O^T O v standing beside it in full.
+    virtual bool residual_from_data() const { return false; }
+    virtual int residual(const double *, double *, cudaStream_t) { return MPI_ERR_INVALID; }
+    // apply_normal after the pending update of p, for operators whose first
     // launch can form it.
     virtual bool takes_direction() const { return false; }
     virtual int apply_direction(const CgDirection &, double *, const double *, double *, cudaStream_t)
