@@ -1838,33 +1838,46 @@ int field_adjoint(const FieldPlan &plan, OUT *out, const double *cg_p, const dou
     return MPI_OK;
 }
 
-bool field_worth(const GridH &g, int64_t T) { return double(T) * g.nx * g.ny >= 3e7; }
+bool field_worth(const GridH &g, int64_t T) { return double(T) * g.nx * g.ny >= 1.5e7; }
 
-// Both sides in microseconds, fitted to GB300 timings.  Direct sums: 25 and
-// 2.3e6 pairs/us (1.05e6 with a general G, whose pairs are all checked).
-// Gridded, per 768 x 768 nodes and per sample: forward 25 + 55 + 0.00019,
-// A^T with the ordering of the samples 40 + 75 + 0.0003.
+// What the direct sums and the gridded operators take, in microseconds,
+// fitted to GB300 timings of both at 24 x 24 to 256 x 256 voxels and 8e6 to
+// 5e8 pairs (fields of view of 24 and 48 mm, three trajectories, fields along
+// the axes and turned; 306 cases).  Choosing by the fit loses 1 % on average
+// against the faster of the two, at most half of a call's time near the line;
+// a fixed rate for the direct sums lost 13 %.
+//
+// A pair of the direct A^T costs by its regime, decided per sample for a
+// warp's box of 16 x 16 voxels: the share of the samples within 12 z units of
+// a box follows from the grid.
+static double near_share(const FieldDev &d)
+{
+    const double px = std::hypot(d.cx[0], d.cx[1]), py = std::hypot(d.cy[0], d.cy[1]);
+    return std::min(1.0, (16.0 + 24.0 / px) / d.x.n) * std::min(1.0, (16.0 + 24.0 / py) / d.y.n);
+}
+static double nodes_768(const FieldDev &d) { return double(d.x.P) * d.y.P / (768.0 * 768.0); }
+
 bool field_route(const FieldPlan &plan)
 {
     const FieldDev &d = plan.d;
-    const double T = double(d.T), pairs = T * d.x.n * d.y.n;
-    const double nodes = double(d.x.P) * d.y.P / (768.0 * 768.0);
-    const double direct = 25.0 + pairs / (d.diag ? 2.3e6 : 1.05e6);
-    const double field = plan.adjoint ? 40.0 + 75.0 * nodes + 0.0003 * T : 25.0 + 55.0 * nodes + 0.00019 * T;
-    return field < direct;
+    const double T = double(d.T), pairs = 1e-6 * T * d.x.n * d.y.n, nodes = nodes_768(d);
+    if (plan.adjoint)
+        return 56.0 + 35.0 * nodes + 278e-6 * T < 40.0 + pairs * ((d.diag ? 0.40 : 0.64) + 2.1 * near_share(d));
+    return 53.0 + 29.0 * nodes + 44e-6 * T < 40.0 + pairs * (d.diag ? 0.51 : 1.07);
 }
 
-// A solve prepares once (60 + 60 and 0.0004 per sample) and applies A^T A:
-// 15 + 75 and 0.0005 per sample against twice 2.4e6 pairs/us and, unless the
-// launches of many frames are shared, 30.
+// A solve prepares once and applies A^T A products times in a replayed graph
+// (shared: direct sums whose launches serve many frames).  15 products at
+// 128 x 128 / 4000 samples: direct 2.63 ms, gridded 1.66 ms; 48 x 48 / 16 000:
+// 2.48 and 1.75 ms; 64 x 64 / 8000: 1.64 and 1.62 ms; 64 x 64 / 4000: 1.16 and
+// 1.60 ms.
 static bool field_route_solve(const FieldPlan &plan, int64_t products, bool shared)
 {
     const FieldDev &d = plan.d;
-    const double T = double(d.T), pairs = T * d.x.n * d.y.n;
-    const double nodes = double(d.x.P) * d.y.P / (768.0 * 768.0);
-    const double direct = (shared ? 0.0 : 30.0) + 2.0 * pairs / (d.diag ? 2.4e6 : 1.05e6);
-    const double field = 15.0 + 75.0 * nodes + 0.0005 * T;
-    return double(products) * (direct - field) > 60.0 + 60.0 * nodes + 0.0004 * T;
+    const double T = double(d.T), pairs = 1e-6 * T * d.x.n * d.y.n, nodes = nodes_768(d);
+    const double direct = (shared ? 0.0 : 55.0) + pairs * ((d.diag ? 0.77 : 1.7) + 3.0 * near_share(d));
+    const double field = 82.0 + 8.0 * nodes * nodes + 100e-6 * T;
+    return double(products) * (direct - field) > 60.0 + 60.0 * nodes + 400e-6 * T;
 }
 
 bool field_solve_plan(const ModelH &m, const GridH &g, int64_t T, int n_iter, int n_cg, bool shared, FieldPlan &plan)
