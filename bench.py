@@ -5,7 +5,9 @@ One step = one full ZeroShot-PnP reconstruction (Algorithm 1) of the
 of 20 CG steps, 5x5 Gaussian denoiser, 5th-percentile trimming) with the
 forward operator A in FP32 and FP64 CG vectors/inner products.  Every step
 applies A and A^T 4201 times; the metric counts (voxel, sample) pairs per
-second over the whole reconstruction.
+second over the whole reconstruction (the FP32 operators reach this size as
+transforms on a grid, so the pairs are those that the sums have, not
+evaluations).
 
 Beside the headline the line carries, each measured (not extrapolated): the
 accuracy of every result (FP32 against the FP64 GPU form, the FP64 form's
@@ -1201,6 +1203,19 @@ def run_ours(args):
                 "bases": kd["bases"], "pipe_rates_per_sm_clk": rates, "kernels": kern,
                 "share_of_step": (fms + ams) / prof_ms if prof_ms else None,
                 "profiled_step_ms": prof_ms}
+
+    if kd["achieved"] and kd["achieved"] > tw["peak"]:
+        # More pairs per second than the pipes could evaluate: the solve ran on
+        # the gridded operators, which evaluate none.  An application is a
+        # chain of short L2-resident launches; its bytes are each input read
+        # once and each output written once.
+        gbytes = (4.0 * N + (16.0 + 4.0 * len(m["p"])) * T) / 1e9
+        hbm = peaks.get("hbm_gbs") or 6800.0
+        rate = gbytes / (kd["avg_launch_ms"] * 1e-3)
+        roofline.update({"bound": "latency", "achieved": rate, "peak": hbm, "unit": "GB/s", "frac": rate / hbm,
+                         "traffic": None, "kernel": "gridded A" if dom == "k_forward" else "gridded A^T",
+                         "peak_basis": "measured copy rate; algorithmic bytes of one application",
+                         "pair_equivalent": {"achieved": kd["achieved"], "pair_bound": tw["peak"], "unit": "Gpair/s"}})
 
     # --- further legs (rank 0, N = 1) -----------------------------------------
     extra = {}
