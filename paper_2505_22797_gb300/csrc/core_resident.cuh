@@ -13,7 +13,7 @@
 //
 // Measured on GB300: 48 x 48 x 24 / 65 536 samples, 20 steps with the setup
 // 1.02 ms (by launches 1.33 ms); 100 x 100 / 1632 samples to the tolerance,
-// 65 steps, 34 us a step (by launches 48 us).  Four (2-D) or five (3-D)
+// 65 to 150 steps, 19 us a step (by launches 48 us).  Four (2-D) or five (3-D)
 // barriers and the L2 latency of what crosses them bound a step.
 #pragma once
 

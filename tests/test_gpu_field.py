@@ -103,8 +103,7 @@ def test_field_unaligned_trajectory(orc):
 
 
 def test_field_solve_single_batch_and_sharded(orc):
-    """Algorithm 1 on the gridded operators (64 x 60, 40 001 samples: the
-    smallest frames that take them) against the oracle, held to the FP32 bar
+    """Algorithm 1 on the gridded operators (64 x 60, 40 001 samples) against the oracle, held to the FP32 bar
     of the well-posed solves; the matched batch (beside a frame that keeps the
     pair sums) bit for bit, and the sharded solve."""
     big, small = _case(64, 60, 40001, 11), _case(20, 24, 900, 12)
