@@ -303,8 +303,10 @@ typedef int (*mpi_allreduce_fn)(double *buf, int64_t count, void *stream, void *
  * (s: [n_ch][T_p]) -- while model, grid, opts and the built-in or callback
  * denoiser are the same on every process.  A of an image gives this process's
  * samples with no exchange; A^T gives a partial image, which the library sums
- * across processes with `allreduce` (N = nx*ny values): once for A^T data and
- * once per CG step.  Every other step (CG vectors, inner products, trimming,
+ * across processes with `allreduce` (N = nx*ny values): once for A^T data and,
+ * in each of the n_iter iterations, once for the initial residual and once per
+ * CG step -- 1 + n_iter (n_cg + 1) calls on every process, whatever the length
+ * of its slice and whether it evaluates its sums pair by pair or on a grid.  Every other step (CG vectors, inner products, trimming,
  * noise estimate, denoiser) runs replicated on the identical reduced vectors,
  * so all processes finish with the same rho_out.  One process with an
  * allreduce that does nothing computes what mpi_pnp_solve computes, up to the

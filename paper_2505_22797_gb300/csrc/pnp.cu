@@ -78,6 +78,13 @@ k_cg_start(int64_t N, const double *__restrict__ r, double *__restrict__ p, doub
     }
 }
 
+// y = a - y.
+__global__ void __launch_bounds__(kVecThreads) k_minuend(int64_t N, const double *__restrict__ a, double *__restrict__ y)
+{
+    const int64_t e0 = (int64_t)blockIdx.x * kVecPerBlock, e1 = min(N, e0 + kVecPerBlock);
+    for (int64_t e = e0 + threadIdx.x; e < e1; e += kVecThreads) y[e] = a[e] - y[e];
+}
+
 // alpha = r.r / p.q;  x += alpha p;  r -= alpha q;  partial sums of the new r.r.
 // Once r.r or p.q is exactly 0 the solve has converged to round-off: the stop
 // flag is set and the remaining steps leave x, r and p untouched.  With a
@@ -273,7 +280,7 @@ int pnp_run(PnPOperator<R> &op, int64_t N, const void *data, const mpi_pnp_opts 
             k_cg_start<<<nblk, kVecThreads, 0, s>>>(N, r, p, rr_part[0], done);
             MPI_CHECK_LAUNCH();
         } else {
-            MPI_TRY(op.apply_normal(x, q, scal + kScalNu, pq_part, s));
+            MPI_TRY(op.apply_start(x, q, scal + kScalNu, pq_part, s));
             MPI_TRY(cg_init_launch(N, b0, x, q, scal + kScalNu, r, p, rr_part[0], done, s));
         }
         for (int i = 0; i < o.n_cg; ++i) {
@@ -352,10 +359,15 @@ struct PnPOp2D final : PnPOperator<R> {
     mpi_denoise_fn den = nullptr;
     void *user = nullptr;
     // Sample-sharded solve: this process's samples only; partial A^T images
-    // are summed across processes by `ar` into `red` (FP64, N values).
+    // are summed across processes by `ar` into `red` (FP64, N values).  The
+    // route follows from this process's own samples (and from whether its
+    // scratch is to be had), so processes may differ in it: both routes reduce
+    // the same quantities in the same sequence, A^T data once and A^T A v for
+    // each product.
     mpi_allreduce_fn ar = nullptr;
     void *ar_user = nullptr;
     double *red = nullptr;
+    double *own = nullptr;  // gridded: A^T of this process's data
 
     int reduce(double *buf, cudaStream_t st)
     {
@@ -368,6 +380,11 @@ struct PnPOp2D final : PnPOperator<R> {
     }
     int rhs(const R *data, double *b0, cudaStream_t st) override
     {
+        if (gridded) {  // (the operand of field_adjoint is still the data)
+            MPI_TRY(field_adjoint<double>(fld, own, nullptr, nullptr, nullptr, st));
+            MPI_TRY_CUDA(cudaMemcpyAsync(b0, own, sizeof(double) * N, cudaMemcpyDeviceToDevice, st));
+            return reduce(b0, st);
+        }
         if (op == MPI_OP_FORWARD) {
             MPI_TRY((launch_adjoint<R, double>(m, g, T, geo, as, data, adj_part, b0, nullptr, nullptr,
                                                nullptr, st)));
@@ -418,12 +435,24 @@ struct PnPOp2D final : PnPOperator<R> {
         return axpy_dot_launch<R>(N, tmp2, dir.p, nu_dev, q, pq_part, st);
     }
     // (the gridded plan holds the data in its samples' order)
-    bool residual_from_data() const override { return gridded; }
+    bool residual_from_data() const override { return gridded && !ar; }
     int residual(const double *v, double *r, cudaStream_t st) override
     {
         MPI_TRY(field_forward_ordered<double>(fld, v, true, st));
-        MPI_TRY(field_adjoint<double>(fld, r, nullptr, nullptr, nullptr, st));
-        return ar ? reduce(r, st) : MPI_OK;
+        return field_adjoint<double>(fld, r, nullptr, nullptr, nullptr, st);
+    }
+    // A sharded gridded solve also forms its part of the residual through its
+    // data, and reduces it as the A^T A v that it stands for, A^T s - A^T (s -
+    // A v): taken from the A^T s that has been reduced, the rounding of A^T s
+    // and of A^T A v cancels to FP64.
+    int apply_start(const double *v, double *q, const double *nu_dev, double *pq_part, cudaStream_t st) override
+    {
+        if (!gridded) return apply_normal(v, q, nu_dev, pq_part, st);
+        MPI_TRY(residual(v, red, st));
+        k_minuend<<<vec_blocks(N), kVecThreads, 0, st>>>(N, own, red);
+        MPI_CHECK_LAUNCH();
+        MPI_TRY(reduce(red, st));
+        return axpy_dot_launch<double>(N, red, v, nu_dev, q, pq_part, st);
     }
     int n_pq() const override
     {
@@ -461,14 +490,15 @@ static int pnp_impl(const ModelH &m, const GridH &g, const mpi_traj *tr, const v
         Scratch fscr(st);
         if (o.op == MPI_OP_FORWARD && field_solve_plan(m, g, S.T, o.n_iter, o.n_cg, false, S.fld)) {
             const size_t o_keep = fscr.reserve(S.fld.keep_bytes), o_work = fscr.reserve(S.fld.work_bytes);
-            const size_t o_sum = ar ? fscr.reserve(sizeof(double) * size_t(S.N)) : 0;
+            const size_t vb = ar ? sizeof(double) * size_t(S.N) : 0;
+            const size_t o_sum = fscr.reserve(vb), o_own = fscr.reserve(vb);
             if (fscr.allocate() == MPI_OK) {
                 S.gridded = true;
-                if (ar) S.red = fscr.at<double>(o_sum);
+                if (ar) S.red = fscr.at<double>(o_sum), S.own = fscr.at<double>(o_own);
                 field_carve(S.fld, fscr.at<char>(o_keep), fscr.at<char>(o_work));
                 const float *r = static_cast<const float *>(tr->r), *v = static_cast<const float *>(tr->v);
                 MPI_TRY(field_prepare(S.fld, nullptr, r, v, st));
-                MPI_TRY(field_order(S.fld, r, v, nullptr, st));
+                MPI_TRY(field_order(S.fld, r, v, ar ? static_cast<const float *>(data) : nullptr, st));
                 MPI_TRY(field_load(S.fld, static_cast<const float *>(data), st));
                 return pnp_run<R>(S, S.N, data, o, rho_out, info, st);
             }

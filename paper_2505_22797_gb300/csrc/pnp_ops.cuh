@@ -64,6 +64,12 @@ struct PnPOperator {
     virtual int apply_normal(const double *v, double *q, const double *nu_dev, double *pq_part,
                              cudaStream_t st) = 0;
     virtual int n_pq() const = 0;
+    // The product from which a solve's initial residual b0 + nu v - q is formed:
+    // apply_normal, or what rounds less and stands for it.
+    virtual int apply_start(const double *v, double *q, const double *nu_dev, double *pq_part, cudaStream_t st)
+    {
+        return apply_normal(v, q, nu_dev, pq_part, st);
+    }
     // r = O^T (data - O v), the residual of the normal equations from x0 = v,
     // for operators that form it this way (they hold the data; rhs is not
     // called).  In exact arithmetic it is b0 + nu v - (O^T O + nu I) v; here the

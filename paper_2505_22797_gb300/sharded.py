@@ -6,8 +6,9 @@ The forward operator and its adjoint are sums over the trajectory samples
 work.  Each process (one GPU) holds its slice of r, v and s; A gives its own
 samples with no exchange, A^T a partial image that the processes sum.  The
 library's mpi_pnp_solve_sharded calls back for that sum once for A^T of the
-data and once per CG step (N = nx * ny FP64 values); everything else runs
-replicated on identical vectors.
+data and, in each iteration, once for the initial residual and once per CG
+step (N = nx * ny FP64 values; the same calls on every process, whatever the
+length of its slice); everything else runs replicated on identical vectors.
 
 This module holds the host logic around that call: the balanced sample
 partition, the all-reduce callables (torch.distributed for processes, a
