@@ -478,10 +478,8 @@ static int prepare_launch(mpi_batch_plan &P)
     auto kf = fwd_kernel(P);
     auto kfp = fwd_kernel_persistent(P);
     auto kap = adj_kernel_persistent(P);
-    if (P.fwd_smem > 48 * 1024) {
-        MPI_TRY_CUDA(cudaFuncSetAttribute(kf, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)P.fwd_smem));
-        MPI_TRY_CUDA(cudaFuncSetAttribute(kfp, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)P.fwd_smem));
-    }
+    MPI_TRY(allow_smem(kf, P.fwd_smem));
+    MPI_TRY(allow_smem(kfp, P.fwd_smem));
     P.fwd_grid_persist = (int)std::min<int64_t>(P.fwd_items, persistent_grid((const void *)kfp, kFwdThreads, P.fwd_smem));
     P.adj_grid_persist = (int)std::min<int64_t>(P.adj_items, persistent_grid((const void *)kap, kAdjThreads, 0));
     return MPI_OK;

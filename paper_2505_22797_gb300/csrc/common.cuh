@@ -38,6 +38,22 @@ const char *last_error();
 void note_launch();
 void note_launches(long long n);
 #ifdef __CUDACC__
+// Opts `kernel` in to more than the default 48 KB of dynamic shared memory.
+// The limit is state of the function on the device, not of a launch: plans of
+// other sizes and other threads share it, so every caller sets the same value,
+// the most a block can have beside the kernel's static shared memory, and none
+// lowers what another has prepared a launch for.
+template <typename K>
+inline int allow_smem(K kernel, size_t bytes)
+{
+    if (bytes <= 48 * 1024) return MPI_OK;
+    cudaFuncAttributes attr;
+    MPI_TRY_CUDA(cudaFuncGetAttributes(&attr, kernel));
+    const int most = 227 * 1024 - (int)attr.sharedSizeBytes;
+    MPI_TRY_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, std::max((int)bytes, most)));
+    return MPI_OK;
+}
+
 // Launches of one dependent chain: the next kernel's launch overlaps the end
 // of the one before (programmatic dependent launch), and every kernel of a
 // chain opens with chain_wait(), which returns once all work before it is

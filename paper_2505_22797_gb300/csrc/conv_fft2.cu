@@ -399,14 +399,6 @@ unsigned block_threads(int lg_n, int lg_c)
 template <typename C>
 constexpr int cols_lg_cb() { return sizeof(C) == 8 ? 2 : 1; }  // one 32-byte sector per row
 
-template <typename K>
-int allow_smem(K kernel, size_t bytes)
-{
-    if (bytes > 48 * 1024)
-        MPI_TRY_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
-    return MPI_OK;
-}
-
 }  // namespace
 
 template <typename C, typename IN>

@@ -231,8 +231,7 @@ static int fft_run_t(const FftPlan &p, C *a, C *b, int n_ch, int64_t dist, const
                (rpb * 2 * most <= kFftThreads || (n_ch + rpb - 1) / rpb > wave))
             rpb *= 2;
         const size_t smem_blk = smem * size_t(rpb);
-        if (smem_blk > 48 * 1024)  // opt in above the default limit (set on the current device)
-            MPI_TRY_CUDA(cudaFuncSetAttribute(k_fft_smem<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_blk));
+        MPI_TRY(allow_smem(k_fft_smem<C>, smem_blk));
         const unsigned blocks = (unsigned)((n_ch + rpb - 1) / rpb);
         k_fft_smem<C><<<blocks, kFftThreads, smem_blk, st>>>(a, (int)p.n, rl, W, dist, n_ch, rpb);
         MPI_CHECK_LAUNCH();

@@ -1597,13 +1597,6 @@ size_t image_smem(const FieldDev &d) { return 2 * sizeof(float2) * smem_fft_elem
 int order_warps(const FieldDev &d) { return std::max(1, std::min<int>(4, 48 * 1024 / (4 * (d.tx * d.ty + 1)))); }
 size_t order_smem(const FieldDev &d) { return sizeof(int) * size_t(d.tx * d.ty + 1) * order_warps(d); }
 
-template <typename K> int allow_smem(K k, size_t bytes)
-{
-    if (bytes > 48 * 1024)
-        MPI_TRY_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
-    return MPI_OK;
-}
-
 // Shared memory above 48 KB is granted per kernel; asked for outside any
 // stream capture (field_prepare), so the launches only launch.
 int allow_all(const FieldDev &d, bool forward, bool adjoint)

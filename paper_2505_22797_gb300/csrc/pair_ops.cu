@@ -438,14 +438,6 @@ static PairFrame<R> base_frame(const ModelH &m, const GridH &g, int64_t T, const
     return f;
 }
 
-template <typename Kern>
-static int set_smem(Kern k, size_t bytes)
-{
-    if (bytes > 48 * 1024)
-        MPI_TRY_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
-    return MPI_OK;
-}
-
 template <typename R, typename CIN, typename OUT>
 int launch_forward(const ModelH &m, const GridH &g, int64_t T, const Geometry<R> &geo,
                    const FwdSplit &sp, const CIN *c, R *part, OUT *s_out, cudaStream_t st)
@@ -466,10 +458,10 @@ int launch_forward(const ModelH &m, const GridH &g, int64_t T, const Geometry<R>
     {
         ProfScope prof(kProfForward, st);
         if (is_diag(m)) {
-            MPI_TRY(set_smem(k_forward<R, CIN, 1, 1>, smem));
+            MPI_TRY(allow_smem(k_forward<R, CIN, 1, 1>, smem));
             k_forward<R, CIN, 1, 1><<<(unsigned)items, kFwdThreads, smem, st>>>(B);
         } else {
-            MPI_TRY(set_smem(k_forward<R, CIN, 0, 1>, smem));
+            MPI_TRY(allow_smem(k_forward<R, CIN, 0, 1>, smem));
             k_forward<R, CIN, 0, 1><<<(unsigned)items, kFwdThreads, smem, st>>>(B);
         }
         MPI_CHECK_LAUNCH();
