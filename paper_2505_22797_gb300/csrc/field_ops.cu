@@ -1294,7 +1294,10 @@ __global__ void __launch_bounds__(kSpreadThreads) k_field_spread(const __grid_co
 }
 
 // Half spectra of node rows 2b, 2b + 1: a node is the sum of the patches of
-// the up to four tiles that reach it, units in order.
+// the up to four tiles that reach it, units in order, in pairs of floats (a
+// tile where the trajectory dwells has thousands of units, whose plain FP32
+// sum would leave 1e-6; four units' loads are in flight).
+constexpr int kUnitsAtOnce = 4;
 __global__ void __launch_bounds__(512) k_field_rows_fwd(const __grid_constant__ FieldDev d)
 {
     chain_wait();
@@ -1307,7 +1310,7 @@ __global__ void __launch_bounds__(512) k_field_rows_fwd(const __grid_constant__ 
     const int ty1 = min(i0 / kTile, d.ty - 1);
     const int ty0 = max(0, (i0 - kPatch + kTile) / kTile);
     for (int i = threadIdx.x; i < P; i += blockDim.x) {
-        float g0[3] = {0.0f, 0.0f, 0.0f}, g1[3] = {0.0f, 0.0f, 0.0f};
+        F2Sum g[2][3] = {};
         if (i < wx) {
             const int tx1 = min(i / kTile, d.tx - 1), tx0 = max(0, (i - kPatch + kTile) / kTile);
             for (int ty = ty0; ty <= ty1; ++ty) {
@@ -1315,15 +1318,30 @@ __global__ void __launch_bounds__(512) k_field_rows_fwd(const __grid_constant__ 
                 for (int tx = tx0; tx <= tx1; ++tx) {
                     const int u0 = d.b.uoff[ty * d.tx + tx], u1 = d.b.uoff[ty * d.tx + tx + 1];
                     const float *p = d.b.upart + int64_t(u0) * 3 * kPatchSize + pr * kPatch + i - tx * kTile;
-                    const int next = pr + 1 < kPatch ? kPatch : 0;
-                    const float on = next ? 1.0f : 0.0f;
-#pragma unroll 2
-                    for (int u = u0; u < u1; ++u, p += 3 * kPatchSize) {
+                    const bool two = pr + 1 < kPatch;
+                    auto load = [&](const float *e, float (&q)[2][3]) {
 #pragma unroll
                         for (int m = 0; m < 3; ++m) {
-                            g0[m] += p[m * kPatchSize];
-                            g1[m] = fmaf(on, p[m * kPatchSize + next], g1[m]);
+                            q[0][m] = e[m * kPatchSize];
+                            q[1][m] = two ? e[m * kPatchSize + kPatch] : 0.0f;
                         }
+                    };
+                    auto add = [&](const float (&q)[2][3]) {
+#pragma unroll
+                        for (int m = 0; m < 3; ++m) g[0][m].add(q[0][m]), g[1][m].add(q[1][m]);
+                    };
+                    int u = u0;
+                    for (; u + kUnitsAtOnce <= u1; u += kUnitsAtOnce, p += kUnitsAtOnce * 3 * kPatchSize) {
+                        float q[kUnitsAtOnce][2][3];
+#pragma unroll
+                        for (int k = 0; k < kUnitsAtOnce; ++k) load(p + k * 3 * kPatchSize, q[k]);
+#pragma unroll
+                        for (int k = 0; k < kUnitsAtOnce; ++k) add(q[k]);
+                    }
+                    for (; u < u1; ++u, p += 3 * kPatchSize) {
+                        float q[2][3];
+                        load(p, q);
+                        add(q);
                     }
                 }
             }
@@ -1331,9 +1349,9 @@ __global__ void __launch_bounds__(512) k_field_rows_fwd(const __grid_constant__ 
         int l = l0 + i;
         l -= l >= P ? P : 0;
         V2<float> *o = a + smem_fft_pad(l) * 3;
-        o[0] = V2<float>{g0[0], g0[1]};
-        o[1] = V2<float>{g1[0], g1[1]};
-        o[2] = V2<float>{g0[2], g1[2]};
+        o[0] = V2<float>{g[0][0].hi + g[0][0].lo, g[0][1].hi + g[0][1].lo};
+        o[1] = V2<float>{g[1][0].hi + g[1][0].lo, g[1][1].hi + g[1][1].lo};
+        o[2] = V2<float>{g[0][2].hi + g[0][2].lo, g[1][2].hi + g[1][2].lo};
     }
     __shared__ V2<float> s_low[kLowY][3];
     __syncthreads();
