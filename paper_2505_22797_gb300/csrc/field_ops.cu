@@ -28,14 +28,17 @@
 // the interpolation's outer sum and the product with W are carried in pairs.
 //
 // Samples beyond the node window (more than 12 z units outside the voxels)
-// are summed directly: there every pair of a diagonal G is in the asymptotic
-// range.
+// are summed directly by blocks of their own beside the interpolation and the
+// spreading, in the pair kernels' form: there every pair of a diagonal G is in
+// the asymptotic range.
 #include <algorithm>
+#include <climits>
 #include <cmath>
 
 #include "field_ops.cuh"
 #include "grid_common.cuh"
 #include "langevin.cuh"
+#include "pair_kernels.cuh"
 
 namespace mpi {
 
@@ -61,9 +64,17 @@ constexpr int kPatchPitch = 28;
 constexpr int kPatchSize = kPatch * kPatch;
 constexpr int kFieldUnit = 224;                 // samples per spreading unit
 constexpr int kSpreadThreads = 384;             // warp = (half of the unit, entry of K, row parity)
+constexpr int kSpreadPerSm = 3;                 // blocks per SM (registers and shared memory)
 constexpr int kRunMin = 128, kRunMax = 512;     // samples per run at least, runs at most
+constexpr int kInterpThreads = 256;
+// Outside sums of A^T: a thread takes kOutRows voxels of one column.
 constexpr int kOutThreads = kSpreadThreads;
-constexpr int kOutVox = 4;                      // voxels per thread of the outside sums
+constexpr int kOutRows = 4;
+// Outside sums of A: kFwdS samples per thread.
+constexpr int kOutStage = kFieldMaxN / 2;       // voxels at a time in shared memory, a row at least (n < Q/2)
+constexpr int kOutFold = 128;                   // columns summed plainly before a compensated add
+constexpr int kOutPerSm = 768;                  // their threads per SM (four blocks at most)
+constexpr int kOutRounds = 3;                   // units per such block at most, if a unit is not all rows
 
 // Kaiser-Bessel window I0(beta sqrt(1 - (x/4)^2))/I0(beta) at x = f + 3 - a
 // for the stencil's points a = 0..3 as polynomials in t = f - 1/2
@@ -103,19 +114,6 @@ __device__ __forceinline__ F2Sum f2_warp(F2Sum v)
     for (int o = 16; o > 0; o >>= 1) v.add(f2_shfl_xor(v, o));
     return v;
 }
-// Sum over the block's threads, valid in thread 0; sh: 32 F2Sum.
-__device__ __forceinline__ F2Sum f2_block(F2Sum v, F2Sum *sh)
-{
-    v = f2_warp(v);
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
-    __syncthreads();
-    F2Sum t{};
-    if (threadIdx.x == 0)
-        for (int w = 0; w < int(blockDim.x >> 5); ++w) t.add(sh[w]);
-    __syncthreads();
-    return t;
-}
-
 struct SampleRec {
     bool in;
     float fx, fy;   // inside: fractions; outside: beta G r
@@ -188,6 +186,12 @@ __device__ double window_inv(int k, int P)
     return s * kKbI0 / (kWin * 0.5 * (exp(s) - exp(-s)));
 }
 
+// Outside samples (unordered plans) and, per out_samples of them, the row runs done.
+__host__ __device__ __forceinline__ int out_counters(const FieldDev &d)
+{
+    return 1 + int((d.T + d.out_samples - 1) / d.out_samples);
+}
+
 // Entry t of the tables laid end to end.
 __device__ void fill_table(const FieldDev &d, int t)
 {
@@ -208,11 +212,16 @@ __device__ void fill_table(const FieldDev &d, int t)
         return;
     }
     t -= d.x.n;
-    if (t < d.y.n) d.b.yrow[t] = V2<float>{float(d.Y0[0] + t * d.cy[0]), float(d.Y0[1] + t * d.cy[1])};
+    if (t < d.y.n) {
+        d.b.yrow[t] = V2<float>{float(d.Y0[0] + t * d.cy[0]), float(d.Y0[1] + t * d.cy[1])};
+        return;
+    }
+    t -= d.y.n;
+    if (d.b.ocount && t < out_counters(d)) d.b.ocount[t] = 0;
 }
 int table_entries(const FieldDev &d)
 {
-    return d.x.P + d.y.P + d.x.Q + d.y.Q + d.x.J + 1 + d.y.J + 1 + d.x.n + d.y.n;
+    return d.x.P + d.y.P + d.x.Q + d.y.Q + d.x.J + 1 + d.y.J + 1 + d.x.n + d.y.n + (d.b.ocount ? out_counters(d) : 0);
 }
 
 // --- ordering the samples by tile ----------------------------------------------
@@ -732,9 +741,41 @@ __global__ void __launch_bounds__(128) k_field_image(const __grid_constant__ Fie
     image_rows(d, 2 * blockIdx.x, c, smem_raw);
 }
 
+// Appends the outside samples among kListPer per thread to olist, in any order
+// (a sample's sum does not depend on its neighbours in the list).
+constexpr int kListPer = 4;
+__device__ void list_outside(const FieldDev &d, int64_t block, const float *__restrict__ r)
+{
+    const int lane = threadIdx.x & 31;
+    const int64_t t0 = block * kListPer * blockDim.x + threadIdx.x;
+    float x[kListPer], y[kListPer];
+#pragma unroll
+    for (int u = 0; u < kListPer; ++u) {
+        const int64_t t = min(t0 + int64_t(u) * blockDim.x, d.T - 1);
+        x[u] = r[2 * t];
+        y[u] = r[2 * t + 1];
+    }
+#pragma unroll
+    for (int u = 0; u < kListPer; ++u) {
+        const int64_t t = t0 + int64_t(u) * blockDim.x;
+        int k;
+        float f;
+        const bool bx = node_coord(d.x, x[u], k, f), by = node_coord(d.y, y[u], k, f);
+        const bool out = t < d.T && !(bx && by);
+        const unsigned mask = __ballot_sync(0xffffffffu, out);
+        if (mask == 0) continue;
+        int base = 0;
+        if (lane == 0) base = atomicAdd(d.b.ocount, __popc(mask));
+        base = __shfl_sync(0xffffffffu, base, 0);
+        if (out) d.b.olist[base + __popc(mask & ((1u << lane) - 1u))] = int(t);
+    }
+}
+
 // The sampled kernel's rows and, behind them, what else needs only the
-// tables: the image's rows (c) or the tiles' prefix sums.
-__global__ void __launch_bounds__(512) k_field_rows(const __grid_constant__ FieldDev d, int n_kernel, const float *c)
+// tables: the image's rows (c) and the list of the outside samples, or the
+// tiles' prefix sums.
+__global__ void __launch_bounds__(512) k_field_rows(const __grid_constant__ FieldDev d, int n_kernel, const float *c,
+                                                    const float *r)
 {
     chain_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -742,7 +783,9 @@ __global__ void __launch_bounds__(512) k_field_rows(const __grid_constant__ Fiel
     if (b < n_kernel) {
         kernel_rows(d, 2 * b, smem_raw);
     } else if (c) {
-        image_rows(d, 2 * (b - n_kernel), c, smem_raw);
+        const int k = b - n_kernel, n_image = (d.y.n + 1) / 2;
+        if (k < n_image) image_rows(d, 2 * k, c, smem_raw);
+        else list_outside(d, k - n_image, r);
     } else {
         const int tile = (b - n_kernel) * int(blockDim.x >> 5) + int(threadIdx.x >> 5);
         if (tile <= d.tx * d.ty) scan_tile(d, tile);
@@ -768,15 +811,213 @@ __device__ __forceinline__ int fast_mod(int k, int n, unsigned mag, int lift)
     return int(u - __umulhi(u, mag) * unsigned(n));
 }
 
+enum { kInterpForward = 0, kInterpOrdered = 1 };
+
+struct InterpArgs {
+    const float *r, *v;   // unordered trajectory
+    float *s;             // [n_ch][T]
+    bool residual;        // ordered: the data minus A c
+};
+
+// One sample's outputs from its channels' sums o (pairs): s, or in an ordered
+// plan the operand of A^T (residual: of the data minus the sums).
+template <int MODE>
+__device__ __forceinline__ void finish_sample(const FieldDev &d, const InterpArgs &A, int64_t t, const df (&o)[2],
+                                              bool inside, float Wx, float Wy)
+{
+    if constexpr (MODE == kInterpForward) {
+#pragma unroll
+        for (int k = 0; k < 2; ++k)
+            if (k < d.n_ch) A.s[int64_t(k) * d.T + t] = o[k].x + o[k].y;
+    } else {
+        const float2 data = A.residual ? d.b.sd[t] : make_float2(0.0f, 0.0f);
+        float ux = 0.0f, uy = 0.0f;
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            if (k >= d.n_ch) break;
+            const float sk = A.residual ? ((k ? data.y : data.x) - o[k].x) - o[k].y : o[k].x + o[k].y;
+            ux += sk * d.p[2 * k];
+            uy += sk * d.p[2 * k + 1];
+        }
+        d.b.q4[t] = inside ? make_float4(ux * Wx, fmaf(ux, Wy, uy * Wx), uy * Wy, 0.0f) : make_float4(ux, uy, 0.0f, 0.0f);
+    }
+}
+
+// Columns [ib, ie) of one staged row for a general G: sa += c f1, (vx, vy) +=
+// c f2 (y.W) y.  FAR: every pair is in the asymptotic range.
+template <bool FAR>
+__device__ __forceinline__ void outside_line(int ib, int ie, const V2<float> *__restrict__ xcol, const V2<float> *xc,
+                                             const float (&ox)[kFwdS], const float (&oy)[kFwdS], const float (&Wx)[kFwdS],
+                                             const float (&Wy)[kFwdS], float (&sa)[kFwdS], float (&vx)[kFwdS], float (&vy)[kFwdS])
+{
+#pragma unroll(FAR ? 4 : 2)
+    for (int i = ib; i < ie; ++i) {
+        const V2<float> x = xcol[i];
+        const float c = xc[i].y;
+#pragma unroll
+        for (int s = 0; s < kFwdS; ++s) {
+            const float yx = x.x + ox[s], yy = x.y + oy[s], u = fmx(yx, yx, yy * yy);
+            float f1, f2;
+            if constexpr (FAR) lang_vfar<float, false>(u, f1, f2);
+            else lang_checked<float, false>(u, f1, f2);
+            sa[s] = fmx(c, f1, sa[s]);
+            const float f = c * f2 * fmx(yx, Wx[s], yy * Wy[s]);
+            vx[s] = fmx(f, yx, vx[s]);
+            vy[s] = fmx(f, yy, vy[s]);
+        }
+    }
+}
+
+// Sums O = sum_x c_x (f1 W + f2 (y.W) y) of the n_out outside samples, by the
+// first out_blocks blocks of a launch: a unit is out_samples samples and a run
+// of rows, a block takes every out_blocks-th; a sample's runs are added, in
+// their order, by the block that ends the last of them.  Bound by the FP32 pipe
+// as the pair sums, whose inner loop it is.  A at 128 x 128 / 65 536 samples, 50
+// and 94 % of them outside: 0.39 and 0.55 ms (pair sums of all samples 0.48 ms;
+// a block summing its samples one after another, as here before, 2.9 ms: bursts
+// of outside samples lie in few blocks); 512 x 512, 84 %: 7.2 ms (6.8, 37.6).
+template <int MODE, typename CIN>
+__device__ __forceinline__ void outside_units(const FieldDev &d, const InterpArgs &A, const CIN *__restrict__ cin,
+                                              int n_out, V2<float> *s_xc, int *s_last)
+{
+    const int first = int(d.T) - n_out;  // (of the ordered samples)
+    const int per = kFwdS * blockDim.x;  // out_samples
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int nx = d.x.n, ny = d.y.n, rs = kOutStage / nx;
+    const int n_grp = (n_out + per - 1) / per;
+    // rows per unit: of the lengths that give 1, 2, .. units per block the one
+    // that ends first (each unit costs about a row more than its rows)
+    int len = ny, best = INT_MAX;
+    for (int q = 1; q <= kOutRounds; ++q) {
+        const int want = min(ny, max(1, q * d.out_blocks / n_grp)), l = (ny + want - 1) / want;
+        const int units = n_grp * ((ny + l - 1) / l), cost = (units + d.out_blocks - 1) / d.out_blocks * (l + 1);
+        if (cost < best) best = cost, len = l;
+    }
+    const int runs = (ny + len - 1) / len;
+#pragma unroll 1
+    for (int u = blockIdx.x; u < n_grp * runs; u += d.out_blocks) {
+        const int g = u / runs, run = u % runs;
+        const int j0 = run * len, j1 = min(ny, j0 + len);
+        const int k0 = g * per + warp * (32 * kFwdS) + lane;  // the thread's samples: k0 + 32 s
+        const bool any = k0 - lane < n_out;                            // of the warp
+        float Rx[kFwdS], Ry[kFwdS], Wx[kFwdS], Wy[kFwdS];
+        float Sa[kFwdS], Vx[kFwdS], Vy[kFwdS], cSa[kFwdS], cVx[kFwdS], cVy[kFwdS];
+#pragma unroll
+        for (int s = 0; s < kFwdS; ++s) {
+            const int k = min(k0 + 32 * s, n_out - 1);
+            if constexpr (MODE == kInterpOrdered) {
+                const float4 rc = d.b.rec[first + k], w = d.b.wv[first + k];
+                Rx[s] = rc.x, Ry[s] = rc.y, Wx[s] = w.x, Wy[s] = w.y;
+            } else {
+                const SampleRec q = make_sample(d, A.r, A.v, d.b.olist[k]);
+                Rx[s] = q.fx, Ry[s] = q.fy, Wx[s] = q.Wx.x, Wy[s] = q.Wy.x;
+            }
+            Sa[s] = Vx[s] = Vy[s] = cSa[s] = cVx[s] = cVy[s] = 0.0f;
+        }
+#pragma unroll 1
+        for (int j = j0; j < j1; j += rs) {
+            const int nr = min(rs, j1 - j);
+            __syncthreads();
+            for (int e = threadIdx.x; e < nr * nx; e += blockDim.x)
+                s_xc[e] = V2<float>{d.b.xcol[e % nx].x, float(cin[int64_t(j) * nx + e])};
+            __syncthreads();
+            if (!any) continue;
+#pragma unroll 1
+            for (int r = 0; r < nr; ++r) {
+                const V2<float> yr = d.b.yrow[j + r];
+                const V2<float> *xc = s_xc + r * nx;
+                float ox[kFwdS], oy[kFwdS], yy2[kFwdS], yyW[kFwdS];
+#pragma unroll
+                for (int s = 0; s < kFwdS; ++s) {
+                    ox[s] = yr.x - Rx[s];
+                    oy[s] = yr.y - Ry[s];
+                    yy2[s] = oy[s] * oy[s];
+                    yyW[s] = oy[s] * Wy[s];
+                }
+#pragma unroll 1
+                for (int ib = 0; ib < nx; ib += kOutFold) {
+                    const int ie = min(nx, ib + kOutFold);
+                    float sa[kFwdS], vx[kFwdS], fy[kFwdS];
+#pragma unroll
+                    for (int s = 0; s < kFwdS; ++s) sa[s] = vx[s] = fy[s] = 0.0f;
+                    if (d.diag) {
+                        fwd_row_vfar<float>(ib, ie, xc, Rx, yy2, Wx, yyW, sa, vx, fy);
+#pragma unroll
+                        for (int s = 0; s < kFwdS; ++s) fy[s] *= oy[s];
+                    } else {
+                        // the columns' positions lie on a line: the closest
+                        // point of its segment decides the form (for the
+                        // warp, so only where its samples are always the
+                        // same ones: not in the unordered list)
+                        const V2<float> b0 = d.b.xcol[ib], b1 = d.b.xcol[ie - 1];
+                        const float ex = b1.x - b0.x, ey = b1.y - b0.y, ee = fmx(ex, ex, ey * ey);
+                        bool far = true;
+#pragma unroll
+                        for (int s = 0; s < kFwdS; ++s) {
+                            const float ax = b0.x + ox[s], ay = b0.y + oy[s];
+                            const float w = ee > 0.0f ? __saturatef(-fmx(ax, ex, ay * ey) / ee) : 0.0f;
+                            const float px = fmx(w, ex, ax), py = fmx(w, ey, ay);
+                            far = far && fmx(px, px, py * py) >= 1.02f * vfar_threshold<float, false>();
+                        }
+                        if (MODE == kInterpOrdered && __all_sync(0xffffffffu, far))
+                            outside_line<true>(ib, ie, d.b.xcol, xc, ox, oy, Wx, Wy, sa, vx, fy);
+                        else
+                            outside_line<false>(ib, ie, d.b.xcol, xc, ox, oy, Wx, Wy, sa, vx, fy);
+                    }
+#pragma unroll
+                    for (int s = 0; s < kFwdS; ++s) {
+                        kahan_add(Sa[s], cSa[s], sa[s]);
+                        kahan_add(Vx[s], cVx[s], vx[s]);
+                        kahan_add(Vy[s], cVy[s], fy[s]);
+                    }
+                }
+            }
+        }
+#pragma unroll
+        for (int s = 0; s < kFwdS; ++s) {
+            const int k = k0 + 32 * s;
+            if (k >= n_out) continue;
+            const float Ox = fmx(Sa[s], Wx[s], Vx[s]), Oy = fmx(Sa[s], Wy[s], Vy[s]);
+            df o[2];
+#pragma unroll
+            for (int c = 0; c < 2; ++c) o[c] = make_float2(fmx(d.p[2 * c], Ox, d.p[2 * c + 1] * Oy), 0.0f);
+            if (runs > 1) {
+#pragma unroll
+                for (int c = 0; c < 2; ++c)
+                    if (c < d.n_ch) d.b.fpart[(int64_t(run) * d.n_ch + c) * n_out + k] = o[c].x;
+            } else {
+                finish_sample<MODE>(d, A, MODE == kInterpOrdered ? first + k : d.b.olist[k], o, false, 0.0f, 0.0f);
+            }
+        }
+        if (runs == 1) continue;
+        __threadfence();
+        __syncthreads();
+        if (threadIdx.x == 0) *s_last = atomicAdd(&d.b.ocount[1 + g], 1) == runs - 1;
+        __syncthreads();
+        if (*s_last == 0) continue;
+        __threadfence();
+        if (threadIdx.x == 0) d.b.ocount[1 + g] = 0;  // for the plan's next application
+        const int k1 = min(n_out, (g + 1) * per);
+        for (int k = g * per + threadIdx.x; k < k1; k += blockDim.x) {
+            df o[2] = {make_float2(0.0f, 0.0f), make_float2(0.0f, 0.0f)};
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                if (c >= d.n_ch) break;
+                F2Sum t{};
+#pragma unroll 8
+                for (int q = 0; q < runs; ++q) t.add(__ldcg(&d.b.fpart[(int64_t(q) * d.n_ch + c) * n_out + k]));
+                o[c] = df_fast_two_sum(t.hi, t.lo);
+            }
+            finish_sample<MODE>(d, A, MODE == kInterpOrdered ? first + k : d.b.olist[k], o, false, 0.0f, 0.0f);
+        }
+    }
+}
+
 // Columns of NC adjacent kx of entry m: DFT of the image rows' spectra along
 // y, times the kernel's spectrum, inverse DFT on the Py nodes; the window's
 // rows are kept.
-template <int NC>
-__global__ void __launch_bounds__(512) k_field_cols_fwd(const __grid_constant__ FieldDev d)
+template <int NC> __device__ __forceinline__ void cols_fwd(const FieldDev &d, unsigned char *smem_raw, float4 (*s_low)[kLowY])
 {
-    chain_wait();
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ float4 s_low[NC][kLowY];
     const int P = d.y.P, Q = d.y.Q, J1 = d.x.J + 1, ny = d.y.n, M = max(P, Q);
     V2<float> *a = reinterpret_cast<V2<float> *>(smem_raw);
     V2<float> *b = a + (smem_fft_pad(M - 1) + 1) * NC;
@@ -844,6 +1085,27 @@ __global__ void __launch_bounds__(512) k_field_cols_fwd(const __grid_constant__ 
         }
         F[int64_t(i) * J1] = f2c(q);
     }
+}
+
+// The columns and then, in the first out_blocks blocks, the outside samples'
+// sums: their loop needs no more registers or shared memory than the columns'
+// transforms, and in-window scans pay one load for it.  (As blocks of their own
+// in the interpolation's launch they cost A at 128 x 128 / 65 536 samples 2 to
+// 3 us of 82, a product of a solve 4 us, with nothing outside.)
+template <int NC, int MODE, typename CIN>
+__global__ void __maxnreg__(80)
+k_field_cols_fwd(const __grid_constant__ FieldDev d, const __grid_constant__ InterpArgs A, const CIN *cin)
+{
+    chain_wait();
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ float4 s_low[NC][kLowY];
+    __shared__ int s_last;
+    // (loaded ahead of the columns' barriers, used behind them)
+    const int n = MODE == kInterpOrdered ? d.b.toff[d.tx * d.ty] : *d.b.ocount;
+    if (int(blockIdx.x) < 3 * d.n_grp) cols_fwd<NC>(d, smem_raw, s_low);
+    if (int(blockIdx.x) >= d.out_blocks) return;
+    const int n_out = MODE == kInterpOrdered ? int(d.T) - n : n;
+    if (n_out > 0) outside_units<MODE, CIN>(d, A, cin, n_out, reinterpret_cast<V2<float> *>(smem_raw), &s_last);
 }
 
 // Node values of window rows 2b, 2b + 1 from their half spectra: xx + i xy of
@@ -928,65 +1190,18 @@ __global__ void __launch_bounds__(512) k_field_rows_inv(const __grid_constant__ 
     }
 }
 
-// Field sums O = sum_x c_x (f1 W + f2 (y.W) y) of one outside sample over all
-// voxels, by the whole block; valid in thread 0.
-template <typename CIN>
-__device__ float2 outside_sum(const FieldDev &d, const CIN *__restrict__ cin, float2 R, float2 W, F2Sum *sh)
-{
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const int nx = d.x.n, ny = d.y.n;
-    float S = 0.0f, Vx = 0.0f, Vy = 0.0f, cS = 0.0f, cVx = 0.0f, cVy = 0.0f;
-    for (int j = warp; j < ny; j += nw) {
-        const V2<float> yr = d.b.yrow[j];
-        const float ox = yr.x - R.x, oy = yr.y - R.y;
-        float s = 0.0f, vx = 0.0f, vy = 0.0f;
-        for (int i0 = 0; i0 < nx; i0 += 32) {
-            const int i = min(i0 + lane, nx - 1);
-            const float c = i0 + lane < nx ? float(cin[int64_t(j) * nx + i]) : 0.0f;
-            const V2<float> xc = d.b.xcol[i];
-            const float yx = xc.x + ox, yy = xc.y + oy;
-            const float u = fmx(yx, yx, yy * yy);
-            float f1, f2;
-            if (d.diag) lang_vfar<float, false>(u, f1, f2);
-            else lang_checked<float, false>(u, f1, f2);
-            s = fmx(c, f1, s);
-            const float f = c * f2 * fmx(yx, W.x, yy * W.y);
-            vx = fmx(f, yx, vx);
-            vy = fmx(f, yy, vy);
-        }
-        kahan_add(S, cS, s);
-        kahan_add(Vx, cVx, vx);
-        kahan_add(Vy, cVy, vy);
-    }
-    const F2Sum a = f2_block(F2Sum{S, -cS}, sh), bx = f2_block(F2Sum{Vx, -cVx}, sh), by = f2_block(F2Sum{Vy, -cVy}, sh);
-    const float s = a.hi + a.lo;
-    return make_float2(fmx(s, W.x, bx.hi + bx.lo), fmx(s, W.y, by.hi + by.lo));
-}
-
-enum { kInterpForward = 0, kInterpOrdered = 1 };
-
-struct InterpArgs {
-    const float *r, *v;   // unordered trajectory
-    float *s;             // [n_ch][T]
-    bool residual;        // ordered: the data minus A c
-};
-
 // The field at the samples and its product with W.  A warp takes 32 samples,
 // eight lanes at a time per sample: lane a holds the stencil's column a (its
 // eight rows are eight independent 16-byte loads; the eight lanes of a row
 // read 128 consecutive bytes), sums its column in FP32 and adds over the
 // lanes in pairs of floats.
-template <int MODE, typename CIN>
-__global__ void __launch_bounds__(256) k_field_interp(const __grid_constant__ FieldDev d, const __grid_constant__ InterpArgs A,
-                                                      const CIN *cin)
+template <int MODE>
+__global__ void __launch_bounds__(kInterpThreads, 4)
+k_field_interp(const __grid_constant__ FieldDev d, const __grid_constant__ InterpArgs A)
 {
     chain_wait();
-    __shared__ float4 s_out[256];
-    __shared__ int s_id[256];
-    __shared__ int s_n;
-    __shared__ F2Sum s_red[32];
     const int lane = threadIdx.x & 31;
-    const int64_t t = int64_t(blockIdx.x) * 256 + threadIdx.x;
+    const int64_t t = int64_t(blockIdx.x) * kInterpThreads + threadIdx.x;
     const bool valid = t < d.T;
     SampleRec q{};
     if (valid) {
@@ -1069,146 +1284,147 @@ __global__ void __launch_bounds__(256) k_field_interp(const __grid_constant__ Fi
             }
         }
     }
-    float sk[2] = {0.0f, 0.0f};
-    const bool residual = MODE == kInterpOrdered && A.residual;
-    auto channels = [&](df Ox, df Oy) {
-        const float2 data = residual ? d.b.sd[t] : make_float2(0.0f, 0.0f);
-        for (int k = 0; k < d.n_ch; ++k) {
-            const float p0 = d.p[2 * k], p1 = d.p[2 * k + 1];
-            const df o = df_add(df_mul(Ox, make_float2(p0, 0.0f)), df_mul(Oy, make_float2(p1, 0.0f)));
-            sk[k] = residual ? ((k ? data.y : data.x) - o.x) - o.y : o.x + o.y;
-        }
-    };
-    auto finish = [&](int64_t tt, float2 W, bool inside) {
-        if constexpr (MODE == kInterpForward) {
-            for (int k = 0; k < d.n_ch; ++k) A.s[int64_t(k) * d.T + tt] = sk[k];
-        } else {
-            float ux = 0.0f, uy = 0.0f;
-            for (int k = 0; k < d.n_ch; ++k) {
-                ux += sk[k] * d.p[2 * k];
-                uy += sk[k] * d.p[2 * k + 1];
-            }
-            d.b.q4[tt] = inside ? make_float4(ux * W.x, fmaf(ux, W.y, uy * W.x), uy * W.y, 0.0f) : make_float4(ux, uy, 0.0f, 0.0f);
-        }
-    };
     if (in) {
-        channels(df_add(df_mul(phi[0], q.Wx), df_mul(phi[1], q.Wy)), df_add(df_mul(phi[1], q.Wx), df_mul(phi[2], q.Wy)));
-        finish(t, make_float2(q.Wx.x, q.Wy.x), true);
-    }
-    if (threadIdx.x == 0) s_n = 0;
-    if (__syncthreads_or(valid && !q.in)) {
-        if (valid && !q.in) {
-            const int k = atomicAdd(&s_n, 1);
-            s_out[k] = make_float4(q.fx, q.fy, q.Wx.x, q.Wy.x);
-            s_id[k] = threadIdx.x;
-        }
-        __syncthreads();
-        const int n = s_n;
-        for (int k = 0; k < n; ++k) {
-            const float4 e = s_out[k];
-            const float2 W = make_float2(e.z, e.w);
-            const float2 O = outside_sum<CIN>(d, cin, make_float2(e.x, e.y), W, s_red);
-            if (threadIdx.x == 0) s_out[k].x = O.x, s_out[k].y = O.y;
-        }
-        __syncthreads();
-        // back to the samples' own threads
-        for (int k = 0; k < n; ++k)
-            if (s_id[k] == int(threadIdx.x)) {
-                channels(make_float2(s_out[k].x, 0.0f), make_float2(s_out[k].y, 0.0f));
-                finish(t, make_float2(q.Wx.x, q.Wy.x), false);
-            }
+        const df Ox = df_add(df_mul(phi[0], q.Wx), df_mul(phi[1], q.Wy)), Oy = df_add(df_mul(phi[1], q.Wx), df_mul(phi[2], q.Wy));
+        df o[2];
+#pragma unroll
+        for (int k = 0; k < 2; ++k)  // (a single channel's second is not stored)
+            o[k] = df_add(df_mul(Ox, make_float2(d.p[2 * k], 0.0f)), df_mul(Oy, make_float2(d.p[2 * k + 1], 0.0f)));
+        finish_sample<MODE>(d, A, t, o, true, q.Wx.x, q.Wy.x);
     }
 }
 
 // --- adjoint --------------------------------------------------------------------
 
-// Blocks below n_unit_max: one spreading unit each -- the patch of the unit's
-// tile, summed over its samples in order.  A warp owns one entry of K on the
+// Chunks of the outside samples' partial images: at least kOutThreads samples each.
+__device__ __forceinline__ int out_chunks_used(const FieldDev &d, int n_out)
+{
+    return n_out > 0 ? min(d.out_chunks, (n_out + kOutThreads - 1) / kOutThreads) : 0;
+}
+
+// Partial image of the ordered outside samples c0 .. c1 - 1 on one tile of the
+// voxels: a thread owns kOutRows voxels of one column, 32 staged samples at a
+// time are summed plainly and added with compensation.  For a diagonal G two
+// samples share packed FP32 arithmetic, as in the pair sums; for a general G
+// their test against the warp's voxels chooses the form.  A^T at 128 x 128 /
+// 65 536 samples, 94 % of them outside: 0.48 ms, before 0.81 ms (pair sums of
+// all samples 0.42 ms); 512 x 512, 84 %: 5.7 ms (7.9, 6.0).
+__device__ __forceinline__ void outside_image(const FieldDev &d, int tile, int c0, int c1, float *s_p, float *__restrict__ out)
+{
+    static_assert(6 * kOutThreads <= 6 * kPatch * kPatchPitch, "staged samples");
+    const int nx = d.x.n, ny = d.y.n, lane = threadIdx.x & 31;
+    const int n_q = nx * ((ny + kOutRows - 1) / kOutRows);
+    const int q0 = tile * kOutThreads + int(threadIdx.x), qc = min(q0, n_q - 1);
+    const int i = qc % nx, jb = qc / nx * kOutRows;
+    const V2<float> xc = d.b.xcol[i];
+    float Yx[kOutRows], Yy[kOutRows], acc[kOutRows], comp[kOutRows];
+#pragma unroll
+    for (int k = 0; k < kOutRows; ++k) {
+        const V2<float> yr = d.b.yrow[min(jb + k, ny - 1)];
+        Yx[k] = yr.x, Yy[k] = yr.y;
+        acc[k] = comp[k] = 0.0f;
+    }
+    float lo[2] = {xc.x + Yx[0], xc.y + Yy[0]}, hi[2] = {lo[0], lo[1]};  // general G: the warp's voxels
+    if (!d.diag) {
+#pragma unroll
+        for (int k = 1; k < kOutRows; ++k) {
+            const float e[2] = {xc.x + Yx[k], xc.y + Yy[k]};
+#pragma unroll
+            for (int a = 0; a < 2; ++a) lo[a] = min(lo[a], e[a]), hi[a] = max(hi[a], e[a]);
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+            for (int a = 0; a < 2; ++a) {
+                lo[a] = min(lo[a], __shfl_xor_sync(0xffffffffu, lo[a], o));
+                hi[a] = max(hi[a], __shfl_xor_sync(0xffffffffu, hi[a], o));
+            }
+    }
+#pragma unroll 1
+    for (int cb = c0; cb < c1; cb += kOutThreads) {
+        const int nb = min(kOutThreads, c1 - cb), nb2 = (nb + 1) & ~1;
+        __syncthreads();
+        if (int(threadIdx.x) < nb2) {
+            const int k = threadIdx.x, t = cb + min(k, nb - 1);
+            const float4 rc = d.b.rec[t], w = d.b.wv[t];
+            const float4 u = k < nb ? d.b.q4[t] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);  // (an odd count: one without weight)
+            const float uW = u.x * w.x + u.y * w.y, Sxx = w.x * u.x, Sxy = w.x * u.y + w.y * u.x, Syy = w.y * u.y;
+            if (d.diag) {  // pairs: (-x, -y), (uW, Sxx), (Sxy, Syy), each entry (even, odd)
+                float *q = s_p + 12 * (k >> 1) + (k & 1);
+                q[0] = -rc.x;
+                q[2] = -rc.y;
+                q[4] = uW;
+                q[6] = Sxx;
+                q[8] = Sxy;
+                q[10] = Syy;
+            } else {
+                float *q = s_p + 6 * k;
+                q[0] = rc.x;
+                q[1] = rc.y;
+                q[2] = uW;
+                q[3] = Sxx;
+                q[4] = Sxy;
+                q[5] = Syy;
+            }
+        }
+        __syncthreads();
+#pragma unroll 1
+        for (int k0 = 0; k0 < nb2; k0 += 32) {
+            const int kn = min(32, nb2 - k0);
+            float blk[kOutRows];
+#pragma unroll
+            for (int k = 0; k < kOutRows; ++k) blk[k] = 0.0f;
+            if (d.diag) {
+                const float4 *pk = reinterpret_cast<const float4 *>(s_p) + 3 * (k0 >> 1);
+                float2 yr2[kOutRows], blk2[kOutRows];
+#pragma unroll
+                for (int k = 0; k < kOutRows; ++k) yr2[k] = make_float2(Yy[k], Yy[k]), blk2[k] = make_float2(0.0f, 0.0f);
+#pragma unroll 2
+                for (int h = 0; h < (kn >> 1); ++h)
+                    adj_pair2_vfar_diag<false>(pk[3 * h], pk[3 * h + 1], pk[3 * h + 2], make_float2(xc.x, xc.x), yr2, blk2);
+#pragma unroll
+                for (int k = 0; k < kOutRows; ++k) blk[k] = blk2[k].x + blk2[k].y;
+            } else {
+                bool far = true;
+                if (lane < kn) {
+                    const float *q = s_p + 6 * (k0 + lane);
+                    const float gx = max(0.0f, max(lo[0] - q[0], q[0] - hi[0])), gy = max(0.0f, max(lo[1] - q[1], q[1] - hi[1]));
+                    far = fmx(gy, gy, gx * gx) >= vfar_threshold<float, false>();
+                }
+                const unsigned mask = __ballot_sync(0xffffffffu, far);
+#pragma unroll 1
+                for (int k = 0; k < kn; ++k) {
+                    const float *q = s_p + 6 * (k0 + k);
+                    const V2<float> rr{q[0], q[1]};
+                    const V4<float> S{q[2], q[3], q[4], q[5]};
+                    if ((mask >> k) & 1u) adj_sample<float, false, false, 2>(rr, S, xc, Yx, Yy, blk);
+                    else adj_sample<float, false, false, 0>(rr, S, xc, Yx, Yy, blk);
+                }
+            }
+#pragma unroll
+            for (int k = 0; k < kOutRows; ++k) kahan_add(acc[k], comp[k], blk[k]);
+        }
+    }
+    if (q0 >= n_q) return;
+#pragma unroll
+    for (int k = 0; k < kOutRows; ++k)
+        if (jb + k < ny) out[int64_t(jb + k) * nx + i] = acc[k];
+}
+
+// One spreading unit u, by one block: the patch of the unit's tile, summed over its samples in order.  A warp owns one entry of K on the
 // patch rows of one parity: a sample's stencil has four such rows of eight
 // points, one per lane, so no two lanes share a node and the order of the
 // additions is the samples' order.  The unit's two halves go to two copies of
 // the patch, added at the end: twice the independent chains of load, FMA and
 // store.  What bounds it is the shared-memory pipe: per sample and warp one load and one store of the patch, and a
 // quarter of three 16-byte loads (weights and addresses of four samples,
-// fetched one step ahead).  The other blocks: partial images of the samples
-// outside the window (none: they return).
+// fetched one step ahead).
 constexpr int kUnitPitch = kFieldUnit + 4;
-__global__ void __launch_bounds__(kSpreadThreads) k_field_spread(const __grid_constant__ FieldDev d)
+__device__ __forceinline__ void spread_unit(const FieldDev &d, int u, float (*s_patch)[3][kPatch * kPatchPitch])
 {
-    chain_wait();
-    __shared__ float s_patch[2][3][kPatch * kPatchPitch];
     __shared__ __align__(16) float s_wx[kWin][kUnitPitch];
     __shared__ __align__(16) float s_c[3][kWin][kUnitPitch];  // entry x row weight, rows by parity
     __shared__ __align__(16) int s_at[kUnitPitch];
-    const int nt = d.tx * d.ty;
-    if (int(blockIdx.x) >= d.n_unit_max) {
-        const int first = d.b.toff[nt];
-        const int n_out = int(d.T) - first;
-        if (n_out <= 0) return;
-        const int job = blockIdx.x - d.n_unit_max;
-        const int used = min(d.out_chunks, (n_out + kOutThreads - 1) / kOutThreads);
-        const int chunk = job / d.out_tiles, tile = job % d.out_tiles;
-        if (chunk >= used) return;
-        const int len = (n_out + used - 1) / used;
-        const int c0 = first + chunk * len, c1 = min(int(d.T), c0 + len);
-        const int64_t N = int64_t(d.x.n) * d.y.n;
-        const int64_t e0 = int64_t(tile) * kOutThreads * kOutVox + threadIdx.x;
-        float vx[kOutVox], vy[kOutVox], acc[kOutVox], comp[kOutVox];
-#pragma unroll
-        for (int k = 0; k < kOutVox; ++k) {
-            const int64_t e = min(N - 1, e0 + int64_t(k) * kOutThreads);
-            const V2<float> xc = d.b.xcol[e % d.x.n], yr = d.b.yrow[e / d.x.n];
-            vx[k] = xc.x + yr.x;
-            vy[k] = xc.y + yr.y;
-            acc[k] = comp[k] = 0.0f;
-        }
-        float *s_p = &s_patch[0][0][0];  // six values per staged sample
-        for (int cb = c0; cb < c1; cb += kOutThreads) {
-            const int nb = min(kOutThreads, c1 - cb);
-            __syncthreads();
-            if (int(threadIdx.x) < nb) {
-                const float4 rc = d.b.rec[cb + threadIdx.x], w = d.b.wv[cb + threadIdx.x], u = d.b.q4[cb + threadIdx.x];
-                float *q = s_p + 6 * threadIdx.x;
-                q[0] = rc.x;
-                q[1] = rc.y;
-                q[2] = u.x * w.x + u.y * w.y;
-                q[3] = w.x * u.x;
-                q[4] = w.x * u.y + w.y * u.x;
-                q[5] = w.y * u.y;
-            }
-            __syncthreads();
-            float blk[kOutVox];
-#pragma unroll
-            for (int k = 0; k < kOutVox; ++k) blk[k] = 0.0f;
-            for (int q = 0; q < nb; ++q) {
-                const float *sv = s_p + 6 * q;
-                const float Rx = sv[0], Ry = sv[1], uW = sv[2], Sxx = sv[3], Sxy = sv[4], Syy = sv[5];
-#pragma unroll
-                for (int k = 0; k < kOutVox; ++k) {
-                    const float yx = vx[k] - Rx, yy = vy[k] - Ry;
-                    const float u = fmx(yx, yx, yy * yy);
-                    const float quad = fmx(yx, fmx(Sxx, yx, Sxy * yy), Syy * yy * yy);
-                    if (d.diag) {
-                        blk[k] = pair_acc_vfar<float, false>(u, uW, quad, blk[k]);
-                    } else {
-                        float f1, f2;
-                        lang_checked<float, false>(u, f1, f2);
-                        blk[k] += fmx(f1, uW, f2 * quad);
-                    }
-                }
-            }
-#pragma unroll
-            for (int k = 0; k < kOutVox; ++k) kahan_add(acc[k], comp[k], blk[k]);
-        }
-#pragma unroll
-        for (int k = 0; k < kOutVox; ++k) {
-            const int64_t e = e0 + int64_t(k) * kOutThreads;
-            if (e < N) d.b.opart[int64_t(chunk) * N + e] = acc[k];
-        }
-        return;
-    }
-    const int u = blockIdx.x;
-    if (u >= d.b.uoff[nt]) return;
     const int tile = d.b.unit_tile[u];
     const int u0 = d.b.uoff[tile], nu = d.b.uoff[tile + 1] - u0;
     const int t0 = d.b.toff[tile], t1 = d.b.toff[tile + 1];
@@ -1290,6 +1506,27 @@ __global__ void __launch_bounds__(kSpreadThreads) k_field_spread(const __grid_co
         const int mm = k / kPatchSize, e = k % kPatchSize;
         const int at = (e / kPatch) * kPatchPitch + e % kPatch;
         out[k] = s_patch[0][mm][at] + s_patch[1][mm][at];
+    }
+}
+
+// The units, one per block, then the outside samples' partial images by the
+// blocks from the last one down (units leave most of them free: their number is
+// only bounded by n_unit_max).
+__global__ void __launch_bounds__(kSpreadThreads, kSpreadPerSm) k_field_spread(const __grid_constant__ FieldDev d)
+{
+    chain_wait();
+    __shared__ __align__(16) float s_patch[2][3][kPatch * kPatchPitch];
+    const int nt = d.tx * d.ty;
+    const int first = d.b.toff[nt], n_unit = d.b.uoff[nt];
+    if (int(blockIdx.x) < n_unit) spread_unit(d, blockIdx.x, s_patch);
+    const int n_out = int(d.T) - first;
+    if (n_out <= 0) return;
+    const int used = out_chunks_used(d, n_out), len = (n_out + used - 1) / used;
+#pragma unroll 1
+    for (int job = int(gridDim.x) - 1 - int(blockIdx.x); job < used * d.out_tiles; job += gridDim.x) {
+        const int chunk = job / d.out_tiles, tile = job % d.out_tiles;
+        const int c0 = first + chunk * len, c1 = min(int(d.T), c0 + len);
+        outside_image(d, tile, c0, c1, &s_patch[0][0][0], d.b.opart + int64_t(chunk) * d.x.n * d.y.n);
     }
 }
 
@@ -1489,7 +1726,7 @@ __global__ void __launch_bounds__(128) k_field_out(const __grid_constant__ Field
     __syncthreads();
     const V2<float> *z = smem_fft<1, 1, float>(a, b, d.fQx, reinterpret_cast<const V2<float> *>(d.b.twQx));
     const int n_out = int(d.T) - d.b.toff[d.tx * d.ty];
-    const int used = n_out > 0 ? min(d.out_chunks, (n_out + kOutThreads - 1) / kOutThreads) : 0;
+    const int used = out_chunks_used(d, n_out);
     const int64_t N = int64_t(nx) * ny;
     double dot = 0.0;
     const double nu = CG ? *nu_dev : 0.0;
@@ -1510,6 +1747,7 @@ __global__ void __launch_bounds__(128) k_field_out(const __grid_constant__ Field
             s.lo += fmaf(v.z, w.x, v.w * w.y);
         }
         const int64_t e = int64_t(j0 + rr) * nx + i;
+#pragma unroll 4
         for (int c = 0; c < used; ++c) s.add(d.b.opart[int64_t(c) * N + e]);
         if constexpr (CG) {
             const double pe = p[e], val = s.value() + nu * pe;
@@ -1608,8 +1846,12 @@ int fft_threads(int nc, int n)
     const int b = (nc * n + 7) / 8, per = (b + 511) / 512;
     return std::max(128, ((b + per - 1) / per + 31) / 32 * 32);
 }
+int cols_threads(const FieldDev &d) { return fft_threads(cols_nc(d), std::max(d.y.P, d.y.Q)); }
 size_t rows_smem(const FieldDev &d) { return 2 * sizeof(float2) * smem_fft_elems(std::max(d.x.P, d.x.Q), 3); }
-size_t cols_smem(const FieldDev &d) { return 2 * sizeof(float2) * smem_fft_elems(std::max(d.y.P, d.y.Q), cols_nc(d)); }
+size_t cols_smem(const FieldDev &d)
+{
+    return std::max(2 * sizeof(float2) * smem_fft_elems(std::max(d.y.P, d.y.Q), cols_nc(d)), sizeof(float2) * kOutStage);
+}
 size_t image_smem(const FieldDev &d) { return 2 * sizeof(float2) * smem_fft_elems(d.x.Q, 1); }
 // Warps per block of the ordering kernels: each has its own tile counters.
 int order_warps(const FieldDev &d) { return std::max(1, std::min<int>(4, 48 * 1024 / (4 * (d.tx * d.ty + 1)))); }
@@ -1624,7 +1866,10 @@ int allow_all(const FieldDev &d, bool forward, bool adjoint)
     MPI_TRY(allow_smem(four ? k_field_kcols<4> : k_field_kcols<2>, cols_smem(d)));
     if (forward) {
         MPI_TRY(allow_smem(k_field_image<double>, image_smem(d)));
-        MPI_TRY(allow_smem(four ? k_field_cols_fwd<4> : k_field_cols_fwd<2>, cols_smem(d)));
+        MPI_TRY(allow_smem(four ? k_field_cols_fwd<4, kInterpForward, float> : k_field_cols_fwd<2, kInterpForward, float>,
+                           cols_smem(d)));
+        MPI_TRY(allow_smem(four ? k_field_cols_fwd<4, kInterpOrdered, double> : k_field_cols_fwd<2, kInterpOrdered, double>,
+                           cols_smem(d)));
         MPI_TRY(allow_smem(k_field_rows_inv, rows_smem(d)));
     }
     if (adjoint) {
@@ -1664,6 +1909,9 @@ void lay_out(FieldPlan &plan, char *keep, char *work, size_t &keep_bytes, size_t
         take(1, b.CL, ny * kFieldLow);
         take(1, b.FL, size_t(3) * d.y.w * kFieldLow);
         take(1, b.FN, size_t(d.y.w) * d.x.w);
+        take(0, b.ocount, out_counters(d));
+        take(1, b.fpart, size_t(d.n_ch) * kOutRounds * d.out_blocks * d.out_samples);
+        if (!plan.adjoint) take(1, b.olist, T1);
     }
     if (plan.adjoint) {
         take(1, b.key, T1); take(1, b.hist, nh); take(1, b.pos, nh); take(1, b.tcnt, nt + 1);
@@ -1702,9 +1950,12 @@ int field_plan(const ModelH &m, const GridH &g, int64_t T, bool forward, bool ad
     d.n_run = (int)((T + d.run_len - 1) / d.run_len);
     const int nt = d.tx * d.ty;
     d.n_unit_max = (int)(T / kFieldUnit + std::min<int64_t>(nt, T));
-    const int64_t N = (int64_t)g.nx * g.ny;
-    d.out_tiles = (int)((N + kOutThreads * kOutVox - 1) / (kOutThreads * kOutVox));
-    d.out_chunks = std::max(1, std::min(32, 2048 / d.out_tiles));
+    const int64_t columns = (int64_t)g.nx * ((g.ny + kOutRows - 1) / kOutRows);
+    d.out_tiles = (int)((columns + kOutThreads - 1) / kOutThreads);
+    const int at_once = kSpreadPerSm * device_sm_count();
+    d.out_chunks = std::max(1, std::min(64, (8 * d.out_tiles <= at_once ? 1 : 3) * at_once / d.out_tiles));
+    d.out_blocks = std::max(1, std::min(4, kOutPerSm / cols_threads(d))) * device_sm_count();
+    d.out_samples = kFwdS * cols_threads(d);
     d.n_ch = m.n_ch;
     d.diag = m.G[1] == 0.0 && m.G[2] == 0.0;
     for (int k = 0; k < 4; ++k) {
@@ -1753,7 +2004,8 @@ int field_prepare(const FieldPlan &plan, const float *c, const float *r, const f
     MPI_CHECK_LAUNCH();
     const int kr = (d.y.P / 2 + 2) / 2, tr = fft_threads(3, d.x.P);
     const int more = c ? (d.y.n + 1) / 2 : plan.adjoint ? (d.tx * d.ty + 1 + tr / 32 - 1) / (tr / 32) : 0;
-    launch_chained(k_field_rows, kr + more, tr, rows_smem(d), st, d, kr, c);
+    const int list = c ? (int)((d.T + tr * kListPer - 1) / (tr * kListPer)) : 0;
+    launch_chained(k_field_rows, kr + more + list, tr, rows_smem(d), st, d, kr, c, r);
     MPI_CHECK_LAUNCH();
     auto cols = cols_nc(d) == 4 ? k_field_kcols<4> : k_field_kcols<2>;
     launch_chained(cols, 3 * d.n_grp + (plan.adjoint ? 1 : 0), fft_threads(cols_nc(d), d.y.P), cols_smem(d), st, d);
@@ -1779,18 +2031,19 @@ int field_load(const FieldPlan &plan, const float *s, cudaStream_t st)
 
 namespace {
 
-// Image rows' spectra -> node values.
-int field_nodes(const FieldDev &d, cudaStream_t st)
+// Image rows' spectra -> node values; the outside samples' sums.
+template <int MODE, typename CIN>
+int field_nodes(const FieldDev &d, const InterpArgs &A, const CIN *c, cudaStream_t st)
 {
-    auto cols = cols_nc(d) == 4 ? k_field_cols_fwd<4> : k_field_cols_fwd<2>;
-    launch_chained(cols, 3 * d.n_grp, fft_threads(cols_nc(d), std::max(d.y.P, d.y.Q)), cols_smem(d), st, d);
+    auto cols = cols_nc(d) == 4 ? k_field_cols_fwd<4, MODE, CIN> : k_field_cols_fwd<2, MODE, CIN>;
+    launch_chained(cols, std::max(3 * d.n_grp, d.out_blocks), cols_threads(d), cols_smem(d), st, d, A, c);
     MPI_CHECK_LAUNCH();
     launch_chained(k_field_rows_inv, (d.y.w + 1) / 2, fft_threads(3, d.x.P), rows_smem(d), st, d);
     MPI_CHECK_LAUNCH();
     return MPI_OK;
 }
 
-unsigned interp_blocks(int64_t T) { return (unsigned)((T + 255) / 256); }
+unsigned interp_blocks(const FieldDev &d) { return unsigned((d.T + kInterpThreads - 1) / kInterpThreads); }
 
 }  // namespace
 
@@ -1798,9 +2051,9 @@ int field_forward(const FieldPlan &plan, const float *c, const float *r, const f
 {
     ProfScope prof(kProfForward, st);
     MPI_TRY(field_prepare(plan, c, r, v, st));
-    MPI_TRY(field_nodes(plan.d, st));
     const InterpArgs A{r, v, s, false};
-    launch_chained(k_field_interp<kInterpForward, float>, interp_blocks(plan.d.T), 256, 0, st, plan.d, A, c);
+    MPI_TRY((field_nodes<kInterpForward>(plan.d, A, c, st)));
+    launch_chained(k_field_interp<kInterpForward>, interp_blocks(plan.d), kInterpThreads, 0, st, plan.d, A);
     MPI_CHECK_LAUNCH();
     return MPI_OK;
 }
@@ -1812,8 +2065,9 @@ int field_forward_ordered(const FieldPlan &plan, const CIN *c, bool residual, cu
     ProfScope prof(kProfForward, st);
     launch_chained(k_field_image<CIN>, (d.y.n + 1) / 2, 128, image_smem(d), st, d, c);
     MPI_CHECK_LAUNCH();
-    MPI_TRY(field_nodes(d, st));
-    launch_chained(k_field_interp<kInterpOrdered, CIN>, interp_blocks(plan.d.T), 256, 0, st, plan.d, InterpArgs{nullptr, nullptr, nullptr, residual}, c);
+    const InterpArgs A{nullptr, nullptr, nullptr, residual};
+    MPI_TRY((field_nodes<kInterpOrdered>(d, A, c, st)));
+    launch_chained(k_field_interp<kInterpOrdered>, interp_blocks(d), kInterpThreads, 0, st, d, A);
     MPI_CHECK_LAUNCH();
     return MPI_OK;
 }
@@ -1826,12 +2080,12 @@ int field_adjoint(const FieldPlan &plan, OUT *out, const double *cg_p, const dou
 {
     const FieldDev &d = plan.d;
     ProfScope prof(kProfAdjoint, st);
-    launch_chained(k_field_spread, d.n_unit_max + d.out_tiles * d.out_chunks, kSpreadThreads, 0, st, d);
+    launch_chained(k_field_spread, std::max(d.n_unit_max, kSpreadPerSm * device_sm_count()), kSpreadThreads, 0, st, d);
     MPI_CHECK_LAUNCH();
     launch_chained(k_field_rows_fwd, (d.y.w + 1) / 2, fft_threads(3, d.x.P), rows_smem(d), st, d);
     MPI_CHECK_LAUNCH();
     auto cols = cols_nc(d) == 4 ? k_field_cols_adj<4> : k_field_cols_adj<2>;
-    launch_chained(cols, 3 * d.n_grp, fft_threads(cols_nc(d), std::max(d.y.P, d.y.Q)), cols_smem(d), st, d);
+    launch_chained(cols, 3 * d.n_grp, cols_threads(d), cols_smem(d), st, d);
     MPI_CHECK_LAUNCH();
     const unsigned nb = (unsigned)field_dot_blocks(d.y.n);
     if constexpr (sizeof(OUT) == sizeof(double)) {

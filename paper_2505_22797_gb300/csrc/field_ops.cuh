@@ -45,6 +45,9 @@ struct FieldBuf {
     float2 *sd;      // the data of a solve, both channels, in the samples' order
     float *upart;    // unit patches
     float *opart;    // outside samples' partial images
+    int *ocount;     // outside samples (unordered), and per group of them the runs of rows done
+    int *olist;      // the outside samples (unordered)
+    float *fpart;    // their partial sums by runs of rows
     float2 *AC;      // [3][ny][Jx + 1]
     float4 *AL;      // [3][ny][kFieldLow]
 };
@@ -60,7 +63,8 @@ struct FieldDev {
     int n_grp;           // groups of adjacent kx in the column transforms
     unsigned magQy;      // floor(2^32 / Qy) + 1
     int n_unit_max;
-    int out_tiles, out_chunks;
+    int out_tiles, out_chunks;  // outside samples, A^T: voxel tiles, partial images
+    int out_blocks, out_samples;  // and A: blocks of the column launch that sum them, samples per block
     int n_ch, diag;
     float p[4];
     float B[4][2];    // beta G as pairs

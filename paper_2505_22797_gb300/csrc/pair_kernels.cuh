@@ -488,7 +488,7 @@ __device__ __forceinline__ void forward_item(const PairBatch<R, MAXF> &B, int64_
 }
 
 // ---------------------------------------------------------------------------
-// One staged sample against this thread's kAdjV voxels of a column (adjoint /
+// One staged sample against this thread's V voxels of a column (adjoint /
 // beta-derivative): blk[v] += f1 (u.W) + f2 y^T S y.  FAR: the warp's voxel
 // box is provably outside the near-FFP range for this sample.
 template <typename R, bool DBETA, int MODE>
@@ -501,17 +501,16 @@ __device__ __forceinline__ void lang_mode(R u, R &f1, R &f2)
 
 // MODE 2: the warp's voxel box is provably in the asymptotic range for this
 // sample; 1: in the closed-form range; 0: near pairs possible.
-template <typename R, bool DIAG, bool DBETA, int MODE>
+template <typename R, bool DIAG, bool DBETA, int MODE, int V>
 __device__ __forceinline__ void adj_sample(const V2<R> rr, const V4<R> q, const V2<R> xc,
-                                           const R (&yrow_x)[kAdjV], const R (&yrow_y)[kAdjV],
-                                           R (&blk)[kAdjV])
+                                           const R (&yrow_x)[V], const R (&yrow_y)[V], R (&blk)[V])
 {
     if (DIAG) {
         const R yx = xc.x - rr.x;
         const R yx2 = yx * yx;
         const R Q0 = q.y * yx2, Q1 = q.z * yx;
 #pragma unroll
-        for (int v = 0; v < kAdjV; ++v) {
+        for (int v = 0; v < V; ++v) {
             const R yy = yrow_y[v] - rr.y;
             const R u = fmx(yy, yy, yx2);
             const R P = fmx(yy, fmx(q.w, yy, Q1), Q0);
@@ -526,7 +525,7 @@ __device__ __forceinline__ void adj_sample(const V2<R> rr, const V4<R> q, const 
     } else {
         const R ox = xc.x - rr.x, oy = xc.y - rr.y;
 #pragma unroll
-        for (int v = 0; v < kAdjV; ++v) {
+        for (int v = 0; v < V; ++v) {
             const R yx = ox + yrow_x[v];
             const R yy = oy + yrow_y[v];
             const R u = fmx(yx, yx, yy * yy);
@@ -543,15 +542,14 @@ __device__ __forceinline__ void adj_sample(const V2<R> rr, const V4<R> q, const 
 }
 
 #ifdef __CUDACC__
-// Two staged samples (2h, 2h + 1) against this thread's kAdjV voxels in the
+// Two staged samples (2h, 2h + 1) against this thread's V voxels in the
 // asymptotic range, diagonal G, packed: a = (-x_e, -x_o, -y_e, -y_o) of B r,
 // b = (uW_e, uW_o, Sxx_e, Sxx_o), c = (S2xy_e, S2xy_o, Syy_e, Syy_o); xc2 =
 // (x_c, x_c) of the thread's column, yr2[v] = (y_v, y_v).  Lane-wise the
 // same operations, in the same order, as adj_sample's MODE 2 on each sample.
-template <bool DBETA>
+template <bool DBETA, int V>
 __device__ __forceinline__ void adj_pair2_vfar_diag(const float4 a, const float4 b, const float4 c,
-                                                    const float2 xc2, const float2 (&yr2)[kAdjV],
-                                                    float2 (&blk2)[kAdjV])
+                                                    const float2 xc2, const float2 (&yr2)[V], float2 (&blk2)[V])
 {
     const float2 nry = make_float2(a.z, a.w);
     const float2 uW = make_float2(b.x, b.y), Sxx = make_float2(b.z, b.w);
@@ -561,7 +559,7 @@ __device__ __forceinline__ void adj_pair2_vfar_diag(const float4 a, const float4
     const float2 Q0 = __fmul2_rn(Sxx, yx2), Q1 = __fmul2_rn(S2xy, yx);
     const float2 nuW = __fmul2_rn(uW, make_float2(-1.0f, -1.0f));
 #pragma unroll
-    for (int v = 0; v < kAdjV; ++v) {
+    for (int v = 0; v < V; ++v) {
         const float2 yy = __fadd2_rn(yr2[v], nry);
         const float2 u = __ffma2_rn(yy, yy, yx2);
         const float2 P = __ffma2_rn(yy, __ffma2_rn(Syy, yy, Q1), Q0);
