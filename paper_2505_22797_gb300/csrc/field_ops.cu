@@ -1550,36 +1550,55 @@ __global__ void __launch_bounds__(512) k_field_rows_fwd(const __grid_constant__ 
         F2Sum g[2][3] = {};
         if (i < wx) {
             const int tx1 = min(i / kTile, d.tx - 1), tx0 = max(0, (i - kPatch + kTile) / kTile);
-            for (int ty = ty0; ty <= ty1; ++ty) {
-                const int pr = i0 - ty * kTile;  // patch row of the first node row
-                for (int tx = tx0; tx <= tx1; ++tx) {
-                    const int u0 = d.b.uoff[ty * d.tx + tx], u1 = d.b.uoff[ty * d.tx + tx + 1];
-                    const float *p = d.b.upart + int64_t(u0) * 3 * kPatchSize + pr * kPatch + i - tx * kTile;
-                    const bool two = pr + 1 < kPatch;
-                    auto load = [&](const float *e, float (&q)[2][3]) {
+            auto load = [&](const float *e, bool two, float (&q)[2][3]) {
 #pragma unroll
-                        for (int m = 0; m < 3; ++m) {
-                            q[0][m] = e[m * kPatchSize];
-                            q[1][m] = two ? e[m * kPatchSize + kPatch] : 0.0f;
-                        }
-                    };
-                    auto add = [&](const float (&q)[2][3]) {
+                for (int m = 0; m < 3; ++m) {
+                    q[0][m] = e[m * kPatchSize];
+                    q[1][m] = two ? e[m * kPatchSize + kPatch] : 0.0f;
+                }
+            };
+            auto add = [&](const float (&q)[2][3]) {
 #pragma unroll
-                        for (int m = 0; m < 3; ++m) g[0][m].add(q[0][m]), g[1][m].add(q[1][m]);
-                    };
-                    int u = u0;
-                    for (; u + kUnitsAtOnce <= u1; u += kUnitsAtOnce, p += kUnitsAtOnce * 3 * kPatchSize) {
-                        float q[kUnitsAtOnce][2][3];
+                for (int m = 0; m < 3; ++m) g[0][m].add(q[0][m]), g[1][m].add(q[1][m]);
+            };
+            // the four tiles' first units at once, then what more they have
+            int u0[4], u1[4];
+            float q[4][2][3];
 #pragma unroll
-                        for (int k = 0; k < kUnitsAtOnce; ++k) load(p + k * 3 * kPatchSize, q[k]);
+            for (int k = 0; k < 4; ++k) {
+                const int ty = ty0 + (k >> 1), tx = tx0 + (k & 1), tile = ty * d.tx + tx;
+                const bool on = ty <= ty1 && tx <= tx1;
+                u0[k] = on ? d.b.uoff[tile] : 0;
+                u1[k] = on ? d.b.uoff[tile + 1] : 0;
+            }
+            auto patch = [&](int k, int u) {
+                const int pr = i0 - (ty0 + (k >> 1)) * kTile;  // patch row of the first node row
+                return d.b.upart + int64_t(u) * 3 * kPatchSize + pr * kPatch + i - (tx0 + (k & 1)) * kTile;
+            };
+            const bool two[2] = {i0 - ty0 * kTile + 1 < kPatch, i0 - ty0 * kTile + 1 < kPatch + kTile};
 #pragma unroll
-                        for (int k = 0; k < kUnitsAtOnce; ++k) add(q[k]);
-                    }
-                    for (; u < u1; ++u, p += 3 * kPatchSize) {
-                        float q[2][3];
-                        load(p, q);
-                        add(q);
-                    }
+            for (int k = 0; k < 4; ++k) {
+                if (u0[k] < u1[k]) {
+                    load(patch(k, u0[k]), two[k >> 1], q[k]);
+                } else {
+#pragma unroll
+                    for (int m = 0; m < 3; ++m) q[k][0][m] = q[k][1][m] = 0.0f;
+                }
+            }
+#pragma unroll
+            for (int k = 0; k < 4; ++k) add(q[k]);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                int u = u0[k] + 1;
+                for (; u + kUnitsAtOnce <= u1[k]; u += kUnitsAtOnce) {
+#pragma unroll
+                    for (int e = 0; e < kUnitsAtOnce; ++e) load(patch(k, u + e), two[k >> 1], q[e]);
+#pragma unroll
+                    for (int e = 0; e < kUnitsAtOnce; ++e) add(q[e]);
+                }
+                for (; u < u1[k]; ++u) {
+                    load(patch(k, u), two[k >> 1], q[0]);
+                    add(q[0]);
                 }
             }
         }
