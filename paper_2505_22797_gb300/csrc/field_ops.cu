@@ -1296,10 +1296,11 @@ k_field_interp(const __grid_constant__ FieldDev d, const __grid_constant__ Inter
 
 // --- adjoint --------------------------------------------------------------------
 
-// Chunks of the outside samples' partial images: at least kOutThreads samples each.
+// Chunks of the outside samples' partial images, of at least 128 samples (13 000
+// on 64 x 64 voxels: 45 us, with 384 a chunk 70).
 __device__ __forceinline__ int out_chunks_used(const FieldDev &d, int n_out)
 {
-    return n_out > 0 ? min(d.out_chunks, (n_out + kOutThreads - 1) / kOutThreads) : 0;
+    return n_out > 0 ? min(d.out_chunks, (n_out + 127) / 128) : 0;
 }
 
 // Partial image of the ordered outside samples c0 .. c1 - 1 on one tile of the
@@ -1766,8 +1767,13 @@ __global__ void __launch_bounds__(128) k_field_out(const __grid_constant__ Field
             s.lo += fmaf(v.z, w.x, v.w * w.y);
         }
         const int64_t e = int64_t(j0 + rr) * nx + i;
-#pragma unroll 4
-        for (int c = 0; c < used; ++c) s.add(d.b.opart[int64_t(c) * N + e]);
+        for (int c = 0; c < used; c += 8) {  // (eight loads in flight)
+            float q[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) q[k] = c + k < used ? d.b.opart[int64_t(c + k) * N + e] : 0.0f;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) s.add(q[k]);
+        }
         if constexpr (CG) {
             const double pe = p[e], val = s.value() + nu * pe;
             dot += pe * val;
