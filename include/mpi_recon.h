@@ -88,11 +88,22 @@ typedef struct {
 /* Forward operator A (Eq. core:formula):  s[k][t] = sum_ij c[j][i] p_k^T
  * beta K(beta G(x_ij - r_t)) G v_t.  c is [ny][nx], s is [n_ch][T].  FP64 and
  * small FP32 problems are summed pair by pair; large FP32 problems are
- * evaluated as convolutions on a grid with interpolation at the samples, to
- * the same accuracy (nothing is truncated: errors are FP32 rounding, about
- * 5e-8 in relative L2).  The route depends on sizes and model only.
- * Deterministic: the same inputs give bit-identical outputs.  T == 0 is a
- * no-op. */
+ * evaluated as convolutions on a grid with interpolation at the samples.
+ * There the kernel's spectrum is cut off at 6.5 rad per unit of |beta G r|
+ * (1e-8), its periodic closure costs 1.4e-9 and the interpolation 1e-9 to
+ * 4e-9, relative to the whole output; beside FP32 rounding this does not show:
+ * in relative L2 4e-8 for dense images, up to 2e-7 for single voxels and
+ * images of both signs (pair sums: 5e-8 and up to 5e-7).  Like any FP32 sum of
+ * terms of both signs, a single small s[k][t] is good to that share of the
+ * larger ones, not of itself.  The route depends on sizes and model, and takes
+ * the pair sums where the grid's scratch is not to be had.  Deterministic: the
+ * same inputs on the same route give bit-identical outputs.  T == 0 is a
+ * no-op.
+ *
+ * FP64 is computed in FP64 throughout; from |beta G r| = 14.5 on exp(-2 |beta G
+ * r|), below 3e-13 of the term, is taken from the FP32 exponential, which
+ * leaves at most 9e-17 (2e-16 in all against 64-bit-exact terms, as with an
+ * FP64 exponential). */
 int mpi_forward(const mpi_model *model, const mpi_grid_desc *grid,
                 const mpi_traj *traj, mpi_dtype dtype, const void *c, void *s,
                 void *stream);
@@ -306,14 +317,15 @@ typedef int (*mpi_allreduce_fn)(double *buf, int64_t count, void *stream, void *
  * across processes with `allreduce` (N = nx*ny values): once for A^T data and,
  * in each of the n_iter iterations, once for the initial residual and once per
  * CG step -- 1 + n_iter (n_cg + 1) calls on every process, whatever the length
- * of its slice and whether it evaluates its sums pair by pair or on a grid.  Every other step (CG vectors, inner products, trimming,
+ * of its slice and whether it evaluates its sums pair by pair or on a grid.
+ * Every other step (CG vectors, inner products, trimming,
  * noise estimate, denoiser) runs replicated on the identical reduced vectors,
  * so all processes finish with the same rho_out.  One process with an
  * allreduce that does nothing computes what mpi_pnp_solve computes, up to the
  * rounding order of the CG inner products.  opts->op must be MPI_OP_FORWARD;
  * allreduce must not be NULL.  A nonzero return of allreduce (or denoise) ends
  * the call with MPI_ERR_CALLBACK.  Allocates scratch like mpi_pnp_solve plus
- * one FP64 image. */
+ * one FP64 image (two on a grid). */
 int mpi_pnp_solve_sharded(const mpi_model *model, const mpi_grid_desc *grid,
                           const mpi_traj *traj, mpi_dtype dtype, const void *data,
                           const mpi_pnp_opts *opts, mpi_denoise_fn denoise, void *user,

@@ -2131,7 +2131,7 @@ int field_adjoint(const FieldPlan &plan, OUT *out, const double *cg_p, const dou
     const unsigned nb = (unsigned)field_dot_blocks(d.y.n);
     if constexpr (sizeof(OUT) == sizeof(double)) {
         if (cg_p) {
-                    launch_chained(k_field_out<double, true>, nb, 128, image_smem(d), st, d, out, cg_p, nu_dev, dot_part);
+            launch_chained(k_field_out<double, true>, nb, 128, image_smem(d), st, d, out, cg_p, nu_dev, dot_part);
             MPI_CHECK_LAUNCH();
             return MPI_OK;
         }

@@ -898,9 +898,10 @@ struct Resident2 {
 };
 
 // The 2-D Core Stage operator: (1/T) M^T M through the binned records and
-// the 5-point Laplacian of each component.  A step is two launches: the unit
-// sums of M^T M p (from the FP32 copy of p on the FP32 path) beside l1 = Lap p,
-// then q with gamma Lap l1 and the <p, q> partials.  The CG vectors are FP64
+// the 5-point Laplacian of each component.  A step forms q in two launches
+// (the two vector passes follow): the unit sums of M^T M p (from the FP32 copy
+// of p on the FP32 path) beside l1 = Lap p, then q with gamma Lap l1 and the
+// <p, q> partials.  The CG vectors are FP64
 // (FP64 path) or double-float pairs (FP32 path: E = float2).
 template <typename R>
 struct GridOp2 final : CoreStageOp<typename CsElem<R>::type> {

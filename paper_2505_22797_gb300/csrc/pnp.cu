@@ -1,7 +1,8 @@
 // ZeroShot-PnP deconvolution (Algorithm 1) on the GPU, with the forward
 // operator A or the trace-kernel convolution C as the data-fidelity operator:
 // CG vector kernels with deterministic FP64 inner products, the percentile
-// trimming and noise estimate (one single-block kernel), the built-in 5-tap
+// trimming and noise estimate (one block, from 4096 values a cluster of
+// eight), the built-in 5-tap
 // Gaussian denoiser, and the mpi_pnp_solve / mpi_conv /
 // mpi_denoise_gaussian5 entry points.  All PnP scalars (nu, lambda, sigma,
 // the CG alpha/beta) stay on the device, so a solve enqueues without any host
