@@ -1532,7 +1532,7 @@ __global__ void __launch_bounds__(kSpreadThreads, kSpreadPerSm) k_field_spread(c
 }
 
 // Half spectra of node rows 2b, 2b + 1: a node is the sum of the patches of
-// the up to four tiles that reach it, units in order, in pairs of floats (a
+// the up to four tiles that reach it, in a fixed order, in pairs of floats (a
 // tile where the trajectory dwells has thousands of units, whose plain FP32
 // sum would leave 1e-6).  Bound by the latency of those loads: the tiles' first
 // units, then four of a tile, are in flight at once (A^T at 128 x 128 / 65 536
@@ -1948,9 +1948,11 @@ void lay_out(FieldPlan &plan, char *keep, char *work, size_t &keep_bytes, size_t
         take(1, b.CR, ny * (d.x.Q / 2 + 1));
         take(1, b.CL, ny * kFieldLow);
         take(1, b.FL, size_t(3) * d.y.w * kFieldLow);
-        take(1, b.FN, size_t(d.y.w) * d.x.w);
+        // (the outside samples' partial sums are done before the nodes are formed)
+        const size_t n_part = size_t(d.n_ch) * kOutRounds * d.out_blocks * d.out_samples;
+        take(1, b.FN, std::max(size_t(d.y.w) * d.x.w, (n_part + 3) / 4));
+        b.fpart = reinterpret_cast<float *>(b.FN);
         take(0, b.ocount, out_counters(d));
-        take(1, b.fpart, size_t(d.n_ch) * kOutRounds * d.out_blocks * d.out_samples);
         if (!plan.adjoint) take(1, b.olist, T1);
     }
     if (plan.adjoint) {

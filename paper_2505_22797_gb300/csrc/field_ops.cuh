@@ -47,7 +47,7 @@ struct FieldBuf {
     float *opart;    // outside samples' partial images
     int *ocount;     // outside samples (unordered), and per group of them the runs of rows done
     int *olist;      // the outside samples (unordered)
-    float *fpart;    // their partial sums by runs of rows
+    float *fpart;    // their partial sums by runs of rows (in FN's memory)
     float2 *AC;      // [3][ny][Jx + 1]
     float4 *AL;      // [3][ny][kFieldLow]
 };
