@@ -1412,14 +1412,15 @@ __device__ __forceinline__ void outside_image(const FieldDev &d, int tile, int c
         if (jb + k < ny) out[int64_t(jb + k) * nx + i] = acc[k];
 }
 
-// One spreading unit u, by one block: the patch of the unit's tile, summed over its samples in order.  A warp owns one entry of K on the
-// patch rows of one parity: a sample's stencil has four such rows of eight
-// points, one per lane, so no two lanes share a node and the order of the
-// additions is the samples' order.  The unit's two halves go to two copies of
-// the patch, added at the end: twice the independent chains of load, FMA and
-// store.  What bounds it is the shared-memory pipe: per sample and warp one load and one store of the patch, and a
-// quarter of three 16-byte loads (weights and addresses of four samples,
-// fetched one step ahead).
+// One spreading unit u, by one block: the patch of the unit's tile, summed over
+// its samples in order.  A warp owns one entry of K on the patch rows of one
+// parity: a sample's stencil has four such rows of eight points, one per lane,
+// so no two lanes share a node and the order of the additions is the samples'
+// order.  The unit's two halves go to two copies of the patch, added at the
+// end: twice the independent chains of load, FMA and store.  What bounds it is
+// the shared-memory pipe: per sample and warp one load and one store of the
+// patch, and a quarter of three 16-byte loads (weights and addresses of four
+// samples, fetched one step ahead).
 constexpr int kUnitPitch = kFieldUnit + 4;
 __device__ __forceinline__ void spread_unit(const FieldDev &d, int u, float (*s_patch)[3][kPatch * kPatchPitch])
 {
